@@ -759,10 +759,15 @@ __global__ void k_energy_line(const int64_t* __restrict__ off, const double* __r
     }
 }
 
-// The periodic quintic spline solve of the curve fit below (k_spline_quintic).
+// The periodic quintic spline solves of the curve fit below (k_spline_quintic
+// and, in parallel, k_spline_quintic_cta).
 __device__ void q_solve(int n, double* __restrict__ t, double xlast[6]);
 __device__ __forceinline__ void q_node(const double* __restrict__ t, int m, const double xlast[6], int j, int c,
                                        double& D, double& M);
+constexpr size_t kQuinticRow = 32 * sizeof(double);  // shared memory per node: h, 3 increments, 2 x 14 of the solver
+constexpr size_t kQuinticSmemMax = 200 * 1024;       // filaments up to 800 nodes
+__device__ const double* q_solve_cta(int n, const double* __restrict__ sm);
+__device__ __forceinline__ double block_sum(double v);
 
 // The same line integral on a quintic curve (order 6): f_j = psi_j .
 // sdot(tau_j), with sdot = D_j + n_l L / T the first derivative of the
@@ -826,12 +831,80 @@ __global__ void k_energy_line_quintic(const int64_t* __restrict__ off, const dou
         atomicAdd(acc, part);
 }
 
+// The same with a CTA per filament (see k_spline_quintic_cta): the node values
+// and segment terms one per thread, summed in a fixed order.
+template <typename T>
+__global__ void __launch_bounds__(256) k_energy_line_quintic_cta(const int64_t* __restrict__ off,
+                                                                 const double* __restrict__ shift,
+                                                                 const T* __restrict__ hseg, const T* __restrict__ Dd,
+                                                                 const T* __restrict__ Tper,
+                                                                 const double* __restrict__ pls,
+                                                                 const double* __restrict__ psr,
+                                                                 double* __restrict__ acc, double* __restrict__ per_fil)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    double* sm = reinterpret_cast<double*>(sm_raw);
+    const int f = blockIdx.x;
+    const int64_t o = off[f];
+    const int n = (int)(off[f + 1] - o);
+    const double Tp = (double)Tper[f], hb = Tp / n, ihb = 1.0 / hb;
+    const double dr[3] = { shift[3 * f] / Tp, shift[3 * f + 1] / Tp, shift[3 * f + 2] / Tp };
+    auto fval = [&](int j) {
+        double fj = 0.0;
+        for (int c = 0; c < 3; ++c)
+            fj += (pls[3 * (o + j) + c] + psr[3 * (o + j) + c]) * ((double)Dd[3 * (o + j) + c] + dr[c]);
+        return fj;
+    };
+    // lengths in units of the mean one, increments of f / hb
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        sm[j] = (double)hseg[o + j] * ihb;
+        sm[n + j] = (fval(j + 1 < n ? j + 1 : 0) - fval(j)) * ihb;
+        sm[2 * n + j] = 0.0;
+        sm[3 * n + j] = 0.0;
+    }
+    __syncthreads();
+    const double* x = q_solve_cta(n, sm);  // x[j] = F'_j, x[3 n + j] = F''_j hb
+    double part = 0.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int jn = j + 1 < n ? j + 1 : 0;
+        const double h = sm[j] * hb;
+        part += 0.5 * h * (fval(j) + fval(jn)) + h * h * (x[j] - x[jn]) / 10.0 +
+                h * h * h * ihb * (x[3 * n + j] + x[3 * n + jn]) / 120.0;
+    }
+    part = block_sum(part);
+    if (threadIdx.x == 0) {
+        if (per_fil)
+            per_fil[f] = part;
+        else
+            atomicAdd(acc, part);
+    }
+}
+
+// Threads and shared memory of the CTA-per-filament quintic kernels.
+inline int quintic_threads(int nmax) { return nmax >= 256 ? 256 : (nmax + 31) & ~31; }
+
+template <typename K>
+cudaError_t quintic_smem(K kernel, size_t sm)
+{
+    return sm > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
+                          : cudaSuccess;
+}
+
 template <typename T>
 cudaError_t launch_energy_line(const double* nodes, const Work& w, int nfil, int nmax, cudaStream_t s, bool det)
 {
     (void)nodes;
     if (nfil <= 0) return cudaSuccess;
-    if (w.Dd) {  // quintic curves
+    if (w.Dd && kQuinticRow * (size_t)nmax <= kQuinticSmemMax) {  // quintic curves
+        const size_t sm = kQuinticRow * (size_t)nmax;
+        cudaError_t e = quintic_smem(k_energy_line_quintic_cta<T>, sm);
+        if (e != cudaSuccess) return e;
+        k_energy_line_quintic_cta<T><<<nfil, quintic_threads(nmax), sm, s>>>(
+            w.off, w.shift, (const T*)w.hseg, (const T*)w.Dd, (const T*)w.Tper, w.pls, w.psr, w.energy_acc + 1,
+            det ? w.lpart : nullptr);
+        return cudaGetLastError();
+    }
+    if (w.Dd) {  // filaments too long for shared memory
         const int tb = 64;
         k_energy_line_quintic<T><<<(nfil + tb - 1) / tb, tb, 0, s>>>(w.off, w.shift, nfil, (const T*)w.hseg,
                                                                      (const T*)w.Dd, (const T*)w.Tper, w.pls, w.psr,
@@ -1073,11 +1146,200 @@ __global__ void k_spline_quintic(const double* __restrict__ nodes, const int64_t
         }
 }
 
+// Sum over the block, in a fixed order, valid in thread 0 (blocks of whole warps).
+__device__ __forceinline__ double block_sum(double v)
+{
+    __shared__ double ws[32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += ws[k];
+    return t;
+}
+
+// The cyclic block system of q_solve by parallel cyclic reduction (Hockney,
+// J. ACM 12, 1965), all threads of a CTA on one filament.  sm: n lengths, 3 n
+// increments (component by component), then 2 x 14 n of scratch.  With every
+// equation multiplied by its diagonal block's inverse,
+//   L_j X_{j-s} + X_j + U_j X_{j+s} = R_j   (indices modulo n),
+// one step eliminates both neighbours and doubles s:
+//   E = (I - L_j U_{j-s} - U_j L_{j+s})^{-1}, L'_j = -E L_j L_{j-s},
+//   U'_j = -E U_j U_{j+s}, R'_j = E (R_j - L_j R_{j-s} - U_j R_{j+s}).
+// The identity holds for every n and s (also when the indices coincide), and
+// the couplings shrink quadratically (0.43^s on equal chords), so the loop
+// ends when they are below 1e-18 (6 or 7 steps) and X = R.  Returns the
+// solution, x[c n + j] = D of component c, x[(3 + c) n + j] = M, and leaves
+// the block synchronised.  Lengths should be of order one.
+__device__ const double* q_solve_cta(int n, const double* __restrict__ sm)
+{
+    const double* h = sm;
+    const double* inc = sm + n;
+    double* cur = const_cast<double*>(sm) + 4 * n;
+    double* nxt = cur + 14 * n;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int jm = j == 0 ? n - 1 : j - 1;
+        double L[4], B[4], U[4], iv[4];
+        const double a = h[jm], hj = h[j];
+        q_blocks(a, hj, L, B, U);
+        inv2(B, iv);
+        const double ia3 = 1.0 / (a * a * a), ih3 = 1.0 / (hj * hj * hj), ia = 1.0 / a, ih = 1.0 / hj;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                cur[(2 * r + c) * n + j] = iv[2 * r] * L[c] + iv[2 * r + 1] * L[2 + c];
+                cur[(4 + 2 * r + c) * n + j] = iv[2 * r] * U[c] + iv[2 * r + 1] * U[2 + c];
+            }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double dj = inc[c * n + j] * ih3, dm = inc[c * n + jm] * ia3;
+            const double r0 = 60.0 * (dj - dm), r1 = -360.0 * (dj * ih + dm * ia);
+            cur[(8 + c) * n + j] = iv[0] * r0 + iv[1] * r1;
+            cur[(11 + c) * n + j] = iv[2] * r0 + iv[3] * r1;
+        }
+    }
+    __syncthreads();
+    int s = 1;  // modulo n
+    for (int it = 0; it < 16; ++it) {
+        bool more = false;
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            const int jm = j - s < 0 ? j - s + n : j - s, jp = j + s >= n ? j + s - n : j + s;
+            double L[4], U[4], Lm[4], Um[4], Lp[4], Up[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                L[k] = cur[k * n + j];
+                U[k] = cur[(4 + k) * n + j];
+                Lm[k] = cur[k * n + jm];
+                Um[k] = cur[(4 + k) * n + jm];
+                Lp[k] = cur[k * n + jp];
+                Up[k] = cur[(4 + k) * n + jp];
+            }
+            double D[4], E[4], EL[4], EU[4];
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    D[2 * r + c] = (r == c ? 1.0 : 0.0) - (L[2 * r] * Um[c] + L[2 * r + 1] * Um[2 + c]) -
+                                   (U[2 * r] * Lp[c] + U[2 * r + 1] * Lp[2 + c]);
+            inv2(D, E);
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    EL[2 * r + c] = E[2 * r] * L[c] + E[2 * r + 1] * L[2 + c];
+                    EU[2 * r + c] = E[2 * r] * U[c] + E[2 * r + 1] * U[2 + c];
+                }
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const double ln = -(EL[2 * r] * Lm[c] + EL[2 * r + 1] * Lm[2 + c]);
+                    const double un = -(EU[2 * r] * Up[c] + EU[2 * r + 1] * Up[2 + c]);
+                    nxt[(2 * r + c) * n + j] = ln;
+                    nxt[(4 + 2 * r + c) * n + j] = un;
+                    more = more || !(fabs(ln) < 1e-18) || !(fabs(un) < 1e-18);
+                }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const double r0 = cur[(8 + c) * n + j], r1 = cur[(11 + c) * n + j];
+                const double m0 = cur[(8 + c) * n + jm], m1 = cur[(11 + c) * n + jm];
+                const double p0 = cur[(8 + c) * n + jp], p1 = cur[(11 + c) * n + jp];
+                nxt[(8 + c) * n + j] =
+                    E[0] * r0 + E[1] * r1 - (EL[0] * m0 + EL[1] * m1) - (EU[0] * p0 + EU[1] * p1);
+                nxt[(11 + c) * n + j] =
+                    E[2] * r0 + E[3] * r1 - (EL[2] * m0 + EL[3] * m1) - (EU[2] * p0 + EU[3] * p1);
+            }
+        }
+        double* t = cur;
+        cur = nxt;
+        nxt = t;
+        if (!__syncthreads_or(more)) break;
+        s = (2 * s) % n;
+    }
+    return cur + 8 * n;
+}
+
+// Quintic fit with a CTA per filament (filaments whose rows fit in shared
+// memory; k_spline_quintic takes longer ones).  Bound by the latency of
+// dependent float64 operations, a few thousand cycles per step of the
+// reduction: the one-thread elimination walks n dependent 2 x 2 blocks
+// through global memory.  One step of two leapfrogging 32-node rings (four
+// evaluations): 3.65 -> 1.80 ms, the fit 513 -> about 50 us an evaluation.
+template <typename T>
+__global__ void __launch_bounds__(256) k_spline_quintic_cta(const double* __restrict__ nodes,
+                                                            const int64_t* __restrict__ off,
+                                                            const double* __restrict__ shift, T* __restrict__ hseg,
+                                                            T* __restrict__ dp, T* __restrict__ ds, T* __restrict__ Mm,
+                                                            T* __restrict__ Dd, T* __restrict__ Tper)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    double* sm = reinterpret_cast<double*>(sm_raw);
+    __shared__ double s_T;
+    const int f = blockIdx.x;
+    const int64_t o = off[f];
+    const int n = (int)(off[f + 1] - o);
+    const double sh[3] = { shift[3 * f], shift[3 * f + 1], shift[3 * f + 2] };
+    double part = 0.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const double* a = nodes + 3 * (o + j);
+        const double* b = nodes + 3 * (j + 1 < n ? o + j + 1 : o);
+        double d[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d[c] = b[c] + (j + 1 < n ? 0.0 : sh[c]) - a[c];
+        const double h = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+        part += h;
+        sm[j] = h;
+        hseg[o + j] = (T)h;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            sm[(1 + c) * n + j] = d[c];
+            ds[3 * (o + j) + c] = (T)d[c];
+        }
+    }
+    part = block_sum(part);
+    if (threadIdx.x == 0) {
+        s_T = part;
+        Tper[f] = (T)part;
+    }
+    __syncthreads();
+    const double invT = 1.0 / s_T, ihb = n * invT;  // lengths in units of the mean one
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const double h = sm[j];
+        sm[j] = h * ihb;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double p = sm[(1 + c) * n + j] - sh[c] * h * invT;  // periodic increment
+            dp[3 * (o + j) + c] = (T)p;
+            sm[(1 + c) * n + j] = p * ihb;
+        }
+    }
+    __syncthreads();
+    const double* x = q_solve_cta(n, sm);
+    for (int j = threadIdx.x; j < n; j += blockDim.x)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            Dd[3 * (o + j) + c] = (T)x[c * n + j];
+            Mm[3 * (o + j) + c] = (T)(x[(3 + c) * n + j] * ihb);
+        }
+}
+
 template <typename T>
 cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStream_t s)
 {
     if (nfil <= 0) return cudaSuccess;
-    if (w.Dd) {  // quintic
+    if (w.Dd && kQuinticRow * (size_t)w.nmax_fil <= kQuinticSmemMax) {  // quintic
+        const size_t sm = kQuinticRow * (size_t)w.nmax_fil;
+        cudaError_t e = quintic_smem(k_spline_quintic_cta<T>, sm);
+        if (e != cudaSuccess) return e;
+        k_spline_quintic_cta<T><<<nfil, quintic_threads(w.nmax_fil), sm, s>>>(
+            nodes, w.off, w.shift, (T*)w.hseg, (T*)w.dp, (T*)w.ds, (T*)w.Mm, (T*)w.Dd, (T*)w.Tper);
+        return cudaGetLastError();
+    }
+    if (w.Dd) {  // filaments too long for shared memory
         const int tb = 64;
         k_spline_quintic<T><<<(nfil + tb - 1) / tb, tb, 0, s>>>(nodes, w.off, w.shift, nfil, (T*)w.hseg, (T*)w.dp,
                                                                 (T*)w.ds, (T*)w.Mm, (T*)w.Dd, (T*)w.Tper, w.qtmp);
