@@ -1164,6 +1164,7 @@ int bs_create(bs_ctx** out, const bs_params* p, void* stream)
     }
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = set_fft_constants();
+    if (e == cudaSuccess) e = set_short_tables();
     // the short-range branch runs at the highest stream priority: its few
     // CTAs are dispatched ahead of the long-range kernels' waiting ones, so
     // the branch ends while the spread is still running

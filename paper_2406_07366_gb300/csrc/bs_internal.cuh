@@ -393,6 +393,7 @@ cudaError_t launch_spread_zfft(const SpZP& P, const Work& w, cudaStream_t s);
 template <typename T>
 size_t col_pt_bytes(int w);
 cudaError_t set_fft_constants();
+cudaError_t set_short_tables();
 template <typename T>
 cudaError_t launch_fft_y(const FftYP& P, const Work& w, void* f2, int sign, cudaStream_t s,
                          const CUtensorMap* tm_f1 = nullptr);

@@ -20,6 +20,8 @@
 // k_short (larger m): one warp per node walks the (2m+1)^2 neighbour rows.
 #include <math.h>
 
+#include <mutex>
+
 #include "bs_internal.cuh"
 
 namespace bsw {
@@ -82,6 +84,60 @@ __device__ __forceinline__ float erfc_e<float>(float x, float e) { return e * er
 template <>
 __device__ __forceinline__ double erfc_e<double>(double x, double) { return erfc(x); }
 
+// The float64 pair term without library calls.  float64 runs at 1/64 of the
+// float32 rate here, and 1/sqrt, exp and erfc cost it about 130 operations
+// per pair (6.1 ms on the 1e5-node tangle, float64 pipe saturated).  Instead:
+//   1/r from the hardware's approximate reciprocal square root and one step
+//   of Householder's third-order iteration (y += y e (1/2 + 3 e / 8), e = 1 -
+//   r2 y^2; the seed's 2^-20 becomes below 2^-58), 5 operations;
+//   g^(n)(x) and erfc(x) from tables of degree-8 polynomials on intervals of
+//   width 1/16 centred at i / 16, i = 0..128, written once per device from
+//   Chebyshev interpolation of the functions in extended precision
+//   (set_short_tables): 8 operations each, interpolation error below 2^-60
+//   of the largest value on the interval.
+// Beyond x = 8 the library functions are called.
+constexpr int kSgN = 129, kSgDeg = 8, kSgStride = 132;
+constexpr int kSgTable = (kSgDeg + 1) * kSgStride;  // doubles per function, degree-major
+__device__ double g_sg_tab[2 * kSgTable];           // g^(n), then erfc
+
+__device__ __forceinline__ double rsqrt_h(double a)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// Value at the table argument: t in [-1/2, 1/2], interval i.
+__device__ __forceinline__ double sg_poly(const double* __restrict__ tab, int i, double t)
+{
+    double v = tab[kSgDeg * kSgStride + i];
+#pragma unroll
+    for (int k = kSgDeg - 1; k >= 0; --k) v = fma(v, t, tab[k * kSgStride + i]);
+    return v;
+}
+
+// double of a small integer without a conversion instruction (exact)
+__device__ __forceinline__ double i2d(int k)
+{
+    return __hiloint2double(0x43300000, k ^ 0x80000000) - 4503601774854144.0;  // 2^52 + 2^31
+}
+
+// Copies the tables into shared memory (float64; the whole block).
+template <typename T>
+__device__ __forceinline__ const double* sg_stage(int want_psi)
+{
+    if constexpr (sizeof(T) == 8) {
+        __shared__ double s_tab[2 * kSgTable];
+        const int n = want_psi ? 2 * kSgTable : kSgTable;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) s_tab[i] = g_sg_tab[i];
+        __syncthreads();
+        return s_tab;
+    } else {
+        return nullptr;
+    }
+}
+
 // Adds the pair term of source (position rel, charge q) seen from the node at
 // distance vector r (source - node), |r| = sqrt(r2).
 template <typename T>
@@ -122,7 +178,7 @@ template <typename T>
 __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __restrict__ tgt,
                                              const int* __restrict__ prev, const int* __restrict__ start,
                                              const SrRec<T>* __restrict__ src, double* __restrict__ vsr,
-                                             double* __restrict__ psr, int bid)
+                                             double* __restrict__ psr, int bid, const double* __restrict__ tab)
 {
     const int lane = threadIdx.x & 31;
     const int wslot = threadIdx.x >> 5;  // the warp's slot in the CTA's row tables
@@ -143,6 +199,7 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
     const T L0 = (T)P.L[0], L1 = (T)P.L[1], L2 = (T)P.L[2];
     const T rc2 = (T)P.rc2;
     const T alpha = (T)P.alpha;
+    const double alpha16 = 16.0 * P.alpha;  // float64: the tables' argument
     const T two_over_sqrtpi = (T)1.12837916709551257390;
     const int m = P.m;
     // neighbour ranges per axis: all cells when 2m+1 >= n
@@ -254,7 +311,11 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
             T rx, ry, rz;
             if (!wrap) {
                 const int4 of = s_ofs[wslot][own];
-                rx = (T)(S.cx + (first ? of.x : of.y)) * h0 + (S.o[0] - t.o[0]);
+                const int dcx = S.cx + (first ? of.x : of.y);
+                if constexpr (sizeof(T) == 8)
+                    rx = fma(i2d(dcx), (double)h0, (double)(S.o[0] - t.o[0]));
+                else
+                    rx = (T)dcx * h0 + (S.o[0] - t.o[0]);
                 ry = s_dh[wslot][own][0] + (S.o[1] - t.o[1]);
                 rz = s_dh[wslot][own][1] + (S.o[2] - t.o[2]);
             } else {
@@ -269,12 +330,29 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
             }
             const T r2 = rx * rx + ry * ry + rz * rz;
             if (r2 >= rc2 || r2 == (T)0) continue;
-            const T ir = rsqrt_t(r2);
-            const T rr = r2 * ir;
-            const T x = alpha * rr;
-            const T e = exp_t(-x * x);
-            const T ec = erfc_e(x, e);
-            const T g = ec + two_over_sqrtpi * x * e;
+            T ir, g, ec = (T)0;
+            if constexpr (sizeof(T) == 8) {
+                ir = rsqrt_h(r2);
+                const double xs = alpha16 * (r2 * ir);  // 16 x
+                if (xs < 128.0) {
+                    const double mi = xs + 4503599627370496.0;  // 2^52: the low word is rint(xs)
+                    const double tt = xs - (mi - 4503599627370496.0);
+                    const int it = __double2loint(mi);
+                    g = sg_poly(tab, it, tt);
+                    if (P.want_psi) ec = sg_poly(tab + kSgTable, it, tt);
+                } else {
+                    const double x = 0.0625 * xs;
+                    ec = erfc(x);
+                    g = ec + two_over_sqrtpi * x * exp(-x * x);
+                }
+            } else {
+                ir = rsqrt_t(r2);
+                const T rr = r2 * ir;
+                const T x = alpha * rr;
+                const T e = exp_t(-x * x);
+                ec = erfc_e(x, e);
+                g = ec + two_over_sqrtpi * x * e;
+            }
             const T fv = g * ir * ir * ir;
             v0 += fv * (ry * S.q[2] - rz * S.q[1]);
             v1 += fv * (rz * S.q[0] - rx * S.q[2]);
@@ -319,7 +397,13 @@ __global__ void __launch_bounds__(256) k_short(ShortP P, const SrTgt<T>* __restr
                                                const int* __restrict__ start, const SrRec<T>* __restrict__ src,
                                                double* __restrict__ vsr, double* __restrict__ psr)
 {
-    k_short_body<T>(P, tgt, prev, start, src, vsr, psr, blockIdx.x);
+    const double* tab = sg_stage<T>(P.want_psi);
+    if constexpr (sizeof(T) == 8) {  // several groups of nodes per CTA: the tables are staged once
+        for (int b = blockIdx.x; b * kShortWarps < P.N; b += gridDim.x)
+            k_short_body<T>(P, tgt, prev, start, src, vsr, psr, b, tab);
+    } else {
+        k_short_body<T>(P, tgt, prev, start, src, vsr, psr, blockIdx.x, tab);
+    }
 }
 
 template <typename T>
@@ -327,7 +411,8 @@ __global__ void __launch_bounds__(256) k_short_b(const ShortD<T>* __restrict__ d
 {
     int bid, nb;
     const ShortD<T>& a = d[batch_member(bs, n, bid, nb)];
-    k_short_body<T>(a.P, a.tgt, a.prev, a.start, a.src, a.vsr, a.psr, bid);
+    const double* tab = sg_stage<T>(a.P.want_psi);
+    k_short_body<T>(a.P, a.tgt, a.prev, a.start, a.src, a.vsr, a.psr, bid, tab);
 }
 
 // ---------------------------------------------------------------------------
@@ -687,8 +772,10 @@ cudaError_t launch_short(const ShortP& P, const Work& w, cudaStream_t s)
     const bool tiled = P.m <= kShortTileMaxM && P.kernel == 1;
     if (!tiled) {
         const int tb = 32 * kShortWarps;  // one warp per target
-        const long long threads = 32LL * P.N;
-        k_short<T><<<(unsigned)((threads + tb - 1) / tb), tb, 0, s>>>(
+        const long long blocks = (P.N + kShortWarps - 1LL) / kShortWarps;
+        // float64: at most 16 CTAs per SM, each on several groups of nodes
+        const unsigned g = (unsigned)(sizeof(T) == 8 && blocks > 16 * 152 ? 16 * 152 : blocks);
+        k_short<T><<<g, tb, 0, s>>>(
             P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt, (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
         return cudaGetLastError();
     }
@@ -719,6 +806,52 @@ template cudaError_t launch_short_b<float>(const BatchL&, cudaStream_t);
 template cudaError_t launch_short_b<double>(const BatchL&, cudaStream_t);
 template cudaError_t launch_short<float>(const ShortP&, const Work&, cudaStream_t);
 template cudaError_t launch_short<double>(const ShortP&, const Work&, cudaStream_t);
+
+static long double sg_erfc(long double x) { return erfcl(x); }
+static long double sg_near(long double x)
+{
+    return erfcl(x) + 1.12837916709551257389615890312154517L * x * expl(-x * x);
+}
+
+// Degree-d monomial coefficients in t of the polynomial through f at the
+// Chebyshev points of x = (i + t) / 16, t in [-1/2, 1/2] (divided differences,
+// extended precision).
+static void sg_fit(long double (*f)(long double), int i, double* out, int stride)
+{
+    constexpr int n = kSgDeg + 1;
+    long double t[n], c[n], p[n] = {};
+    for (int k = 0; k < n; ++k) {
+        t[k] = 0.5L * cosl(3.14159265358979323846264338327950288L * (k + 0.5L) / n);
+        c[k] = f((i + t[k]) / 16.0L);
+    }
+    for (int j = 1; j < n; ++j)
+        for (int k = n - 1; k >= j; --k) c[k] = (c[k] - c[k - 1]) / (t[k] - t[k - j]);
+    for (int k = n - 1; k >= 0; --k) {  // p <- p (t - t_k) + c_k
+        for (int j = n - 1; j > 0; --j) p[j] = p[j - 1] - t[k] * p[j];
+        p[0] = c[k] - t[k] * p[0];
+    }
+    for (int j = 0; j < n; ++j) out[j * stride] = (double)p[j];
+}
+
+// The float64 pair term's tables, once per device.
+cudaError_t set_short_tables()
+{
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
+    static double tab[2 * kSgTable];
+    for (int i = 0; i < kSgN; ++i) {
+        sg_fit(sg_near, i, tab + i, kSgStride);
+        sg_fit(sg_erfc, i, tab + kSgTable + i, kSgStride);
+    }
+    e = cudaMemcpyToSymbol(g_sg_tab, tab, sizeof tab);
+    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+    return e;
+}
 
 // The float32 complementary error function as the short-range kernels take
 // it (erfc_e with e = expf(-x^2)), one thread per argument.

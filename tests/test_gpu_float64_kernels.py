@@ -43,3 +43,22 @@ def test_quintic_fit_at_the_edges_of_its_size_rule(n):
     d -= f.L * np.round(d / f.L)
     assert np.abs(d).max() < 1e-12 * f.L.max()
     assert np.abs(qq.cpu().numpy() - g.qq).max() < 1e-11 * np.abs(g.qq).max()
+
+
+@pytest.mark.parametrize("beta", [0.3, 3.5, 7.99, 8.01, 12.0])
+def test_float64_short_range_over_the_table_and_beyond(beta):
+    """The pair functions come from tables up to alpha r = 8 and from the
+    library beyond; every r up to the cut-off against the oracle's brute
+    force, 1e-12 relative to the largest velocity (the tolerance of the
+    float64 parity tests)."""
+    B, f = _B(), W.ellipses(6, 48, seed=3)
+    rc = 2.0
+    p = B.make_params(f.L, M=32, Q=2, w=8, precision=B.BS_FP64, alpha=beta / rc, rc=rc, flags=B.BS_WANT_PSI)
+    bs = B.BiotSavart(p, f.offsets, f.closing)
+    parts, psi = bs.parts(torch.from_numpy(f.nodes).cuda(), want_psi=True)
+    torch.cuda.synchronize()
+    bs.close()
+    g = oracle.geometry(f.nodes, f.offsets, f.closing, f.L, 4, 2)
+    v, ps = oracle.short_range(g, f.L, 1.0, p.alpha, p.rc)
+    assert np.abs(parts[1].cpu().numpy() - v).max() < 1e-12 * np.abs(v).max()
+    assert np.abs(psi[1].cpu().numpy() - ps).max() < 1e-12 * np.abs(ps).max()
