@@ -230,6 +230,14 @@ __device__ __forceinline__ void dft(typename Cx<T>::t* x)
         C t;
         t.x = x[0].x - (T)0.5 * s.x;
         t.y = x[0].y - (T)0.5 * s.y;
+        if constexpr (sizeof(T) == 8) {  // t +- i h d in fused form
+            x[0] = cadd(x[0], s);
+            x[1].x = fma(-h, d.y, t.x);
+            x[1].y = fma(h, d.x, t.y);
+            x[2].x = fma(h, d.y, t.x);
+            x[2].y = fma(-h, d.x, t.y);
+            return;
+        }
         C u;  // i h d
         u.x = -h * d.y;
         u.y = h * d.x;
@@ -249,6 +257,26 @@ __device__ __forceinline__ void dft(typename Cx<T>::t* x)
         dft<T, 4, S>(e);
         dft<T, 4, S>(o);
         const T r2 = (T)0.70710678118654752440;
+        if constexpr (sizeof(T) == 8) {
+            // e +- w8^m o with the factor sqrt(1/2) fused into the sums
+            const T sg = (T)sign;
+            const T p1 = fma(-sg, o[1].y, o[1].x), q1 = fma(sg, o[1].x, o[1].y);
+            const T p3 = -fma(sg, o[3].y, o[3].x), q3 = fma(sg, o[3].x, -o[3].y);
+            o[2] = cmuli(o[2], sign);
+            x[0] = cadd(e[0], o[0]);
+            x[4] = csub(e[0], o[0]);
+            x[1].x = fma(r2, p1, e[1].x);
+            x[1].y = fma(r2, q1, e[1].y);
+            x[5].x = fma(-r2, p1, e[1].x);
+            x[5].y = fma(-r2, q1, e[1].y);
+            x[2] = cadd(e[2], o[2]);
+            x[6] = csub(e[2], o[2]);
+            x[3].x = fma(r2, p3, e[3].x);
+            x[3].y = fma(r2, q3, e[3].y);
+            x[7].x = fma(-r2, p3, e[3].x);
+            x[7].y = fma(-r2, q3, e[3].y);
+            return;
+        }
         // w8^m = e^{sign 2 pi i m / 8}
         C w1;
         w1.x = r2;
@@ -323,6 +351,18 @@ template <typename T, int R, int S>
 __device__ __forceinline__ void apply_twiddles(typename Cx<T>::t* x, const typename Cx<T>::t* __restrict__ tw, int m)
 {
     using C = typename Cx<T>::t;
+    if constexpr (sizeof(T) == 8) {
+        // float64 (1/64 of the float32 rate): every power from the table, a
+        // broadcast read; the products that make the powers were a fifth of
+        // the transform's operations (y pass on 384^3: 3.47 -> 2.96 ms)
+#pragma unroll
+        for (int q = 1; q < R; ++q) {
+            C wq = tw[q * m];
+            if constexpr (S > 0) wq.y = -wq.y;
+            x[q] = cmul(x[q], wq);
+        }
+        return;
+    }
     C w[R];
     w[1] = tw[m];
     if constexpr (S > 0) w[1].y = -w[1].y;
@@ -1083,6 +1123,23 @@ __device__ __forceinline__ void k_spread_zfft_body(const SpZP& P, const int* __r
     constexpr int RC = spz_rec_chunk<T>();
     const int s0 = cstart[bid * P.nzb], s1 = cstart[(bid + 1) * P.nzb];
     const int nslot = Ty * W;
+    if (s0 == s1) {
+        // no point reaches the block: its modes are zero, no transform (a few
+        // curves in a box leave most columns empty; with the interpolation's
+        // early return a batch of 256 tangles of 250-650 nodes takes 2.67 ms
+        // in place of 3.02)
+        const int nk = P.K[2] + 1;
+        C zero;
+        zero.x = 0;
+        zero.y = 0;
+        for (int i = tid; i < nreal * nk; i += blockDim.x) {
+            const int rl = i / nk, k = i - rl * nk;
+            const int c = fdiv(rl, P.d_txy), rem = rl - c * txy;
+            const int lx = fdiv(rem, P.d_ty), ly = rem - lx * Ty;
+            F1[(((size_t)c * P.ng[0] + bx * Tx + lx) * P.ng[1] + by * Ty + ly) * nk + k] = zero;
+        }
+        return;
+    }
     if (P.nzb > 1) {
         __syncthreads();  // the lines are zeroed
         switch (Tx) {
@@ -1808,6 +1865,8 @@ __device__ __forceinline__ void k_zfft_interp_body(const SpZP& P, const int* __r
     // the home ranges are fetched while the buffer is cleared
     int rb0, rlen;
     const int nr = home_fetch(P, cstart, bx, by, H, rb0, rlen);
+    // no node near the block (rlen is 0 past the ranges): nothing to transform
+    if (!__syncthreads_or(rlen > 0)) return;
     zero_cx(cb, ncl * CS);
     if (tid < kHomeMax) {
         r_beg[tid] = rb0;
