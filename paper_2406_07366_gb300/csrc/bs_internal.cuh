@@ -204,7 +204,12 @@ struct ColP {
     int n2;   // grid points along z
     double zeta;   // kernel shape parameter
     double inorm;  // 1 / (1 - e^{-2 zeta}), the kernel's normalisation
+    const double* kbc;  // float64: the kernel's polynomials (kb_weights)
 };
+
+// Degree of the float64 kernel's polynomials on one grid spacing, and their
+// coefficients per pair of support points.
+constexpr int kKbDeg = 22;
 
 struct SpZP {
     int det;  // deterministic accumulation: each warp owns a z-range and adds in record order
@@ -279,11 +284,13 @@ struct InterpP {
     int w;
     double zeta, inorm;
     int want_psi;
+    const double* kbc;  // as in ColP
 };
 
 // Workspace buffers (device) of one context; T-typed buffers are void*.
 struct Work {
     // topology
+    double* kbc = nullptr;  // the float64 kernel's polynomials (w / 2 x (kKbDeg + 1))
     int64_t* off = nullptr;
     int* fil_of = nullptr;
     int* prev = nullptr;
