@@ -318,6 +318,16 @@ int derive(const bs_params* p, Derived* d)
         txy *= 2;
         d->zthreads = 512;
     }
+    if (rb == 8) {
+        // float64: the largest block of at most 8 columns that leaves room for
+        // two CTAs per SM.  Measured on the 384^3 grid of the 1e5-node tangle:
+        // 2 x 4 against 1 x 4 columns take the spread from 8.5 to 7.2 ms and
+        // the interpolation from 6.2 to 5.1; on the 96^3 grid of 40 ellipses
+        // 2 x 4 against 4 x 4, 225 to 213 us and 139 to 115 us.
+        const size_t rec = 128 * (32 + 24 * (size_t)p->nufft_w);
+        for (txy = 8; txy > 2 && 24 * (size_t)txy * (size_t)(d->ng[2] + 33) + rec > 112 * 1024; txy /= 2) {
+        }
+    }
     d->ty = std::min(4, txy);
     d->tx = txy / d->ty;
     if (p->block_x > 0 || p->block_y > 0 || p->block_threads > 0) {

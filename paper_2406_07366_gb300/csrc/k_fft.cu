@@ -398,8 +398,10 @@ __device__ __forceinline__ void fft_pass(typename Cx<T>::t* __restrict__ buf, in
     // numbered as a full group with the extra lines idle: then each group
     // covers G lines at one offset, which an odd line stride spreads over all
     // banks.
+    // Not in float64: an idle lane costs the float64 pipe as much as a busy
+    // one, more than the conflicts do (x pass at 6 lines, 384^3: 6.09 ms padded).
     constexpr int G = sizeof(C) == 8 ? 16 : 8;
-    const bool pad = nlines < G && (G % nlines) != 0 && 2 * nlines > G;
+    const bool pad = sizeof(C) == 8 && nlines < G && (G % nlines) != 0 && 2 * nlines > G;
     const int tot = (pad ? G : nlines) * nb;
     const int L = st * R;
     for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
