@@ -391,6 +391,23 @@ int derive(const bs_params* p, Derived* d)
 
 }  // namespace
 
+void bsw::cheb_fit(long double (*f)(long double), long double c, long double w, int deg, double* out, int stride)
+{
+    long double t[32], v[32], p[32] = {};
+    const int n = deg + 1;
+    for (int k = 0; k < n; ++k) {
+        t[k] = 0.5L * cosl(3.14159265358979323846264338327950288L * (k + 0.5L) / n);
+        v[k] = f(c + w * t[k]);
+    }
+    for (int j = 1; j < n; ++j)
+        for (int k = n - 1; k >= j; --k) v[k] = (v[k] - v[k - 1]) / (t[k] - t[k - j]);
+    for (int k = n - 1; k >= 0; --k) {  // p <- p (t - t_k) + v_k
+        for (int j = n - 1; j > 0; --j) p[j] = p[j - 1] - t[k] * p[j];
+        p[0] = v[k] - t[k] * p[0];
+    }
+    for (int j = 0; j < n; ++j) out[j * stride] = (double)p[j];
+}
+
 void bsw::set_last_error(const char* msg) { g_err = msg ? msg : ""; }
 
 struct bs_ctx {
@@ -1211,6 +1228,7 @@ int bs_create(bs_ctx** out, const bs_params* p, void* stream)
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = set_fft_constants();
     if (e == cudaSuccess) e = set_short_tables();
+    if (e == cudaSuccess) e = set_node_tables();
     // the short-range branch runs at the highest stream priority: its few
     // CTAs are dispatched ahead of the long-range kernels' waiting ones, so
     // the branch ends while the spread is still running

@@ -80,6 +80,29 @@ template <> struct __align__(16) LrRec<double> {
     int pad[3];
 };
 
+// ---- float64 helpers (float64 runs at 1/64 of the float32 rate: library
+// square roots, divisions and conversions are avoided where they are many) ----
+// 1 / sqrt(a), a > 0 normal: the hardware's approximation and one step of
+// Householder's third-order iteration.
+__device__ __forceinline__ double rsqrt_h(double a)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// double of a 32-bit integer without a conversion instruction (exact)
+__device__ __forceinline__ double i2d(int k)
+{
+    return __hiloint2double(0x43300000, k ^ 0x80000000) - 4503601774854144.0;  // 2^52 + 2^31
+}
+
+// Monomial coefficients in t (stride apart) of the degree-deg polynomial
+// through f(c + w t) at the Chebyshev points t of [-1/2, 1/2] (divided
+// differences, extended precision; host, deg < 32).
+void cheb_fit(long double (*f)(long double), long double c, long double w, int deg, double* out, int stride);
+
 // Parameters of the geometry / node kernel.
 struct GeomP {
     double L[3];
@@ -401,6 +424,7 @@ template <typename T>
 size_t col_pt_bytes(int w);
 cudaError_t set_fft_constants();
 cudaError_t set_short_tables();
+cudaError_t set_node_tables();
 template <typename T>
 cudaError_t launch_fft_y(const FftYP& P, const Work& w, void* f2, int sign, cudaStream_t s,
                          const CUtensorMap* tm_f1 = nullptr);

@@ -28,6 +28,8 @@
 // T-precision offset from the cell origin.
 #include <math.h>
 
+#include <mutex>
+
 #include "bs_internal.cuh"
 
 namespace bsw {
@@ -348,28 +350,84 @@ __device__ __forceinline__ void make_poly(SegPoly<T>& P, const T* __restrict__ h
             P.c4[c] = ((T)7 * B - (T)15 * A - C) * ih;
             P.c5[c] = ((T)6 * A - (T)3 * B + (T)0.5 * C) * ih * ih;
         } else {
-            P.b[c] = dp[3 * j + c] * ih - h * ((T)2 * Mj + Mn) / (T)6;
-            P.c3[c] = (Mn - Mj) * ih / (T)6;
+            if constexpr (sizeof(T) == 8) {  // a product: six float64 divisions cost more than the rest
+                P.b[c] = dp[3 * j + c] * ih - h * ((T)2 * Mj + Mn) * (T)(1.0 / 6.0);
+                P.c3[c] = (Mn - Mj) * ih * (T)(1.0 / 6.0);
+            } else {
+                P.b[c] = dp[3 * j + c] * ih - h * ((T)2 * Mj + Mn) / (T)6;
+                P.c3[c] = (Mn - Mj) * ih / (T)6;
+            }
             P.c4[c] = 0;
             P.c5[c] = 0;
         }
     }
 }
 
-// Accumulate the self terms of one C_0 point: r from the node, charge q.
-template <typename T>
-__device__ __forceinline__ void self_add(const T r[3], const T q[3], T alpha, T* vs, T* ps)
+// The float64 self term's functions without library calls (erf, exp, a square
+// root and two divisions cost it about 150 float64 operations a point): E(u) =
+// g^(f)(x) / x^3 and P(u) = erf(x) / x are entire functions of u = x^2, taken
+// from degree-8 polynomials on intervals of 1/4 centred at i / 4, i = 0..64
+// (interpolation error below 2^-55), written once per device
+// (set_node_tables).  Beyond u = 16 the library forms below.
+constexpr int kSelfN = 65, kSelfDeg = 8;
+__device__ double g_self_tab[2][(kSelfDeg + 1) * kSelfN];  // E, P; degree-major
+
+__device__ __forceinline__ double self_poly(const double* __restrict__ tab, int i, double t)
 {
-    const T rr = tsqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-    const T x = alpha * rr;
-    const T fv = g_far(x) / (rr * rr * rr);
-    const T fp = erf(x) / rr;
-    vs[0] += fv * (r[1] * q[2] - r[2] * q[1]);
-    vs[1] += fv * (r[2] * q[0] - r[0] * q[2]);
-    vs[2] += fv * (r[0] * q[1] - r[1] * q[0]);
-    ps[0] += fp * q[0];
-    ps[1] += fp * q[1];
-    ps[2] += fp * q[2];
+    double v = __ldg(tab + kSelfDeg * kSelfN + i);
+#pragma unroll
+    for (int k = kSelfDeg - 1; k >= 0; --k) v = fma(v, t, __ldg(tab + k * kSelfN + i));
+    return v;
+}
+
+// sqrt(a), a >= 0: float64 through rsqrt_h.
+template <typename T>
+__device__ __forceinline__ T sqrt_n(T a)
+{
+    if constexpr (sizeof(T) == 8)
+        return a > 0.0 ? a * rsqrt_h(a) : 0.0;
+    else
+        return tsqrt(a);
+}
+
+// Accumulate the self terms of one C_0 point: r from the node, charge q (in
+// float64 ps only with want_psi).
+template <typename T>
+__device__ __forceinline__ void self_add(const T r[3], const T q[3], T alpha, int want_psi, T* vs, T* ps)
+{
+    if constexpr (sizeof(T) == 8) {
+        const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+        const double u = alpha * alpha * r2;
+        double fv, fp = 0.0;
+        if (u < 15.9) {
+            const double m = fma(4.0, u, 4503599627370496.0);  // 2^52: the low word is rint(4 u)
+            const double t = fma(4.0, u, -(m - 4503599627370496.0));
+            const int i = __double2loint(m);
+            fv = self_poly(g_self_tab[0], i, t) * (alpha * alpha * alpha);
+            if (want_psi) fp = self_poly(g_self_tab[1], i, t) * alpha;
+        } else {
+            const double rr = tsqrt(r2), x = alpha * rr;
+            fv = g_far(x) / (rr * rr * rr);
+            if (want_psi) fp = erf(x) / rr;
+        }
+        vs[0] += fv * (r[1] * q[2] - r[2] * q[1]);
+        vs[1] += fv * (r[2] * q[0] - r[0] * q[2]);
+        vs[2] += fv * (r[0] * q[1] - r[1] * q[0]);
+        ps[0] += fp * q[0];
+        ps[1] += fp * q[1];
+        ps[2] += fp * q[2];
+    } else {
+        const T rr = tsqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+        const T x = alpha * rr;
+        const T fv = g_far(x) / (rr * rr * rr);
+        const T fp = erf(x) / rr;
+        vs[0] += fv * (r[1] * q[2] - r[2] * q[1]);
+        vs[1] += fv * (r[2] * q[0] - r[0] * q[2]);
+        vs[2] += fv * (r[0] * q[1] - r[1] * q[0]);
+        ps[0] += fp * q[0];
+        ps[1] += fp * q[1];
+        ps[2] += fp * q[2];
+    }
 }
 
 template <typename T>
@@ -415,8 +473,8 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
         S.eval(u, del, sd);
         const T wq = (T)P.gw[i] * S.h;
         T q[3] = { wq * sd[0], wq * sd[1], wq * sd[2] };
-        lp += wq * tsqrt(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
-        self_add(del, q, alpha, vs, ps);
+        lp += wq * sqrt_n(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
+        self_add(del, q, alpha, P.want_psi, vs, ps);
 
         // the point is near the wrapped node: it is mostly in the box already
         bool b2 = false;
@@ -477,9 +535,9 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
             R.eval(u, del, sd);
             const T wq = (T)P.gw[i] * R.h;
             const T q[3] = { wq * sd[0], wq * sd[1], wq * sd[2] };
-            lm += wq * tsqrt(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
+            lm += wq * sqrt_n(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
             const T r[3] = { del[0] - dsx, del[1] - dsy, del[2] - dsz };
-            self_add(r, q, alpha, vs, ps);
+            self_add(r, q, alpha, P.want_psi, vs, ps);
         }
     }
 
@@ -499,9 +557,9 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
             const T gh = (T)P.gh[i], gw = (T)P.gw[i];
             T del[3], sd[3];
             S.eval(gh * fr * S.h, del, sd);
-            lp += gw * fr * S.h * tsqrt(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
+            lp += gw * fr * S.h * sqrt_n(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
             R.eval(((T)1 - fr + gh * fr) * R.h, del, sd);
-            lm += gw * fr * R.h * tsqrt(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
+            lm += gw * fr * R.h * sqrt_n(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
         }
         for (int side = 0; side < 2; ++side) {
             const SegPoly<T>& Gs = side == 0 ? S : R;
@@ -518,14 +576,26 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
 #pragma unroll
                     for (int c = 0; c < 3; ++c) r[c] = side == 0 ? del[c] : del[c] - dsp[c];
                     const T q[3] = { wt * sd[0], wt * sd[1], wt * sd[2] };
-                    const T rr = tsqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-                    const T ir3 = (T)1 / (rr * rr * rr);
-                    vd[0] += (r[1] * q[2] - r[2] * q[1]) * ir3;
-                    vd[1] += (r[2] * q[0] - r[0] * q[2]) * ir3;
-                    vd[2] += (r[0] * q[1] - r[1] * q[0]) * ir3;
-                    pd[0] += q[0] / rr;
-                    pd[1] += q[1] / rr;
-                    pd[2] += q[2] / rr;
+                    if constexpr (sizeof(T) == 8) {
+                        const double ir = rsqrt_h(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]), ir3 = ir * ir * ir;
+                        vd[0] += (r[1] * q[2] - r[2] * q[1]) * ir3;
+                        vd[1] += (r[2] * q[0] - r[0] * q[2]) * ir3;
+                        vd[2] += (r[0] * q[1] - r[1] * q[0]) * ir3;
+                        if (P.want_psi) {
+                            pd[0] += q[0] * ir;
+                            pd[1] += q[1] * ir;
+                            pd[2] += q[2] * ir;
+                        }
+                    } else {
+                        const T rr = tsqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+                        const T ir3 = (T)1 / (rr * rr * rr);
+                        vd[0] += (r[1] * q[2] - r[2] * q[1]) * ir3;
+                        vd[1] += (r[2] * q[0] - r[0] * q[2]) * ir3;
+                        vd[2] += (r[0] * q[1] - r[1] * q[0]) * ir3;
+                        pd[0] += q[0] / rr;
+                        pd[1] += q[1] / rr;
+                        pd[2] += q[2] / rr;
+                    }
                 }
                 x0 = x1;
             }
@@ -1397,5 +1467,57 @@ template cudaError_t launch_export_quadrature<float>(const GeomP&, const double*
                                                      cudaStream_t);
 template cudaError_t launch_export_quadrature<double>(const GeomP&, const double*, const Work&, double*, double*,
                                                       cudaStream_t);
+
+// E(u) and P(u) of the self term: the series (2/sqrt(pi)) sum_{n>=1}
+// (-1)^{n+1} 2n u^{n-1} / (n! (2n+1)) and its counterpart below u = 2 (the closed
+// forms cancel there), the closed forms above.
+static long double self_e(long double u)
+{
+    const long double c = 1.12837916709551257389615890312154517L;
+    if (u < 2.0L) {
+        long double s = 0, p = 1;  // p = (-u)^{n-1} / n!
+        for (int n = 1; n < 60; ++n) {
+            p = n == 1 ? 1.0L : -p * u / n;
+            s += p * (2.0L * n) / (2.0L * n + 1.0L);
+        }
+        return c * s;
+    }
+    const long double x = sqrtl(u);
+    return (erfl(x) - c * x * expl(-u)) / (x * u);
+}
+static long double self_p(long double u)
+{
+    const long double c = 1.12837916709551257389615890312154517L;
+    if (u < 2.0L) {
+        long double s = 0, p = 1;  // p = (-u)^n / n!
+        for (int n = 0; n < 60; ++n) {
+            if (n > 0) p *= -u / n;
+            s += p / (2.0L * n + 1.0L);
+        }
+        return c * s;
+    }
+    const long double x = sqrtl(u);
+    return erfl(x) / x;
+}
+
+// The float64 self term's tables, once per device.
+cudaError_t set_node_tables()
+{
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
+    static double tab[2][(kSelfDeg + 1) * kSelfN];
+    for (int i = 0; i < kSelfN; ++i) {
+        cheb_fit(self_e, i / 4.0L, 1 / 4.0L, kSelfDeg, tab[0] + i, kSelfN);
+        cheb_fit(self_p, i / 4.0L, 1 / 4.0L, kSelfDeg, tab[1] + i, kSelfN);
+    }
+    e = cudaMemcpyToSymbol(g_self_tab, tab, sizeof tab);
+    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+    return e;
+}
 
 }  // namespace bsw

@@ -100,14 +100,6 @@ constexpr int kSgN = 129, kSgDeg = 8, kSgStride = 132;
 constexpr int kSgTable = (kSgDeg + 1) * kSgStride;  // doubles per function, degree-major
 __device__ double g_sg_tab[2 * kSgTable];           // g^(n), then erfc
 
-__device__ __forceinline__ double rsqrt_h(double a)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double e = fma(-(a * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 // Value at the table argument: t in [-1/2, 1/2], interval i.
 __device__ __forceinline__ double sg_poly(const double* __restrict__ tab, int i, double t)
 {
@@ -115,12 +107,6 @@ __device__ __forceinline__ double sg_poly(const double* __restrict__ tab, int i,
 #pragma unroll
     for (int k = kSgDeg - 1; k >= 0; --k) v = fma(v, t, tab[k * kSgStride + i]);
     return v;
-}
-
-// double of a small integer without a conversion instruction (exact)
-__device__ __forceinline__ double i2d(int k)
-{
-    return __hiloint2double(0x43300000, k ^ 0x80000000) - 4503601774854144.0;  // 2^52 + 2^31
 }
 
 // Copies the tables into shared memory (float64; the whole block).
@@ -813,26 +799,6 @@ static long double sg_near(long double x)
     return erfcl(x) + 1.12837916709551257389615890312154517L * x * expl(-x * x);
 }
 
-// Degree-d monomial coefficients in t of the polynomial through f at the
-// Chebyshev points of x = (i + t) / 16, t in [-1/2, 1/2] (divided differences,
-// extended precision).
-static void sg_fit(long double (*f)(long double), int i, double* out, int stride)
-{
-    constexpr int n = kSgDeg + 1;
-    long double t[n], c[n], p[n] = {};
-    for (int k = 0; k < n; ++k) {
-        t[k] = 0.5L * cosl(3.14159265358979323846264338327950288L * (k + 0.5L) / n);
-        c[k] = f((i + t[k]) / 16.0L);
-    }
-    for (int j = 1; j < n; ++j)
-        for (int k = n - 1; k >= j; --k) c[k] = (c[k] - c[k - 1]) / (t[k] - t[k - j]);
-    for (int k = n - 1; k >= 0; --k) {  // p <- p (t - t_k) + c_k
-        for (int j = n - 1; j > 0; --j) p[j] = p[j - 1] - t[k] * p[j];
-        p[0] = c[k] - t[k] * p[0];
-    }
-    for (int j = 0; j < n; ++j) out[j * stride] = (double)p[j];
-}
-
 // The float64 pair term's tables, once per device.
 cudaError_t set_short_tables()
 {
@@ -845,8 +811,8 @@ cudaError_t set_short_tables()
     if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
     static double tab[2 * kSgTable];
     for (int i = 0; i < kSgN; ++i) {
-        sg_fit(sg_near, i, tab + i, kSgStride);
-        sg_fit(sg_erfc, i, tab + kSgTable + i, kSgStride);
+        cheb_fit(sg_near, i / 16.0L, 1 / 16.0L, kSgDeg, tab + i, kSgStride);
+        cheb_fit(sg_erfc, i / 16.0L, 1 / 16.0L, kSgDeg, tab + kSgTable + i, kSgStride);
     }
     e = cudaMemcpyToSymbol(g_sg_tab, tab, sizeof tab);
     if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
