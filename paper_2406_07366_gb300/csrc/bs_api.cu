@@ -925,27 +925,35 @@ int run(bs_ctx* c, const double* nodes, double* vel, double* psi, double* parts,
     ColP CP;
     fill_colp(c, CP);
     const bool fused = d.fuse_interp && !spectrum && !coarse;
+    const bool pruned = !(p.flags & BS_FFT_CUFFT);
 
     rec(c, 0, s);
     CE(launch_spline<T>(nodes, w, c->nfil, s));
     CE(launch_nodes<T>(G, nodes, w, parts ? parts : nullptr, parts ? parts + 3 * N3 : nullptr,
-                       psi_parts ? psi_parts : nullptr, psi_parts ? psi_parts + 3 * N3 : nullptr, s));
+                       psi_parts ? psi_parts : nullptr, psi_parts ? psi_parts + 3 * N3 : nullptr, s,
+                       pruned ? w.col_cnt : nullptr, pruned ? CP.ncols * CP.nzb + 1 : 0));
     rec(c, 1, s);
 
-    // short range on the side stream (not for the spectrum or the grid field)
-    if (!spectrum && !coarse) {
-    CE(cudaEventRecord(c->ev_fork, s));
-    CE(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
-    cudaStream_t ss = c->side;
-    CE(launch_sort_sr<T>(w, (int)c->NQ, (int)d.ncells, ss, det));
-    rec(c, 2, ss);
-    ShortP S;
-    fill_short(c, want_psi, S);
-    CE(launch_short<T>(S, w, ss));
-    rec(c, 3, ss);
-    if (fused) CE(launch_node_bin<T>(CP, I, nodes, w, ss));
-    CE(cudaEventRecord(c->ev_join, ss));
-    }
+    // Short range and node binning on the side stream (not for the spectrum or
+    // the grid field).  The fork is here; the pruned path issues them after its
+    // own first kernels, the longer chain: a small evaluation is bound by the
+    // launches, and the main stream should not wait for the side's.
+    auto side_branch = [&]() -> int {
+        cudaStream_t ss = c->side;
+        CE(cudaStreamWaitEvent(ss, c->ev_fork, 0));
+        if (fused) CE(launch_node_clear<T>(CP, I, w, (int)d.ncells, ss));
+        CE(launch_sort_sr<T>(w, (int)c->NQ, (int)d.ncells, ss, det, fused));
+        rec(c, 2, ss);
+        ShortP S;
+        fill_short(c, want_psi, S);
+        CE(launch_short<T>(S, w, ss));
+        rec(c, 3, ss);
+        if (fused) CE(launch_node_bin<T>(CP, I, nodes, w, ss));
+        CE(cudaEventRecord(c->ev_join, ss));
+        return BS_OK;
+    };
+    if (!spectrum && !coarse) CE(cudaEventRecord(c->ev_fork, s));
+    if (!spectrum && !coarse && !pruned) TRY(side_branch());
 
     // long range on the main stream
     if (p.flags & BS_FFT_CUFFT) {
@@ -979,12 +987,13 @@ int run(bs_ctx* c, const double* nodes, double* vel, double* psi, double* parts,
         TRY(fft_inv<T>(c, w.spec, s));
         rec(c, 8, s);
     } else {
-        CE(launch_col_sort<T>(CP, w, (int)c->NQ, s, det));
+        CE(launch_col_sort<T>(CP, w, (int)c->NQ, s, det, true));
         rec(c, 4, s);
         SpZP SZ;
         fill_spzp<T>(c, det, SZ);
         CE(launch_spread_zfft<T>(SZ, w, s));
         rec(c, 5, s);
+        if (!spectrum && !coarse) TRY(side_branch());
         FftYP YP;
         fill_fftyp<T>(c, YP);
         CE(launch_fft_y<T>(YP, w, w.f2, -1, s, tmap_y<T>(c, YP)));

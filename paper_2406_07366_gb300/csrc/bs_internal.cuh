@@ -398,12 +398,12 @@ template <typename T>
 cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStream_t s);
 template <typename T>
 cudaError_t launch_nodes(const GeomP& P, const double* nodes, const Work& w, double* part_local, double* part_self,
-                         double* psi_local, double* psi_self, cudaStream_t s);
+                         double* psi_local, double* psi_self, cudaStream_t s, int* clr, int nclr);
 template <typename T>
 cudaError_t launch_export_quadrature(const GeomP& P, const double* nodes, const Work& w, double* qX, double* qq,
                                      cudaStream_t s);
 template <typename T>
-cudaError_t launch_sort_sr(const Work& w, int NQ, int ncells, cudaStream_t s, bool det);
+cudaError_t launch_sort_sr(const Work& w, int NQ, int ncells, cudaStream_t s, bool det, bool cleared);
 template <typename T>
 cudaError_t launch_sort_lr(const Work& w, int NQ, int ntiles, cudaStream_t s);
 template <typename T>
@@ -417,7 +417,7 @@ cudaError_t launch_interp(const InterpP& P, const double* nodes, const Work& w, 
                           double* out, double* part_long, cudaStream_t s);
 
 template <typename T>
-cudaError_t launch_col_sort(const ColP& P, const Work& w, int NQ, cudaStream_t s, bool det);
+cudaError_t launch_col_sort(const ColP& P, const Work& w, int NQ, cudaStream_t s, bool det, bool cleared);
 template <typename T>
 cudaError_t launch_spread_zfft(const SpZP& P, const Work& w, cudaStream_t s);
 template <typename T>
@@ -425,6 +425,11 @@ size_t col_pt_bytes(int w);
 cudaError_t set_fft_constants();
 cudaError_t set_short_tables();
 cudaError_t set_node_tables();
+
+// Threads per CTA of a kernel with a thread per item: whole warps spread over
+// the SMs while there are fewer than two warps per scheduler (float64 and the
+// kernel weights are serial chains: 64 nodes on one SM wait for each other).
+inline int item_threads(long long items, int most) { return items <= 152 * 256 ? 32 : most; }
 template <typename T>
 cudaError_t launch_fft_y(const FftYP& P, const Work& w, void* f2, int sign, cudaStream_t s,
                          const CUtensorMap* tm_f1 = nullptr);
@@ -467,6 +472,8 @@ template <typename T>
 cudaError_t launch_zfft_interp(const SpZP& P, const Work& w, cudaStream_t s);
 template <typename T>
 cudaError_t launch_node_bin(const ColP& P, const InterpP& I, const double* nodes, const Work& w, cudaStream_t s);
+template <typename T>
+cudaError_t launch_node_clear(const ColP& P, const InterpP& I, const Work& w, int ncells, cudaStream_t s);
 template <typename T>
 size_t nd_rec_bytes(int w);
 template <typename T>
@@ -670,7 +677,8 @@ cudaError_t launch_scatter_b(const BatchL& L, cudaStream_t s);
 
 // Exclusive scan of n ints in place (cnt[n] receives the total); tmp holds
 // scan_blocks(n) ints.
-cudaError_t scan_exclusive(int* cnt, int n, int* tmp, cudaStream_t s);
+cudaError_t scan_exclusive(int* cnt, int n, int* tmp, cudaStream_t s, int* cur = nullptr);
+cudaError_t launch_clear(int* a, long long na, int* b, long long nb, int* c, long long nc, cudaStream_t s);
 int scan_blocks(int n);
 
 }  // namespace bsw

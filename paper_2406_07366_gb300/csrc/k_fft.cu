@@ -2135,7 +2135,8 @@ static cudaError_t col_scatter_w(const ColP& P, const Work& w, int NQ, cudaStrea
     // deterministic: the copies' entries go to the second buffer, then every
     // column block is put in increasing source order
     static_assert(sizeof(SpPt<T, W>) % 16 == 0, "records are gathered as 16-byte words");
-    k_col_scatter<T, W><<<(NQ + kThreads - 1) / kThreads, kThreads, 0, s>>>(
+    const int tb = item_threads(NQ, kThreads);
+    k_col_scatter<T, W><<<(NQ + tb - 1) / tb, tb, 0, s>>>(
         P, (const LrRec<T>*)w.lr_rec, NQ, w.col_cur, det ? w.col_rec2 : w.col_rec, (SpPt<T, W>*)w.col_pts);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !det) return e;
@@ -2159,16 +2160,14 @@ static cudaError_t launch_col_scatter_w(const ColP& P, const Work& w, int NQ, cu
 }
 
 template <typename T>
-cudaError_t launch_col_sort(const ColP& P, const Work& w, int NQ, cudaStream_t s, bool det)
+cudaError_t launch_col_sort(const ColP& P, const Work& w, int NQ, cudaStream_t s, bool det, bool cleared)
 {
     const int nbins = P.ncols * P.nzb;
-    cudaError_t e = cudaMemsetAsync(w.col_cnt, 0, sizeof(int) * (size_t)(nbins + 1), s);
+    cudaError_t e = cleared ? cudaSuccess : cudaMemsetAsync(w.col_cnt, 0, sizeof(int) * (size_t)(nbins + 1), s);
     if (e != cudaSuccess) return e;
-    if (NQ > 0) k_col_count<T><<<(NQ + kThreads - 1) / kThreads, kThreads, 0, s>>>(P, (const LrRec<T>*)w.lr_rec, NQ,
-                                                                                  w.col_cnt);
-    e = scan_exclusive(w.col_cnt, nbins, w.scan_tmp2, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(w.col_cur, w.col_cnt, sizeof(int) * (size_t)nbins, cudaMemcpyDeviceToDevice, s);
+    const int tb = item_threads(NQ, kThreads);
+    if (NQ > 0) k_col_count<T><<<(NQ + tb - 1) / tb, tb, 0, s>>>(P, (const LrRec<T>*)w.lr_rec, NQ, w.col_cnt);
+    e = scan_exclusive(w.col_cnt, nbins, w.scan_tmp2, s, w.col_cur);
     if (e != cudaSuccess) return e;
     if (NQ > 0)
         e = launch_col_scatter_w<T>(P, w, NQ, s, det);
@@ -2179,25 +2178,31 @@ template <typename T, int W>
 static cudaError_t node_bin_w(const ColP& P, const InterpP& I, const double* nodes, const Work& w, cudaStream_t s)
 {
     const int N = I.N;
-    const int g = (N + kThreads - 1) / kThreads;
-    k_node_w<T, W><<<g, kThreads, 0, s>>>(I, P.tx, P.ty, P.nbx, nodes, (NdW<T, W>*)w.nd_rec, w.nd_key, w.nd_rank,
+    const int tb = item_threads(N, kThreads), g = (N + tb - 1) / tb;
+    k_node_w<T, W><<<g, tb, 0, s>>>(I, P.tx, P.ty, P.nbx, nodes, (NdW<T, W>*)w.nd_rec, w.nd_key, w.nd_rank,
                                            w.ncol_cnt);
     cudaError_t e = scan_exclusive(w.ncol_cnt, P.ncols, w.scan_tmp, s);
     if (e != cudaSuccess) return e;
-    k_node_scatter<T, W><<<g, kThreads, 0, s>>>(N, (const NdW<T, W>*)w.nd_rec, w.nd_key, w.nd_rank, w.ncol_cnt,
+    k_node_scatter<T, W><<<g, tb, 0, s>>>(N, (const NdW<T, W>*)w.nd_rec, w.nd_key, w.nd_rank, w.ncol_cnt,
                                                  (NdW<T, W>*)w.nd_sorted);
     return cudaGetLastError();
 }
 
+// Clears the interpolation's accumulator and the counters of the node binning
+// and of the short range's cells, in one launch.
+template <typename T>
+cudaError_t launch_node_clear(const ColP& P, const InterpP& I, const Work& w, int ncells, cudaStream_t s)
+{
+    return launch_clear((int*)w.vacc, 3 * (long long)I.N * (int)(sizeof(T) / 4), w.ncol_cnt, P.ncols + 1LL, w.cell_cnt,
+                        ncells + 1LL, s);
+}
+
 // Sorts the nodes with their weights by the z-column block of their grid
-// cell for the fused inverse-z interpolation, and clears the accumulator it
-// adds into.
+// cell for the fused inverse-z interpolation (after launch_node_clear).
 template <typename T>
 cudaError_t launch_node_bin(const ColP& P, const InterpP& I, const double* nodes, const Work& w, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(w.vacc, 0, sizeof(T) * 3 * (size_t)I.N, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.ncol_cnt, 0, sizeof(int) * (size_t)(P.ncols + 1), s);
-    if (e != cudaSuccess || I.N == 0) return e;
+    if (I.N == 0) return cudaSuccess;
     switch (P.w) {
     case 2: return node_bin_w<T, 2>(P, I, nodes, w, s);
     case 4: return node_bin_w<T, 4>(P, I, nodes, w, s);
@@ -2747,14 +2752,16 @@ BSW_INST_B(float)
 BSW_INST_B(double)
 #undef BSW_INST_B
 
-template cudaError_t launch_col_sort<float>(const ColP&, const Work&, int, cudaStream_t, bool);
-template cudaError_t launch_col_sort<double>(const ColP&, const Work&, int, cudaStream_t, bool);
+template cudaError_t launch_col_sort<float>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
+template cudaError_t launch_col_sort<double>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
 template cudaError_t launch_spread_zfft<float>(const SpZP&, const Work&, cudaStream_t);
 template cudaError_t launch_spread_zfft<double>(const SpZP&, const Work&, cudaStream_t);
 template cudaError_t launch_zfft_interp<float>(const SpZP&, const Work&, cudaStream_t);
 template cudaError_t launch_zfft_interp<double>(const SpZP&, const Work&, cudaStream_t);
 template cudaError_t launch_node_bin<float>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
+template cudaError_t launch_node_clear<float>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
 template cudaError_t launch_node_bin<double>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
+template cudaError_t launch_node_clear<double>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
 template size_t nd_rec_bytes<float>(int);
 template size_t nd_rec_bytes<double>(int);
 template cudaError_t launch_fft_x_kspace<float>(const FftXP&, const Work&, bool, cudaStream_t, const CUtensorMap*);

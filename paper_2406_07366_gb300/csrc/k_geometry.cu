@@ -250,9 +250,15 @@ __device__ __forceinline__ void k_spline_warp_body(const double* __restrict__ no
     if (lane < 4) {
         T* r = sh_r + lane * nmax;
         const T a0 = hl, cn = hl;
-        T cprev = 0, dprev = 0, hm = hl;
+        // the chain per node is two dependent products and a reciprocal; the
+        // operands come a step ahead so that no shared-memory read is in it
+        T cprev = 0, dprev = 0, hm = hl, hnx = sh_h[0], rnx = r[0];
         for (int j = 0; j < n; ++j) {
-            const T hj = sh_h[j];
+            const T hj = hnx, rj = rnx;
+            if (j + 1 < n) {
+                hnx = sh_h[j + 1];
+                rnx = r[j + 1];
+            }
             const T a = (j == 0) ? (T)0 : hm;
             T bb = (T)2 * (hm + hj);
             if (j == 0) bb -= gamma;
@@ -260,15 +266,21 @@ __device__ __forceinline__ void k_spline_warp_body(const double* __restrict__ no
             const T c = (j == n - 1) ? (T)0 : hj;
             const T im = (T)1 / (bb - a * cprev);
             cprev = c * im;
-            dprev = (r[j] - a * dprev) * im;
+            dprev = (rj - a * dprev) * im;
             if (lane == 0) sh_cp[j] = cprev;
             r[j] = dprev;
             hm = hj;
         }
         __syncwarp(0xfu);
         T x = r[n - 1];
+        T rb = n > 1 ? r[n - 2] : (T)0, cb = n > 1 ? sh_cp[n - 2] : (T)0;
         for (int j = n - 2; j >= 0; --j) {
-            x = r[j] - sh_cp[j] * x;
+            const T rj = rb, cj = cb;
+            if (j > 0) {
+                rb = r[j - 1];
+                cb = sh_cp[j - 1];
+            }
+            x = rj - cj * x;
             r[j] = x;
         }
     }
@@ -672,8 +684,10 @@ __global__ void k_nodes(GeomP P, const double* __restrict__ nodes, const int* __
                         SrTgt<T>* __restrict__ tgt, double* __restrict__ vls, double* __restrict__ pls,
                         double* __restrict__ part_local, double* __restrict__ part_self,
                         double* __restrict__ psi_local, double* __restrict__ psi_self, int* __restrict__ status,
-                        const T* __restrict__ Dd)
+                        const T* __restrict__ Dd, int* __restrict__ clr, int nclr)
 {
+    // the bin counters of the kernels that follow (they are idle here)
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nclr; i += gridDim.x * blockDim.x) clr[i] = 0;
     k_nodes_body<T>(P, nodes, fil_of, prev, off, shift, hseg, dp, ds, Mm, Tper, sr_rec, sr_key, lr_rec, lr_key, tgt,
         vls, pls, part_local, part_self, psi_local, psi_self, status, Dd, blockIdx.x);
 }
@@ -822,6 +836,113 @@ __global__ void k_energy_line(const int64_t* __restrict__ off, const double* __r
 #pragma unroll
     for (int k = 16; k > 0; k >>= 1) part += __shfl_xor_sync(0xffffffffu, part, k);
     if (lane == 0) {
+        if (per_fil)
+            per_fil[f] = part;  // deterministic: summed in filament order on the host
+        else
+            atomicAdd(acc, part);
+    }
+}
+
+// The cyclic tridiagonal moment system of the periodic cubic spline,
+//   h_{j-1} M_{j-1} + 2 (h_{j-1} + h_j) M_j + h_j M_{j+1} = R_j,
+// for NR right-hand sides by parallel cyclic reduction (as q_solve_cta, the
+// couplings start at 1/4 each on equal chords and square every step: 5 or 6
+// steps).  h: n lengths; buf: (2 + NR) 2 n of scratch with R of component c at
+// buf + (2 + c) n.  All threads of the block, synchronised before; returns the
+// moments, component c at c n, and leaves the block synchronised.
+template <int NR>
+__device__ const double* m_solve_cta(int n, const double* __restrict__ h, double* buf)
+{
+    double* cur = buf;
+    double* nxt = buf + (2 + NR) * n;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const double a = h[j == 0 ? n - 1 : j - 1], hj = h[j], id = 1.0 / (2.0 * (a + hj));
+        cur[j] = a * id;
+        cur[n + j] = hj * id;
+#pragma unroll
+        for (int c = 0; c < NR; ++c) cur[(2 + c) * n + j] *= id;
+    }
+    __syncthreads();
+    int s = 1;  // modulo n
+    for (int it = 0; it < 16; ++it) {
+        bool more = false;
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            const int jm = j - s < 0 ? j - s + n : j - s, jp = j + s >= n ? j + s - n : j + s;
+            const double l = cur[j], u = cur[n + j];
+            const double e = 1.0 / (1.0 - l * cur[n + jm] - u * cur[jp]);
+            const double el = e * l, eu = e * u;
+            const double ln = -el * cur[jm], un = -eu * cur[n + jp];
+            nxt[j] = ln;
+            nxt[n + j] = un;
+            more = more || !(fabs(ln) < 1e-18) || !(fabs(un) < 1e-18);
+#pragma unroll
+            for (int c = 0; c < NR; ++c) {
+                const double* r = cur + (2 + c) * n;
+                nxt[(2 + c) * n + j] = e * r[j] - el * r[jm] - eu * r[jp];
+            }
+        }
+        double* t = cur;
+        cur = nxt;
+        nxt = t;
+        if (!__syncthreads_or(more)) break;
+        s = (2 * s) % n;
+    }
+    return cur + 2 * n;
+}
+
+constexpr size_t kCubicSmemMax = 200 * 1024;
+constexpr size_t kCubicRow = 14 * sizeof(double);  // shared memory per node of the float64 fit
+constexpr size_t kLineRow = 8 * sizeof(double);    // and of the energy line integral
+__device__ __forceinline__ double block_sum(double v);
+
+// The energy line integral with a CTA per filament (up to 3200 nodes; longer
+// filaments: one warp, serial sweeps).  Bound by the latency of the sweeps:
+// 40 filaments of 64 nodes took 51 us with them.
+template <typename T>
+__global__ void __launch_bounds__(256) k_energy_line_cta(const int64_t* __restrict__ off,
+                                                         const double* __restrict__ shift,
+                                                         const T* __restrict__ hseg, const T* __restrict__ dp,
+                                                         const T* __restrict__ Mm, const T* __restrict__ Tper,
+                                                         const double* __restrict__ pls, const double* __restrict__ psr,
+                                                         double* __restrict__ acc, double* __restrict__ per_fil)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    const int f = blockIdx.x;
+    const int64_t o = off[f];
+    const int n = (int)(off[f + 1] - o);
+    double* sh_h = reinterpret_cast<double*>(sm_raw);
+    double* sh_f = sh_h + n;
+    double* buf = sh_f + n;
+    const double iT = 1.0 / (double)Tper[f];
+    const double dr[3] = { shift[3 * f] * iT, shift[3 * f + 1] * iT, shift[3 * f + 2] * iT };
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int jn = (j + 1 < n) ? j + 1 : 0;
+        const double h = (double)hseg[o + j], ih = 1.0 / h;
+        sh_h[j] = h;
+        double fj = 0.0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double Mj = (double)Mm[3 * (o + j) + c], Mn = (double)Mm[3 * (o + jn) + c];
+            const double sdot = (double)dp[3 * (o + j) + c] * ih - h * (2.0 * Mj + Mn) * (1.0 / 6.0) + dr[c];
+            fj += (pls[3 * (o + j) + c] + psr[3 * (o + j) + c]) * sdot;
+        }
+        sh_f[j] = fj;
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int jm = j == 0 ? n - 1 : j - 1, jn = (j + 1 < n) ? j + 1 : 0;
+        buf[2 * n + j] = 6.0 * ((sh_f[jn] - sh_f[j]) / sh_h[j] - (sh_f[j] - sh_f[jm]) / sh_h[jm]);
+    }
+    __syncthreads();
+    const double* m = m_solve_cta<1>(n, sh_h, buf);
+    double part = 0.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int jn = (j + 1 < n) ? j + 1 : 0;
+        const double h = sh_h[j];
+        part += 0.5 * h * (sh_f[j] + sh_f[jn]) - h * h * h * (m[j] + m[jn]) * (1.0 / 24.0);
+    }
+    part = block_sum(part);
+    if (threadIdx.x == 0) {
         if (per_fil)
             per_fil[f] = part;  // deterministic: summed in filament order on the host
         else
@@ -979,6 +1100,16 @@ cudaError_t launch_energy_line(const double* nodes, const Work& w, int nfil, int
         k_energy_line_quintic<T><<<(nfil + tb - 1) / tb, tb, 0, s>>>(w.off, w.shift, nfil, (const T*)w.hseg,
                                                                      (const T*)w.Dd, (const T*)w.Tper, w.pls, w.psr,
                                                                      w.qtmp, w.energy_acc + 1, det ? w.lpart : nullptr);
+        return cudaGetLastError();
+    }
+    if (kLineRow * (size_t)nmax <= kCubicSmemMax) {
+        const size_t sc = kLineRow * (size_t)nmax;
+        cudaError_t e = quintic_smem(k_energy_line_cta<T>, sc);
+        if (e != cudaSuccess) return e;
+        k_energy_line_cta<T><<<nfil, quintic_threads(nmax), sc, s>>>(w.off, w.shift, (const T*)w.hseg,
+                                                                     (const T*)w.dp, (const T*)w.Mm, (const T*)w.Tper,
+                                                                     w.pls, w.psr, w.energy_acc + 1,
+                                                                     det ? w.lpart : nullptr);
         return cudaGetLastError();
     }
     const size_t sm = 5 * (size_t)nmax * sizeof(double);
@@ -1397,6 +1528,68 @@ __global__ void __launch_bounds__(256) k_spline_quintic_cta(const double* __rest
         }
 }
 
+// Cubic fit in float64 with a CTA per filament (m_solve_cta).  float32 keeps
+// the serial sweeps: their rounding is the fit's, and the chain is short there.
+__global__ void __launch_bounds__(256) k_spline_cta(const double* __restrict__ nodes, const int64_t* __restrict__ off,
+                                                    const double* __restrict__ shift, double* __restrict__ hseg,
+                                                    double* __restrict__ dp, double* __restrict__ ds,
+                                                    double* __restrict__ Mm, double* __restrict__ Tper)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ double s_T;
+    const int f = blockIdx.x;
+    const int64_t o = off[f];
+    const int n = (int)(off[f + 1] - o);
+    double* sh_h = reinterpret_cast<double*>(sm_raw);
+    double* sh_d = sh_h + n;      // 3 n: increments over the lengths
+    double* buf = sh_d + 3 * n;   // 10 n
+    const double sh[3] = { shift[3 * f], shift[3 * f + 1], shift[3 * f + 2] };
+    double part = 0.0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const double* a = nodes + 3 * (o + j);
+        const double* b = nodes + 3 * (j + 1 < n ? o + j + 1 : o);
+        double d[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d[c] = b[c] + (j + 1 < n ? 0.0 : sh[c]) - a[c];
+        const double h = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+        part += h;
+        sh_h[j] = h;
+        hseg[o + j] = h;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            sh_d[c * n + j] = d[c];
+            ds[3 * (o + j) + c] = d[c];
+        }
+    }
+    part = block_sum(part);
+    if (threadIdx.x == 0) {
+        s_T = part;
+        Tper[f] = part;
+    }
+    __syncthreads();
+    const double invT = 1.0 / s_T;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const double h = sh_h[j], ih = 1.0 / h;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double p = sh_d[c * n + j] - sh[c] * h * invT;  // periodic increment
+            dp[3 * (o + j) + c] = p;
+            sh_d[c * n + j] = p * ih;
+        }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int jm = j == 0 ? n - 1 : j - 1;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) buf[(2 + c) * n + j] = 6.0 * (sh_d[c * n + j] - sh_d[c * n + jm]);
+    }
+    __syncthreads();
+    const double* m = m_solve_cta<3>(n, sh_h, buf);
+    for (int j = threadIdx.x; j < n; j += blockDim.x)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Mm[3 * (o + j) + c] = m[c * n + j];
+}
+
 template <typename T>
 cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStream_t s)
 {
@@ -1414,6 +1607,16 @@ cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStre
         k_spline_quintic<T><<<(nfil + tb - 1) / tb, tb, 0, s>>>(nodes, w.off, w.shift, nfil, (T*)w.hseg, (T*)w.dp,
                                                                 (T*)w.ds, (T*)w.Mm, (T*)w.Dd, (T*)w.Tper, w.qtmp);
         return cudaGetLastError();
+    }
+    if constexpr (sizeof(T) == 8) {
+        const size_t sc = kCubicRow * (size_t)w.nmax_fil;
+        if (sc <= kCubicSmemMax) {
+            cudaError_t e = quintic_smem(k_spline_cta, sc);
+            if (e != cudaSuccess) return e;
+            k_spline_cta<<<nfil, quintic_threads(w.nmax_fil), sc, s>>>(nodes, w.off, w.shift, (T*)w.hseg, (T*)w.dp,
+                                                                     (T*)w.ds, (T*)w.Mm, (T*)w.Tper);
+            return cudaGetLastError();
+        }
     }
     const size_t sm = 9 * (size_t)w.nmax_fil * sizeof(T);
     if (sm <= kSplineSmemMax) {
@@ -1434,14 +1637,15 @@ cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStre
 
 template <typename T>
 cudaError_t launch_nodes(const GeomP& P, const double* nodes, const Work& w, double* part_local, double* part_self,
-                         double* psi_local, double* psi_self, cudaStream_t s)
+                         double* psi_local, double* psi_self, cudaStream_t s, int* clr, int nclr)
 {
-    if (P.N <= 0) return cudaSuccess;
-    const int tb = 128;
+    if (P.N <= 0) return nclr > 0 ? cudaMemsetAsync(clr, 0, sizeof(int) * (size_t)nclr, s) : cudaSuccess;
+    const int tb = item_threads(P.N, 128);
     k_nodes<T><<<(P.N + tb - 1) / tb, tb, 0, s>>>(
         P, nodes, w.fil_of, w.prev, w.off, w.shift, (const T*)w.hseg, (const T*)w.dp, (const T*)w.ds,
         (const T*)w.Mm, (const T*)w.Tper, (SrRec<T>*)w.sr_rec, w.sr_key, (LrRec<T>*)w.lr_rec, w.lr_key,
-        (SrTgt<T>*)w.tgt, w.vls, w.pls, part_local, part_self, psi_local, psi_self, w.status, (const T*)w.Dd);
+        (SrTgt<T>*)w.tgt, w.vls, w.pls, part_local, part_self, psi_local, psi_self, w.status, (const T*)w.Dd, clr,
+        nclr);
     return cudaGetLastError();
 }
 
@@ -1460,9 +1664,9 @@ cudaError_t launch_export_quadrature(const GeomP& P, const double* nodes, const 
 template cudaError_t launch_spline<float>(const double*, const Work&, int, cudaStream_t);
 template cudaError_t launch_spline<double>(const double*, const Work&, int, cudaStream_t);
 template cudaError_t launch_nodes<float>(const GeomP&, const double*, const Work&, double*, double*, double*, double*,
-                                         cudaStream_t);
+                                         cudaStream_t, int*, int);
 template cudaError_t launch_nodes<double>(const GeomP&, const double*, const Work&, double*, double*, double*, double*,
-                                          cudaStream_t);
+                                          cudaStream_t, int*, int);
 template cudaError_t launch_export_quadrature<float>(const GeomP&, const double*, const Work&, double*, double*,
                                                      cudaStream_t);
 template cudaError_t launch_export_quadrature<double>(const GeomP&, const double*, const Work&, double*, double*,

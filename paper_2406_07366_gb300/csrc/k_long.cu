@@ -216,13 +216,18 @@ __global__ void k_kspace(KspaceP P, typename Cplx<T>::t* __restrict__ spec, type
 //   out = add_d (float64: local - self) + add_t (short range, float64) + interp.
 // part (optional) receives the interpolated long-range part alone.  The
 // weights of the last two axes live in registers (static indices); those of
-// the first axis are computed in the outer loop.
-template <typename T, int W>
+// the first axis are computed in the outer loop.  NC = 3: a thread per node;
+// NC = 1: a thread per node and component, three times the threads while the
+// nodes alone leave most of the GPU idle (2560 nodes, 32-thread blocks: 82 us
+// with one thread a node in 128-thread blocks).  Either way a component is
+// summed over the W^3 points in the same order, which is its float32 rounding.
+template <typename T, int W, int NC>
 __global__ void __launch_bounds__(128) k_interp(InterpP P, const double* __restrict__ nodes, const T* __restrict__ grid,
                                                 const double* __restrict__ add_d, const double* __restrict__ add_t,
                                                 double* __restrict__ out, double* __restrict__ part)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = NC == 3 ? i0 : i0 / 3, c0 = NC == 3 ? 0 : i0 - 3 * j;  // node, first component
     if (j >= P.N) return;
     constexpr int H = W / 2;
     const T zeta = (T)P.zeta;
@@ -255,7 +260,8 @@ __global__ void __launch_bounds__(128) k_interp(InterpP P, const double* __restr
         iz[t] = gz < 0 ? gz + P.ng[2] : (gz >= P.ng[2] ? gz - P.ng[2] : gz);
     }
     const size_t gsz = (size_t)P.ng[0] * P.ng[1] * P.ng[2];
-    T a0 = 0, a1 = 0, a2 = 0;
+    grid += c0 * gsz;
+    T a[NC] = {};
 #pragma unroll 1
     for (int p = 0; p < W; ++p) {
         const T kx = kb_eval((fr[0] + (T)(H - 1 - p)) * ((T)2 / (T)W), zeta, inorm);
@@ -270,32 +276,96 @@ __global__ void __launch_bounds__(128) k_interp(InterpP P, const double* __restr
             for (int r = 0; r < W; ++r) {
                 const size_t gi = row + iz[r];
                 const T wv = wpq * kz[r];
-                a0 += wv * grid[gi];
-                a1 += wv * grid[gsz + gi];
-                a2 += wv * grid[2 * gsz + gi];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) a[c] += wv * grid[c * gsz + gi];
             }
         }
     }
-    if (part) {
-        part[3 * j + 0] = (double)a0;
-        part[3 * j + 1] = (double)a1;
-        part[3 * j + 2] = (double)a2;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const size_t i = 3 * (size_t)j + c0 + c;
+        if (part) part[i] = (double)a[c];
+        if (out) {
+            double o = (double)a[c];
+            if (add_t) o += add_t[i];
+            if (add_d) o += add_d[i];
+            out[i] = o;
+        }
     }
-    if (out) {
-        double o0 = (double)a0, o1 = (double)a1, o2 = (double)a2;
-        if (add_t) {
-            o0 += (double)add_t[3 * j + 0];
-            o1 += (double)add_t[3 * j + 1];
-            o2 += (double)add_t[3 * j + 2];
+}
+
+// The same in float64: a group of G lanes takes a node, lane t its z position t: the group reads whole
+// runs of a grid row, each lane evaluates one weight per axis (passed round
+// by shuffles) and the z sums are reduced over the group.
+constexpr int interp_group(int W) { return W <= 2 ? 2 : (W <= 4 ? 4 : (W <= 8 ? 8 : 16)); }
+template <typename T, int W>
+__global__ void __launch_bounds__(128) k_interp_g(InterpP P, const double* __restrict__ nodes, const T* __restrict__ grid,
+                                                const double* __restrict__ add_d, const double* __restrict__ add_t,
+                                                double* __restrict__ out, double* __restrict__ part)
+{
+    constexpr int G = interp_group(W);
+    const int t = threadIdx.x & (G - 1);
+    const long long jj = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const bool live = jj < P.N;  // the lanes past the end follow the last node
+    const int j = live ? (int)jj : P.N - 1;
+    constexpr int H = W / 2;
+    int ib[3];
+    T kw[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        double x = nodes[3 * (size_t)j + d];
+        if (!isfinite(x)) x = 0.0;
+        double xw = x - P.L[d] * floor(x * P.iL[d]);
+        if (xw >= P.L[d]) xw -= P.L[d];
+        if (xw < 0.0) xw = 0.0;
+        const double g = xw * P.ihg[d];
+        int k = (int)floor(g);
+        k = k < 0 ? 0 : (k >= P.ng[d] ? P.ng[d] - 1 : k);
+        double f = g - (double)k;
+        f = f < 0.0 ? 0.0 : (f > 1.0 ? 1.0 : f);
+        ib[d] = k;
+        kw[d] = t < W ? kb_eval(((T)f + (T)(H - 1 - t)) * ((T)2 / (T)W), (T)P.zeta, (T)P.inorm) : (T)0;
+    }
+    auto wrap = [](int g, int n) { return g < 0 ? g + n : (g >= n ? g - n : g); };
+    const int iz = wrap(ib[2] - H + 1 + (t < W ? t : 0), P.ng[2]);
+    const size_t gsz = (size_t)P.ng[0] * P.ng[1] * P.ng[2];
+    T a0 = 0, a1 = 0, a2 = 0;
+#pragma unroll 1
+    for (int p = 0; p < W; ++p) {
+        const T kx = __shfl_sync(0xffffffffu, kw[0], p, G);
+        const size_t plane = (size_t)wrap(ib[0] - H + 1 + p, P.ng[0]) * P.ng[1];
+#pragma unroll
+        for (int q = 0; q < W; ++q) {
+            const T wpq = kx * __shfl_sync(0xffffffffu, kw[1], q, G);
+            const size_t gi = (plane + wrap(ib[1] - H + 1 + q, P.ng[1])) * P.ng[2] + iz;
+            a0 += wpq * grid[gi];
+            a1 += wpq * grid[gsz + gi];
+            a2 += wpq * grid[2 * gsz + gi];
         }
-        if (add_d) {
-            o0 += add_d[3 * j + 0];
-            o1 += add_d[3 * j + 1];
-            o2 += add_d[3 * j + 2];
+    }
+    a0 *= kw[2];
+    a1 *= kw[2];
+    a2 *= kw[2];
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+        a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+        a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+    }
+    // lane c < 3 of the group writes component c (G = 2: lane 0 all three)
+    if (!live) return;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (t != (G >= 4 ? c : 0)) continue;
+        const T a = c == 0 ? a0 : (c == 1 ? a1 : a2);
+        const size_t i = 3 * (size_t)j + c;
+        if (part) part[i] = (double)a;
+        if (out) {
+            double o = (double)a;
+            if (add_t) o += add_t[i];
+            if (add_d) o += add_d[i];
+            out[i] = o;
         }
-        out[3 * j + 0] = o0;
-        out[3 * j + 1] = o1;
-        out[3 * j + 2] = o2;
     }
 }
 
@@ -360,8 +430,17 @@ template <typename T, int W>
 static cudaError_t interp_w(const InterpP& P, const double* nodes, const void* grid, const double* add_d, const double* add_t,
                             double* out, double* part, cudaStream_t s)
 {
-    const int tb = 128;
-    k_interp<T, W><<<(P.N + tb - 1) / tb, tb, 0, s>>>(P, nodes, (const T*)grid, add_d, add_t, out, part);
+    if constexpr (sizeof(T) == 8) {
+        constexpr int tb = 128;
+        const long long g = ((long long)P.N * interp_group(W) + tb - 1) / tb;
+        k_interp_g<T, W><<<(unsigned)g, tb, 0, s>>>(P, nodes, (const T*)grid, add_d, add_t, out, part);
+    } else if (P.N <= 152 * 256) {
+        const int tb = item_threads(3LL * P.N, 128);
+        k_interp<T, W, 1><<<(3 * P.N + tb - 1) / tb, tb, 0, s>>>(P, nodes, (const T*)grid, add_d, add_t, out, part);
+    } else {
+        const int tb = 128;
+        k_interp<T, W, 3><<<(P.N + tb - 1) / tb, tb, 0, s>>>(P, nodes, (const T*)grid, add_d, add_t, out, part);
+    }
     return cudaGetLastError();
 }
 

@@ -88,9 +88,38 @@ __device__ __forceinline__ void scan_parts_body(int* __restrict__ part, int nb)
 
 __global__ void k_scan_parts(int* __restrict__ part, int nb) { scan_parts_body(part, nb); }
 
+// Exclusive scan of a whole short array by one block, tile after tile, cnt[n]
+// the total; cur (if non-null) takes a copy of the n starts.
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(int* __restrict__ cnt, int n, int* __restrict__ cur)
+{
+    __shared__ int sh[32];
+    int carry = 0;
+    for (int t0 = 0; t0 <= n; t0 += kScanTile) {
+        const int base = t0 + threadIdx.x * kScanItems;
+        int v[kScanItems];
+        int s = 0;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            v[k] = (base + k < n) ? cnt[base + k] : 0;
+            s += v[k];
+        }
+        int total;
+        const int inc = block_scan_incl(s, sh, total);
+        int run = carry + inc - s;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            if (base + k <= n) cnt[base + k] = run;
+            if (cur && base + k < n) cur[base + k] = run;
+            run += v[k];
+        }
+        carry += total;
+    }
+}
+
 // Phase 3: exclusive scan within each tile plus its offset, in place over
 // cnt[0..n]; cnt[n] becomes the grand total.
-__device__ __forceinline__ void scan_apply_body(int* __restrict__ cnt, int n, const int* __restrict__ part, int bid)
+__device__ __forceinline__ void scan_apply_body(int* __restrict__ cnt, int n, const int* __restrict__ part, int bid,
+                                                int* __restrict__ cur = nullptr, bool raw = false)
 {
     __shared__ int sh[32];
     const int base = bid * kScanTile + threadIdx.x * kScanItems;
@@ -103,27 +132,67 @@ __device__ __forceinline__ void scan_apply_body(int* __restrict__ cnt, int n, co
         s += v[k];
     }
     int total;
+    int before;  // sum of the tiles before this one
+    if (raw) {   // part holds the tiles' own sums
+        int q = 0;
+        for (int i = threadIdx.x; i < bid; i += blockDim.x) q += part[i];
+        block_scan_incl(q, sh, before);
+    } else {
+        before = part[bid];
+    }
     const int inc = block_scan_incl(s, sh, total);
-    int run = part[bid] + inc - s;
+    int run = before + inc - s;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
         const int i = base + k;
         if (i <= n) cnt[i] = run;
+        if (cur && i < n) cur[i] = run;
         run += v[k];
     }
 }
 
-__global__ void k_scan_apply(int* __restrict__ cnt, int n, const int* __restrict__ part)
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(int* __restrict__ cnt, int n,
+                                                             const int* __restrict__ part, int* __restrict__ cur,
+                                                             bool raw)
 {
-    scan_apply_body(cnt, n, part, blockIdx.x);
+    scan_apply_body(cnt, n, part, blockIdx.x, cur, raw);
 }
 
-cudaError_t scan_exclusive(int* cnt, int n, int* tmp, cudaStream_t s)
+// Exclusive scan of cnt[0..n) in place, cnt[n] the total; cur (optional)
+// takes a copy of the starts.  Launches, not bytes, are what a scan costs
+// here (2.5-4 us each): up to 4 tiles one block does it all; up to 2048 tiles
+// every block of the last phase sums the tiles before it (at most two loads
+// a thread) in place of a middle launch; beyond that three phases.
+cudaError_t scan_exclusive(int* cnt, int n, int* tmp, cudaStream_t s, int* cur)
 {
     const int nb = scan_blocks(n);
+    if (nb <= 4) {
+        k_scan_one<<<1, kScanThreads, 0, s>>>(cnt, n, cur);
+        return cudaGetLastError();
+    }
+    const bool raw = nb <= 2048;
     k_scan_reduce<<<nb, kScanThreads, 0, s>>>(cnt, n, tmp);
-    k_scan_parts<<<1, kScanThreads, 0, s>>>(tmp, nb);
-    k_scan_apply<<<nb, kScanThreads, 0, s>>>(cnt, n, tmp);
+    if (!raw) k_scan_parts<<<1, kScanThreads, 0, s>>>(tmp, nb);
+    k_scan_apply<<<nb, kScanThreads, 0, s>>>(cnt, n, tmp, cur, raw);
+    return cudaGetLastError();
+}
+
+// Clears up to three arrays of 32-bit words in one launch.
+__global__ void k_clear(int* __restrict__ a, long long na, int* __restrict__ b, long long nb, int* __restrict__ c,
+                        long long nc)
+{
+    const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, st = (long long)gridDim.x * blockDim.x;
+    for (long long i = i0; i < na; i += st) a[i] = 0;
+    for (long long i = i0; i < nb; i += st) b[i] = 0;
+    for (long long i = i0; i < nc; i += st) c[i] = 0;
+}
+
+cudaError_t launch_clear(int* a, long long na, int* b, long long nb, int* c, long long nc, cudaStream_t s)
+{
+    const long long most = na > nb ? (na > nc ? na : nc) : (nb > nc ? nb : nc);
+    if (most <= 0) return cudaSuccess;
+    const long long g = (most + kThreads - 1) / kThreads;
+    k_clear<<<(unsigned)(g < 152 * 8 ? g : 152 * 8), kThreads, 0, s>>>(a, na, b, nb, c, nc);
     return cudaGetLastError();
 }
 
@@ -301,17 +370,15 @@ cudaError_t launch_segsort(const int* start, int nseg, const R* in, const int* k
 
 template <typename R>
 static cudaError_t sort_records(const int* key, const R* in, R* out, int n, int* cnt, int* cur, int nbins, int* tmp,
-                                cudaStream_t s, int* idx_out = nullptr)
+                                cudaStream_t s, int* idx_out = nullptr, bool cleared = false)
 {
-    cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)(nbins + 1), s);
+    cudaError_t e = cleared ? cudaSuccess : cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)(nbins + 1), s);
     if (e != cudaSuccess) return e;
     if (n > 0) {
         const int g = (n + kThreads - 1) / kThreads;
         k_count<<<g, kThreads, 0, s>>>(key, n, cnt);
     }
-    e = scan_exclusive(cnt, nbins, tmp, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(cur, cnt, sizeof(int) * (size_t)nbins, cudaMemcpyDeviceToDevice, s);
+    e = scan_exclusive(cnt, nbins, tmp, s, cur);
     if (e != cudaSuccess) return e;
     if (n > 0) {
         const int g = (n + kThreads - 1) / kThreads;
@@ -321,15 +388,15 @@ static cudaError_t sort_records(const int* key, const R* in, R* out, int n, int*
 }
 
 template <typename T>
-cudaError_t launch_sort_sr(const Work& w, int NQ, int ncells, cudaStream_t s, bool det)
+cudaError_t launch_sort_sr(const Work& w, int NQ, int ncells, cudaStream_t s, bool det, bool cleared)
 {
     if (!det)
         return sort_records<SrRec<T>>(w.sr_key, (const SrRec<T>*)w.sr_rec, (SrRec<T>*)w.sr_sorted, NQ, w.cell_cnt,
-                                      w.cell_cur, ncells, w.scan_tmp, s);
+                                      w.cell_cur, ncells, w.scan_tmp, s, nullptr, cleared);
     // deterministic: bin into the second buffer with the source indices, then
     // order every cell by source index
     cudaError_t e = sort_records<SrRec<T>>(w.sr_key, (const SrRec<T>*)w.sr_rec, (SrRec<T>*)w.sr_sorted2, NQ,
-                                           w.cell_cnt, w.cell_cur, ncells, w.scan_tmp, s, w.sr_idx);
+                                           w.cell_cnt, w.cell_cur, ncells, w.scan_tmp, s, w.sr_idx, cleared);
     if (e != cudaSuccess) return e;
     return launch_segsort<SrRec<T>>(w.cell_cnt, ncells, (const SrRec<T>*)w.sr_sorted2, w.sr_idx,
                                     (SrRec<T>*)w.sr_sorted, s);
@@ -342,8 +409,8 @@ cudaError_t launch_sort_lr(const Work& w, int NQ, int ntiles, cudaStream_t s)
                                   w.tile_cur, ntiles, w.scan_tmp2, s);
 }
 
-template cudaError_t launch_sort_sr<float>(const Work&, int, int, cudaStream_t, bool);
-template cudaError_t launch_sort_sr<double>(const Work&, int, int, cudaStream_t, bool);
+template cudaError_t launch_sort_sr<float>(const Work&, int, int, cudaStream_t, bool, bool);
+template cudaError_t launch_sort_sr<double>(const Work&, int, int, cudaStream_t, bool, bool);
 template cudaError_t launch_sort_lr<float>(const Work&, int, int, cudaStream_t);
 template cudaError_t launch_sort_lr<double>(const Work&, int, int, cudaStream_t);
 

@@ -62,3 +62,57 @@ def test_float64_short_range_over_the_table_and_beyond(beta):
     v, ps = oracle.short_range(g, f.L, 1.0, p.alpha, p.rc)
     assert np.abs(parts[1].cpu().numpy() - v).max() < 1e-12 * np.abs(v).max()
     assert np.abs(psi[1].cpu().numpy() - ps).max() < 1e-12 * np.abs(ps).max()
+
+
+@pytest.mark.parametrize("n", [4, 5, 31, 32, 33, 256, 257, 1828, 1829])
+def test_float64_cubic_fit_at_the_edges_of_its_size_rule(n):
+    """Parallel cyclic reduction up to 1828 nodes per filament, the serial
+    sweeps beyond: 1e-12 of the box and 1e-11 of the largest charge against the
+    oracle's collocation, as for the quintic fit."""
+    B, f = _B(), _uneven_ring(n, n) if n > 5 else W.ring(R=0.3, N=n)
+    p = B.make_params(f.L, M=32, Q=2, w=8, precision=B.BS_FP64)
+    bs = B.BiotSavart(p, f.offsets, f.closing)
+    v = bs.velocity(torch.from_numpy(f.nodes).cuda())
+    qX, qq = bs.quadrature(torch.from_numpy(f.nodes).cuda())
+    torch.cuda.synchronize()
+    bs.close()
+    assert torch.isfinite(v).all()
+    g = oracle.geometry(f.nodes, f.offsets, f.closing, f.L, 4, 2)
+    d = qX.cpu().numpy() - g.qX
+    d -= f.L * np.round(d / f.L)
+    assert np.abs(d).max() < 1e-12 * f.L.max()
+    assert np.abs(qq.cpu().numpy() - g.qq).max() < 1e-11 * np.abs(g.qq).max()
+
+
+def test_energy_line_on_both_sides_of_its_size_rule():
+    """A ring of 3200 nodes (a CTA per filament) and one of 3201 (a warp):
+    between them the local terms' O(l^2) error, 4e-6 here, changes by 6e-4 of
+    itself, 3e-9 of the energy."""
+    B = _B()
+    E = []
+    for n in (3200, 3201):
+        f = W.ring(N=n)
+        p = B.make_params(f.L, M=32, Q=2, w=8, precision=B.BS_FP64, flags=B.BS_WANT_PSI)
+        bs = B.BiotSavart(p, f.offsets, f.closing)
+        E.append(bs.energy(torch.from_numpy(f.nodes).cuda()))
+        bs.close()
+    assert abs(E[0] - E[1]) < 1e-8 * abs(E[0])
+
+
+@pytest.mark.parametrize("sigma", [1.25, 1.5, 2.0])
+@pytest.mark.parametrize("w", [2, 4, 6, 8, 10, 12, 14, 16])
+def test_float64_kernel_polynomials_equal_the_kernel(w, sigma):
+    """The long-range part with polynomial kernel weights (the default path,
+    every column block shape the sizes give) against the full-transform path,
+    which evaluates the kernel itself.  Weight errors are below 3e-15 of the
+    peak on either side; a part is a sum of such terms: 1e-12 of its largest value."""
+    B, f = _B(), W.ellipses(3, 40, seed=11)
+    nodes = torch.from_numpy(f.nodes).cuda()
+    parts = []
+    for flags in (0, B.BS_FFT_CUFFT):
+        p = B.make_params(f.L, M=33, Q=2, w=w, sigma=sigma, precision=B.BS_FP64, flags=flags)
+        bs = B.BiotSavart(p, f.offsets, f.closing)
+        parts.append(bs.parts(nodes)[2].clone())
+        torch.cuda.synchronize()
+        bs.close()
+    assert float((parts[0] - parts[1]).abs().max()) < 1e-12 * float(parts[1].abs().max())
