@@ -1883,8 +1883,17 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, kThreads, 0);
     }
-    {   // 8 short range (warp per node)
+    {   // 8 short range (warp per node, or per pair when most nodes can pair)
         std::vector<ShortD<T>> D;
+        const int prec = sizeof(T) == 8 ? BS_FP64 : BS_MIXED;
+        long long can = 0, all = 0;
+        for (size_t m = 0; m < nm; ++m) {
+            ShortP P;
+            fill_short(mem[m], false, P);
+            all += P.N;
+            can += short_can_pair(P, prec) ? P.N : 0;
+        }
+        const bool kind = 2 * can > all;
         for (size_t m = 0; m < nm; ++m) {
             const Work& w = mem[m]->w;
             ShortD<T> e;
@@ -1896,9 +1905,10 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
             e.vsr = w.vsr;
             e.psr = w.psr;
             D.push_back(e);
-            blk.push_back(cdiv(32LL * mem[m]->N, 256));
+            blk.push_back(short_blocks(e.P, kind && short_can_pair(e.P, prec)));
         }
         add(D, 256, 0);
+        st.back().kind = kind;
     }
     auto col_cnt = [](bs_ctx* c) { return c->w.col_cnt; };
     auto colb_n = [](bs_ctx* c) { return c->d.ncolb; };  // spread bins: blocks x z-buckets

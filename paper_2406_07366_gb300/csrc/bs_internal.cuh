@@ -425,6 +425,9 @@ size_t col_pt_bytes(int w);
 cudaError_t set_fft_constants();
 cudaError_t set_short_tables();
 cudaError_t set_node_tables();
+// CTAs of the warp-per-node (or pair) short range.
+bool short_can_pair(const ShortP& P, int precision);
+int short_blocks(const ShortP& P, bool pairs);
 
 // Threads per CTA of a kernel with a thread per item: whole warps spread over
 // the SMs while there are fewer than two warps per scheduler (float64 and the
@@ -544,6 +547,7 @@ struct BatchL {
     int total;    // CTAs of the launch
     int threads;  // threads per CTA
     size_t smem;  // dynamic shared memory per CTA (the largest member's)
+    int kind = 0;  // variant of the kernel (short range: 1 for pairs of nodes)
 };
 
 // Descriptors of the batched stages (one per member).

@@ -151,6 +151,16 @@ __device__ __forceinline__ void st_pair(T rx, T ry, T rz, T r2, const T* q, T al
 
 constexpr int kShortWarps = 8;  // warps per CTA of the warp-per-node kernel
 
+// Row tables of a CTA, per warp: a round's non-empty rows (first source of
+// each run, run lengths, first candidate), the x-cell offsets of the two runs
+// and the y and z cell offsets, and the latter times the cell edges (of both
+// nodes in the paired kernel).
+template <typename T> struct ShortRows {
+    int4 row[kShortWarps][32];
+    int4 ofs[kShortWarps][32];
+    T dh[kShortWarps][32][sizeof(T) == 4 ? 4 : 2];
+};
+
 // One warp per target node.  The lanes first list the source ranges of the
 // (2m+1)^2 neighbour rows (32 rows at a time; a row wrapping around the box
 // gives two ranges; rows and row ends beyond r_c are cut), prefix-sum their
@@ -164,17 +174,11 @@ template <typename T>
 __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __restrict__ tgt,
                                              const int* __restrict__ prev, const int* __restrict__ start,
                                              const SrRec<T>* __restrict__ src, double* __restrict__ vsr,
-                                             double* __restrict__ psr, int bid, const double* __restrict__ tab)
+                                             double* __restrict__ psr, int j, const double* __restrict__ tab,
+                                             ShortRows<T>& rows)
 {
     const int lane = threadIdx.x & 31;
     const int wslot = threadIdx.x >> 5;  // the warp's slot in the CTA's row tables
-    // per warp: a round's non-empty rows (first source of each run, run
-    // lengths, first candidate) and their y, z cell offsets
-    __shared__ int4 s_row[kShortWarps][32];
-    __shared__ int4 s_ofs[kShortWarps][32];   // x-cell offsets of the two runs, y and z cell offsets
-    __shared__ T s_dh[kShortWarps][32][2];    // y and z cell offsets times the cell edges
-    const int j = (int)((bid * (size_t)blockDim.x + threadIdx.x) >> 5);
-    if (j >= P.N) return;  // whole warps exit together
     const SrTgt<T> t = tgt[j];
     const int jp = prev[j];
     const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
@@ -269,10 +273,10 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
         const unsigned nonempty = __ballot_sync(0xffffffffu, nr > 0);
         if (nr > 0) {
             const int ci = __popc(nonempty & ((1u << lane) - 1u));
-            s_row[wslot][ci] = make_int4(s0, n0, s1, ex);
-            s_ofs[wslot][ci] = make_int4(xo0, xo1, dyi, dzi);
-            s_dh[wslot][ci][0] = (T)dyi * h1;
-            s_dh[wslot][ci][1] = (T)dzi * h2;
+            rows.row[wslot][ci] = make_int4(s0, n0, s1, ex);
+            rows.ofs[wslot][ci] = make_int4(xo0, xo1, dyi, dzi);
+            rows.dh[wslot][ci][0] = (T)dyi * h1;
+            rows.dh[wslot][ci][1] = (T)dzi * h2;
         }
         __syncwarp();
         // Candidate c belongs to the last non-empty row starting at or before
@@ -288,7 +292,7 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
             const int own = jr + __popc(M & upto);
             jr += __popc(M);
             if (c >= total) continue;
-            const int4 rw = s_row[wslot][own];
+            const int4 rw = rows.row[wslot][own];
             const int local = c - rw.w;
             const bool first = local < rw.y;
             const int k = first ? rw.x + local : rw.z + (local - rw.y);
@@ -296,16 +300,16 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
             if (S.seg == j || S.seg == jp) continue;  // C_0 of the node (Eq. BS_on_vortex)
             T rx, ry, rz;
             if (!wrap) {
-                const int4 of = s_ofs[wslot][own];
+                const int4 of = rows.ofs[wslot][own];
                 const int dcx = S.cx + (first ? of.x : of.y);
                 if constexpr (sizeof(T) == 8)
                     rx = fma(i2d(dcx), (double)h0, (double)(S.o[0] - t.o[0]));
                 else
                     rx = (T)dcx * h0 + (S.o[0] - t.o[0]);
-                ry = s_dh[wslot][own][0] + (S.o[1] - t.o[1]);
-                rz = s_dh[wslot][own][1] + (S.o[2] - t.o[2]);
+                ry = rows.dh[wslot][own][0] + (S.o[1] - t.o[1]);
+                rz = rows.dh[wslot][own][1] + (S.o[2] - t.o[2]);
             } else {
-                const int4 of = s_ofs[wslot][own];
+                const int4 of = rows.ofs[wslot][own];
                 rx = (T)cdiff(S.cx, cx, nc0) * h0 + (S.o[0] - t.o[0]);
                 ry = (T)of.z * h1 + (S.o[1] - t.o[1]);
                 rz = (T)of.w * h2 + (S.o[2] - t.o[2]);
@@ -378,27 +382,271 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_short(ShortP P, const SrTgt<T>* __restrict__ tgt, const int* __restrict__ prev,
-                                               const int* __restrict__ start, const SrRec<T>* __restrict__ src,
-                                               double* __restrict__ vsr, double* __restrict__ psr)
+// Two consecutive nodes of a filament per warp (float32), in cells at most one
+// apart along each axis: their neighbourhoods are almost the same (node
+// spacings are a fraction of the cut-off), so one walk over the union of their
+// rows serves both: the row search, the candidate's table look-up and its
+// record are paid once for two pair terms.  Every pair term is the one of
+// k_short_body, rounded alike; a lane adds each node's terms by itself.
+// Needs at least 2 (m + 2) cells per axis (no axis taken whole, the nearest
+// cell image is the minimum image of every candidate for both nodes).
+__device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>& ta, const SrTgt<float>& tb, int dx,
+                                             int dy, int dz, const int* __restrict__ prev,
+                                             const int* __restrict__ start, const SrRec<float>* __restrict__ src,
+                                             double* __restrict__ vsr, double* __restrict__ psr, int j,
+                                             ShortRows<float>& rows)
 {
-    const double* tab = sg_stage<T>(P.want_psi);
-    if constexpr (sizeof(T) == 8) {  // several groups of nodes per CTA: the tables are staged once
-        for (int b = blockIdx.x; b * kShortWarps < P.N; b += gridDim.x)
-            k_short_body<T>(P, tgt, prev, start, src, vsr, psr, b, tab);
-    } else {
-        k_short_body<T>(P, tgt, prev, start, src, vsr, psr, blockIdx.x, tab);
+    const int lane = threadIdx.x & 31;
+    const int wslot = threadIdx.x >> 5;
+    const int jp[2] = { prev[j], prev[j + 1] };
+    const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
+    const int cx = ta.cell % nc0;
+    const int cy = (ta.cell / nc0) % nc1;
+    const int cz = ta.cell / (nc0 * nc1);
+    const float h0 = (float)P.hc[0], h1 = (float)P.hc[1], h2 = (float)P.hc[2];
+    const float rc2 = (float)P.rc2;
+    const float alpha = (float)P.alpha;
+    const float two_over_sqrtpi = 1.12837916709551257390f;
+    const int m = P.m;
+    const int ny = 2 * m + 1 + abs(dy), nz = 2 * m + 1 + abs(dz);
+    const int y0 = min(dy, 0) - m, z0 = min(dz, 0) - m;  // first row offsets from the first node's cell
+    const int nrows = ny * nz;
+    const float rcm2 = rc2 * 1.0001f;
+    const float ih0 = 1.0f / h0;
+    const float dxf = (float)dx;
+    // the nodes' positions in their cells
+    const float ox[2] = { ta.o[0] + 0.5f * h0, tb.o[0] + 0.5f * h0 };
+    const float oy[2] = { ta.o[1] + 0.5f * h1, tb.o[1] + 0.5f * h1 };
+    const float oz[2] = { ta.o[2] + 0.5f * h2, tb.o[2] + 0.5f * h2 };
+    float v[2][3] = {}, ps[2][3] = {};
+    for (int rb = 0; rb < nrows; rb += 32) {
+        const int r = rb + lane;
+        int s0 = 0, n0 = 0, s1 = 0, n1r = 0, dyi = 0, dzi = 0;
+        int xo0 = 0, xo1 = 0;
+        if (r < nrows) {
+            const int iz = r / ny, iy = r - iz * ny;
+            dyi = y0 + iy;
+            dzi = z0 + iz;
+            // union of the two nodes' x ranges, offsets from the first node's cell
+            int lo = m + 2, hi = -m - 2;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int ey = dyi - (e ? dy : 0), ez = dzi - (e ? dz : 0);
+                float gy = ey > 0 ? ey * h1 - oy[e] : (ey < 0 ? oy[e] - (ey + 1) * h1 : 0.0f);
+                float gz = ez > 0 ? ez * h2 - oz[e] : (ez < 0 ? oz[e] - (ez + 1) * h2 : 0.0f);
+                gy = gy > 0.0f ? gy : 0.0f;
+                gz = gz > 0.0f ? gz : 0.0f;
+                const float d2 = gy * gy + gz * gz;
+                if (d2 < rcm2) {
+                    const float ext = sqrtf(rcm2 - d2);
+                    const int l = (int)floorf((ox[e] - ext) * ih0), u = (int)floorf((ox[e] + ext) * ih0);
+                    lo = min(lo, (l < -m ? -m : l) + (e ? dx : 0));
+                    hi = max(hi, (u > m ? m : u) + (e ? dx : 0));
+                }
+            }
+            if (lo <= hi) {
+                int zc = cz + dzi, yc = cy + dyi;
+                zc = zc < 0 ? zc + nc2 : (zc >= nc2 ? zc - nc2 : zc);
+                yc = yc < 0 ? yc + nc1 : (yc >= nc1 ? yc - nc1 : yc);
+                lo += cx;
+                hi += cx;
+                int xa0 = lo, xb0 = hi, xa1 = 0, xb1 = -1;
+                xo0 = -cx;
+                if (lo < 0) {
+                    xa0 = lo + nc0;
+                    xb0 = nc0 - 1;
+                    xb1 = hi;
+                    xo0 = -nc0 - cx;
+                    xo1 = -cx;
+                    if (hi < 0) {  // the whole run lies across the boundary
+                        xb0 = hi + nc0;
+                        xb1 = -1;
+                    }
+                } else if (hi >= nc0) {
+                    xb0 = nc0 - 1;
+                    xb1 = hi - nc0;
+                    xo1 = nc0 - cx;
+                    if (lo >= nc0) {
+                        xa0 = lo - nc0;
+                        xb0 = hi - nc0;
+                        xb1 = -1;
+                        xo0 = nc0 - cx;
+                    }
+                }
+                const int row = (zc * nc1 + yc) * nc0;
+                s0 = start[row + xa0];
+                n0 = start[row + xb0 + 1] - s0;
+                if (xb1 >= xa1) {
+                    s1 = start[row + xa1];
+                    n1r = start[row + xb1 + 1] - s1;
+                }
+            }
+        }
+        // the table and the walk over the candidates as in k_short_body
+        const int nr = n0 + n1r;
+        int inc = nr;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        const int total = __shfl_sync(0xffffffffu, inc, 31);
+        const int ex = inc - nr;
+        const unsigned nonempty = __ballot_sync(0xffffffffu, nr > 0);
+        if (nr > 0) {
+            const int ci = __popc(nonempty & ((1u << lane) - 1u));
+            rows.row[wslot][ci] = make_int4(s0, n0, s1, ex);
+            rows.ofs[wslot][ci] = make_int4(xo0, xo1, 0, 0);
+            *reinterpret_cast<float4*>(rows.dh[wslot][ci]) =
+                make_float4((float)dyi * h1, (float)dzi * h2, (float)(dyi - dy) * h1, (float)(dzi - dz) * h2);
+        }
+        __syncwarp();
+        const unsigned upto = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);
+        int jr = -1;
+        for (int cb = 0; cb < total; cb += 32) {  // warp-uniform trip count
+            const unsigned bit = (nr > 0 && ex >= cb && ex < cb + 32) ? (1u << (ex - cb)) : 0u;
+            const unsigned M = __reduce_or_sync(0xffffffffu, bit);
+            const int c = cb + lane;
+            const int own = jr + __popc(M & upto);
+            jr += __popc(M);
+            if (c >= total) continue;
+            const int4 rw = rows.row[wslot][own];
+            const int local = c - rw.w;
+            const bool first = local < rw.y;
+            const int k = first ? rw.x + local : rw.z + (local - rw.y);
+            const SrRec<float> S = src[k];
+            const int2 of = *reinterpret_cast<const int2*>(&rows.ofs[wslot][own]);
+            const float4 dh = *reinterpret_cast<const float4*>(rows.dh[wslot][own]);
+            const float xc = (float)(S.cx + (first ? of.x : of.y));
+            float rx[2], ry[2], rz[2], r2[2];
+            rx[0] = xc * h0 + (S.o[0] - ta.o[0]);
+            ry[0] = dh.x + (S.o[1] - ta.o[1]);
+            rz[0] = dh.y + (S.o[2] - ta.o[2]);
+            rx[1] = (xc - dxf) * h0 + (S.o[0] - tb.o[0]);
+            ry[1] = dh.z + (S.o[1] - tb.o[1]);
+            rz[1] = dh.w + (S.o[2] - tb.o[2]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) r2[e] = rx[e] * rx[e] + ry[e] * ry[e] + rz[e] * rz[e];
+            // C_0 of each node is left out
+            const bool in0 = r2[0] < rc2 && r2[0] != 0.0f && S.seg != j && S.seg != jp[0];
+            const bool in1 = r2[1] < rc2 && r2[1] != 0.0f && S.seg != j + 1 && S.seg != jp[1];
+            if (!(in0 || in1)) continue;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float ir = rsqrt_t(r2[e]);
+                const float rr = r2[e] * ir;
+                const float x = alpha * rr;
+                const float ee = exp_t(-x * x);
+                const float ec = erfc_e(x, ee);
+                const float g = ec + two_over_sqrtpi * x * ee;
+                float fv = g * ir * ir * ir;
+                fv = (e ? in1 : in0) ? fv : 0.0f;
+                v[e][0] += fv * (ry[e] * S.q[2] - rz[e] * S.q[1]);
+                v[e][1] += fv * (rz[e] * S.q[0] - rx[e] * S.q[2]);
+                v[e][2] += fv * (rx[e] * S.q[1] - ry[e] * S.q[0]);
+                if (P.want_psi) {
+                    const float fp = (e ? in1 : in0) ? ec * ir : 0.0f;
+                    ps[e][0] += fp * S.q[0];
+                    ps[e][1] += fp * S.q[1];
+                    ps[e][2] += fp * S.q[2];
+                }
+            }
+        }
+        __syncwarp();  // the table is rewritten by the next round of rows
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                v[e][c] += __shfl_xor_sync(0xffffffffu, v[e][c], o);
+                if (P.want_psi) ps[e][c] += __shfl_xor_sync(0xffffffffu, ps[e][c], o);
+            }
+    if (lane == 0) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                vsr[3 * (j + e) + c] = P.pref * (double)v[e][c];
+                if (P.want_psi) psr[3 * (j + e) + c] = P.pref * (double)ps[e][c];
+            }
     }
 }
 
+// Nodes per warp: pairs in float32 on grids wide enough for k_short_pair.
 template <typename T>
-__global__ void __launch_bounds__(256) k_short_b(const ShortD<T>* __restrict__ d, const int* __restrict__ bs, int n)
+__host__ __device__ __forceinline__ bool short_pairs(const ShortP& P)
 {
+    const int need = 2 * (P.m + 2);
+    return sizeof(T) == 4 && P.nc[0] >= need && P.nc[1] >= need && P.nc[2] >= need;
+}
+
+// One warp of the kernels below: a node, or with PAIR a pair of nodes where
+// the grid allows (pairs whose cells are further apart one after the other).
+// The two are separate kernels: the paired walk's registers would cost the
+// small grids that cannot use it half of their warps.
+template <typename T, bool PAIR>
+__device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __restrict__ tgt,
+                                             const int* __restrict__ prev, const int* __restrict__ start,
+                                             const SrRec<T>* __restrict__ src, double* __restrict__ vsr,
+                                             double* __restrict__ psr, int w, const double* __restrict__ tab,
+                                             ShortRows<T>& rows)
+{
+    int j = w, je = w + 1;
+    if constexpr (PAIR) {
+        if (short_pairs<T>(P)) {
+            j = 2 * w;
+            je = j + 2;
+            if (j + 1 < P.N) {
+                const SrTgt<float> ta = tgt[j], tb = tgt[j + 1];
+                const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
+                const int dx = cdiff(tb.cell % nc0, ta.cell % nc0, nc0);
+                const int dy = cdiff((tb.cell / nc0) % nc1, (ta.cell / nc0) % nc1, nc1);
+                const int dz = cdiff(tb.cell / (nc0 * nc1), ta.cell / (nc0 * nc1), nc2);
+                if (abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1) {
+                    k_short_pair(P, ta, tb, dx, dy, dz, prev, start, src, vsr, psr, j, rows);
+                    return;
+                }
+            }
+        }
+    }
+    for (; j < je && j < P.N; ++j) k_short_body<T>(P, tgt, prev, start, src, vsr, psr, j, tab, rows);
+}
+
+template <typename T, bool PAIR>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (PAIR ? 4 : 5) : 3) k_short(ShortP P, const SrTgt<T>* __restrict__ tgt, const int* __restrict__ prev,
+                                               const int* __restrict__ start, const SrRec<T>* __restrict__ src,
+                                               double* __restrict__ vsr, double* __restrict__ psr)
+{
+    __shared__ ShortRows<T> rows;
+    const double* tab = sg_stage<T>(P.want_psi);
+    const int wid = threadIdx.x >> 5;
+    if constexpr (sizeof(T) == 8) {  // several groups of nodes per CTA: the tables are staged once
+        for (int b = blockIdx.x; b * kShortWarps < P.N; b += gridDim.x)
+            k_short_warp<T, PAIR>(P, tgt, prev, start, src, vsr, psr, b * kShortWarps + wid, tab, rows);
+    } else {
+        k_short_warp<T, PAIR>(P, tgt, prev, start, src, vsr, psr, blockIdx.x * kShortWarps + wid, tab, rows);
+    }
+}
+
+template <typename T, bool PAIR>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (PAIR ? 4 : 5) : 3) k_short_b(const ShortD<T>* __restrict__ d, const int* __restrict__ bs, int n)
+{
+    __shared__ ShortRows<T> rows;
     int bid, nb;
     const ShortD<T>& a = d[batch_member(bs, n, bid, nb)];
     const double* tab = sg_stage<T>(a.P.want_psi);
-    k_short_body<T>(a.P, a.tgt, a.prev, a.start, a.src, a.vsr, a.psr, bid, tab);
+    k_short_warp<T, PAIR>(a.P, a.tgt, a.prev, a.start, a.src, a.vsr, a.psr,
+                          bid * kShortWarps + (int)(threadIdx.x >> 5), tab, rows);
+}
+
+bool short_can_pair(const ShortP& P, int precision) { return precision == BS_MIXED && short_pairs<float>(P); }
+
+int short_blocks(const ShortP& P, bool pairs)
+{
+    const long long warps = pairs ? (P.N + 1LL) / 2 : P.N;
+    return (int)((warps + kShortWarps - 1) / kShortWarps);
 }
 
 // ---------------------------------------------------------------------------
@@ -758,11 +1006,19 @@ cudaError_t launch_short(const ShortP& P, const Work& w, cudaStream_t s)
     const bool tiled = P.m <= kShortTileMaxM && P.kernel == 1;
     if (!tiled) {
         const int tb = 32 * kShortWarps;  // one warp per target
-        const long long blocks = (P.N + kShortWarps - 1LL) / kShortWarps;
+        const bool pairs = short_can_pair(P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED);
+        const long long blocks = short_blocks(P, pairs);
         // float64: at most 16 CTAs per SM, each on several groups of nodes
         const unsigned g = (unsigned)(sizeof(T) == 8 && blocks > 16 * 152 ? 16 * 152 : blocks);
-        k_short<T><<<g, tb, 0, s>>>(
-            P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt, (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
+        if constexpr (sizeof(T) == 4) {
+            if (pairs) {
+                k_short<T, true><<<g, tb, 0, s>>>(P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt,
+                                                  (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
+                return cudaGetLastError();
+            }
+        }
+        k_short<T, false><<<g, tb, 0, s>>>(P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt,
+                                           (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
         return cudaGetLastError();
     }
     // nodes by target block: count, scan, scatter
@@ -784,7 +1040,14 @@ cudaError_t launch_short(const ShortP& P, const Work& w, cudaStream_t s)
 template <typename T>
 cudaError_t launch_short_b(const BatchL& L, cudaStream_t s)
 {
-    if (L.total > 0) k_short_b<T><<<L.total, 32 * kShortWarps, 0, s>>>((const ShortD<T>*)L.desc, L.bstart, L.n);
+    if (L.total <= 0) return cudaSuccess;
+    if constexpr (sizeof(T) == 4) {
+        if (L.kind) {
+            k_short_b<T, true><<<L.total, 32 * kShortWarps, 0, s>>>((const ShortD<T>*)L.desc, L.bstart, L.n);
+            return cudaGetLastError();
+        }
+    }
+    k_short_b<T, false><<<L.total, 32 * kShortWarps, 0, s>>>((const ShortD<T>*)L.desc, L.bstart, L.n);
     return cudaGetLastError();
 }
 
