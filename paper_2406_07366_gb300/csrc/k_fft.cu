@@ -1148,6 +1148,162 @@ __device__ __forceinline__ void spread_bucketed(const SpZP& P, int s0, int s1, c
     flush(hi, zs + W + t);
 }
 
+// Two float32 values in a register pair and their packed arithmetic (each
+// half rounded as the scalar operation).
+__device__ __forceinline__ unsigned long long pk2(float lo, float hi)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 upk2(unsigned long long v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// The bucketed loop in float32.  It is bound by the instructions per copy (65
+// in spread_bucketed, 12 copies per point on the 4e6-node tangle), so the
+// index work is done once per copy while it is staged and not by every lane
+// at every copy: four lanes per copy pick the weights that the block needs
+// out of the point's record and lay them down at fixed places, weights
+// outside the support as zeros, the z weights rotated so that lane t finds
+// its own at place t, charges and x weights twice for packed arithmetic.  A
+// lane's two cells are the halves of a register pair: per column one packed
+// product and three packed multiply-adds.  About 25 instructions per copy.
+// The next chunk's words are in registers while this one is added.
+constexpr int kSpzShare = 16;  // copies per warp before another warp of the CTA takes part
+template <int W, int TX>
+constexpr int spz_head() { return (6 + 2 * TX + 1 + 3) & ~3; }  // charges, x weights, z start: words
+template <int W, int TX>
+constexpr int spz_stride() { return (spz_head<W, TX>() + 4 + W + 3) & ~3; }
+
+template <int W, int TX>
+__device__ __forceinline__ void spread_bucketed_f(const SpZP& P, int s0, int s1, const int2* __restrict__ cidx,
+                                                  const SpPt<float, W>* __restrict__ pts, float* sbuf, float* accf)
+{
+    using U = unsigned long long;
+    constexpr int RCW = kSpzWarpChunk, A = spz_head<W, TX>(), ST = spz_stride<W, TX>(), NZ = (W + 3) / 4;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int n2 = P.ng[2], Ty = P.ty, CS = P.cls;
+    const int sx = Ty * CS, sc = TX * Ty * CS;  // float offsets of lx + 1 and of component c + 1
+    const int n = s1 - s0;
+    const int nw = min((int)(blockDim.x >> 5), (n + kSpzShare - 1) / kSpzShare);
+    if (wid >= nw) return;
+    const int e0 = s0 + (int)((wid * (long long)n) / nw), e1 = s0 + (int)(((wid + 1) * (long long)n) / nw);
+    if (e0 >= e1) return;
+    float* wb = sbuf + wid * RCW * ST;
+    const int ly = lane / W, t = lane - ly * W;
+    const bool slot = lane < Ty * W;
+    const float* wyp = wb + A + (slot ? ly : 0);
+    const float* wzp = wb + A + 4 + t;
+    const int ab0 = ((ly >> 1) * CS) * 2 + (ly & 1);  // float offset of (lx 0, ly, z 0, component 0)
+    U acc[TX][3];  // (cell at zs + t, cell at zs + W + t)
+#pragma unroll
+    for (int a = 0; a < TX; ++a)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[a][c] = 0;
+    auto flush = [&](int half, int z) {
+        z = z >= n2 ? z - n2 : z;
+        if (slot) {
+            const int ab = ab0 + 2 * z;
+#pragma unroll
+            for (int a = 0; a < TX; ++a)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const float2 v = upk2(acc[a][c]);
+                    atomicAdd(&accf[ab + a * sx + c * sc], half ? v.y : v.x);
+                }
+        }
+    };
+    const int cp = lane >> 2, p = lane & 3;  // staging: copy of the chunk, part
+    float nq = 0, nwx = 0, nwy = 0, nwz[NZ];
+    int nmeta = 0;
+    auto entry = [&](int c0) { return c0 + cp < e1 ? __ldg(cidx + c0 + cp) : make_int2(-1, 0); };
+    auto fetch = [&](int2 e) {
+        nq = nwx = nwy = 0;
+#pragma unroll
+        for (int i = 0; i < NZ; ++i) nwz[i] = 0;
+        if (e.x < 0) return;
+        const float* rec = reinterpret_cast<const float*>(pts + e.x);  // base, q, wx, wy, wz
+        const int jx = p - ((e.y & 255) - 128), jy = p - (((e.y >> 8) & 255) - 128), d = (e.y >> 16) & 15;
+        if (p < 3) nq = __ldg(rec + 1 + p);
+        if (p < TX && (unsigned)jx < (unsigned)W) nwx = __ldg(rec + 4 + jx);
+        if (p < Ty && (unsigned)jy < (unsigned)W) nwy = __ldg(rec + 4 + W + jy);
+#pragma unroll
+        for (int i = 0; i < NZ; ++i) {
+            const int tt = p + 4 * i, j = tt - d < 0 ? tt - d + W : tt - d;
+            if (tt < W) nwz[i] = __ldg(rec + 4 + 2 * W + j);
+        }
+        nmeta = ((e.y >> 20) << 4) | d;
+    };
+    auto put = [&]() {
+        float* d = wb + cp * ST;
+        if (p < 3) *reinterpret_cast<float2*>(d + 2 * p) = make_float2(nq, nq);
+        if (p < TX) *reinterpret_cast<float2*>(d + 6 + 2 * p) = make_float2(nwx, nwx);
+        if (p == 3) reinterpret_cast<int*>(d)[6 + 2 * TX] = nmeta;
+        d[A + p] = nwy;
+#pragma unroll
+        for (int i = 0; i < NZ; ++i)
+            if (p + 4 * i < W) d[A + 4 + p + 4 * i] = nwz[i];
+    };
+    int zs = -1;  // start of the warp's current bucket (none yet)
+    fetch(entry(e0));
+    int2 en = entry(e0 + RCW);
+    for (int c0 = e0; c0 < e1; c0 += RCW) {
+        put();
+        __syncwarp();
+        fetch(en);  // the next chunk, and the entries of the one after
+        en = entry(c0 + 2 * RCW);
+        const int nch = min(RCW, e1 - c0);
+#pragma unroll 1
+        for (int k = 0; k < nch; ++k) {
+            const float* r = wb + k * ST;
+            const ulonglong2 q01 = *reinterpret_cast<const ulonglong2*>(r);  // charges, each twice
+            const U q2 = *reinterpret_cast<const U*>(r + 4);
+            const int meta = reinterpret_cast<const int*>(r)[6 + 2 * TX];
+            const float wyz = wyp[k * ST] * wzp[k * ST];
+            const int zsb = meta >> 4;
+            if (zsb != zs) {  // the same in the whole warp
+                if (zs >= 0) {
+                    flush(0, zs + t);
+                    if (zsb != zs + W) flush(1, zs + W + t);
+#pragma unroll
+                    for (int a = 0; a < TX; ++a)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) acc[a][c] = zsb == zs + W ? pk2(upk2(acc[a][c]).y, 0.f) : 0;
+                }
+                zs = zsb;
+            }
+            const bool first = t >= (meta & 15);
+            const U wlh = pk2(first ? wyz : 0.f, first ? 0.f : wyz);
+#pragma unroll
+            for (int a = 0; a < TX; ++a) {
+                const U v = mul2(*reinterpret_cast<const U*>(r + 6 + 2 * a), wlh);
+                acc[a][0] = fma2(v, q01.x, acc[a][0]);
+                acc[a][1] = fma2(v, q01.y, acc[a][1]);
+                acc[a][2] = fma2(v, q2, acc[a][2]);
+            }
+        }
+        __syncwarp();  // every lane is done with the buffer before it is refilled
+    }
+    flush(0, zs + t);
+    flush(1, zs + W + t);
+}
+
 template <typename T, int W, int RM>
 __device__ __forceinline__ void k_spread_zfft_body(const SpZP& P, const int* __restrict__ cstart,
                                                    const int2* __restrict__ cidx,
@@ -1193,10 +1349,19 @@ __device__ __forceinline__ void k_spread_zfft_body(const SpZP& P, const int* __r
     }
     if (P.nzb > 1) {
         __syncthreads();  // the lines are zeroed
-        switch (Tx) {
-        case 1: spread_bucketed<T, W, 1>(P, s0, s1, cidx, pts, sbuf, accf); break;
-        case 2: spread_bucketed<T, W, 2>(P, s0, s1, cidx, pts, sbuf, accf); break;
-        default: spread_bucketed<T, W, 4>(P, s0, s1, cidx, pts, sbuf, accf); break;
+        if constexpr (sizeof(T) == 4) {
+            float* sf = reinterpret_cast<float*>(sbuf);
+            switch (Tx) {
+            case 1: spread_bucketed_f<W, 1>(P, s0, s1, cidx, pts, sf, accf); break;
+            case 2: spread_bucketed_f<W, 2>(P, s0, s1, cidx, pts, sf, accf); break;
+            default: spread_bucketed_f<W, 4>(P, s0, s1, cidx, pts, sf, accf); break;
+            }
+        } else {
+            switch (Tx) {
+            case 1: spread_bucketed<T, W, 1>(P, s0, s1, cidx, pts, sbuf, accf); break;
+            case 2: spread_bucketed<T, W, 2>(P, s0, s1, cidx, pts, sbuf, accf); break;
+            default: spread_bucketed<T, W, 4>(P, s0, s1, cidx, pts, sbuf, accf); break;
+            }
         }
         __syncthreads();
         fft_fwd_dif<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
