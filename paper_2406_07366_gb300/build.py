@@ -23,6 +23,8 @@ LIB = os.path.join(LIBDIR, "libbsewald.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["bs_api.cu", "k_geometry.cu", "k_sort.cu", "k_short.cu", "k_long.cu", "k_fft.cu", "k_static_short.cu", "k_rk4.cu",
            "k_peak.cu"]
+# sources compiled a second time with a macro: the transform kernels, an object per precision
+VARIANTS = [("k_fft.cu", "k_fft_f64.o", ["-DBSW_FFT_DOUBLE"])]
 
 
 def _nvcc() -> str:
@@ -57,12 +59,13 @@ def build_library(verbose: bool = False, extra_flags=None, force: bool = False) 
     flags = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC,
                     "--expt-relaxed-constexpr"] + list(extra_flags or [])
     objs, jobs = [], []
-    for src in SOURCES:
+    units = [(src, src.replace(".cu", ".o"), []) for src in SOURCES] + VARIANTS
+    for src, obj, extra in sorted(units, key=lambda u: u[0] != "k_fft.cu"):  # the longest first
         s = os.path.join(CSRC, src)
-        o = os.path.join(BUILD, src.replace(".cu", ".o"))
+        o = os.path.join(BUILD, obj)
         objs.append(o)
         if force or _stale(o, [s] + headers):
-            jobs.append([nvcc, "-c", s, "-o", o] + flags)
+            jobs.append([nvcc, "-c", s, "-o", o] + flags + extra)
 
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)

@@ -135,6 +135,12 @@ FftPlan make_plan(int n, int maxr)
     pl.n = n;
     std::vector<int> cur, best;
     plan_search(n, maxr, 0, cur, best);
+    // a 6 goes last: the kernels' boundary passes are built on it
+    const auto six = std::find(best.begin(), best.end(), 6);
+    if (six != best.end()) {
+        best.erase(six);
+        best.push_back(6);
+    }
     pl.nr = (int)best.size();
     for (int s = 0; s < pl.nr; ++s) pl.r[s] = best[s];
     int L = n;
@@ -1235,7 +1241,7 @@ int bs_create(bs_ctx** out, const bs_params* p, void* stream)
         return rc;
     }
     cudaError_t e = cudaGetDevice(&c->device);
-    if (e == cudaSuccess) e = set_fft_constants();
+    if (e == cudaSuccess) e = p->precision == BS_FP64 ? set_fft_constants<double>() : set_fft_constants<float>();
     if (e == cudaSuccess) e = set_short_tables();
     if (e == cudaSuccess) e = set_node_tables();
     // the short-range branch runs at the highest stream priority: its few

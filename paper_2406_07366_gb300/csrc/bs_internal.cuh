@@ -422,6 +422,7 @@ template <typename T>
 cudaError_t launch_spread_zfft(const SpZP& P, const Work& w, cudaStream_t s);
 template <typename T>
 size_t col_pt_bytes(int w);
+template <typename T>
 cudaError_t set_fft_constants();
 cudaError_t set_short_tables();
 cudaError_t set_node_tables();

@@ -187,8 +187,8 @@ __device__ __forceinline__ unsigned char* smem_align128(unsigned char* p)
 // (set_fft_constants).  Indices are compile-time constants after unrolling,
 // so the factors come straight from the constant bank.
 constexpr int kTwOff6 = 0, kTwOff9 = 6, kTwOff12 = 15, kTwOff16 = 27, kTwOff24 = 43, kTwOff32 = 67, kTwCount = 99;
-__constant__ float2 c_twf[kTwCount];
-__constant__ double2 c_twd[kTwCount];
+static __constant__ float2 c_twf[kTwCount];
+static __constant__ double2 c_twd[kTwCount];
 
 template <int R> struct TwOff;
 template <> struct TwOff<6> { static constexpr int v = kTwOff6; };
@@ -463,22 +463,27 @@ __device__ __forceinline__ void fft_pass_c(typename Cx<T>::t* __restrict__ buf, 
     }
 }
 
-// Transform of plan (Rs...) with N = product of the radices and NL lines:
-// forward passes in plan order (stride N / R0 first), inverse in reverse.
+// Passes of plan (Rs...) with N = product of the radices and NL lines, all but
+// the last radix's (which the boundary passes below take): forward in plan
+// order (stride N / R0 first), inverse in reverse.
 template <typename T, bool TR, int NL, int N, int ST, int TWS, int R, int... Rest>
 __device__ __forceinline__ void fft_c_fwd(typename Cx<T>::t* buf, int ls, const typename Cx<T>::t* __restrict__ tw)
 {
-    fft_pass_c<T, R, true, N, ST / R, TWS, NL, TR>(buf, ls, tw);
-    __syncthreads();
-    if constexpr (sizeof...(Rest) > 0) fft_c_fwd<T, TR, NL, N, ST / R, TWS * R, Rest...>(buf, ls, tw);
+    if constexpr (sizeof...(Rest) > 0) {
+        fft_pass_c<T, R, true, N, ST / R, TWS, NL, TR>(buf, ls, tw);
+        __syncthreads();
+        fft_c_fwd<T, TR, NL, N, ST / R, TWS * R, Rest...>(buf, ls, tw);
+    }
 }
 
 template <typename T, bool TR, int NL, int N, int ST, int TWS, int R, int... Rest>
 __device__ __forceinline__ void fft_c_inv(typename Cx<T>::t* buf, int ls, const typename Cx<T>::t* __restrict__ tw)
 {
-    if constexpr (sizeof...(Rest) > 0) fft_c_inv<T, TR, NL, N, ST / R, TWS * R, Rest...>(buf, ls, tw);
-    fft_pass_c<T, R, false, N, ST / R, TWS, NL, TR>(buf, ls, tw);
-    __syncthreads();
+    if constexpr (sizeof...(Rest) > 0) {
+        fft_c_inv<T, TR, NL, N, ST / R, TWS * R, Rest...>(buf, ls, tw);
+        fft_pass_c<T, R, false, N, ST / R, TWS, NL, TR>(buf, ls, tw);
+        __syncthreads();
+    }
 }
 
 template <typename T, bool DIF, bool TR, int NL, int... Rs>
@@ -503,8 +508,8 @@ __device__ __forceinline__ bool plan_is(const FftPlan& pl)
 }
 
 // Plans with a compiled form (float): 384 = 8 x 8 x 6 at 12, 16 or 24 lines
-// (the 1e5-node tangle), 768 = 8 x 6 x 4 x 4 at 6, 8, 12 or 16 lines (the 4e6-node
-// tangle), 192 = 8 x 6 x 4 at 16 or 24 lines (the largest batch members).
+// (the 1e5-node tangle), 768 = 8 x 4 x 4 x 6 at 6, 8, 12 or 16 lines (the 4e6-node
+// tangle), 192 = 8 x 4 x 6 at 16 or 24 lines (the largest batch members).
 template <typename T, bool DIF, bool TR = false>
 __device__ __forceinline__ bool fft_const(typename Cx<T>::t* buf, int nlines, int ls, const FftPlan& pl,
                                           const typename Cx<T>::t* __restrict__ tw)
@@ -517,18 +522,18 @@ __device__ __forceinline__ bool fft_const(typename Cx<T>::t* buf, int nlines, in
             case 24: fft_c<T, DIF, TR, 24, 8, 8, 6>(buf, ls, tw); return true;
             default: break;
             }
-        } else if (plan_is<8, 6, 4, 4>(pl)) {
+        } else if (plan_is<8, 4, 4, 6>(pl)) {
             switch (nlines) {
-            case 6: fft_c<T, DIF, TR, 6, 8, 6, 4, 4>(buf, ls, tw); return true;
-            case 8: fft_c<T, DIF, TR, 8, 8, 6, 4, 4>(buf, ls, tw); return true;
-            case 12: fft_c<T, DIF, TR, 12, 8, 6, 4, 4>(buf, ls, tw); return true;
-            case 16: fft_c<T, DIF, TR, 16, 8, 6, 4, 4>(buf, ls, tw); return true;
+            case 6: fft_c<T, DIF, TR, 6, 8, 4, 4, 6>(buf, ls, tw); return true;
+            case 8: fft_c<T, DIF, TR, 8, 8, 4, 4, 6>(buf, ls, tw); return true;
+            case 12: fft_c<T, DIF, TR, 12, 8, 4, 4, 6>(buf, ls, tw); return true;
+            case 16: fft_c<T, DIF, TR, 16, 8, 4, 4, 6>(buf, ls, tw); return true;
             default: break;
             }
-        } else if (plan_is<8, 6, 4>(pl)) {
+        } else if (plan_is<8, 4, 6>(pl)) {
             switch (nlines) {
-            case 16: fft_c<T, DIF, TR, 16, 8, 6, 4>(buf, ls, tw); return true;
-            case 24: fft_c<T, DIF, TR, 24, 8, 6, 4>(buf, ls, tw); return true;
+            case 16: fft_c<T, DIF, TR, 16, 8, 4, 6>(buf, ls, tw); return true;
+            case 24: fft_c<T, DIF, TR, 24, 8, 4, 6>(buf, ls, tw); return true;
             default: break;
             }
         }
@@ -565,7 +570,6 @@ template <typename T, int RM, bool TR = false>
 __device__ __forceinline__ void fft_fwd_dif(typename Cx<T>::t* buf, int nlines, const FastDiv& dl, int ls, const FftPlan& pl,
                             const typename Cx<T>::t* __restrict__ tw)
 {
-    if (fft_const<T, true, TR>(buf, nlines, ls, pl, tw)) return;
     for (int s = 0; s < pl.nr; ++s) fft_stage<T, true, RM, TR>(buf, nlines, dl, ls, pl, s, tw);
 }
 
@@ -575,10 +579,118 @@ template <typename T, int RM, bool TR = false>
 __device__ __forceinline__ void fft_inv_dit(typename Cx<T>::t* buf, int nlines, const FastDiv& dl, int ls, const FftPlan& pl,
                             const typename Cx<T>::t* __restrict__ tw)
 {
-    if (fft_const<T, false, TR>(buf, nlines, ls, pl, tw)) return;
     for (int s = pl.nr - 1; s >= 0; --s) fft_stage<T, false, RM, TR>(buf, nlines, dl, ls, pl, s, tw);
 }
 
+// ---- boundary passes ----
+// The transforms keep the frequencies |k| <= K < n / 3 only.  With a last
+// radix of 6 (stride 1, no twiddles) butterfly c holds, at positions rev(c) ..
+// rev(c) + 5, the frequencies c + q B, q = 0..5, B = n / 6, of which q = 2 and 3
+// are never kept.  So that pass need not go through shared memory: the forward
+// transform's last pass hands its outputs straight to whoever consumes the
+// modes, the inverse one's first pass takes its inputs straight from their
+// source, the x pass's two meet in registers around the k-space step, and the
+// zero padding is never written or read.  These kernels are bound by shared
+// memory (65-70 % of its bandwidth on the 384^3 grid), and this removes 2 of 7
+// (y), 4 of 14 (x) and about a third (z) of their accesses.
+// The other plans (no factor 3, or K >= n / 3) take the general passes.
+template <typename P>
+__device__ __forceinline__ bool fuse6(const P& pl, int K)
+{
+    return pl.nr >= 2 && pl.r[pl.nr - 1] == 6 && 3 * K < pl.n;
+}
+
+// All forward passes but the last; all inverse passes but the first.
+template <typename T, int RM, bool TR = false>
+__device__ __forceinline__ void fft_fwd_head(typename Cx<T>::t* buf, int nlines, const FastDiv& dl, int ls,
+                                             const FftPlan& pl, const typename Cx<T>::t* __restrict__ tw)
+{
+    if (fft_const<T, true, TR>(buf, nlines, ls, pl, tw)) return;
+    for (int s = 0; s < pl.nr - 1; ++s) fft_stage<T, true, RM, TR>(buf, nlines, dl, ls, pl, s, tw);
+}
+template <typename T, int RM, bool TR = false>
+__device__ __forceinline__ void fft_inv_tail(typename Cx<T>::t* buf, int nlines, const FastDiv& dl, int ls,
+                                             const FftPlan& pl, const typename Cx<T>::t* __restrict__ tw)
+{
+    if (fft_const<T, false, TR>(buf, nlines, ls, pl, tw)) return;
+    for (int s = pl.nr - 2; s >= 0; --s) fft_stage<T, false, RM, TR>(buf, nlines, dl, ls, pl, s, tw);
+}
+
+// dft<T, 6, +1> of an input whose x[2] and x[3] are zero (not read).
+template <typename T>
+__device__ __forceinline__ void idft6p(typename Cx<T>::t* x)
+{
+    using C = typename Cx<T>::t;
+    const T h = (T)0.86602540378443864676;
+    C y[2][3];  // 3-point transforms of (x0, 0, x4) and (x1, 0, x5)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        const C u = x[b], v = x[4 + b];
+        C t;
+        t.x = u.x - (T)0.5 * v.x;
+        t.y = u.y - (T)0.5 * v.y;
+        y[b][0] = cadd(u, v);
+        y[b][1].x = t.x + h * v.y;
+        y[b][1].y = t.y - h * v.x;
+        y[b][2].x = t.x - h * v.y;
+        y[b][2].y = t.y + h * v.x;
+    }
+#pragma unroll
+    for (int k = 1; k < 3; ++k) {
+        C w = ctw<T>(TwOff<6>::v + k);  // e^{-2 pi i k / 6}
+        w.y = -w.y;
+        y[1][k] = cmul(y[1][k], w);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        x[k] = cadd(y[0][k], y[1][k]);
+        x[k + 3] = csub(y[0][k], y[1][k]);
+    }
+}
+
+// Butterflies c and B - c of a pair of real z-lines A, B packed as A + i B hold
+// between them the modes c, B + c, B - c and 2 B - c and their mirrors.
+// Inverse: from the modes m[] = {c, B + c, B - c, 2 B - c} of both rows (zero
+// beyond K) the two butterflies' outputs X (c) and Y (B - c).
+template <typename T>
+__device__ __forceinline__ void z_pair_inverse(const typename Cx<T>::t* A, const typename Cx<T>::t* Bv, int c,
+                                               typename Cx<T>::t* X, typename Cx<T>::t* Y)
+{
+    using C = typename Cx<T>::t;
+    C p[4], m[4];  // Z at the modes and at their mirrors
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        p[e].x = A[e].x - Bv[e].y;
+        p[e].y = A[e].y + Bv[e].x;
+        m[e].x = A[e].x + Bv[e].y;
+        m[e].y = -A[e].y + Bv[e].x;
+    }
+    if (c == 0) {
+        p[0].x = A[0].x;
+        p[0].y = Bv[0].x;
+    }
+    X[0] = p[0];
+    X[1] = p[1];
+    X[4] = m[3];
+    X[5] = m[2];
+    Y[0] = p[2];
+    Y[1] = p[3];
+    Y[4] = m[1];
+    Y[5] = m[0];
+    idft6p<T>(X);
+    idft6p<T>(Y);
+}
+
+// Items of a z boundary pass: i -> line l and c = 0..B/2, four consecutive c
+// on consecutive lanes (a 32-byte sector of a mode row), then the lines
+// (distinct banks at the odd line stride).  c > B/2: no item.
+__device__ __forceinline__ void z_item(int i, int ncl, const FastDiv& d_ncl, int& l, int& c)
+{
+    const int j = i >> 2, g = fdiv(j, d_ncl);
+    l = j - g * ncl;
+    c = 4 * g + (i & 3);
+}
+__device__ __forceinline__ int z_items(int B, int ncl) { return ((B / 2 + 4) >> 2) * 4 * ncl; }
 
 // Digit-reversed positions of 8 consecutive frequencies 8q + d (and of
 // n - 8q - d) when the plan's first radix is 8 (stride st0 = n / 8): the first
@@ -984,6 +1096,76 @@ __device__ __forceinline__ void spz_unpack(const SpZP& P, const typename Cx<T>::
     }
 }
 
+// The forward boundary pass of a spread block: the last pass of every complex
+// z-line, the separation of its two real lines and the store of their modes.
+template <typename T>
+__device__ __forceinline__ void spz_tail6(const SpZP& P, const typename Cx<T>::t* cb, typename Cx<T>::t* F1, int bx,
+                                          int by)
+{
+    using C = typename Cx<T>::t;
+    const int Tx = P.tx, Ty = P.ty, n2 = P.ng[2], CS = P.cls, K = P.K[2];
+    const int txy = Tx * Ty, ncl = 3 * txy / 2, B = n2 / 6, nk = K + 1;
+    const int tot = z_items(B, ncl);
+    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+        int l, c;
+        z_item(i, ncl, P.d_ncl, l, c);
+        if (2 * c > B) continue;
+        C X[6], Y[6];
+        const C* px = cb + l * CS + P.rev[c];
+        const C* py = cb + l * CS + P.rev[c == 0 ? 0 : B - c];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) X[q] = px[q];
+        dft<T, 6, -1>(X);
+        if (c == 0) {  // its own mirror: mode 0 with itself, B with -B
+            Y[5] = X[0];
+            Y[4] = X[5];
+        } else {
+#pragma unroll
+            for (int q = 0; q < 6; ++q) Y[q] = py[q];
+            dft<T, 6, -1>(Y);
+        }
+        C* dst[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int rl = 2 * l + r;
+            const int cc = fdiv(rl, P.d_txy), rem = rl - cc * txy;
+            const int lx = fdiv(rem, P.d_ty), ly = rem - lx * Ty;
+            dst[r] = F1 + (((size_t)cc * P.ng[0] + bx * Tx + lx) * P.ng[1] + by * Ty + ly) * nk;
+        }
+        auto put = [&](int m, const C& zk, const C& zn) {
+            if (m > K) return;
+            C o;  // A_k = (Z_k + conj Z_{-k}) / 2, B_k = (Z_k - conj Z_{-k}) / (2i)
+            o.x = (T)0.5 * (zk.x + zn.x);
+            o.y = (T)0.5 * (zk.y - zn.y);
+            dst[0][m] = o;
+            o.x = (T)0.5 * (zk.y + zn.y);
+            o.y = (T)0.5 * (zn.x - zk.x);
+            dst[1][m] = o;
+        };
+        put(c, X[0], Y[5]);
+        put(B + c, X[1], Y[4]);
+        if (c > 0 && 2 * c < B) {
+            put(B - c, Y[0], X[5]);
+            put(2 * B - c, Y[1], X[4]);
+        }
+    }
+}
+
+// z transform of a spread block's lines and the store of their modes.
+template <typename T, int RM>
+__device__ __forceinline__ void spz_transform(const SpZP& P, typename Cx<T>::t* cb, int ncl, int CS,
+                                              const typename Cx<T>::t* __restrict__ tw2, typename Cx<T>::t* F1, int bx,
+                                              int by)
+{
+    if (fuse6(P.plan2, P.K[2])) {
+        fft_fwd_head<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
+        spz_tail6<T>(P, cb, F1, bx, by);
+    } else {
+        fft_fwd_dif<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
+        spz_unpack<T>(P, cb, F1, bx, by);
+    }
+}
+
 // Bytes of a block's complex z-lines in shared memory, rounded up to 16 so
 // that the record buffer after them takes 16-byte copies (an odd count of
 // float32 lines at an odd stride would leave it 8-byte aligned).
@@ -1364,8 +1546,7 @@ __device__ __forceinline__ void k_spread_zfft_body(const SpZP& P, const int* __r
             }
         }
         __syncthreads();
-        fft_fwd_dif<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
-        spz_unpack<T>(P, cb, F1, bx, by);
+        spz_transform<T, RM>(P, cb, ncl, CS, tw2, F1, bx, by);
         return;
     }
     // deterministic mode: warp wid owns z in [zlo, zhi) and adds every record
@@ -1484,8 +1665,7 @@ __device__ __forceinline__ void k_spread_zfft_body(const SpZP& P, const int* __r
         }
     }
     __syncthreads();
-    fft_fwd_dif<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
-    spz_unpack<T>(P, cb, F1, bx, by);
+    spz_transform<T, RM>(P, cb, ncl, CS, tw2, F1, bx, by);
 }
 
 template <typename T, int W, int RM>
@@ -1503,6 +1683,55 @@ __global__ void __launch_bounds__(z_threads_max<T>(), 2) k_spread_zfft(SpZP P, c
 // forward: F1[c][x][y][mz] -> F2[c][x][my'][mz], my' = my + K1, |my| <= K1
 // inverse: F2 -> F1 (zero-padded to n1)
 // ---------------------------------------------------------------------------
+// Boundary passes along y: a thread per (butterfly c, mode l), the lanes on
+// consecutive modes.  Row y of line l sits at y MC + l (TR) or l LS + y.
+template <typename T, bool TR>
+__device__ __forceinline__ void y_tail6(const FftYP& P, const typename Cx<T>::t* a, typename Cx<T>::t* __restrict__ F2,
+                                        int cx, int mz0, int mcount)
+{
+    using C = typename Cx<T>::t;
+    const int B = P.ng[1] / 6, K1 = P.K[1], nk = P.K[2] + 1, MC = 1 << P.lmc, es = TR ? MC : 1;
+    const int l = threadIdx.x & (MC - 1);
+    if (l >= mcount) return;
+    C* dst = F2 + ((size_t)cx * (2 * K1 + 1) + K1) * nk + mz0 + l;  // row my = 0
+    for (int c = threadIdx.x >> P.lmc; c < B; c += blockDim.x >> P.lmc) {
+        const C* p = a + (TR ? (size_t)P.rev[c] * MC + l : (size_t)l * P.ls + P.rev[c]);
+        C x[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) x[q] = p[q * es];
+        dft<T, 6, -1>(x);
+        if (c <= K1) dst[(long long)c * nk] = x[0];
+        if (c + B <= K1) dst[(long long)(c + B) * nk] = x[1];
+        if (2 * B - c <= K1) dst[(long long)(c - 2 * B) * nk] = x[4];
+        if (B - c <= K1) dst[(long long)(c - B) * nk] = x[5];
+    }
+}
+template <typename T, bool TR>
+__device__ __forceinline__ void y_head6(const FftYP& P, typename Cx<T>::t* a, const typename Cx<T>::t* __restrict__ F2,
+                                        int cx, int mz0, int mcount)
+{
+    using C = typename Cx<T>::t;
+    const int B = P.ng[1] / 6, K1 = P.K[1], nk = P.K[2] + 1, MC = 1 << P.lmc, es = TR ? MC : 1;
+    const int l = threadIdx.x & (MC - 1);
+    const bool live = l < mcount;
+    const C* src = F2 + ((size_t)cx * (2 * K1 + 1) + K1) * nk + mz0 + l;  // row my = 0
+    C zero;
+    zero.x = 0;
+    zero.y = 0;
+#pragma unroll 2
+    for (int c = threadIdx.x >> P.lmc; c < B; c += blockDim.x >> P.lmc) {
+        C x[6];
+        x[0] = live && c <= K1 ? src[(long long)c * nk] : zero;
+        x[1] = live && c + B <= K1 ? src[(long long)(c + B) * nk] : zero;
+        x[4] = live && 2 * B - c <= K1 ? src[(long long)(c - 2 * B) * nk] : zero;
+        x[5] = live && B - c <= K1 ? src[(long long)(c - B) * nk] : zero;
+        idft6p<T>(x);
+        C* p = a + (TR ? (size_t)P.rev[c] * MC + l : (size_t)l * P.ls + P.rev[c]);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) p[q * es] = x[q];
+    }
+}
+
 template <typename T, int RM>
 __device__ __forceinline__ void k_fft_y_tma(const FftYP& P, typename Cx<T>::t* __restrict__ F1,
                                             typename Cx<T>::t* __restrict__ F2,
@@ -1552,6 +1781,11 @@ __device__ __forceinline__ void k_fft_y_body(const FftYP& P, typename Cx<T>::t* 
         }
         cp_async_wait_all();
         __syncthreads();
+        if (fuse6(P.plan1, K1)) {
+            fft_fwd_head<T, RM>(a, MC, P.d_lines, LS, P.plan1, tw1);
+            y_tail6<T, false>(P, a, F2, cx, mz0, mcount);
+            return;
+        }
         fft_fwd_dif<T, RM>(a, MC, P.d_lines, LS, P.plan1, tw1);
         if (live) {
             C* dst = F2 + ((size_t)cx * ny2 + r0) * nk + mz0 + l;
@@ -1561,6 +1795,11 @@ __device__ __forceinline__ void k_fft_y_body(const FftYP& P, typename Cx<T>::t* 
             }
         }
     } else {
+        if (fuse6(P.plan1, K1)) {
+            y_head6<T, false>(P, a, F2, cx, mz0, mcount);
+            __syncthreads();
+            fft_inv_tail<T, RM>(a, MC, P.d_lines, LS, P.plan1, tw1);
+        } else {
         const C* src = F2 + ((size_t)cx * ny2) * nk + mz0 + l;
         for (int y = r0; y < n1; y += rstep) {  // y: frequency index
             const int my = y <= n1 / 2 ? y : y - n1;
@@ -1573,6 +1812,7 @@ __device__ __forceinline__ void k_fft_y_body(const FftYP& P, typename Cx<T>::t* 
         cp_async_wait_all();
         __syncthreads();
         fft_inv_dit<T, RM>(a, MC, P.d_lines, LS, P.plan1, tw1);
+        }
         if (live) {
             C* dst = F1 + ((size_t)cx * n1 + r0) * nk + mz0 + l;
             const size_t dstep = (size_t)rstep * nk;
@@ -1624,6 +1864,11 @@ __device__ __forceinline__ void k_fft_y_tma(const FftYP& P, typename Cx<T>::t* _
             if (threadIdx.x == 0) atomicOr(status, ST_TIMEOUT);
             return;
         }
+        if (fuse6(P.plan1, K1)) {
+            fft_fwd_head<T, RM, true>(a, MC, P.d_lines, 0, P.plan1, tw1);
+            y_tail6<T, true>(P, a, F2, cx, mz0, mcount);
+            return;
+        }
         fft_fwd_dif<T, RM, true>(a, MC, P.d_lines, 0, P.plan1, tw1);
         if (live) {
             C* dst = F2 + ((size_t)cx * ny2 + r0) * nk + mz0 + l;
@@ -1634,6 +1879,11 @@ __device__ __forceinline__ void k_fft_y_tma(const FftYP& P, typename Cx<T>::t* _
             }
         }
     } else {
+        if (fuse6(P.plan1, K1)) {
+            y_head6<T, true>(P, a, F2, cx, mz0, mcount);
+            __syncthreads();
+            fft_inv_tail<T, RM, true>(a, MC, P.d_lines, 0, P.plan1, tw1);
+        } else {
         C zero;
         zero.x = 0;
         zero.y = 0;
@@ -1649,6 +1899,7 @@ __device__ __forceinline__ void k_fft_y_tma(const FftYP& P, typename Cx<T>::t* _
         cp_async_wait_all();
         __syncthreads();
         fft_inv_dit<T, RM, true>(a, MC, P.d_lines, 0, P.plan1, tw1);
+        }
         fence_proxy_async_smem();
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -1665,6 +1916,88 @@ __global__ void __launch_bounds__(kThreads, 2) k_fft_y(FftYP P, typename Cx<T>::
                                                     const __grid_constant__ CUtensorMap tm, int* status)
 {
     k_fft_y_body<T, RM>(P, F1, F2, tw1, sign, blockIdx.x, P.tnb > 0 ? &tm : nullptr, status);
+}
+
+// The x pass's two boundary passes with the k-space step between them, in
+// registers: a thread per (butterfly c, mode lk) takes the three components'
+// forward butterflies, their kept frequencies through the k-space step, and
+// the inverse butterflies (of the streamfunction too with PSI).  Row p of line
+// (comp, lk) sits at p NL + comp MC + lk (TR) or (comp MC + lk) LS + p.
+template <typename T, bool TR, bool PSI>
+__device__ __forceinline__ void x_mid6(const FftXP& P, typename Cx<T>::t* a, int myp, int mz0, int mcount,
+                                       const T* __restrict__ tab0, const T* __restrict__ tab1,
+                                       const T* __restrict__ tab2, double& esum)
+{
+    using C = typename Cx<T>::t;
+    const int B = P.ng[0] / 6, K0 = P.K[0], MC = 1 << P.lmc;
+    const int es = TR ? 3 * MC : 1, cs = TR ? MC : MC * P.ls;  // strides of a row and of a component
+    const int my = myp - P.K[1], amy = my < 0 ? -my : my;
+    const T kk0 = (T)P.kk[0], kk1 = (T)P.kk[1], kk2 = (T)P.kk[2];  // 2 pi / L_d
+    const T scale = (T)P.scale;
+    const int lk = threadIdx.x & (MC - 1), mz = mz0 + lk;
+    const bool live = lk < mcount;
+    const T k1 = kk1 * (T)my, k2 = kk2 * (T)mz;
+    for (int c = threadIdx.x >> P.lmc; c < B; c += blockDim.x >> P.lmc) {
+        C* p = a + (TR ? P.rev[c] * es + lk : lk * P.ls + P.rev[c]);
+        C w[3][6], s[PSI ? 3 : 1][6];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+#pragma unroll
+            for (int q = 0; q < 6; ++q) w[d][q] = p[d * cs + q * es];
+            dft<T, 6, -1>(w[d]);
+        }
+        const int mxs[4] = { c, c + B, c - 2 * B, c - B };
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int q = e < 2 ? e : e + 2;
+            const int mx = mxs[e], amx = mx < 0 ? -mx : mx;
+            if (!live || amx > K0 || (mx == 0 && my == 0 && mz == 0)) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    w[d][q].x = w[d][q].y = (T)0;
+                    if (PSI) s[d][q] = w[d][q];
+                }
+                continue;
+            }
+            C w0 = w[0][q], w1 = w[1][q], w2 = w[2][q];
+            const T k0 = kk0 * (T)mx;
+            const T ksq = k0 * k0 + k1 * k1 + k2 * k2;
+            const T mult = scale * tab0[amx] * tab1[amy] * tab2[mz] / ksq;
+            if (P.energy) {
+                // (1/2) e^{-k^2/4a^2} |omega|^2 / k^2 = (kappa/V) mult |F|^2 / 2; the
+                // half spectrum holds the pair (k, -k) once when mz > 0
+                const double f2 = (double)w0.x * w0.x + (double)w0.y * w0.y + (double)w1.x * w1.x +
+                                  (double)w1.y * w1.y + (double)w2.x * w2.x + (double)w2.y * w2.y;
+                esum += (mz > 0 ? 1.0 : 0.5) * P.scale * (double)mult * f2;
+            }
+            w0.x *= mult; w0.y *= mult;
+            w1.x *= mult; w1.y *= mult;
+            w2.x *= mult; w2.y *= mult;
+            if (PSI) {
+                s[0][q] = w0;
+                s[PSI ? 1 : 0][q] = w1;
+                s[PSI ? 2 : 0][q] = w2;
+            }
+            // i k x w
+            const T cr0 = k1 * w2.x - k2 * w1.x, ci0 = k1 * w2.y - k2 * w1.y;
+            const T cr1 = k2 * w0.x - k0 * w2.x, ci1 = k2 * w0.y - k0 * w2.y;
+            const T cr2 = k0 * w1.x - k1 * w0.x, ci2 = k0 * w1.y - k1 * w0.y;
+            w[0][q].x = -ci0; w[0][q].y = cr0;
+            w[1][q].x = -ci1; w[1][q].y = cr1;
+            w[2][q].x = -ci2; w[2][q].y = cr2;
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            idft6p<T>(w[d]);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) p[d * cs + q * es] = w[d][q];
+            if constexpr (PSI) {
+                idft6p<T>(s[d]);
+#pragma unroll
+                for (int q = 0; q < 6; ++q) p[(3 + d) * cs + q * es] = s[d][q];
+            }
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1715,7 +2048,11 @@ __device__ __forceinline__ void k_fft_x_kspace_body(const FftXP& P, typename Cx<
     }
     cp_async_wait_all();
     __syncthreads();
-    fft_fwd_dif<T, RM>(a, 3 * MC, P.d_lines, LS, P.plan0, tw0);
+    const bool fused = !P.spectrum && fuse6(P.plan0, K0);
+    if (fused)
+        fft_fwd_head<T, RM>(a, 3 * MC, P.d_lines, LS, P.plan0, tw0);
+    else
+        fft_fwd_dif<T, RM>(a, 3 * MC, P.d_lines, LS, P.plan0, tw0);
     // k-space pass: frequency (mx, my, mz) sits at position rev(xi) of line (c, l)
     const int my = myp - K1;
     const int amy = my < 0 ? -my : my;
@@ -1754,9 +2091,13 @@ __device__ __forceinline__ void k_fft_x_kspace_body(const FftXP& P, typename Cx<
     double esum = 0.0;  // energy of this thread's modes (float64 reduction)
     // a thread takes 8 consecutive x frequencies of one line, the lanes on
     // consecutive groups (distinct banks at the digit-reversed positions)
-    const int nq = n0 >> 3;
+    const int nq = fused ? 0 : n0 >> 3;
     const T kk0 = (T)P.kk[0], kk1 = (T)P.kk[1], kk2 = (T)P.kk[2];  // 2 pi / L_d
     const T scale = (T)P.scale;
+    if (fused && want_psi)
+        x_mid6<T, false, true>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+    else if (fused)
+        x_mid6<T, false, false>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
     for (int i = threadIdx.x; i < nq * MC; i += blockDim.x) {
         const int lk = i / nq, q = i - lk * nq;
         const int mz = mz0 + lk;
@@ -1829,7 +2170,10 @@ __device__ __forceinline__ void k_fft_x_kspace_body(const FftXP& P, typename Cx<
         }
     }
     __syncthreads();
-    fft_inv_dit<T, RM>(a, (want_psi ? 6 : 3) * MC, want_psi ? P.d_lines_psi : P.d_lines, LS, P.plan0, tw0);
+    if (fused)
+        fft_inv_tail<T, RM>(a, (want_psi ? 6 : 3) * MC, want_psi ? P.d_lines_psi : P.d_lines, LS, P.plan0, tw0);
+    else
+        fft_inv_dit<T, RM>(a, (want_psi ? 6 : 3) * MC, want_psi ? P.d_lines_psi : P.d_lines, LS, P.plan0, tw0);
     if (live) {
 #pragma unroll 1
         for (int c = 0; c < 3; ++c) {
@@ -1886,7 +2230,11 @@ __device__ __forceinline__ void k_fft_x_tma(const FftXP& P, typename Cx<T>::t* _
         if (threadIdx.x == 0) atomicOr(status, ST_TIMEOUT);
         return;
     }
-    fft_fwd_dif<T, RM, true>(a, NL, P.d_lines, 0, P.plan0, tw0);
+    const bool fused = fuse6(P.plan0, K0);
+    if (fused)
+        fft_fwd_head<T, RM, true>(a, NL, P.d_lines, 0, P.plan0, tw0);
+    else
+        fft_fwd_dif<T, RM, true>(a, NL, P.d_lines, 0, P.plan0, tw0);
     // k-space pass: frequency (mx, my, mz) of line (c, lk) sits at position
     // p with irev[p] = xi
     const int my = myp - K1;
@@ -1897,7 +2245,8 @@ __device__ __forceinline__ void k_fft_x_tma(const FftXP& P, typename Cx<T>::t* _
     C zero;
     zero.x = 0;
     zero.y = 0;
-    for (int i = threadIdx.x; i < (n0 << lmc); i += blockDim.x) {
+    if (fused) x_mid6<T, true, false>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+    for (int i = threadIdx.x; !fused && i < (n0 << lmc); i += blockDim.x) {
         const int lk = i & (MC - 1), p = i >> lmc;
         const int xi = P.irev[p];
         const int mx = xi <= n0 / 2 ? xi : xi - n0;
@@ -1937,7 +2286,10 @@ __device__ __forceinline__ void k_fft_x_tma(const FftXP& P, typename Cx<T>::t* _
         if ((threadIdx.x & 31) == 0 && esum != 0.0) atomicAdd(P.energy, esum);
     }
     __syncthreads();
-    fft_inv_dit<T, RM, true>(a, NL, P.d_lines, 0, P.plan0, tw0);
+    if (fused)
+        fft_inv_tail<T, RM, true>(a, NL, P.d_lines, 0, P.plan0, tw0);
+    else
+        fft_inv_dit<T, RM, true>(a, NL, P.d_lines, 0, P.plan0, tw0);
     fence_proxy_async_smem();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1982,6 +2334,33 @@ __global__ void __launch_bounds__(kThreads, 2) k_fft_z_c2r(FftZP P, const typena
     C zero;
     zero.x = 0;
     zero.y = 0;
+    if (fuse6(P.plan2, P.K[2])) {
+        const int B = n2 / 6, K = nk - 1, tot = z_items(B, ncl);
+        for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+            int l, c;
+            z_item(i, ncl, P.d_ncl, l, c);
+            if (2 * c > B) continue;
+            const C* rowA = F1 + ((size_t)cx * n1 + y0 + 2 * l) * nk;
+            const int md[4] = { c, B + c, B - c, 2 * B - c };
+            C A[4], Bv[4], X[6], Y[6];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                A[e] = md[e] <= K ? rowA[md[e]] : zero;
+                Bv[e] = md[e] <= K ? rowA[nk + md[e]] : zero;
+            }
+            z_pair_inverse<T>(A, Bv, c, X, Y);
+            C* px = a + l * CS + P.rev[c];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) px[q] = X[q];
+            if (c > 0 && 2 * c < B) {
+                C* py = a + l * CS + P.rev[B - c];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) py[q] = Y[q];
+            }
+        }
+        __syncthreads();
+        fft_inv_tail<T, RM>(a, ncl, P.d_ncl, CS, P.plan2, tw2);
+    } else {
     for (int i = threadIdx.x; i < ncl * CS; i += blockDim.x) a[i] = zero;
     __syncthreads();
     // Z_k = A_k + i B_k, Z_{n-k} = conj(A_k) + i conj(B_k), k = 0..K2, at rev
@@ -2023,6 +2402,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_fft_z_c2r(FftZP P, const typena
     }
     __syncthreads();
     fft_inv_dit<T, RM>(a, ncl, P.d_ncl, CS, P.plan2, tw2);
+    }
     const size_t gsz = (size_t)P.ng[0] * n1 * n2;
     const int c = fdiv(cx, P.d_n0), x = cx - c * P.ng[0];
     TO* gout = grid + c * gsz + ((size_t)x * n1 + y0) * n2;
@@ -2083,13 +2463,50 @@ __device__ __forceinline__ void k_zfft_interp_body(const SpZP& P, const int* __r
     const int nr = home_fetch(P, cstart, bx, by, H, rb0, rlen);
     // no node near the block (rlen is 0 past the ranges): nothing to transform
     if (!__syncthreads_or(rlen > 0)) return;
-    zero_cx(cb, ncl * CS);
+    const bool fused = fuse6(P.plan2, P.K[2]);
+    if (!fused) zero_cx(cb, ncl * CS);
     if (tid < kHomeMax) {
         r_beg[tid] = rb0;
         r_pre[tid + 1] = rlen;
     }
     __syncthreads();
     home_prefix(r_pre);
+    if (fused) {
+        // the inverse boundary pass, modes straight from the two rows
+        const int B = n2 / 6, K = nk - 1, tot = z_items(B, ncl);
+        for (int i = tid; i < tot; i += blockDim.x) {
+            int l, c;
+            z_item(i, ncl, P.d_ncl, l, c);
+            if (2 * c > B) continue;
+            const C* row[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int rl = 2 * l + r;
+                const int cc = fdiv(rl, P.d_txy), rem = rl - cc * txy;
+                const int lx = fdiv(rem, P.d_ty), ly = rem - lx * Ty;
+                row[r] = F1 + (((size_t)cc * n0 + bx * Tx + lx) * n1 + by * Ty + ly) * nk;
+            }
+            const int md[4] = { c, B + c, B - c, 2 * B - c };
+            C A[4], Bv[4], X[6], Y[6];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                A[e].x = A[e].y = Bv[e].x = Bv[e].y = (T)0;
+                if (md[e] <= K) {
+                    A[e] = row[0][md[e]];
+                    Bv[e] = row[1][md[e]];
+                }
+            }
+            z_pair_inverse<T>(A, Bv, c, X, Y);
+            C* px = cb + l * CS + P.rev[c];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) px[q] = X[q];
+            if (c > 0 && 2 * c < B) {
+                C* py = cb + l * CS + P.rev[B - c];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) py[q] = Y[q];
+            }
+        }
+    } else {
     // Z_k = A_k + i B_k, Z_{n-k} = conj(A_k) + i conj(B_k) at the digit-reversed
     // positions, 8 consecutive k of one line pair per thread
     const int nq = (nk + 7) >> 3;
@@ -2123,9 +2540,13 @@ __device__ __forceinline__ void k_zfft_interp_body(const SpZP& P, const int* __r
             }
         }
     }
+    }
     __syncthreads();
     const int ncand = r_pre[nr];
-    fft_inv_dit<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
+    if (fused)
+        fft_inv_tail<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
+    else
+        fft_inv_dit<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
     // periodic halo: positions n2 .. n2 + W - 2 of every line repeat 0 .. W - 2
     // (the line stride leaves room), so a node's W positions from its support
     // start taken modulo n2 are contiguous
@@ -2586,8 +3007,6 @@ bool make_tmap_y(void* F1, const FftYP& P, CUtensorMap* tm)
                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
-template bool make_tmap_y<float>(void*, const FftYP&, CUtensorMap*);
-template bool make_tmap_y<double>(void*, const FftYP&, CUtensorMap*);
 
 template <typename T>
 bool make_tmap_x(void* F2, const FftXP& P, CUtensorMap* tm)
@@ -2610,8 +3029,6 @@ bool make_tmap_x(void* F2, const FftXP& P, CUtensorMap* tm)
                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
-template bool make_tmap_x<float>(void*, const FftXP&, CUtensorMap*);
-template bool make_tmap_x<double>(void*, const FftXP&, CUtensorMap*);
 
 template <typename T>
 struct FftXLaunch {
@@ -2913,32 +3330,16 @@ cudaError_t launch_zfft_interp_b(int w, const BatchL& L, cudaStream_t s)
     template size_t fft_y_smem<T>(const FftYP&);                                       \
     template size_t fft_x_smem<T>(const FftXP&);                                       \
     template size_t zfft_interp_smem<T>(const SpZP&);
-BSW_INST_B(float)
+#ifdef BSW_FFT_DOUBLE
 BSW_INST_B(double)
+#else
+BSW_INST_B(float)
+#endif
 #undef BSW_INST_B
 
-template cudaError_t launch_col_sort<float>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
-template cudaError_t launch_col_sort<double>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
-template cudaError_t launch_spread_zfft<float>(const SpZP&, const Work&, cudaStream_t);
-template cudaError_t launch_spread_zfft<double>(const SpZP&, const Work&, cudaStream_t);
-template cudaError_t launch_zfft_interp<float>(const SpZP&, const Work&, cudaStream_t);
-template cudaError_t launch_zfft_interp<double>(const SpZP&, const Work&, cudaStream_t);
-template cudaError_t launch_node_bin<float>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
-template cudaError_t launch_node_clear<float>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
-template cudaError_t launch_node_bin<double>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
-template cudaError_t launch_node_clear<double>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
-template size_t nd_rec_bytes<float>(int);
-template size_t nd_rec_bytes<double>(int);
-template cudaError_t launch_fft_x_kspace<float>(const FftXP&, const Work&, bool, cudaStream_t, const CUtensorMap*);
-template cudaError_t launch_fft_x_kspace<double>(const FftXP&, const Work&, bool, cudaStream_t, const CUtensorMap*);
-template cudaError_t launch_fft_y<float>(const FftYP&, const Work&, void*, int, cudaStream_t, const CUtensorMap*);
-template cudaError_t launch_fft_y<double>(const FftYP&, const Work&, void*, int, cudaStream_t, const CUtensorMap*);
-template cudaError_t launch_fft_x_kspace<float>(const FftXP&, const Work&, bool, cudaStream_t);
-template cudaError_t launch_fft_x_kspace<double>(const FftXP&, const Work&, bool, cudaStream_t);
-template cudaError_t launch_fft_z_c2r<float>(const FftZP&, const Work&, cudaStream_t, double*);
-template cudaError_t launch_fft_z_c2r<double>(const FftZP&, const Work&, cudaStream_t, double*);
 // Writes the composite-radix twiddles into the current device's constant
 // bank (once per device).
+template <typename T>
 cudaError_t set_fft_constants()
 {
     static std::mutex mu;
@@ -2958,15 +3359,47 @@ cudaError_t set_fft_constants()
             hd[offs[k] + m] = make_double2(cos(ph), sin(ph));
             hf[offs[k] + m] = make_float2((float)cos(ph), (float)sin(ph));
         }
-    e = cudaMemcpyToSymbol(c_twf, hf, sizeof hf);
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_twd, hd, sizeof hd);
+    if constexpr (sizeof(T) == 4)
+        e = cudaMemcpyToSymbol(c_twf, hf, sizeof hf);
+    else
+        e = cudaMemcpyToSymbol(c_twd, hd, sizeof hd);
     if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
     return e;
 }
 
-template size_t col_pt_bytes<float>(int);
+// One object per precision (the two compile in parallel): BSW_FFT_DOUBLE.
+#ifdef BSW_FFT_DOUBLE
+template bool make_tmap_y<double>(void*, const FftYP&, CUtensorMap*);
+template bool make_tmap_x<double>(void*, const FftXP&, CUtensorMap*);
+template cudaError_t launch_col_sort<double>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
+template cudaError_t launch_spread_zfft<double>(const SpZP&, const Work&, cudaStream_t);
+template cudaError_t launch_zfft_interp<double>(const SpZP&, const Work&, cudaStream_t);
+template cudaError_t launch_node_bin<double>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
+template cudaError_t launch_node_clear<double>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
+template size_t nd_rec_bytes<double>(int);
+template cudaError_t launch_fft_x_kspace<double>(const FftXP&, const Work&, bool, cudaStream_t, const CUtensorMap*);
+template cudaError_t launch_fft_y<double>(const FftYP&, const Work&, void*, int, cudaStream_t, const CUtensorMap*);
+template cudaError_t launch_fft_x_kspace<double>(const FftXP&, const Work&, bool, cudaStream_t);
+template cudaError_t launch_fft_z_c2r<double>(const FftZP&, const Work&, cudaStream_t, double*);
 template size_t col_pt_bytes<double>(int);
-template size_t spread_zfft_smem<float>(const SpZP&);
 template size_t spread_zfft_smem<double>(const SpZP&);
+template cudaError_t set_fft_constants<double>();
+#else
+template bool make_tmap_y<float>(void*, const FftYP&, CUtensorMap*);
+template bool make_tmap_x<float>(void*, const FftXP&, CUtensorMap*);
+template cudaError_t launch_col_sort<float>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
+template cudaError_t launch_spread_zfft<float>(const SpZP&, const Work&, cudaStream_t);
+template cudaError_t launch_zfft_interp<float>(const SpZP&, const Work&, cudaStream_t);
+template cudaError_t launch_node_bin<float>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
+template cudaError_t launch_node_clear<float>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
+template size_t nd_rec_bytes<float>(int);
+template cudaError_t launch_fft_x_kspace<float>(const FftXP&, const Work&, bool, cudaStream_t, const CUtensorMap*);
+template cudaError_t launch_fft_y<float>(const FftYP&, const Work&, void*, int, cudaStream_t, const CUtensorMap*);
+template cudaError_t launch_fft_x_kspace<float>(const FftXP&, const Work&, bool, cudaStream_t);
+template cudaError_t launch_fft_z_c2r<float>(const FftZP&, const Work&, cudaStream_t, double*);
+template size_t col_pt_bytes<float>(int);
+template size_t spread_zfft_smem<float>(const SpZP&);
+template cudaError_t set_fft_constants<float>();
+#endif
 
 }  // namespace bsw

@@ -42,3 +42,31 @@ def test_short_range_of_node_pairs(sizes, rc_over_L):
     a = _parts(B, f, precision=B.BS_MIXED, **kw)[1]
     b = _parts(B, f, precision=B.BS_FP64, **kw)[1]
     assert np.sqrt(((a - b) ** 2).mean()) <= 1e-5 * np.sqrt((b ** 2).mean())
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("sigma", [1.25, 1.5])
+@pytest.mark.parametrize("M", [15, 31, 33, 43, 47, 63, 64, 85, 95, 97, 127, 130])
+def test_boundary_passes_equal_full_transforms(M, sigma, prec):
+    """The passes that start and end the transforms at the kept modes (grids
+    with a factor 3 and K < n / 3, which sigma = 1.5 gives and 1.25 does not)
+    and the general ones (powers of two, sigma = 1.25), with and without psi,
+    against full cuFFT transforms.  Velocity and psi of the long range: 1e-12 of
+    the largest value in float64; float32 transforms of 30 to 200 points, three
+    axes both ways and sums of w^3 = 512 float32 terms, about 30 roundings of
+    6e-8: 2e-6."""
+    B, tol = _B(), 2e-6 if prec == "mixed" else 1e-12
+    f = W.ellipses(3, 40, seed=M)
+    nodes = torch.from_numpy(f.nodes).cuda()
+    got = []
+    for flags in (0, B.BS_WANT_PSI, B.BS_WANT_PSI | B.BS_FFT_CUFFT):
+        p = B.make_params(f.L, M=M, Q=2, w=8, sigma=sigma, flags=flags, alpha=1.2, rc=3.0,
+                          precision=B.BS_MIXED if prec == "mixed" else B.BS_FP64)
+        bs = B.BiotSavart(p, f.offsets, f.closing)
+        v = bs.parts(nodes, want_psi=bool(flags))
+        got.append([x[2].clone() for x in (v if flags else (v,))])
+        torch.cuda.synchronize()
+        bs.close()
+    ref = got[2]
+    for x, r in ((got[0][0], ref[0]), (got[1][0], ref[0]), (got[1][1], ref[1])):
+        assert float((x - r).abs().max()) < tol * float(r.abs().max())
