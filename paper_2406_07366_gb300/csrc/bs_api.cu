@@ -103,7 +103,8 @@ int fft_friendly(int n)
 // for nl >= slots an odd stride suffices.
 int line_stride(int n, int nl, int slots)
 {
-    const int target = nl >= slots ? 1 : (slots % nl == 0 ? slots / nl : 1);
+    // 24 lines of float2 are taken 8 at a time at two positions (fft_pass)
+    const int target = nl == 24 && slots == 16 ? 2 : nl >= slots ? 1 : (slots % nl == 0 ? slots / nl : 1);
     return n + (((target - n) % slots) + slots) % slots;
 }
 
@@ -135,7 +136,15 @@ FftPlan make_plan(int n, int maxr)
     pl.n = n;
     std::vector<int> cur, best;
     plan_search(n, maxr, 0, cur, best);
-    // a 6 goes last: the kernels' boundary passes are built on it
+    // a 6 goes last (the kernels' boundary passes take 4, 6 or 8 there)
+    if (n % 6 == 0 && std::find(best.begin(), best.end(), 6) == best.end()) {
+        std::vector<int> c2, with6;
+        plan_search(n / 6, maxr, 0, c2, with6);
+        if (with6.size() + 1 <= best.size()) {
+            best = with6;
+            best.push_back(6);
+        }
+    }
     const auto six = std::find(best.begin(), best.end(), 6);
     if (six != best.end()) {
         best.erase(six);

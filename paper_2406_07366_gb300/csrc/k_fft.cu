@@ -404,9 +404,14 @@ __device__ __forceinline__ void fft_pass(typename Cx<T>::t* __restrict__ buf, in
     const bool pad = sizeof(C) == 8 && nlines < G && (G % nlines) != 0 && 2 * nlines > G;
     const int tot = (pad ? G : nlines) * nb;
     const int L = st * R;
+    const bool tri = sizeof(C) == 8 && !TR && nlines == 24 && (nb & 1) == 0;  // see fft_pass_c
     for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
         int i, line;
-        if (pad) {
+        if (tri) {
+            const int rest = idx >> 4, lg = rest % 3;
+            i = 2 * (rest / 3) + ((idx >> 3) & 1);
+            line = 8 * lg + (idx & 7);
+        } else if (pad) {
             i = idx / G;
             line = idx & (G - 1);
             if (line >= nlines) continue;
@@ -443,10 +448,15 @@ __device__ __forceinline__ void fft_pass_c(typename Cx<T>::t* __restrict__ buf, 
     constexpr int nb = N / R;
     constexpr int tot = NLV * nb;
     constexpr int L = ST * R;
+    // 24 lines are neither a multiple of the 16 lanes that shared memory serves
+    // at a time nor padded: line by line a third of the half-warps would mix two
+    // positions and collide.  A half-warp takes 8 lines at two neighbouring
+    // positions (line stride 2 modulo 16: 16 distinct banks).
+    constexpr bool tri = sizeof(C) == 8 && !TR && NL == 24 && nb % 2 == 0;
 #pragma unroll 1
     for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-        const int i = idx / NLV;
-        const int line = idx % NLV;
+        const int i = tri ? 2 * (idx / 48) + ((idx >> 3) & 1) : idx / NLV;
+        const int line = tri ? 8 * ((idx >> 4) % 3) + (idx & 7) : idx % NLV;
         if (pad && line >= NL) continue;
         const int b = i / ST;
         const int j = i % ST;
@@ -584,21 +594,25 @@ __device__ __forceinline__ void fft_inv_dit(typename Cx<T>::t* buf, int nlines, 
 
 // ---- boundary passes ----
 // The transforms keep the frequencies |k| <= K < n / 3 only.  With a last
-// radix of 6 (stride 1, no twiddles) butterfly c holds, at positions rev(c) ..
-// rev(c) + 5, the frequencies c + q B, q = 0..5, B = n / 6, of which q = 2 and 3
-// are never kept.  So that pass need not go through shared memory: the forward
-// transform's last pass hands its outputs straight to whoever consumes the
-// modes, the inverse one's first pass takes its inputs straight from their
-// source, the x pass's two meet in registers around the k-space step, and the
-// zero padding is never written or read.  These kernels are bound by shared
-// memory (65-70 % of its bandwidth on the 384^3 grid), and this removes 2 of 7
-// (y), 4 of 14 (x) and about a third (z) of their accesses.
-// The other plans (no factor 3, or K >= n / 3) take the general passes.
+// radix R (stride 1, no twiddles) butterfly c holds, at positions rev(c) ..
+// rev(c) + R - 1, the frequencies c + q B, q = 0..R-1, B = n / R; q < H and q >=
+// R - H can be kept, H = 2 for R = 4 and 6, 3 for R = 8.  That pass need not go
+// through shared memory: the forward transform's last pass hands its outputs
+// straight to whoever consumes the modes, the inverse one's first pass takes
+// its inputs straight from their source, the x pass's two meet in registers
+// around the k-space step, and the zero padding is never written or read.
+// These kernels are bound by shared memory (65-70 % of its bandwidth on the
+// 384^3 grid), and this removes 2 of 7 (y), 4 of 14 (x) and about a third (z)
+// of their accesses.  Other plans (K >= n / 3, odd last radices) take the
+// general passes.
 template <typename P>
-__device__ __forceinline__ bool fuse6(const P& pl, int K)
+__device__ __forceinline__ int boundary_radix(const P& pl, int K)
 {
-    return pl.nr >= 2 && pl.r[pl.nr - 1] == 6 && 3 * K < pl.n;
+    const int r = pl.r[pl.nr - 1];
+    return pl.nr >= 2 && 3 * K < pl.n && (r == 4 || r == 6 || r == 8) ? r : 0;
 }
+template <int R>
+constexpr int kept_half() { return R == 8 ? 3 : 2; }
 
 // All forward passes but the last; all inverse passes but the first.
 template <typename T, int RM, bool TR = false>
@@ -648,37 +662,50 @@ __device__ __forceinline__ void idft6p(typename Cx<T>::t* x)
     }
 }
 
+// dft<T, R, +1> of an input that is zero outside the kept halves.
+template <typename T, int R>
+__device__ __forceinline__ void idft_kept(typename Cx<T>::t* x)
+{
+    if constexpr (R == 6) {
+        idft6p<T>(x);
+    } else {
+#pragma unroll
+        for (int q = kept_half<R>(); q < R - kept_half<R>(); ++q) x[q].x = x[q].y = (T)0;
+        dft<T, R, 1>(x);
+    }
+}
+
 // Butterflies c and B - c of a pair of real z-lines A, B packed as A + i B hold
-// between them the modes c, B + c, B - c and 2 B - c and their mirrors.
-// Inverse: from the modes m[] = {c, B + c, B - c, 2 B - c} of both rows (zero
+// between them the modes c + e B and (e + 1) B - c, e < H, and their mirrors.
+// Inverse: from those modes of both rows (the first H, then the second H; zero
 // beyond K) the two butterflies' outputs X (c) and Y (B - c).
-template <typename T>
+template <typename T, int R>
 __device__ __forceinline__ void z_pair_inverse(const typename Cx<T>::t* A, const typename Cx<T>::t* Bv, int c,
                                                typename Cx<T>::t* X, typename Cx<T>::t* Y)
 {
     using C = typename Cx<T>::t;
-    C p[4], m[4];  // Z at the modes and at their mirrors
+    constexpr int H = kept_half<R>();
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        p[e].x = A[e].x - Bv[e].y;
-        p[e].y = A[e].y + Bv[e].x;
-        m[e].x = A[e].x + Bv[e].y;
-        m[e].y = -A[e].y + Bv[e].x;
+    for (int e = 0; e < 2 * H; ++e) {
+        C p, m;  // Z at the mode and at its mirror
+        p.x = A[e].x - Bv[e].y;
+        p.y = A[e].y + Bv[e].x;
+        m.x = A[e].x + Bv[e].y;
+        m.y = -A[e].y + Bv[e].x;
+        if (e == 0 && c == 0) {
+            p.x = A[0].x;
+            p.y = Bv[0].x;
+        }
+        if (e < H) {
+            X[e] = p;
+            Y[R - 1 - e] = m;
+        } else {
+            Y[e - H] = p;
+            X[R - 1 - (e - H)] = m;
+        }
     }
-    if (c == 0) {
-        p[0].x = A[0].x;
-        p[0].y = Bv[0].x;
-    }
-    X[0] = p[0];
-    X[1] = p[1];
-    X[4] = m[3];
-    X[5] = m[2];
-    Y[0] = p[2];
-    Y[1] = p[3];
-    Y[4] = m[1];
-    Y[5] = m[0];
-    idft6p<T>(X);
-    idft6p<T>(Y);
+    idft_kept<T, R>(X);
+    idft_kept<T, R>(Y);
 }
 
 // Items of a z boundary pass: i -> line l and c = 0..B/2, four consecutive c
@@ -691,6 +718,43 @@ __device__ __forceinline__ void z_item(int i, int ncl, const FastDiv& d_ncl, int
     c = 4 * g + (i & 3);
 }
 __device__ __forceinline__ int z_items(int B, int ncl) { return ((B / 2 + 4) >> 2) * 4 * ncl; }
+
+// The inverse boundary pass of ncl pairs of rows into the lines at cb (stride
+// CS); rows(l, A, B) gives the mode rows of pair l.
+template <typename T, int R, typename Rows>
+__device__ __forceinline__ void z_head(typename Cx<T>::t* cb, int CS, int ncl, const FastDiv& d_ncl, int n2, int K,
+                                       const int* __restrict__ rev, Rows rows)
+{
+    using C = typename Cx<T>::t;
+    constexpr int H = kept_half<R>();
+    const int B = n2 / R, tot = z_items(B, ncl);
+    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+        int l, c;
+        z_item(i, ncl, d_ncl, l, c);
+        if (2 * c > B) continue;
+        const C *ra, *rb;
+        rows(l, ra, rb);
+        C A[2 * H], Bv[2 * H], X[R], Y[R];
+#pragma unroll
+        for (int e = 0; e < 2 * H; ++e) {
+            const int m = e < H ? c + e * B : (e - H + 1) * B - c;
+            A[e].x = A[e].y = Bv[e].x = Bv[e].y = (T)0;
+            if (m <= K) {
+                A[e] = ra[m];
+                Bv[e] = rb[m];
+            }
+        }
+        z_pair_inverse<T, R>(A, Bv, c, X, Y);
+        C* px = cb + l * CS + rev[c];
+#pragma unroll
+        for (int q = 0; q < R; ++q) px[q] = X[q];
+        if (c > 0 && 2 * c < B) {
+            C* py = cb + l * CS + rev[B - c];
+#pragma unroll
+            for (int q = 0; q < R; ++q) py[q] = Y[q];
+        }
+    }
+}
 
 // Digit-reversed positions of 8 consecutive frequencies 8q + d (and of
 // n - 8q - d) when the plan's first radix is 8 (stride st0 = n / 8): the first
@@ -1098,31 +1162,32 @@ __device__ __forceinline__ void spz_unpack(const SpZP& P, const typename Cx<T>::
 
 // The forward boundary pass of a spread block: the last pass of every complex
 // z-line, the separation of its two real lines and the store of their modes.
-template <typename T>
-__device__ __forceinline__ void spz_tail6(const SpZP& P, const typename Cx<T>::t* cb, typename Cx<T>::t* F1, int bx,
+template <typename T, int R>
+__device__ __forceinline__ void spz_tail(const SpZP& P, const typename Cx<T>::t* cb, typename Cx<T>::t* F1, int bx,
                                           int by)
 {
     using C = typename Cx<T>::t;
+    constexpr int H = kept_half<R>();
     const int Tx = P.tx, Ty = P.ty, n2 = P.ng[2], CS = P.cls, K = P.K[2];
-    const int txy = Tx * Ty, ncl = 3 * txy / 2, B = n2 / 6, nk = K + 1;
+    const int txy = Tx * Ty, ncl = 3 * txy / 2, B = n2 / R, nk = K + 1;
     const int tot = z_items(B, ncl);
     for (int i = threadIdx.x; i < tot; i += blockDim.x) {
         int l, c;
         z_item(i, ncl, P.d_ncl, l, c);
         if (2 * c > B) continue;
-        C X[6], Y[6];
+        C X[R], Y[R];
         const C* px = cb + l * CS + P.rev[c];
         const C* py = cb + l * CS + P.rev[c == 0 ? 0 : B - c];
 #pragma unroll
-        for (int q = 0; q < 6; ++q) X[q] = px[q];
-        dft<T, 6, -1>(X);
-        if (c == 0) {  // its own mirror: mode 0 with itself, B with -B
-            Y[5] = X[0];
-            Y[4] = X[5];
+        for (int q = 0; q < R; ++q) X[q] = px[q];
+        dft<T, R, -1>(X);
+        if (c == 0) {  // its own mirror: mode 0 with itself, e B with -e B
+#pragma unroll
+            for (int e = 0; e < H; ++e) Y[R - 1 - e] = X[e ? R - e : 0];
         } else {
 #pragma unroll
-            for (int q = 0; q < 6; ++q) Y[q] = py[q];
-            dft<T, 6, -1>(Y);
+            for (int q = 0; q < R; ++q) Y[q] = py[q];
+            dft<T, R, -1>(Y);
         }
         C* dst[2];
 #pragma unroll
@@ -1142,11 +1207,10 @@ __device__ __forceinline__ void spz_tail6(const SpZP& P, const typename Cx<T>::t
             o.y = (T)0.5 * (zn.x - zk.x);
             dst[1][m] = o;
         };
-        put(c, X[0], Y[5]);
-        put(B + c, X[1], Y[4]);
-        if (c > 0 && 2 * c < B) {
-            put(B - c, Y[0], X[5]);
-            put(2 * B - c, Y[1], X[4]);
+#pragma unroll
+        for (int e = 0; e < H; ++e) {
+            put(c + e * B, X[e], Y[R - 1 - e]);
+            if (c > 0 && 2 * c < B) put((e + 1) * B - c, Y[e], X[R - 1 - e]);
         }
     }
 }
@@ -1157,9 +1221,14 @@ __device__ __forceinline__ void spz_transform(const SpZP& P, typename Cx<T>::t* 
                                               const typename Cx<T>::t* __restrict__ tw2, typename Cx<T>::t* F1, int bx,
                                               int by)
 {
-    if (fuse6(P.plan2, P.K[2])) {
+    const int br = boundary_radix(P.plan2, P.K[2]);
+    if (br) {
         fft_fwd_head<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
-        spz_tail6<T>(P, cb, F1, bx, by);
+        switch (br) {
+        case 4: spz_tail<T, 4>(P, cb, F1, bx, by); break;
+        case 6: spz_tail<T, 6>(P, cb, F1, bx, by); break;
+        default: spz_tail<T, 8>(P, cb, F1, bx, by); break;
+        }
     } else {
         fft_fwd_dif<T, RM>(cb, ncl, P.d_ncl, CS, P.plan2, tw2);
         spz_unpack<T>(P, cb, F1, bx, by);
@@ -1328,33 +1397,6 @@ __device__ __forceinline__ void spread_bucketed(const SpZP& P, int s0, int s1, c
     }
     flush(lo, zs + t);
     flush(hi, zs + W + t);
-}
-
-// Two float32 values in a register pair and their packed arithmetic (each
-// half rounded as the scalar operation).
-__device__ __forceinline__ unsigned long long pk2(float lo, float hi)
-{
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 upk2(unsigned long long v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
-{
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
 }
 
 // The bucketed loop in float32.  It is bound by the instructions per copy (65
@@ -1685,33 +1727,35 @@ __global__ void __launch_bounds__(z_threads_max<T>(), 2) k_spread_zfft(SpZP P, c
 // ---------------------------------------------------------------------------
 // Boundary passes along y: a thread per (butterfly c, mode l), the lanes on
 // consecutive modes.  Row y of line l sits at y MC + l (TR) or l LS + y.
-template <typename T, bool TR>
-__device__ __forceinline__ void y_tail6(const FftYP& P, const typename Cx<T>::t* a, typename Cx<T>::t* __restrict__ F2,
+template <typename T, int R, bool TR>
+__device__ __forceinline__ void y_tail(const FftYP& P, const typename Cx<T>::t* a, typename Cx<T>::t* __restrict__ F2,
                                         int cx, int mz0, int mcount)
 {
     using C = typename Cx<T>::t;
-    const int B = P.ng[1] / 6, K1 = P.K[1], nk = P.K[2] + 1, MC = 1 << P.lmc, es = TR ? MC : 1;
+    const int B = P.ng[1] / R, K1 = P.K[1], nk = P.K[2] + 1, MC = 1 << P.lmc, es = TR ? MC : 1;
     const int l = threadIdx.x & (MC - 1);
     if (l >= mcount) return;
     C* dst = F2 + ((size_t)cx * (2 * K1 + 1) + K1) * nk + mz0 + l;  // row my = 0
     for (int c = threadIdx.x >> P.lmc; c < B; c += blockDim.x >> P.lmc) {
         const C* p = a + (TR ? (size_t)P.rev[c] * MC + l : (size_t)l * P.ls + P.rev[c]);
-        C x[6];
+        C x[R];
 #pragma unroll
-        for (int q = 0; q < 6; ++q) x[q] = p[q * es];
-        dft<T, 6, -1>(x);
-        if (c <= K1) dst[(long long)c * nk] = x[0];
-        if (c + B <= K1) dst[(long long)(c + B) * nk] = x[1];
-        if (2 * B - c <= K1) dst[(long long)(c - 2 * B) * nk] = x[4];
-        if (B - c <= K1) dst[(long long)(c - B) * nk] = x[5];
+        for (int q = 0; q < R; ++q) x[q] = p[q * es];
+        dft<T, R, -1>(x);
+#pragma unroll
+        for (int e = 0; e < kept_half<R>(); ++e) {
+            const int up = c + e * B, dn = (e + 1) * B - c;  // my = up and my = -dn
+            if (up <= K1) dst[(long long)up * nk] = x[e];
+            if (dn <= K1) dst[-(long long)dn * nk] = x[R - 1 - e];
+        }
     }
 }
-template <typename T, bool TR>
-__device__ __forceinline__ void y_head6(const FftYP& P, typename Cx<T>::t* a, const typename Cx<T>::t* __restrict__ F2,
+template <typename T, int R, bool TR>
+__device__ __forceinline__ void y_head(const FftYP& P, typename Cx<T>::t* a, const typename Cx<T>::t* __restrict__ F2,
                                         int cx, int mz0, int mcount)
 {
     using C = typename Cx<T>::t;
-    const int B = P.ng[1] / 6, K1 = P.K[1], nk = P.K[2] + 1, MC = 1 << P.lmc, es = TR ? MC : 1;
+    const int B = P.ng[1] / R, K1 = P.K[1], nk = P.K[2] + 1, MC = 1 << P.lmc, es = TR ? MC : 1;
     const int l = threadIdx.x & (MC - 1);
     const bool live = l < mcount;
     const C* src = F2 + ((size_t)cx * (2 * K1 + 1) + K1) * nk + mz0 + l;  // row my = 0
@@ -1720,15 +1764,38 @@ __device__ __forceinline__ void y_head6(const FftYP& P, typename Cx<T>::t* a, co
     zero.y = 0;
 #pragma unroll 2
     for (int c = threadIdx.x >> P.lmc; c < B; c += blockDim.x >> P.lmc) {
-        C x[6];
-        x[0] = live && c <= K1 ? src[(long long)c * nk] : zero;
-        x[1] = live && c + B <= K1 ? src[(long long)(c + B) * nk] : zero;
-        x[4] = live && 2 * B - c <= K1 ? src[(long long)(c - 2 * B) * nk] : zero;
-        x[5] = live && B - c <= K1 ? src[(long long)(c - B) * nk] : zero;
-        idft6p<T>(x);
+        C x[R];
+#pragma unroll
+        for (int e = 0; e < kept_half<R>(); ++e) {
+            const int up = c + e * B, dn = (e + 1) * B - c;
+            x[e] = live && up <= K1 ? src[(long long)up * nk] : zero;
+            x[R - 1 - e] = live && dn <= K1 ? src[-(long long)dn * nk] : zero;
+        }
+        idft_kept<T, R>(x);
         C* p = a + (TR ? (size_t)P.rev[c] * MC + l : (size_t)l * P.ls + P.rev[c]);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) p[q * es] = x[q];
+        for (int q = 0; q < R; ++q) p[q * es] = x[q];
+    }
+}
+
+template <typename T, bool TR>
+__device__ __forceinline__ void y_tail_r(int r, const FftYP& P, const typename Cx<T>::t* a,
+                                         typename Cx<T>::t* __restrict__ F2, int cx, int mz0, int mcount)
+{
+    switch (r) {
+    case 4: y_tail<T, 4, TR>(P, a, F2, cx, mz0, mcount); break;
+    case 6: y_tail<T, 6, TR>(P, a, F2, cx, mz0, mcount); break;
+    default: y_tail<T, 8, TR>(P, a, F2, cx, mz0, mcount); break;
+    }
+}
+template <typename T, bool TR>
+__device__ __forceinline__ void y_head_r(int r, const FftYP& P, typename Cx<T>::t* a,
+                                         const typename Cx<T>::t* __restrict__ F2, int cx, int mz0, int mcount)
+{
+    switch (r) {
+    case 4: y_head<T, 4, TR>(P, a, F2, cx, mz0, mcount); break;
+    case 6: y_head<T, 6, TR>(P, a, F2, cx, mz0, mcount); break;
+    default: y_head<T, 8, TR>(P, a, F2, cx, mz0, mcount); break;
     }
 }
 
@@ -1781,9 +1848,9 @@ __device__ __forceinline__ void k_fft_y_body(const FftYP& P, typename Cx<T>::t* 
         }
         cp_async_wait_all();
         __syncthreads();
-        if (fuse6(P.plan1, K1)) {
+        if (const int br = boundary_radix(P.plan1, K1)) {
             fft_fwd_head<T, RM>(a, MC, P.d_lines, LS, P.plan1, tw1);
-            y_tail6<T, false>(P, a, F2, cx, mz0, mcount);
+            y_tail_r<T, false>(br, P, a, F2, cx, mz0, mcount);
             return;
         }
         fft_fwd_dif<T, RM>(a, MC, P.d_lines, LS, P.plan1, tw1);
@@ -1795,8 +1862,8 @@ __device__ __forceinline__ void k_fft_y_body(const FftYP& P, typename Cx<T>::t* 
             }
         }
     } else {
-        if (fuse6(P.plan1, K1)) {
-            y_head6<T, false>(P, a, F2, cx, mz0, mcount);
+        if (const int br = boundary_radix(P.plan1, K1)) {
+            y_head_r<T, false>(br, P, a, F2, cx, mz0, mcount);
             __syncthreads();
             fft_inv_tail<T, RM>(a, MC, P.d_lines, LS, P.plan1, tw1);
         } else {
@@ -1864,9 +1931,9 @@ __device__ __forceinline__ void k_fft_y_tma(const FftYP& P, typename Cx<T>::t* _
             if (threadIdx.x == 0) atomicOr(status, ST_TIMEOUT);
             return;
         }
-        if (fuse6(P.plan1, K1)) {
+        if (const int br = boundary_radix(P.plan1, K1)) {
             fft_fwd_head<T, RM, true>(a, MC, P.d_lines, 0, P.plan1, tw1);
-            y_tail6<T, true>(P, a, F2, cx, mz0, mcount);
+            y_tail_r<T, true>(br, P, a, F2, cx, mz0, mcount);
             return;
         }
         fft_fwd_dif<T, RM, true>(a, MC, P.d_lines, 0, P.plan1, tw1);
@@ -1879,8 +1946,8 @@ __device__ __forceinline__ void k_fft_y_tma(const FftYP& P, typename Cx<T>::t* _
             }
         }
     } else {
-        if (fuse6(P.plan1, K1)) {
-            y_head6<T, true>(P, a, F2, cx, mz0, mcount);
+        if (const int br = boundary_radix(P.plan1, K1)) {
+            y_head_r<T, true>(br, P, a, F2, cx, mz0, mcount);
             __syncthreads();
             fft_inv_tail<T, RM, true>(a, MC, P.d_lines, 0, P.plan1, tw1);
         } else {
@@ -1923,33 +1990,34 @@ __global__ void __launch_bounds__(kThreads, 2) k_fft_y(FftYP P, typename Cx<T>::
 // forward butterflies, their kept frequencies through the k-space step, and
 // the inverse butterflies (of the streamfunction too with PSI).  Row p of line
 // (comp, lk) sits at p NL + comp MC + lk (TR) or (comp MC + lk) LS + p.
-template <typename T, bool TR, bool PSI>
-__device__ __forceinline__ void x_mid6(const FftXP& P, typename Cx<T>::t* a, int myp, int mz0, int mcount,
+template <typename T, int R, bool TR, bool PSI, bool EN>
+__device__ __forceinline__ void x_mid(const FftXP& P, typename Cx<T>::t* a, int myp, int mz0, int mcount,
                                        const T* __restrict__ tab0, const T* __restrict__ tab1,
                                        const T* __restrict__ tab2, double& esum)
 {
     using C = typename Cx<T>::t;
-    const int B = P.ng[0] / 6, K0 = P.K[0], MC = 1 << P.lmc;
+    const int B = P.ng[0] / R, K0 = P.K[0], MC = 1 << P.lmc;
     const int es = TR ? 3 * MC : 1, cs = TR ? MC : MC * P.ls;  // strides of a row and of a component
     const int my = myp - P.K[1], amy = my < 0 ? -my : my;
     const T kk0 = (T)P.kk[0], kk1 = (T)P.kk[1], kk2 = (T)P.kk[2];  // 2 pi / L_d
     const T scale = (T)P.scale;
     const int lk = threadIdx.x & (MC - 1), mz = mz0 + lk;
     const bool live = lk < mcount;
-    const T k1 = kk1 * (T)my, k2 = kk2 * (T)mz;
+    const T k1 = kk1 * (T)my, k2 = kk2 * (T)mz, k12 = k1 * k1 + k2 * k2;
+    const T st = live ? scale * tab1[amy] * tab2[mz] : (T)0;
     for (int c = threadIdx.x >> P.lmc; c < B; c += blockDim.x >> P.lmc) {
         C* p = a + (TR ? P.rev[c] * es + lk : lk * P.ls + P.rev[c]);
-        C w[3][6], s[PSI ? 3 : 1][6];
+        C w[3][R], s[PSI ? 3 : 1][R];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
 #pragma unroll
-            for (int q = 0; q < 6; ++q) w[d][q] = p[d * cs + q * es];
-            dft<T, 6, -1>(w[d]);
+            for (int q = 0; q < R; ++q) w[d][q] = p[d * cs + q * es];
+            dft<T, R, -1>(w[d]);
         }
         const int mxs[4] = { c, c + B, c - 2 * B, c - B };
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int q = e < 2 ? e : e + 2;
+            const int q = e < 2 ? e : e + R - 4;
             const int mx = mxs[e], amx = mx < 0 ? -mx : mx;
             if (!live || amx > K0 || (mx == 0 && my == 0 && mz == 0)) {
 #pragma unroll
@@ -1961,9 +2029,8 @@ __device__ __forceinline__ void x_mid6(const FftXP& P, typename Cx<T>::t* a, int
             }
             C w0 = w[0][q], w1 = w[1][q], w2 = w[2][q];
             const T k0 = kk0 * (T)mx;
-            const T ksq = k0 * k0 + k1 * k1 + k2 * k2;
-            const T mult = scale * tab0[amx] * tab1[amy] * tab2[mz] / ksq;
-            if (P.energy) {
+            const T mult = st * tab0[amx] / (k0 * k0 + k12);
+            if (EN && P.energy) {
                 // (1/2) e^{-k^2/4a^2} |omega|^2 / k^2 = (kappa/V) mult |F|^2 / 2; the
                 // half spectrum holds the pair (k, -k) once when mz > 0
                 const double f2 = (double)w0.x * w0.x + (double)w0.y * w0.y + (double)w1.x * w1.x +
@@ -1988,13 +2055,13 @@ __device__ __forceinline__ void x_mid6(const FftXP& P, typename Cx<T>::t* a, int
         }
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            idft6p<T>(w[d]);
+            idft_kept<T, R>(w[d]);
 #pragma unroll
-            for (int q = 0; q < 6; ++q) p[d * cs + q * es] = w[d][q];
+            for (int q = 0; q < R; ++q) p[d * cs + q * es] = w[d][q];
             if constexpr (PSI) {
-                idft6p<T>(s[d]);
+                idft_kept<T, R>(s[d]);
 #pragma unroll
-                for (int q = 0; q < 6; ++q) p[(3 + d) * cs + q * es] = s[d][q];
+                for (int q = 0; q < R; ++q) p[(3 + d) * cs + q * es] = s[d][q];
             }
         }
     }
@@ -2048,7 +2115,8 @@ __device__ __forceinline__ void k_fft_x_kspace_body(const FftXP& P, typename Cx<
     }
     cp_async_wait_all();
     __syncthreads();
-    const bool fused = !P.spectrum && fuse6(P.plan0, K0);
+    const int br = P.spectrum ? 0 : boundary_radix(P.plan0, K0);
+    const bool fused = br == 4 || br == 6;  // radix 8 would hold 24 values a thread
     if (fused)
         fft_fwd_head<T, RM>(a, 3 * MC, P.d_lines, LS, P.plan0, tw0);
     else
@@ -2094,10 +2162,24 @@ __device__ __forceinline__ void k_fft_x_kspace_body(const FftXP& P, typename Cx<
     const int nq = fused ? 0 : n0 >> 3;
     const T kk0 = (T)P.kk[0], kk1 = (T)P.kk[1], kk2 = (T)P.kk[2];  // 2 pi / L_d
     const T scale = (T)P.scale;
-    if (fused && want_psi)
-        x_mid6<T, false, true>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
-    else if (fused)
-        x_mid6<T, false, false>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+    if (fused && (want_psi || P.energy)) {
+        if (want_psi) {
+            if (br == 6)
+                x_mid<T, 6, false, true, true>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+            else
+                x_mid<T, 4, false, true, true>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+        } else {
+            if (br == 6)
+                x_mid<T, 6, false, false, true>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+            else
+                x_mid<T, 4, false, false, true>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+        }
+    } else if (fused) {
+        if (br == 6)
+            x_mid<T, 6, false, false, false>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+        else
+            x_mid<T, 4, false, false, false>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+    }
     for (int i = threadIdx.x; i < nq * MC; i += blockDim.x) {
         const int lk = i / nq, q = i - lk * nq;
         const int mz = mz0 + lk;
@@ -2230,7 +2312,8 @@ __device__ __forceinline__ void k_fft_x_tma(const FftXP& P, typename Cx<T>::t* _
         if (threadIdx.x == 0) atomicOr(status, ST_TIMEOUT);
         return;
     }
-    const bool fused = fuse6(P.plan0, K0);
+    const int br = boundary_radix(P.plan0, K0);
+    const bool fused = br == 4 || br == 6;
     if (fused)
         fft_fwd_head<T, RM, true>(a, NL, P.d_lines, 0, P.plan0, tw0);
     else
@@ -2245,7 +2328,14 @@ __device__ __forceinline__ void k_fft_x_tma(const FftXP& P, typename Cx<T>::t* _
     C zero;
     zero.x = 0;
     zero.y = 0;
-    if (fused) x_mid6<T, true, false>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+    if (br == 6 && P.energy)
+        x_mid<T, 6, true, false, true>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+    else if (br == 4 && P.energy)
+        x_mid<T, 4, true, false, true>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+    else if (br == 6)
+        x_mid<T, 6, true, false, false>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
+    else if (br == 4)
+        x_mid<T, 4, true, false, false>(P, a, myp, mz0, mcount, tab0, tab1, tab2, esum);
     for (int i = threadIdx.x; !fused && i < (n0 << lmc); i += blockDim.x) {
         const int lk = i & (MC - 1), p = i >> lmc;
         const int xi = P.irev[p];
@@ -2298,8 +2388,14 @@ __device__ __forceinline__ void k_fft_x_tma(const FftXP& P, typename Cx<T>::t* _
     }
 }
 
+// Threads of an x-pass CTA.
+template <typename T>
+constexpr int x_threads_max()
+{
+    return z_threads_max<T>();
+}
 template <typename T, int RM>
-__global__ void __launch_bounds__(z_threads_max<T>(), 2) k_fft_x_kspace(FftXP P, typename Cx<T>::t* __restrict__ F2,
+__global__ void __launch_bounds__(x_threads_max<T>(), 2) k_fft_x_kspace(FftXP P, typename Cx<T>::t* __restrict__ F2,
                                                            typename Cx<T>::t* __restrict__ F2psi,
                                                            const typename Cx<T>::t* __restrict__ tw0,
                                                            const T* __restrict__ tab0, const T* __restrict__ tab1,
@@ -2334,29 +2430,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_fft_z_c2r(FftZP P, const typena
     C zero;
     zero.x = 0;
     zero.y = 0;
-    if (fuse6(P.plan2, P.K[2])) {
-        const int B = n2 / 6, K = nk - 1, tot = z_items(B, ncl);
-        for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-            int l, c;
-            z_item(i, ncl, P.d_ncl, l, c);
-            if (2 * c > B) continue;
-            const C* rowA = F1 + ((size_t)cx * n1 + y0 + 2 * l) * nk;
-            const int md[4] = { c, B + c, B - c, 2 * B - c };
-            C A[4], Bv[4], X[6], Y[6];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                A[e] = md[e] <= K ? rowA[md[e]] : zero;
-                Bv[e] = md[e] <= K ? rowA[nk + md[e]] : zero;
-            }
-            z_pair_inverse<T>(A, Bv, c, X, Y);
-            C* px = a + l * CS + P.rev[c];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) px[q] = X[q];
-            if (c > 0 && 2 * c < B) {
-                C* py = a + l * CS + P.rev[B - c];
-#pragma unroll
-                for (int q = 0; q < 6; ++q) py[q] = Y[q];
-            }
+    const int br = boundary_radix(P.plan2, P.K[2]);
+    if (br) {
+        auto rows = [&](int l, const C*& ra, const C*& rb) {
+            ra = F1 + ((size_t)cx * n1 + y0 + 2 * l) * nk;
+            rb = ra + nk;
+        };
+        switch (br) {
+        case 4: z_head<T, 4>(a, CS, ncl, P.d_ncl, n2, nk - 1, P.rev, rows); break;
+        case 6: z_head<T, 6>(a, CS, ncl, P.d_ncl, n2, nk - 1, P.rev, rows); break;
+        default: z_head<T, 8>(a, CS, ncl, P.d_ncl, n2, nk - 1, P.rev, rows); break;
         }
         __syncthreads();
         fft_inv_tail<T, RM>(a, ncl, P.d_ncl, CS, P.plan2, tw2);
@@ -2463,7 +2546,7 @@ __device__ __forceinline__ void k_zfft_interp_body(const SpZP& P, const int* __r
     const int nr = home_fetch(P, cstart, bx, by, H, rb0, rlen);
     // no node near the block (rlen is 0 past the ranges): nothing to transform
     if (!__syncthreads_or(rlen > 0)) return;
-    const bool fused = fuse6(P.plan2, P.K[2]);
+    const int fused = boundary_radix(P.plan2, P.K[2]);
     if (!fused) zero_cx(cb, ncl * CS);
     if (tid < kHomeMax) {
         r_beg[tid] = rb0;
@@ -2473,11 +2556,7 @@ __device__ __forceinline__ void k_zfft_interp_body(const SpZP& P, const int* __r
     home_prefix(r_pre);
     if (fused) {
         // the inverse boundary pass, modes straight from the two rows
-        const int B = n2 / 6, K = nk - 1, tot = z_items(B, ncl);
-        for (int i = tid; i < tot; i += blockDim.x) {
-            int l, c;
-            z_item(i, ncl, P.d_ncl, l, c);
-            if (2 * c > B) continue;
+        auto rows = [&](int l, const C*& ra, const C*& rb) {
             const C* row[2];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
@@ -2486,25 +2565,13 @@ __device__ __forceinline__ void k_zfft_interp_body(const SpZP& P, const int* __r
                 const int lx = fdiv(rem, P.d_ty), ly = rem - lx * Ty;
                 row[r] = F1 + (((size_t)cc * n0 + bx * Tx + lx) * n1 + by * Ty + ly) * nk;
             }
-            const int md[4] = { c, B + c, B - c, 2 * B - c };
-            C A[4], Bv[4], X[6], Y[6];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                A[e].x = A[e].y = Bv[e].x = Bv[e].y = (T)0;
-                if (md[e] <= K) {
-                    A[e] = row[0][md[e]];
-                    Bv[e] = row[1][md[e]];
-                }
-            }
-            z_pair_inverse<T>(A, Bv, c, X, Y);
-            C* px = cb + l * CS + P.rev[c];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) px[q] = X[q];
-            if (c > 0 && 2 * c < B) {
-                C* py = cb + l * CS + P.rev[B - c];
-#pragma unroll
-                for (int q = 0; q < 6; ++q) py[q] = Y[q];
-            }
+            ra = row[0];
+            rb = row[1];
+        };
+        switch (fused) {
+        case 4: z_head<T, 4>(cb, CS, ncl, P.d_ncl, n2, nk - 1, P.rev, rows); break;
+        case 6: z_head<T, 6>(cb, CS, ncl, P.d_ncl, n2, nk - 1, P.rev, rows); break;
+        default: z_head<T, 8>(cb, CS, ncl, P.d_ncl, n2, nk - 1, P.rev, rows); break;
         }
     } else {
     // Z_k = A_k + i B_k, Z_{n-k} = conj(A_k) + i conj(B_k) at the digit-reversed
@@ -3064,7 +3131,7 @@ struct FftXLaunch {
         const T* tab0 = (const T*)w.ktab + (P.single_decon ? ntab : 0);
         const T* tab1 = tab0 + (P.K[0] + 1);
         const T* tab2 = tab1 + (P.K[1] + 1);
-        const int nt = P.nthreads > 0 && P.nthreads <= z_threads_max<T>() ? P.nthreads : kThreads;
+        const int nt = P.nthreads > 0 ? std::min(P.nthreads, x_threads_max<T>()) : kThreads;
         k_fft_x_kspace<T, RM><<<(2 * P.K[1] + 1) * nch, nt, sm, s>>>(
             Q, (C*)w.f2, want_psi ? (C*)w.f2psi : nullptr, (const C*)w.tw, tab0, tab1, tab2, map, w.status);
         return cudaGetLastError();
@@ -3158,7 +3225,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_fft_y_b(const FftYD<T>* __restr
 }
 
 template <typename T, int RM>
-__global__ void __launch_bounds__(z_threads_max<T>(), 2) k_fft_x_kspace_b(const FftXD<T>* __restrict__ d,
+__global__ void __launch_bounds__(x_threads_max<T>(), 2) k_fft_x_kspace_b(const FftXD<T>* __restrict__ d,
                                                                         const int* __restrict__ bs, int n)
 {
     using C = typename Cx<T>::t;
@@ -3273,7 +3340,8 @@ cudaError_t launch_fft_x_kspace_b(const BatchL& L, cudaStream_t s)
     cudaError_t e =
         cudaFuncSetAttribute(k_fft_x_kspace_b<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
     if (e != cudaSuccess) return e;
-    k_fft_x_kspace_b<T, 8><<<L.total, L.threads, L.smem, s>>>((const FftXD<T>*)L.desc, L.bstart, L.n);
+    const int nt = std::min(L.threads, x_threads_max<T>());
+    k_fft_x_kspace_b<T, 8><<<L.total, nt, L.smem, s>>>((const FftXD<T>*)L.desc, L.bstart, L.n);
     return cudaGetLastError();
 }
 
