@@ -57,6 +57,28 @@ __device__ __forceinline__ float erfcx_f(float x)
     return v;
 }
 
+// erfcx_f of two arguments; 1 / (1 + x/2) from the hardware's approximation
+// and one Newton step (the correctly rounded value but for rare last places).
+__device__ __forceinline__ unsigned long long erfcx_2(unsigned long long x)
+{
+    using U = unsigned long long;
+    constexpr float c[11] = { 1.441113045e-05f, 2.817091850e-01f, 2.866406861e-01f, 2.157398867e-01f,
+                              3.128657818e-01f, -3.176314365e-01f, 7.893466267e-01f, -1.078447950e+00f,
+                              7.163310796e-01f, -2.393311398e-01f, 3.276285984e-02f };
+    const U d = fma2(dup2(0.5f), x, dup2(1.0f));
+    const float2 df = upk2(d);
+    float t0, t1;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(df.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(df.y));
+    const U y = pk2(t0, t1);
+    const U e = fma2(pk2(-df.x, -df.y), y, dup2(1.0f));
+    const U t = fma2(y, e, y);
+    U v = dup2(c[10]);
+#pragma unroll
+    for (int k = 9; k >= 0; --k) v = fma2(v, t, dup2(c[k]));
+    return v;
+}
+
 // 1 / sqrt(x) and exp(x) of the pair terms: float32 through the hardware
 // approximations (reciprocal square root; exp as 2^(x log2 e), whose scaled
 // argument costs about |x| 2^-24 relative, below 1e-6 for the |x| <= beta^2
@@ -386,8 +408,9 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
 // apart along each axis: their neighbourhoods are almost the same (node
 // spacings are a fraction of the cut-off), so one walk over the union of their
 // rows serves both: the row search, the candidate's table look-up and its
-// record are paid once for two pair terms.  Every pair term is the one of
-// k_short_body, rounded alike; a lane adds each node's terms by itself.
+// record are paid once for two pair terms, and the two are computed together
+// in packed float32 arithmetic.  Every pair term is the one of k_short_body,
+// operation by operation.
 // Needs at least 2 (m + 2) cells per axis (no axis taken whole, the nearest
 // cell image is the minimum image of every candidate for both nodes).
 __device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>& ta, const SrTgt<float>& tb, int dx,
@@ -406,7 +429,6 @@ __device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>
     const float h0 = (float)P.hc[0], h1 = (float)P.hc[1], h2 = (float)P.hc[2];
     const float rc2 = (float)P.rc2;
     const float alpha = (float)P.alpha;
-    const float two_over_sqrtpi = 1.12837916709551257390f;
     const int m = P.m;
     const int ny = 2 * m + 1 + abs(dy), nz = 2 * m + 1 + abs(dz);
     const int y0 = min(dy, 0) - m, z0 = min(dz, 0) - m;  // first row offsets from the first node's cell
@@ -418,7 +440,10 @@ __device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>
     const float ox[2] = { ta.o[0] + 0.5f * h0, tb.o[0] + 0.5f * h0 };
     const float oy[2] = { ta.o[1] + 0.5f * h1, tb.o[1] + 0.5f * h1 };
     const float oz[2] = { ta.o[2] + 0.5f * h2, tb.o[2] + 0.5f * h2 };
-    float v[2][3] = {}, ps[2][3] = {};
+    using U = unsigned long long;
+    const U h00 = dup2(h0), alpha2 = dup2(alpha), two2 = dup2(1.12837916709551257390f);
+    const U mox = pk2(-ta.o[0], -tb.o[0]), moy = pk2(-ta.o[1], -tb.o[1]), moz = pk2(-ta.o[2], -tb.o[2]);
+    U v[3] = {}, ps[3] = {};
     for (int rb = 0; rb < nrows; rb += 32) {
         const int r = rb + lane;
         int s0 = 0, n0 = 0, s1 = 0, n1r = 0, dyi = 0, dzi = 0;
@@ -518,41 +543,48 @@ __device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>
             const int2 of = *reinterpret_cast<const int2*>(&rows.ofs[wslot][own]);
             const float4 dh = *reinterpret_cast<const float4*>(rows.dh[wslot][own]);
             const float xc = (float)(S.cx + (first ? of.x : of.y));
-            float rx[2], ry[2], rz[2], r2[2];
-            rx[0] = xc * h0 + (S.o[0] - ta.o[0]);
-            ry[0] = dh.x + (S.o[1] - ta.o[1]);
-            rz[0] = dh.y + (S.o[2] - ta.o[2]);
-            rx[1] = (xc - dxf) * h0 + (S.o[0] - tb.o[0]);
-            ry[1] = dh.z + (S.o[1] - tb.o[1]);
-            rz[1] = dh.w + (S.o[2] - tb.o[2]);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) r2[e] = rx[e] * rx[e] + ry[e] * ry[e] + rz[e] * rz[e];
+            // both nodes at once: (first node, second node) in register pairs
+            const U sx = dup2(S.o[0]), sy = dup2(S.o[1]), sz = dup2(S.o[2]);
+            const U rx = fma2(pk2(xc, xc - dxf), h00, add2(sx, mox));
+            const U ry = add2(pk2(dh.x, dh.z), add2(sy, moy));
+            const U rz = add2(pk2(dh.y, dh.w), add2(sz, moz));
+            const U r2 = fma2(rz, rz, fma2(rx, rx, mul2(ry, ry)));
+            const float2 r2f = upk2(r2);
             // C_0 of each node is left out
-            const bool in0 = r2[0] < rc2 && r2[0] != 0.0f && S.seg != j && S.seg != jp[0];
-            const bool in1 = r2[1] < rc2 && r2[1] != 0.0f && S.seg != j + 1 && S.seg != jp[1];
+            const bool in0 = r2f.x < rc2 && r2f.x != 0.0f && S.seg != j && S.seg != jp[0];
+            const bool in1 = r2f.y < rc2 && r2f.y != 0.0f && S.seg != j + 1 && S.seg != jp[1];
             if (!(in0 || in1)) continue;
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const float ir = rsqrt_t(r2[e]);
-                const float rr = r2[e] * ir;
-                const float x = alpha * rr;
-                const float ee = exp_t(-x * x);
-                const float ec = erfc_e(x, ee);
-                const float g = ec + two_over_sqrtpi * x * ee;
-                float fv = g * ir * ir * ir;
-                fv = (e ? in1 : in0) ? fv : 0.0f;
-                v[e][0] += fv * (ry[e] * S.q[2] - rz[e] * S.q[1]);
-                v[e][1] += fv * (rz[e] * S.q[0] - rx[e] * S.q[2]);
-                v[e][2] += fv * (rx[e] * S.q[1] - ry[e] * S.q[0]);
-                if (P.want_psi) {
-                    const float fp = (e ? in1 : in0) ? ec * ir : 0.0f;
-                    ps[e][0] += fp * S.q[0];
-                    ps[e][1] += fp * S.q[1];
-                    ps[e][2] += fp * S.q[2];
-                }
+            const U ir = pk2(rsqrt_t(r2f.x), rsqrt_t(r2f.y));
+            const U x = mul2(alpha2, mul2(r2, ir));
+            const float2 xx = upk2(mul2(x, x));
+            const U ee = pk2(exp_t(-xx.x), exp_t(-xx.y));
+            const U ec = mul2(ee, erfcx_2(x));
+            const U g = fma2(mul2(two2, x), ee, ec);
+            const float2 ff = upk2(mul2(mul2(mul2(g, ir), ir), ir));
+            const U fv = pk2(in0 ? ff.x : 0.0f, in1 ? ff.y : 0.0f);
+            const U q0 = dup2(S.q[0]), q1 = dup2(S.q[1]), q2 = dup2(S.q[2]);
+            const U n0 = dup2(-S.q[0]), n1 = dup2(-S.q[1]), n2 = dup2(-S.q[2]);
+            v[0] = fma2(fv, fma2(ry, q2, mul2(rz, n1)), v[0]);
+            v[1] = fma2(fv, fma2(rz, q0, mul2(rx, n2)), v[1]);
+            v[2] = fma2(fv, fma2(rx, q1, mul2(ry, n0)), v[2]);
+            if (P.want_psi) {
+                const float2 pf = upk2(mul2(ec, ir));
+                const U fp = pk2(in0 ? pf.x : 0.0f, in1 ? pf.y : 0.0f);
+                ps[0] = fma2(fp, q0, ps[0]);
+                ps[1] = fma2(fp, q1, ps[1]);
+                ps[2] = fma2(fp, q2, ps[2]);
             }
         }
         __syncwarp();  // the table is rewritten by the next round of rows
+    }
+    float vf[2][3], pf[2][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float2 a = upk2(v[c]), b = upk2(ps[c]);
+        vf[0][c] = a.x;
+        vf[1][c] = a.y;
+        pf[0][c] = b.x;
+        pf[1][c] = b.y;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
@@ -560,16 +592,16 @@ __device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>
         for (int e = 0; e < 2; ++e)
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                v[e][c] += __shfl_xor_sync(0xffffffffu, v[e][c], o);
-                if (P.want_psi) ps[e][c] += __shfl_xor_sync(0xffffffffu, ps[e][c], o);
+                vf[e][c] += __shfl_xor_sync(0xffffffffu, vf[e][c], o);
+                if (P.want_psi) pf[e][c] += __shfl_xor_sync(0xffffffffu, pf[e][c], o);
             }
     if (lane == 0) {
 #pragma unroll
         for (int e = 0; e < 2; ++e)
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                vsr[3 * (j + e) + c] = P.pref * (double)v[e][c];
-                if (P.want_psi) psr[3 * (j + e) + c] = P.pref * (double)ps[e][c];
+                vsr[3 * (j + e) + c] = P.pref * (double)vf[e][c];
+                if (P.want_psi) psr[3 * (j + e) + c] = P.pref * (double)pf[e][c];
             }
     }
 }
