@@ -704,6 +704,8 @@ void fill_geom(const bs_ctx* c, GeomP& G)
     }
     G.kappa = p.kappa;
     G.a = p.a;
+    G.pv = p.kappa / (4.0 * kPi);
+    G.pp = p.kappa / (2.0 * kPi);
     G.log2a = std::log(2.0 / p.a);
     G.delta = p.delta;
     G.alpha = p.alpha;

@@ -132,6 +132,21 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
 }
 __device__ __forceinline__ unsigned long long dup2(float a) { return pk2(a, a); }
 
+// x wrapped into [0, L) (iL = 1/L); non-finite input maps to 0 and raises the
+// flag.  The comparisons are made on the bits (float64 comparisons share the
+// slow pipe).
+__device__ __forceinline__ double wrap_box(double x, double L, double iL, bool& bad)
+{
+    if ((__double2hiint(x) & 0x7ff00000) == 0x7ff00000) {
+        bad = true;
+        return 0.0;
+    }
+    double y = x - L * floor(x * iL);
+    if (__double_as_longlong(y) >= __double_as_longlong(L)) y -= L;  // L > 0, a negative y is below
+    if (__double2hiint(y) < 0) y = 0.0;
+    return y;
+}
+
 // Monomial coefficients in t (stride apart) of the degree-deg polynomial
 // through f(c + w t) at the Chebyshev points t of [-1/2, 1/2] (divided
 // differences, extended precision; host, deg < 32).
@@ -157,6 +172,7 @@ struct GeomP {
     double iL[3], ihc[3], ihg[3];  // reciprocals of L, hc, hg (binning multiplies: float64 division is slow here)
     int want_psi;
     double local_frac;  // subdivided local segments (0: off)
+    double pv, pp;      // kappa / (4 pi), kappa / (2 pi): a float64 division per node saved
     double log2a;       // log(2 / a): the local term's logarithm is log(l- l+) / 2 + log(2 / a)
 };
 

@@ -1273,10 +1273,12 @@ __host__ __device__ __forceinline__ size_t zlines_bytes(int ncl, int cls)
 // bucket adds both.  The lines see 3 TX atomic adds per lane and bucket
 // instead of per lane and copy.  Needs an even Ty, Ty W <= 32 and n2 >= 2 W
 // (the 2 W cells of a lane's window are distinct planes).
-template <typename T, int W, int TX>
-__device__ __forceinline__ void spread_bucketed(const SpZP& P, int s0, int s1, const int2* __restrict__ cidx,
-                                                const SpPt<T, W>* __restrict__ pts, SpPt<T, W>* sbuf, T* accf)
+template <int W, int TX>
+__device__ __forceinline__ void spread_bucketed_d(const SpZP& P, int s0, int s1, const int2* __restrict__ cidx,
+                                                const SpPt<double, W>* __restrict__ pts, SpPt<double, W>* sbuf,
+                                                  double* accf)
 {
+    using T = double;
     constexpr int RCW = kSpzWarpChunk;
     constexpr int kWords = (int)(sizeof(SpPt<T, W>) / 16);
     constexpr int kIt = (RCW * kWords + 31) / 32;
@@ -1364,30 +1366,24 @@ __device__ __forceinline__ void spread_bucketed(const SpZP& P, int s0, int s1, c
                 const bool first = t >= d;
                 const int tz = (W & (W - 1)) == 0 ? ((t - d) & (W - 1)) : (first ? t - d : t - d + W);
                 const T wyz = R.wy[jy] * R.wz[tz];
-                const T wl = first ? wyz : (T)0, wh = first ? (T)0 : wyz;
-                T q0, q1, q2;
-                if constexpr (sizeof(T) == 4) {
-                    const float4 bq = *reinterpret_cast<const float4*>(&R);  // base, q[0..2]
-                    q0 = bq.y;
-                    q1 = bq.z;
-                    q2 = bq.w;
-                } else {
-                    q0 = R.q[0];
-                    q1 = R.q[1];
-                    q2 = R.q[2];
-                }
+                const T q0 = R.q[0], q1 = R.q[1], q2 = R.q[2];
+                // a lane adds to one of its two cells: picked by selects (the
+                // float64 pipe is the bound, and adding zeros to the other
+                // cell was 3 of 8 operations)
 #pragma unroll
                 for (int a = 0; a < TX; ++a) {
                     const int jx = a - r0;  // the same in the whole warp
                     if ((unsigned)jx < (unsigned)W) {
-                        const T wx = R.wx[jx];
-                        const T vl = wx * wl, vh = wx * wh;
-                        lo[a][0] += vl * q0;
-                        lo[a][1] += vl * q1;
-                        lo[a][2] += vl * q2;
-                        hi[a][0] += vh * q0;
-                        hi[a][1] += vh * q1;
-                        hi[a][2] += vh * q2;
+                        const T v = R.wx[jx] * wyz;
+                        const T s0 = fma(v, q0, first ? lo[a][0] : hi[a][0]);
+                        const T s1 = fma(v, q1, first ? lo[a][1] : hi[a][1]);
+                        const T s2 = fma(v, q2, first ? lo[a][2] : hi[a][2]);
+                        lo[a][0] = first ? s0 : lo[a][0];
+                        lo[a][1] = first ? s1 : lo[a][1];
+                        lo[a][2] = first ? s2 : lo[a][2];
+                        hi[a][0] = first ? hi[a][0] : s0;
+                        hi[a][1] = first ? hi[a][1] : s1;
+                        hi[a][2] = first ? hi[a][2] : s2;
                     }
                 }
             }
@@ -1400,7 +1396,7 @@ __device__ __forceinline__ void spread_bucketed(const SpZP& P, int s0, int s1, c
 }
 
 // The bucketed loop in float32.  It is bound by the instructions per copy (65
-// in spread_bucketed, 12 copies per point on the 4e6-node tangle), so the
+// in the float64 form, 12 copies per point on the 4e6-node tangle), so the
 // index work is done once per copy while it is staged and not by every lane
 // at every copy: four lanes per copy pick the weights that the block needs
 // out of the point's record and lay them down at fixed places, weights
@@ -1582,9 +1578,9 @@ __device__ __forceinline__ void k_spread_zfft_body(const SpZP& P, const int* __r
             }
         } else {
             switch (Tx) {
-            case 1: spread_bucketed<T, W, 1>(P, s0, s1, cidx, pts, sbuf, accf); break;
-            case 2: spread_bucketed<T, W, 2>(P, s0, s1, cidx, pts, sbuf, accf); break;
-            default: spread_bucketed<T, W, 4>(P, s0, s1, cidx, pts, sbuf, accf); break;
+            case 1: spread_bucketed_d<W, 1>(P, s0, s1, cidx, pts, sbuf, accf); break;
+            case 2: spread_bucketed_d<W, 2>(P, s0, s1, cidx, pts, sbuf, accf); break;
+            default: spread_bucketed_d<W, 4>(P, s0, s1, cidx, pts, sbuf, accf); break;
             }
         }
         __syncthreads();
@@ -2713,18 +2709,14 @@ __device__ __forceinline__ void k_node_w_body(const InterpP& P, int tx, int ty, 
         T fr[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            double x = nodes[3 * j + d];
-            if (!isfinite(x)) x = 0.0;
-            double xw = x - P.L[d] * floor(x * P.iL[d]);
-            if (xw >= P.L[d]) xw -= P.L[d];
-            if (xw < 0.0) xw = 0.0;
+            bool bad = false;
+            const double xw = wrap_box(nodes[3 * j + d], P.L[d], P.iL[d], bad);
             const double g = xw * P.ihg[d];
-            int k = (int)floor(g);
-            k = k < 0 ? 0 : (k >= P.ng[d] ? P.ng[d] - 1 : k);
-            double f = g - (double)k;
-            f = f < 0.0 ? 0.0 : (f > 1.0 ? 1.0 : f);
+            int k = (int)g;  // g >= 0
+            k = k >= P.ng[d] ? P.ng[d] - 1 : k;
+            const T f = (T)(g - i2d(k));
             ib[d] = k;
-            fr[d] = (T)f;
+            fr[d] = f > (T)1 ? (T)1 : f;
         }
         kb_weights<T, W>(fr, P.zeta, P.inorm, P.kbc, R.wx, R.wy, R.wz);
         R.base = ib[0] | (ib[1] << 10) | (ib[2] << 20);
