@@ -829,6 +829,7 @@ void fill_spzp(const bs_ctx* c, bool det, SpZP& SZ)
     SZ.nzb = d.nzb;
     // room for the interpolation's periodic halo of w - 1 positions
     SZ.cls = line_stride(d.ng[2] + p.nufft_w - 1, 3 * d.tx * d.ty / 2, 128 / (2 * (int)sizeof(T)));
+    SZ.scls = line_stride(d.ng[2], 3 * d.tx * d.ty / 2, 128 / (2 * (int)sizeof(T)));
     SZ.ls = d.lsz;
     while (SZ.ls < SZ.cls) SZ.ls += 32;  // the real region also holds the complex lines
     SZ.zeta = d.zeta;
@@ -1975,6 +1976,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
             const Work& w = c->w;
             SpzD<T> e;
             fill_spzp<T>(c, false, e.P);
+            e.P.cls = e.P.scls;
             e.cstart = w.col_cnt;
             e.recs = w.col_rec;
             e.pts = w.col_pts;

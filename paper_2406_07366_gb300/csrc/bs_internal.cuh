@@ -293,7 +293,8 @@ struct SpZP {
     int w;
     int nzb;            // z-buckets per block: > 1 selects the bucketed record loop
     int ls;             // padded stride of the real z-lines in shared memory
-    int cls;            // complex line stride of the z FFT buffers
+    int cls;            // complex line stride of the z FFT buffers (the interpolation's, with its halo)
+    int scls;           // the same of the spread
     double zeta;
     FftPlan plan2;
     const int* rev;  // position of frequency k after the forward transform, k < n

@@ -1972,8 +1972,10 @@ __device__ __forceinline__ void k_fft_y_tma(const FftYP& P, typename Cx<T>::t* _
     }
 }
 
+// Four CTAs per SM in float32 (64 registers): the loads' latency is the bound
+// (768^3: 1.38 -> 1.30 ms forward, 1.73 -> 1.55 inverse against 72 registers).
 template <typename T, int RM>
-__global__ void __launch_bounds__(kThreads, 2) k_fft_y(FftYP P, typename Cx<T>::t* __restrict__ F1,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_fft_y(FftYP P, typename Cx<T>::t* __restrict__ F1,
                                                     typename Cx<T>::t* __restrict__ F2,
                                                     const typename Cx<T>::t* __restrict__ tw1, int sign,
                                                     const __grid_constant__ CUtensorMap tm, int* status)
@@ -2880,9 +2882,15 @@ size_t nd_rec_bytes(int w)
 template <typename T>
 size_t spread_zfft_smem(const SpZP& P)
 {
-    using C = typename Cx<T>::t;
-    const int ncl = 3 * P.tx * P.ty / 2;
-    return zlines_bytes<T>(ncl, P.cls) + 2 * spz_rec_chunk<T>() * col_pt_bytes<T>(P.w);  // two record chunks
+    const size_t lines = zlines_bytes<T>(3 * P.tx * P.ty / 2, P.cls);
+    if (sizeof(T) == 4 && P.nzb > 1) {
+        // bucketed float32 loop: a staged chunk per warp.  Half of the general
+        // loop's buffers: three CTAs become four on 192^3 grids, one becomes
+        // two on 512^3
+        const int stride = (((6 + 2 * P.tx + 1 + 3) & ~3) + 4 + P.w + 3) & ~3;  // spz_stride
+        return lines + (size_t)(z_threads<T>(P) / 32) * kSpzWarpChunk * stride * sizeof(T);
+    }
+    return lines + 2 * spz_rec_chunk<T>() * col_pt_bytes<T>(P.w);  // two record chunks
 }
 
 // Register-budget class of a plan: the largest radix it uses, rounded up to
@@ -2931,8 +2939,10 @@ static cudaError_t spz_w(const SpZP& P, const Work& w, cudaStream_t s)
 }
 
 template <typename T>
-cudaError_t launch_spread_zfft(const SpZP& P, const Work& w, cudaStream_t s)
+cudaError_t launch_spread_zfft(const SpZP& P0, const Work& w, cudaStream_t s)
 {
+    SpZP P = P0;
+    P.cls = P0.scls;
     switch (P.w) {
     case 2: return spz_w<T, 2>(P, w, s);
     case 4: return spz_w<T, 4>(P, w, s);
