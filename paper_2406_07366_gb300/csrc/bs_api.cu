@@ -1727,11 +1727,13 @@ BatchL stage(Arena& A, const std::vector<D>& desc, const std::vector<int>& block
 {
     std::vector<int> bs(desc.size() + 1, 0);
     for (size_t m = 0; m < desc.size(); ++m) bs[m + 1] = bs[m] + blocks[m];
+    const int total = bs.back();
+    for (size_t m = 0; m < desc.size(); ++m) bs.insert(bs.end(), blocks[m], (int)m);  // each CTA's member
     BatchL L;
     L.desc = (const void*)A.put(desc.data(), sizeof(D) * desc.size());
     L.bstart = (const int*)A.put(bs.data(), sizeof(int) * bs.size());
     L.n = (int)desc.size();
-    L.total = bs.back();
+    L.total = total;
     L.threads = threads;
     L.smem = smem;
     return L;

@@ -791,14 +791,18 @@ __device__ __forceinline__ int rev8_neg(const Rev8& r, const int* __restrict__ r
     return r.ok ? (d == 0 ? r.pa : r.pb + (8 - d) * r.st0) : rev[k == 0 ? 0 : n - k];
 }
 
-template <typename T>
-__device__ __forceinline__ T kb_val(T z, T zeta, T inorm)
+// The kernel at z (float32): 2 e^{-zeta} sinh(zeta s) / s.  Where 2 zeta s > 20 the
+// second exponential is lost against 1 (expm1f returns -1 there): whole warps
+// skip it at the inner support points.
+__device__ __forceinline__ float kb_val(float z, float zeta, float inorm)
 {
-    T s2 = (T)1 - z * z;
-    s2 = s2 > (T)0 ? s2 : (T)0;
-    const T s = sqrt(s2);
-    const T num = (s > (T)1e-6) ? -expm1((T)-2 * zeta * s) / s : (T)2 * zeta;
-    return exp(zeta * (s - (T)1)) * num * inorm;
+    float s2 = 1.0f - z * z;
+    s2 = s2 > 0.0f ? s2 : 0.0f;
+    const float s = sqrt(s2);
+    const float a = -2.0f * zeta * s;
+    const float em = a < -20.0f ? -1.0f : expm1f(a);
+    const float num = (s > 1e-6f) ? -em / s : 2.0f * zeta;
+    return exp(zeta * (s - 1.0f)) * num * inorm;
 }
 
 // The 3 W kernel weights of a point at grid fractions f (support point t at
@@ -3215,7 +3219,7 @@ __global__ void __launch_bounds__(z_threads_max<T>(), 2) k_spread_zfft_b(const S
 }
 
 template <typename T, int RM>
-__global__ void __launch_bounds__(kThreads, 2) k_fft_y_b(const FftYD<T>* __restrict__ d, const int* __restrict__ bs,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_fft_y_b(const FftYD<T>* __restrict__ d, const int* __restrict__ bs,
                                                       int n)
 {
     using C = typename Cx<T>::t;
