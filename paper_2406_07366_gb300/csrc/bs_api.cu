@@ -385,6 +385,9 @@ int derive(const bs_params* p, Derived* d)
     const size_t mcy = 50000 / ((size_t)(d->ng[1] + 1) * cb);
     d->lmcy = 0;
     while (d->lmcy < 4 && ((size_t)2 << d->lmcy) <= mcy) ++d->lmcy;
+    // 17 to 20 modes: one chunk of 32 in place of a full one and one with 1 to 4
+    // modes (grids of 33 to 39 modes a side, the small members of batches)
+    if (d->lmcy == 4 && d->K[2] + 1 > 16 && d->K[2] + 1 <= 20 && 32 <= mcy) d->lmcy = 5;
     const int lines_x = (p->flags & BS_WANT_PSI) ? 6 : 3;
     // the x pass gets the same larger CTAs as the z-column blocks (two
     // 512-thread CTAs per SM; measured on the 384^3 grid: 0.29 ms against
@@ -1850,40 +1853,43 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         add(D, 128, 0);
     }
     // counting sorts: zero the counts, count, scan, copy to the cursors, scatter
-    auto zero_stage = [&](auto cnt_of, auto n_of) {
-        std::vector<ZeroD> Z;
-        for (size_t m = 0; m < nm; ++m) {
-            Z.push_back({ cnt_of(mem[m]), n_of(mem[m]) + 1 });
-            blk.push_back(std::min(cdiv(n_of(mem[m]) + 1, 256), 256));
-        }
-        add(Z, 256, 0);
-    };
-    auto scan_stage = [&](auto cnt_of, auto n_of, auto tmp_of) {
+    // exclusive scan of a counter array per member, the starts copied to cur_of
+    // (null: no copy); the second list has one CTA per member: members of up to
+    // 8 tiles are scanned by one CTA each in one launch
+    auto scan_stage = [&](auto cnt_of, auto n_of, auto tmp_of, auto cur_of) {
         std::vector<ScanD> S;
         std::vector<int> one;
+        int most = 0;
         for (size_t m = 0; m < nm; ++m) {
             const int n = n_of(mem[m]);
-            S.push_back({ cnt_of(mem[m]), n, tmp_of(mem[m]), scan_blocks(n) });
+            S.push_back({ cnt_of(mem[m]), n, tmp_of(mem[m]), scan_blocks(n), cur_of(mem[m]) });
             blk.push_back(scan_blocks(n));
             one.push_back(1);
+            most = std::max(most, scan_blocks(n));
         }
         add(S, 1024, 0);
         blk = one;
         add(S, 1024, 0);
-    };
-    auto copy_stage = [&](auto cnt_of, auto n_of, auto cur_of) {
-        std::vector<CopyD> Cd;
-        for (size_t m = 0; m < nm; ++m) {
-            Cd.push_back({ cnt_of(mem[m]), cur_of(mem[m]), n_of(mem[m]) });
-            blk.push_back(std::min(cdiv(n_of(mem[m]), 256), 256));
-        }
-        add(Cd, 256, 0);
+        st.back().kind = most <= 8;
     };
     auto cell_cnt = [](bs_ctx* c) { return c->w.cell_cnt; };
     auto cell_n = [](bs_ctx* c) { return (int)c->d.ncells; };
     auto cell_tmp = [](bs_ctx* c) { return c->w.scan_tmp; };
     auto cell_cur = [](bs_ctx* c) { return c->w.cell_cur; };
-    zero_stage(cell_cnt, cell_n);                                                          // 2 zero
+    {   // 2 zero: the bin counters and the interpolation's sums
+        std::vector<ZeroD> Z;
+        for (size_t m = 0; m < nm; ++m) {
+            const bs_ctx* c = mem[m];
+            const int n4[4] = { (int)c->d.ncells + 1, c->d.ncolb + 1, c->d.ncols + 1,
+                                (int)(3 * c->N * (sizeof(T) / 4)) };
+            int* const p4[4] = { c->w.cell_cnt, c->w.col_cnt, c->w.ncol_cnt, (int*)c->w.vacc };
+            for (int k = 0; k < 4; ++k) {
+                Z.push_back({ p4[k], n4[k] });
+                blk.push_back(std::min(cdiv(n4[k], 256), 256));
+            }
+        }
+        add(Z, 256, 0);
+    }
     {   // 3 count
         std::vector<CountD> D;
         for (size_t m = 0; m < nm; ++m) {
@@ -1892,9 +1898,8 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, kThreads, 0);
     }
-    scan_stage(cell_cnt, cell_n, cell_tmp);                                                // 4, 5 scan
-    copy_stage(cell_cnt, cell_n, cell_cur);                                                // 6 copy
-    {   // 7 scatter
+    scan_stage(cell_cnt, cell_n, cell_tmp, cell_cur);                                      // 4, 5 scan
+    {   // 6 scatter
         std::vector<ScatterD<SrRec<T>>> D;
         for (size_t m = 0; m < nm; ++m) {
             const Work& w = mem[m]->w;
@@ -1903,7 +1908,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, kThreads, 0);
     }
-    {   // 8 short range (warp per node, or per pair when most nodes can pair)
+    {   // 7 short range (warp per node, or per pair when most nodes can pair)
         std::vector<ShortD<T>> D;
         const int prec = sizeof(T) == 8 ? BS_FP64 : BS_MIXED;
         long long can = 0, all = 0;
@@ -1935,8 +1940,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
     auto col_n = [](bs_ctx* c) { return c->d.ncols; };   // node bins: blocks
     auto col_tmp = [](bs_ctx* c) { return c->w.scan_tmp2; };
     auto col_cur = [](bs_ctx* c) { return c->w.col_cur; };
-    zero_stage(col_cnt, colb_n);                                                           // 9 zero
-    {   // 10 column count, 13 column scatter share the descriptor shape
+    {   // 8 column count, 11 column scatter share the descriptor shape
         std::vector<ColD<T>> D;
         for (size_t m = 0; m < nm; ++m) {
             const Work& w = mem[m]->w;
@@ -1952,9 +1956,8 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, kThreads, 0);
     }
-    scan_stage(col_cnt, colb_n, col_tmp);                                                  // 11, 12 scan
-    copy_stage(col_cnt, colb_n, col_cur);                                                  // 13 copy
-    {   // 14 column scatter
+    scan_stage(col_cnt, colb_n, col_tmp, col_cur);                                         // 9, 10 scan
+    {   // 11 column scatter
         std::vector<ColD<T>> D;
         for (size_t m = 0; m < nm; ++m) {
             const Work& w = mem[m]->w;
@@ -1970,7 +1973,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, kThreads, 0);
     }
-    {   // 15 spread + z transform
+    {   // 12 spread + z transform
         std::vector<SpzD<T>> D;
         size_t sm = 0;
         for (size_t m = 0; m < nm; ++m) {
@@ -2010,8 +2013,8 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, kThreads, sm);
     };
-    ffty(-1);  // 16
-    {   // 17 x transform + k-space pass + inverse x transform
+    ffty(-1);  // 13
+    {   // 14 x transform + k-space pass + inverse x transform
         std::vector<FftXD<T>> D;
         size_t sm = 0;
         for (size_t m = 0; m < nm; ++m) {
@@ -2031,19 +2034,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, zt, sm);
     }
-    ffty(+1);  // 18
-    {   // 19 zero: the interpolation sums and the node-block counts
-        std::vector<ZeroD> Z;
-        for (size_t m = 0; m < nm; ++m) {
-            const bs_ctx* c = mem[m];
-            const int nv = (int)(3 * c->N * (long long)sizeof(T) / sizeof(int));
-            Z.push_back({ (int*)c->w.vacc, nv });
-            blk.push_back(std::min(cdiv(nv, 256), 256));
-            Z.push_back({ c->w.ncol_cnt, c->d.ncols + 1 });
-            blk.push_back(std::min(cdiv(c->d.ncols + 1, 256), 256));
-        }
-        add(Z, 256, 0);
-    }
+    ffty(+1);  // 15
     std::vector<NodeWD<T>> NW;
     for (size_t m = 0; m < nm; ++m) {
         const bs_ctx* c = mem[m];
@@ -2062,13 +2053,13 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         NW.push_back(e);
         blk.push_back(cdiv(c->N, kThreads));
     }
-    add(NW, kThreads, 0);                                                                  // 20 node weights
+    add(NW, kThreads, 0);                                                                  // 16 node weights
     auto nb_cnt = [](bs_ctx* c) { return c->w.ncol_cnt; };
     auto nb_tmp = [](bs_ctx* c) { return c->w.scan_tmp; };
-    scan_stage(nb_cnt, col_n, nb_tmp);                                                     // 21, 22 scan
+    scan_stage(nb_cnt, col_n, nb_tmp, [](bs_ctx*) { return (int*)nullptr; });              // 17, 18 scan
     for (size_t m = 0; m < nm; ++m) blk.push_back(cdiv(mem[m]->N, kThreads));
-    add(NW, kThreads, 0);                                                                  // 23 node scatter
-    {   // 24 inverse z transform + interpolation
+    add(NW, kThreads, 0);                                                                  // 19 node scatter
+    {   // 20 inverse z transform + interpolation
         std::vector<SpzD<T>> D;
         size_t sm = 0;
         for (size_t m = 0; m < nm; ++m) {
@@ -2088,7 +2079,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, zt, sm);
     }
-    {   // 25 final sum
+    {   // 21 final sum
         std::vector<SumD<T>> D;
         for (size_t m = 0; m < nm; ++m) {
             const bs_ctx* c = mem[m];
@@ -2132,35 +2123,32 @@ int batch_issue_staged(bs_batch* b, cudaStream_t s)
             w = b->ctx[i]->p.nufft_w;
             break;
         }
+    // the short range and the node binning on a side stream, issued after the
+    // main chain's first kernels, as in run()
+    cudaStream_t ss = b->side;
+    CE(launch_zero_b(L[2], s));
     CE(launch_spline_b<T>(L[0], s));
     CE(launch_nodes_b<T>(L[1], s));
-    // the short range and the node binning on a side stream, as in run()
-    cudaStream_t ss = b->side;
     CE(cudaEventRecord(b->ev_side, s));
+    CE(launch_col_count_b<T>(L[8], s));
+    CE(launch_scan_b(L[9], L[10], s));
+    CE(launch_col_scatter_b<T>(w, L[11], s));
+    CE(launch_spread_zfft_b<T>(w, L[12], s));
     CE(cudaStreamWaitEvent(ss, b->ev_side, 0));
-    CE(launch_zero_b(L[2], ss));
     CE(launch_count_b(L[3], ss));
     CE(launch_scan_b(L[4], L[5], ss));
-    CE(launch_copy_b(L[6], ss));
-    CE(launch_scatter_b<SrRec<T>>(L[7], ss));
-    CE(launch_short_b<T>(L[8], ss));
-    CE(launch_zero_b(L[19], ss));
-    CE(launch_node_w_b<T>(w, L[20], ss));
-    CE(launch_scan_b(L[21], L[22], ss));
-    CE(launch_node_scatter_b<T>(w, L[23], ss));
+    CE(launch_scatter_b<SrRec<T>>(L[6], ss));
+    CE(launch_short_b<T>(L[7], ss));
+    CE(launch_node_w_b<T>(w, L[16], ss));
+    CE(launch_scan_b(L[17], L[18], ss));
+    CE(launch_node_scatter_b<T>(w, L[19], ss));
     CE(cudaEventRecord(b->ev_side, ss));
-    CE(launch_zero_b(L[9], s));
-    CE(launch_col_count_b<T>(L[10], s));
-    CE(launch_scan_b(L[11], L[12], s));
-    CE(launch_copy_b(L[13], s));
-    CE(launch_col_scatter_b<T>(w, L[14], s));
-    CE(launch_spread_zfft_b<T>(w, L[15], s));
-    CE(launch_fft_y_b<T>(L[16], s));
-    CE(launch_fft_x_kspace_b<T>(L[17], s));
-    CE(launch_fft_y_b<T>(L[18], s));
+    CE(launch_fft_y_b<T>(L[13], s));
+    CE(launch_fft_x_kspace_b<T>(L[14], s));
+    CE(launch_fft_y_b<T>(L[15], s));
     CE(cudaStreamWaitEvent(s, b->ev_side, 0));
-    CE(launch_zfft_interp_b<T>(w, L[24], s));
-    CE(launch_interp_sum_b<T>(L[25], s));
+    CE(launch_zfft_interp_b<T>(w, L[20], s));
+    CE(launch_interp_sum_b<T>(L[21], s));
     return BS_OK;
 }
 

@@ -597,14 +597,13 @@ struct BatchL {
     int total;    // CTAs of the launch
     int threads;  // threads per CTA
     size_t smem;  // dynamic shared memory per CTA (the largest member's)
-    int kind = 0;  // variant of the kernel (short range: 1 for pairs of nodes)
+    int kind = 0;  // variant of the kernel (short range: pairs of nodes; scan: one CTA per member)
 };
 
 // Descriptors of the batched stages (one per member).
 struct ZeroD { int* p; int n; };                  // p[0..n) = 0
-struct CopyD { const int* src; int* dst; int n; };
 struct CountD { const int* key; int n; int* cnt; };
-struct ScanD { int* cnt; int n; int* part; int nb; };
+struct ScanD { int* cnt; int n; int* part; int nb; int* cur; };
 template <typename R> struct ScatterD { const int* key; const R* in; int n; int* cur; R* out; };
 
 template <typename T> struct SplineD {
@@ -721,7 +720,6 @@ template <typename T>
 size_t zfft_interp_smem(const SpZP& P);
 
 cudaError_t launch_zero_b(const BatchL& L, cudaStream_t s);
-cudaError_t launch_copy_b(const BatchL& L, cudaStream_t s);
 cudaError_t launch_count_b(const BatchL& L, cudaStream_t s);
 // the three phases of the exclusive scan, per member: L1 over each member's
 // scan tiles (scan_blocks(n)), L2 one CTA per member

@@ -90,7 +90,7 @@ __global__ void k_scan_parts(int* __restrict__ part, int nb) { scan_parts_body(p
 
 // Exclusive scan of a whole short array by one block, tile after tile, cnt[n]
 // the total; cur (if non-null) takes a copy of the n starts.
-__global__ void __launch_bounds__(kScanThreads) k_scan_one(int* __restrict__ cnt, int n, int* __restrict__ cur)
+__device__ __forceinline__ void scan_one_body(int* __restrict__ cnt, int n, int* __restrict__ cur)
 {
     __shared__ int sh[32];
     int carry = 0;
@@ -114,6 +114,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_one(int* __restrict__ cnt
         }
         carry += total;
     }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(int* __restrict__ cnt, int n, int* __restrict__ cur)
+{
+    scan_one_body(cnt, n, cur);
 }
 
 // Phase 3: exclusive scan within each tile plus its offset, in place over
@@ -225,13 +230,6 @@ __global__ void k_zero_b(const ZeroD* __restrict__ d, const int* __restrict__ bs
     for (int i = bid * blockDim.x + threadIdx.x; i < a.n; i += nb * blockDim.x) a.p[i] = 0;
 }
 
-__global__ void k_copy_b(const CopyD* __restrict__ d, const int* __restrict__ bs, int n)
-{
-    int bid, nb;
-    const CopyD& a = d[batch_member(bs, n, bid, nb)];
-    for (int i = bid * blockDim.x + threadIdx.x; i < a.n; i += nb * blockDim.x) a.dst[i] = a.src[i];
-}
-
 __global__ void k_count_b(const CountD* __restrict__ d, const int* __restrict__ bs, int n)
 {
     int bid, nb;
@@ -246,6 +244,12 @@ __global__ void k_scan_reduce_b(const ScanD* __restrict__ d, const int* __restri
     scan_reduce_body(a.cnt, a.n, a.part, bid);
 }
 
+__global__ void __launch_bounds__(kScanThreads) k_scan_one_b(const ScanD* __restrict__ d)
+{
+    const ScanD& a = d[blockIdx.x];
+    scan_one_body(a.cnt, a.n, a.cur);
+}
+
 __global__ void k_scan_parts_b(const ScanD* __restrict__ d, int n)
 {
     const ScanD& a = d[blockIdx.x];
@@ -256,7 +260,7 @@ __global__ void k_scan_apply_b(const ScanD* __restrict__ d, const int* __restric
 {
     int bid, nb;
     const ScanD& a = d[batch_member(bs, n, bid, nb)];
-    scan_apply_body(a.cnt, a.n, a.part, bid);
+    scan_apply_body(a.cnt, a.n, a.part, bid, a.cur);
 }
 
 template <typename R>
@@ -273,12 +277,6 @@ cudaError_t launch_zero_b(const BatchL& L, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_copy_b(const BatchL& L, cudaStream_t s)
-{
-    if (L.total > 0) k_copy_b<<<L.total, L.threads, 0, s>>>((const CopyD*)L.desc, L.bstart, L.n);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_count_b(const BatchL& L, cudaStream_t s)
 {
     if (L.total > 0) k_count_b<<<L.total, L.threads, 0, s>>>((const CountD*)L.desc, L.bstart, L.n);
@@ -288,6 +286,10 @@ cudaError_t launch_count_b(const BatchL& L, cudaStream_t s)
 cudaError_t launch_scan_b(const BatchL& L1, const BatchL& L2, cudaStream_t s)
 {
     if (L1.total <= 0) return cudaSuccess;
+    if (L2.kind) {
+        k_scan_one_b<<<L2.n, kScanThreads, 0, s>>>((const ScanD*)L2.desc);
+        return cudaGetLastError();
+    }
     k_scan_reduce_b<<<L1.total, kScanThreads, 0, s>>>((const ScanD*)L1.desc, L1.bstart, L1.n);
     k_scan_parts_b<<<L2.n, kScanThreads, 0, s>>>((const ScanD*)L2.desc, L2.n);
     k_scan_apply_b<<<L1.total, kScanThreads, 0, s>>>((const ScanD*)L1.desc, L1.bstart, L1.n);
