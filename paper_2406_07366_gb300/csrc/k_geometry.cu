@@ -452,7 +452,11 @@ __device__ __forceinline__ double bin_wrap(double x, double L, double iL, bool& 
     }
 }
 
-template <typename T, bool PLAIN>
+// LN lanes per node (float64 on few nodes): the quadrature points of the two
+// segments and of the subdivided parts are dealt to the lanes and the sums
+// reduced.  Bound by the chain of float64 operations of one node: two 32-node
+// rings with subdivided segments 114 us with a thread a node, 48 with 8 lanes.
+template <typename T, bool PLAIN, int LN>
 __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __restrict__ nodes,
                                              const int* __restrict__ fil_of, const int* __restrict__ prev,
                                              const int64_t* __restrict__ off, const double* __restrict__ shift,
@@ -466,8 +470,14 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
                                              double* __restrict__ psi_local, double* __restrict__ psi_self,
                                              int* __restrict__ status, const T* __restrict__ Dd, int bid)
 {
-    const int j = bid * blockDim.x + threadIdx.x;
-    if (j >= P.N) return;
+    int j = bid * blockDim.x + threadIdx.x;
+    const int ln = LN == 1 ? 0 : (int)(threadIdx.x & (LN - 1));
+    if constexpr (LN > 1) {
+        j /= LN;
+        if (j >= P.N) j = P.N - 1;  // whole groups repeat the last node (the same values)
+    } else {
+        if (j >= P.N) return;
+    }
     const int f = fil_of[j];
     const int jp = prev[j];
     const int jn = (j + 1 < (int)off[f + 1]) ? j + 1 : (int)off[f];
@@ -489,7 +499,7 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
     const T alpha = (T)P.alpha;
 
     // Outgoing segment j: sources for both ranges, self term, l^+.
-    for (int i = 0; i < P.Q; ++i) {
+    for (int i = LN == 1 ? 0 : ln; i < P.Q; i += LN) {
         const T u = (T)P.gh[i] * S.h;
         T del[3], sd[3];
         S.eval(u, del, sd);
@@ -560,7 +570,7 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
         SegPoly<T> R;
         make_poly(R, hseg, dp, Mm, jp, j, drift, Dd);
         const T dsx = ds[3 * jp], dsy = ds[3 * jp + 1], dsz = ds[3 * jp + 2];
-        for (int i = 0; i < P.Q; ++i) {
+        for (int i = LN == 1 ? 0 : ((ln + LN / 2) & (LN - 1)); i < P.Q; i += LN) {
             const T u = (T)P.gh[i] * R.h;
             T del[3], sd[3];
             R.eval(u, del, sd);
@@ -584,7 +594,7 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
         const T dsp[3] = { ds[3 * jp], ds[3 * jp + 1], ds[3 * jp + 2] };
         lp = 0;
         lm = 0;
-        for (int i = 0; i < P.Q; ++i) {
+        for (int i = LN == 1 ? 0 : ln; i < P.Q; i += LN) {
             const T gh = (T)P.gh[i], gw = (T)P.gw[i];
             T del[3], sd[3];
             S.eval(gh * fr * S.h, del, sd);
@@ -592,44 +602,77 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
             R.eval(((T)1 - fr + gh * fr) * R.h, del, sd);
             lm += gw * fr * R.h * sqrt_n(sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2]);
         }
-        for (int side = 0; side < 2; ++side) {
+        // one point at the fraction x of [x0, x1]
+        auto point = [&](int side, T x0, T x1, int i) {
             const SegPoly<T>& Gs = side == 0 ? S : R;
-            T x0 = fr;
-            for (int piece = 0; piece < 64 && x0 < (T)1; ++piece) {
-                const T x1 = (T)2 * x0 < (T)1 ? (T)2 * x0 : (T)1;
-                for (int i = 0; i < P.Q; ++i) {
-                    const T x = x0 + (x1 - x0) * (T)P.gh[i];  // fraction from the node
-                    const T u = side == 0 ? x * Gs.h : ((T)1 - x) * Gs.h;
-                    const T wt = (x1 - x0) * Gs.h * (T)P.gw[i];
-                    T del[3], sd[3];
-                    Gs.eval(u, del, sd);
-                    T r[3];
+            const T x = x0 + (x1 - x0) * (T)P.gh[i];  // fraction from the node
+            const T u = side == 0 ? x * Gs.h : ((T)1 - x) * Gs.h;
+            const T wt = (x1 - x0) * Gs.h * (T)P.gw[i];
+            T del[3], sd[3];
+            Gs.eval(u, del, sd);
+            T r[3];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) r[c] = side == 0 ? del[c] : del[c] - dsp[c];
-                    const T q[3] = { wt * sd[0], wt * sd[1], wt * sd[2] };
-                    if constexpr (sizeof(T) == 8) {
-                        const double ir = rsqrt_h(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]), ir3 = ir * ir * ir;
-                        vd[0] += (r[1] * q[2] - r[2] * q[1]) * ir3;
-                        vd[1] += (r[2] * q[0] - r[0] * q[2]) * ir3;
-                        vd[2] += (r[0] * q[1] - r[1] * q[0]) * ir3;
-                        if (P.want_psi) {
-                            pd[0] += q[0] * ir;
-                            pd[1] += q[1] * ir;
-                            pd[2] += q[2] * ir;
-                        }
-                    } else {
-                        const T rr = tsqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-                        const T ir3 = (T)1 / (rr * rr * rr);
-                        vd[0] += (r[1] * q[2] - r[2] * q[1]) * ir3;
-                        vd[1] += (r[2] * q[0] - r[0] * q[2]) * ir3;
-                        vd[2] += (r[0] * q[1] - r[1] * q[0]) * ir3;
-                        pd[0] += q[0] / rr;
-                        pd[1] += q[1] / rr;
-                        pd[2] += q[2] / rr;
-                    }
+            for (int c = 0; c < 3; ++c) r[c] = side == 0 ? del[c] : del[c] - dsp[c];
+            const T q[3] = { wt * sd[0], wt * sd[1], wt * sd[2] };
+            if constexpr (sizeof(T) == 8) {
+                const double ir = rsqrt_h(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]), ir3 = ir * ir * ir;
+                vd[0] += (r[1] * q[2] - r[2] * q[1]) * ir3;
+                vd[1] += (r[2] * q[0] - r[0] * q[2]) * ir3;
+                vd[2] += (r[0] * q[1] - r[1] * q[0]) * ir3;
+                if (P.want_psi) {
+                    pd[0] += q[0] * ir;
+                    pd[1] += q[1] * ir;
+                    pd[2] += q[2] * ir;
                 }
-                x0 = x1;
+            } else {
+                const T rr = tsqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+                const T ir3 = (T)1 / (rr * rr * rr);
+                vd[0] += (r[1] * q[2] - r[2] * q[1]) * ir3;
+                vd[1] += (r[2] * q[0] - r[0] * q[2]) * ir3;
+                vd[2] += (r[0] * q[1] - r[1] * q[0]) * ir3;
+                pd[0] += q[0] / rr;
+                pd[1] += q[1] / rr;
+                pd[2] += q[2] / rr;
             }
+        };
+        if constexpr (LN > 1) {  // the points of all pieces of a side dealt to the lanes
+            int np = 0;
+            for (T x0 = fr; np < 64 && x0 < (T)1; x0 += x0) ++np;
+            for (int side = 0; side < 2; ++side)
+                for (int t = ln; t < np * P.Q; t += LN) {
+                    const int piece = t / P.Q;
+                    const T x0 = fr * (T)__longlong_as_double((long long)(1023 + piece) << 52);  // fr 2^piece
+                    point(side, x0, (T)2 * x0 < (T)1 ? (T)2 * x0 : (T)1, t - piece * P.Q);
+                }
+        } else {
+            for (int side = 0; side < 2; ++side) {
+                T x0 = fr;
+                for (int piece = 0; piece < 64 && x0 < (T)1; ++piece) {
+                    const T x1 = (T)2 * x0 < (T)1 ? (T)2 * x0 : (T)1;
+                    for (int i = 0; i < P.Q; ++i) point(side, x0, x1, i);
+                    x0 = x1;
+                }
+            }
+        }
+    }
+
+    if constexpr (LN > 1) {
+#pragma unroll
+        for (int o = LN / 2; o > 0; o >>= 1) {
+            lp += __shfl_xor_sync(0xffffffffu, lp, o);
+            lm += __shfl_xor_sync(0xffffffffu, lm, o);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                vs[c] += __shfl_xor_sync(0xffffffffu, vs[c], o);
+                ps[c] += __shfl_xor_sync(0xffffffffu, ps[c], o);
+                vd[c] += __shfl_xor_sync(0xffffffffu, vd[c], o);
+                pd[c] += __shfl_xor_sync(0xffffffffu, pd[c], o);
+            }
+        }
+        if (ln != 0) {  // the node's own results: lane 0
+            if (bad || bad_node) flags |= ST_NONFINITE;
+            if (flags) atomicOr(status, flags);
+            return;
         }
     }
 
@@ -697,7 +740,7 @@ __device__ __forceinline__ void k_nodes_body(const GeomP& P, const double* __res
     if (flags) atomicOr(status, flags);
 }
 
-template <typename T>
+template <typename T, int LN>
 __global__ void k_nodes(GeomP P, const double* __restrict__ nodes, const int* __restrict__ fil_of,
                         const int* __restrict__ prev, const int64_t* __restrict__ off, const double* __restrict__ shift,
                         const T* __restrict__ hseg, const T* __restrict__ dp, const T* __restrict__ ds,
@@ -710,7 +753,7 @@ __global__ void k_nodes(GeomP P, const double* __restrict__ nodes, const int* __
 {
     // the bin counters of the kernels that follow (they are idle here)
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nclr; i += gridDim.x * blockDim.x) clr[i] = 0;
-    k_nodes_body<T, false>(P, nodes, fil_of, prev, off, shift, hseg, dp, ds, Mm, Tper, sr_rec, sr_key, lr_rec, lr_key, tgt,
+    k_nodes_body<T, false, LN>(P, nodes, fil_of, prev, off, shift, hseg, dp, ds, Mm, Tper, sr_rec, sr_key, lr_rec, lr_key, tgt,
         vls, pls, part_local, part_self, psi_local, psi_self, status, Dd, blockIdx.x);
 }
 
@@ -728,7 +771,7 @@ __global__ void __launch_bounds__(128) k_nodes_b(const NodesD<T>* __restrict__ d
 {
     int bid, nb;
     const NodesD<T>& a = d[batch_member(bs, n, bid, nb)];
-    k_nodes_body<T, sizeof(T) == 4>(a.P, a.nodes, a.fil_of, a.prev, a.off, a.shift, a.hseg, a.dp, a.ds, a.Mm, a.Tper, a.sr_rec,
+    k_nodes_body<T, sizeof(T) == 4, 1>(a.P, a.nodes, a.fil_of, a.prev, a.off, a.shift, a.hseg, a.dp, a.ds, a.Mm, a.Tper, a.sr_rec,
                     a.sr_key, a.lr_rec, a.lr_key, a.tgt, a.vls, a.pls, nullptr, nullptr, nullptr, nullptr, a.status,
                     a.Dd, bid);
 }
@@ -1199,11 +1242,12 @@ __global__ void k_export_quad(GeomP P, const double* __restrict__ nodes, const i
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void q_blocks(double a, double h, double L[4], double B[4], double U[4])
 {
-    const double a2 = a * a, a3 = a2 * a, h2 = h * h, h3 = h2 * h;
-    L[0] = -24.0 / a2; L[1] = -3.0 / a; L[2] = -168.0 / a3; L[3] = -24.0 / a2;
-    B[0] = 36.0 / h2 - 36.0 / a2; B[1] = 9.0 / a + 9.0 / h;
-    B[2] = -192.0 / a3 - 192.0 / h3; B[3] = 36.0 / a2 - 36.0 / h2;
-    U[0] = 24.0 / h2; U[1] = -3.0 / h; U[2] = -168.0 / h3; U[3] = 24.0 / h2;
+    // two reciprocals in place of 14 divisions
+    const double a1 = 1.0 / a, h1 = 1.0 / h, a2 = a1 * a1, a3 = a2 * a1, h2 = h1 * h1, h3 = h2 * h1;
+    L[0] = -24.0 * a2; L[1] = -3.0 * a1; L[2] = -168.0 * a3; L[3] = -24.0 * a2;
+    B[0] = 36.0 * h2 - 36.0 * a2; B[1] = 9.0 * a1 + 9.0 * h1;
+    B[2] = -192.0 * a3 - 192.0 * h3; B[3] = 36.0 * a2 - 36.0 * h2;
+    U[0] = 24.0 * h2; U[1] = -3.0 * h1; U[2] = -168.0 * h3; U[3] = 24.0 * h2;
 }
 
 // inverse of the 2 x 2 matrix m (row major)
@@ -1409,7 +1453,7 @@ __device__ const double* q_solve_cta(int n, const double* __restrict__ sm)
         const double a = h[jm], hj = h[j];
         q_blocks(a, hj, L, B, U);
         inv2(B, iv);
-        const double ia3 = 1.0 / (a * a * a), ih3 = 1.0 / (hj * hj * hj), ia = 1.0 / a, ih = 1.0 / hj;
+        const double ia = 1.0 / a, ih = 1.0 / hj, ia3 = ia * ia * ia, ih3 = ih * ih * ih;
 #pragma unroll
         for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -1663,11 +1707,23 @@ cudaError_t launch_nodes(const GeomP& P, const double* nodes, const Work& w, dou
 {
     if (P.N <= 0) return nclr > 0 ? cudaMemsetAsync(clr, 0, sizeof(int) * (size_t)nclr, s) : cudaSuccess;
     const int tb = item_threads(P.N, 128);
-    k_nodes<T><<<(P.N + tb - 1) / tb, tb, 0, s>>>(
+    auto launch = [&](auto kernel, long long threads, int block) {
+        kernel<<<(unsigned)((threads + block - 1) / block), block, 0, s>>>(
         P, nodes, w.fil_of, w.prev, w.off, w.shift, (const T*)w.hseg, (const T*)w.dp, (const T*)w.ds,
         (const T*)w.Mm, (const T*)w.Tper, (SrRec<T>*)w.sr_rec, w.sr_key, (LrRec<T>*)w.lr_rec, w.lr_key,
         (SrTgt<T>*)w.tgt, w.vls, w.pls, part_local, part_self, psi_local, psi_self, w.status, (const T*)w.Dd, clr,
         nclr);
+    };
+    if constexpr (sizeof(T) == 8) {
+        // Up to 32 nodes per SM 8 lanes take a node: a whole evaluation (local_frac
+        // 0.1) 318 -> 234 us on 640 nodes, 740 -> 682 on 2560, 1542 -> 1515 on 4864,
+        // where the float64 pipes begin to fill and the gain ends.
+        if (P.N <= 152 * 32) {
+            launch(k_nodes<T, 8>, 8LL * P.N, 32);
+            return cudaGetLastError();
+        }
+    }
+    launch(k_nodes<T, 1>, P.N, tb);
     return cudaGetLastError();
 }
 

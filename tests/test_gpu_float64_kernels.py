@@ -116,3 +116,29 @@ def test_float64_kernel_polynomials_equal_the_kernel(w, sigma):
         torch.cuda.synchronize()
         bs.close()
     assert float((parts[0] - parts[1]).abs().max()) < 1e-12 * float(parts[1].abs().max())
+
+
+@pytest.mark.parametrize("local_frac", [0.0, 0.1])
+@pytest.mark.parametrize("order,total", [(4, 4864), (4, 4865), (6, 4865)])
+def test_float64_node_terms_by_lanes_equal_a_thread_per_node(order, total, local_frac):
+    """Up to 4864 nodes 8 lanes share a node's quadrature points, beyond it a
+    thread takes the node.  The local and self terms depend on the node's own
+    filament alone, so a 65-node curve has the same ones by itself and beside
+    others: sums of at most 2 (2 + 4) Q terms in another order, 1e-12 of the
+    largest (the float64 parity tolerance)."""
+    B, a = _B(), _uneven_ring(65, 7)
+    rest = total - 65 - 64 * 73
+    X = [a.nodes] + [_uneven_ring(64, k).nodes for k in range(73)] + [_uneven_ring(rest, 99).nodes]
+    f = W._pack(X, a.L)
+    assert len(f.nodes) == total
+    out = []
+    for s in (a, f):
+        p = B.make_params(s.L, M=32, Q=3, order=order, w=8, precision=B.BS_FP64, alpha=4.0, rc=1.5,
+                          flags=B.BS_WANT_PSI, local_frac=local_frac)
+        bs = B.BiotSavart(p, s.offsets, s.closing)
+        v, psi = bs.parts(torch.from_numpy(s.nodes).cuda(), want_psi=True)
+        torch.cuda.synchronize()
+        bs.close()
+        out.append([x[k, :65].cpu().numpy() for x in (v, psi) for k in (0, 3)])
+    for x, y in zip(*out):
+        assert np.abs(x - y).max() < 1e-12 * np.abs(x).max()
