@@ -653,10 +653,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (PAIR ? 4 : 5) : 3) k_sh
 {
     __shared__ ShortRows<T> rows;
     const double* tab = sg_stage<T>(P.want_psi);
-    const int wid = threadIdx.x >> 5;
+    const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if constexpr (sizeof(T) == 8) {  // several groups of nodes per CTA: the tables are staged once
-        for (int b = blockIdx.x; b * kShortWarps < P.N; b += gridDim.x)
-            k_short_warp<T, PAIR>(P, tgt, prev, start, src, vsr, psr, b * kShortWarps + wid, tab, rows);
+        for (int b = blockIdx.x; b * nw < P.N; b += gridDim.x)
+            k_short_warp<T, PAIR>(P, tgt, prev, start, src, vsr, psr, b * nw + wid, tab, rows);
     } else {
         k_short_warp<T, PAIR>(P, tgt, prev, start, src, vsr, psr, blockIdx.x * kShortWarps + wid, tab, rows);
     }
@@ -1037,9 +1037,15 @@ cudaError_t launch_short(const ShortP& P, const Work& w, cudaStream_t s)
     // ms on the 1e5-node one), the tiled kernel only on request
     const bool tiled = P.m <= kShortTileMaxM && P.kernel == 1;
     if (!tiled) {
-        const int tb = 32 * kShortWarps;  // one warp per target
+        // one warp per target; in float64 few nodes are spread over the SMs (the
+        // warps of a CTA share one slow float64 pipe: 64 nodes
+        // 38.5 -> 27 us)
+        int nw = kShortWarps;
+        if (sizeof(T) == 8)
+            while (nw > 1 && P.N < 152 * nw) nw /= 2;
+        const int tb = 32 * nw;
         const bool pairs = short_can_pair(P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED);
-        const long long blocks = short_blocks(P, pairs);
+        const long long blocks = sizeof(T) == 8 ? (P.N + nw - 1LL) / nw : short_blocks(P, pairs);
         // float64: at most 16 CTAs per SM, each on several groups of nodes
         const unsigned g = (unsigned)(sizeof(T) == 8 && blocks > 16 * 152 ? 16 * 152 : blocks);
         if constexpr (sizeof(T) == 4) {
