@@ -984,16 +984,35 @@ __device__ __forceinline__ void k_col_scatter_body(const ColP& P, const LrRec<T>
         kb_weights<T, W>(R.f, P.zeta, P.inorm, P.kbc, D.wx, D.wy, D.wz);
         pts[i] = D;
     }
-    for (int k = 0; k < nk; ++k) {
-        const bool live = k < nx * ny;
-        const int kyi = live ? k / nx : 0;
-        const int bx = x0 + (k - kyi * nx), by = y0 + kyi;
-        const int b = live ? col_bin(P, col_wrap(bx, P.nbx) + P.nbx * col_wrap(by, P.nby), (R.base >> 20) & 1023) : -1;
-        const int p = warp_rank(b, cur);
-        if (!live) continue;
-        const int r1 = ib1 - H + 1 - by * P.ty;  // support start relative to the block (unwrapped block)
-        const int r0 = ib0 - H + 1 - bx * P.tx;
-        out[p] = make_int2(i, (r0 + 128) | ((r1 + 128) << 8) | zbits);
+    // four copies at a time: their atomics are in flight together (one by one,
+    // each copy waited for the atomic of the one before: 25 -> 19 us in float64
+    // on 192 points, where this is all latency)
+    constexpr int KU = 4;
+    const int lane = threadIdx.x & 31;
+    for (int k0 = 0; k0 < nk; k0 += KU) {
+        int word[KU], rank[KU];
+        unsigned peers[KU];
+#pragma unroll
+        for (int u = 0; u < KU; ++u) {
+            const int k = k0 + u;
+            const bool live = k < nx * ny;
+            const int kyi = live ? k / nx : 0;
+            const int bx = x0 + (k - kyi * nx), by = y0 + kyi;
+            const int b =
+                live ? col_bin(P, col_wrap(bx, P.nbx) + P.nbx * col_wrap(by, P.nby), (R.base >> 20) & 1023) : -1;
+            peers[u] = __match_any_sync(0xffffffffu, b);
+            rank[u] = 0;
+            if (live && lane == __ffs(peers[u]) - 1) rank[u] = atomicAdd(&cur[b], __popc(peers[u]));
+            // support start relative to the block (unwrapped block)
+            const int r1 = ib1 - H + 1 - by * P.ty, r0 = ib0 - H + 1 - bx * P.tx;
+            word[u] = live ? ((r0 + 128) | ((r1 + 128) << 8) | zbits) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < KU; ++u) {
+            const int p = __shfl_sync(0xffffffffu, rank[u], __ffs(peers[u]) - 1) +
+                          __popc(peers[u] & ((1u << lane) - 1u));
+            if (k0 + u < nx * ny) out[p] = make_int2(i, word[u]);
+        }
     }
 }
 
