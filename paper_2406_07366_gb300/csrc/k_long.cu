@@ -214,26 +214,36 @@ __global__ void k_kspace(KspaceP P, typename Cplx<T>::t* __restrict__ spec, type
 
 // Type-2 interpolation at the nodes, plus the epilogue sum
 //   out = add_d (float64: local - self) + add_t (short range, float64) + interp.
-// part (optional) receives the interpolated long-range part alone.  The
-// weights of the last two axes live in registers (static indices); those of
-// the first axis are computed in the outer loop.  NC = 3: a thread per node;
-// NC = 1: a thread per node and component, three times the threads while the
-// nodes alone leave most of the GPU idle (2560 nodes, 32-thread blocks: 82 us
-// with one thread a node in 128-thread blocks).  Either way a component is
-// summed over the W^3 points in the same order, which is its float32 rounding.
-template <typename T, int W, int NC>
-__global__ void __launch_bounds__(128) k_interp(InterpP P, const double* __restrict__ nodes, const T* __restrict__ grid,
-                                                const double* __restrict__ add_d, const double* __restrict__ add_t,
-                                                double* __restrict__ out, double* __restrict__ part)
+// part (optional) receives the interpolated long-range part alone.
+//
+// A warp takes a node: it copies the node's points of the three grids to shared
+// memory, whole runs along z at a time and all loads in flight together, and
+// three lanes sum a component each.  Bound by the latency of the gather on few
+// nodes and by the three lanes' sums on many.  (A thread per node and component
+// gathered straight from the grid: 32 sectors per load and 512 loads in a
+// chain; 2560 nodes, W = 8: 62 us, now 24.)  A component is summed over the W^3 points in
+// order, which fixes its float32 rounding.  PC planes across the first axis are
+// staged at a time, 512 points of a component at most.
+constexpr int kInterpWarps = 4;
+template <typename T, int W>
+__global__ void __launch_bounds__(32 * kInterpWarps) k_interp(InterpP P, const double* __restrict__ nodes,
+                                                              const T* __restrict__ grid,
+                                                              const double* __restrict__ add_d,
+                                                              const double* __restrict__ add_t,
+                                                              double* __restrict__ out, double* __restrict__ part)
 {
-    const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = NC == 3 ? i0 : i0 / 3, c0 = NC == 3 ? 0 : i0 - 3 * j;  // node, first component
-    if (j >= P.N) return;
-    constexpr int H = W / 2;
+    constexpr int H = W / 2, WW = W * W, PC = 512 / WW < W ? 512 / WW : W;
+    constexpr int LD = PC * WW + 4;  // the components' lanes read different banks
+    __shared__ __align__(16) T val_s[kInterpWarps][3][LD];
+    __shared__ T wt_s[kInterpWarps][3][W];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int j = blockIdx.x * (blockDim.x >> 5) + wid;
+    if (j >= P.N) return;  // a whole warp
+    T (*val)[LD] = val_s[wid];
+    T (*wt)[W] = wt_s[wid];
     const T zeta = (T)P.zeta;
     const T inorm = (T)P.inorm;
     int ib[3];
-    T fr[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         double x = nodes[3 * j + d];
@@ -247,46 +257,57 @@ __global__ void __launch_bounds__(128) k_interp(InterpP P, const double* __restr
         double f = g - (double)k;
         f = f < 0.0 ? 0.0 : (f > 1.0 ? 1.0 : f);
         ib[d] = k;
-        fr[d] = (T)f;
+        const T fr = (T)f;
+        if (lane < W) wt[d][lane] = kb_eval((fr + (T)(H - 1 - lane)) * ((T)2 / (T)W), zeta, inorm);
     }
+    __syncwarp();
     T ky[W], kz[W];
-    int iy[W], iz[W];
 #pragma unroll
     for (int t = 0; t < W; ++t) {
-        ky[t] = kb_eval((fr[1] + (T)(H - 1 - t)) * ((T)2 / (T)W), zeta, inorm);
-        kz[t] = kb_eval((fr[2] + (T)(H - 1 - t)) * ((T)2 / (T)W), zeta, inorm);
-        int gy = ib[1] - H + 1 + t, gz = ib[2] - H + 1 + t;
-        iy[t] = gy < 0 ? gy + P.ng[1] : (gy >= P.ng[1] ? gy - P.ng[1] : gy);
-        iz[t] = gz < 0 ? gz + P.ng[2] : (gz >= P.ng[2] ? gz - P.ng[2] : gz);
+        ky[t] = wt[1][t];
+        kz[t] = wt[2][t];
     }
     const size_t gsz = (size_t)P.ng[0] * P.ng[1] * P.ng[2];
-    grid += c0 * gsz;
-    T a[NC] = {};
+    T a = 0;
 #pragma unroll 1
-    for (int p = 0; p < W; ++p) {
-        const T kx = kb_eval((fr[0] + (T)(H - 1 - p)) * ((T)2 / (T)W), zeta, inorm);
-        int gx = ib[0] - H + 1 + p;
-        gx = gx < 0 ? gx + P.ng[0] : (gx >= P.ng[0] ? gx - P.ng[0] : gx);
-        const size_t plane = (size_t)gx * P.ng[1];
+    for (int p0 = 0; p0 < W; p0 += PC) {
+#pragma unroll 8
+        for (int e = lane; e < PC * WW; e += 32) {
+            const int p = e / WW, q = (e / W) % W, r = e % W;
+            if (p0 + p >= W) break;
+            int gx = ib[0] - H + 1 + p0 + p, gy = ib[1] - H + 1 + q, gz = ib[2] - H + 1 + r;
+            gx = gx < 0 ? gx + P.ng[0] : (gx >= P.ng[0] ? gx - P.ng[0] : gx);
+            gy = gy < 0 ? gy + P.ng[1] : (gy >= P.ng[1] ? gy - P.ng[1] : gy);
+            gz = gz < 0 ? gz + P.ng[2] : (gz >= P.ng[2] ? gz - P.ng[2] : gz);
+            const size_t gi = ((size_t)gx * P.ng[1] + gy) * P.ng[2] + gz;
 #pragma unroll
-        for (int q = 0; q < W; ++q) {
-            const T wpq = kx * ky[q];
-            const size_t row = (plane + iy[q]) * P.ng[2];
+            for (int c = 0; c < 3; ++c) val[c][e] = grid[c * gsz + gi];
+        }
+        __syncwarp();
+        if (lane < 3) {
+            const T* v = val[lane];
+#pragma unroll 1
+            for (int p = 0; p < PC && p0 + p < W; ++p) {
+                const T kx = wt[0][p0 + p];
 #pragma unroll
-            for (int r = 0; r < W; ++r) {
-                const size_t gi = row + iz[r];
-                const T wv = wpq * kz[r];
+                for (int q = 0; q < W; ++q) {
+                    const T wpq = kx * ky[q];
 #pragma unroll
-                for (int c = 0; c < NC; ++c) a[c] += wv * grid[c * gsz + gi];
+                    for (int r = 0; r < W; ++r) {
+                        const T wv = wpq * kz[r];
+                        a += wv * v[q * W + r];
+                    }
+                }
+                v += WW;
             }
         }
+        __syncwarp();
     }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        const size_t i = 3 * (size_t)j + c0 + c;
-        if (part) part[i] = (double)a[c];
+    if (lane < 3) {
+        const size_t i = 3 * (size_t)j + lane;
+        if (part) part[i] = (double)a;
         if (out) {
-            double o = (double)a[c];
+            double o = (double)a;
             if (add_t) o += add_t[i];
             if (add_d) o += add_d[i];
             out[i] = o;
@@ -434,12 +455,10 @@ static cudaError_t interp_w(const InterpP& P, const double* nodes, const void* g
         constexpr int tb = 128;
         const long long g = ((long long)P.N * interp_group(W) + tb - 1) / tb;
         k_interp_g<T, W><<<(unsigned)g, tb, 0, s>>>(P, nodes, (const T*)grid, add_d, add_t, out, part);
-    } else if (P.N <= 152 * 256) {
-        const int tb = item_threads(3LL * P.N, 128);
-        k_interp<T, W, 1><<<(3 * P.N + tb - 1) / tb, tb, 0, s>>>(P, nodes, (const T*)grid, add_d, add_t, out, part);
     } else {
-        const int tb = 128;
-        k_interp<T, W, 3><<<(P.N + tb - 1) / tb, tb, 0, s>>>(P, nodes, (const T*)grid, add_d, add_t, out, part);
+        // few nodes: a warp per block, all of them resident at once (9 blocks an SM)
+        const int nw = P.N <= 152 * 8 ? 1 : kInterpWarps;
+        k_interp<T, W><<<(P.N + nw - 1) / nw, 32 * nw, 0, s>>>(P, nodes, (const T*)grid, add_d, add_t, out, part);
     }
     return cudaGetLastError();
 }
