@@ -176,13 +176,17 @@ __global__ void k_spline(const double* __restrict__ nodes, const int64_t* __rest
     }
 }
 
-// The same fit with one warp per filament, staged in shared memory: the
-// lanes compute chords, increments and right-hand sides in parallel; lanes
-// 0..3 then run the four sequential Thomas sweeps (x, y, z and the
-// Sherman-Morrison vector) out of shared memory; all lanes apply the
-// correction and write the moments.  smem: 9 * nmax values of T.
+// The same fit with a CTA per filament, staged in shared memory: the threads
+// compute chords, increments and right-hand sides in parallel; lanes 0..3 of
+// the first warp then run the four sequential Thomas sweeps (x, y, z and the
+// Sherman-Morrison vector) out of shared memory; all threads apply the
+// correction and write the moments.  smem: 9 * nmax values of T.  Bound by
+// latency: the loads, the float64 chords and the sweeps follow one another.
+// With a warp per filament and a second pass over the chords for every curve
+// (a closed curve's increments are its chords: it skips that) 23.3 us on 200
+// filaments of 100 nodes and 14.3 on one of 64, now 14.2 and 11.5.
 template <typename T>
-__device__ __forceinline__ void k_spline_warp_body(const double* __restrict__ nodes, const int64_t* __restrict__ off,
+__device__ __forceinline__ void k_spline_thomas_body(const double* __restrict__ nodes, const int64_t* __restrict__ off,
                                                    const double* __restrict__ shift, int nfil, int nmax,
                                                    T* __restrict__ hseg, T* __restrict__ dp, T* __restrict__ ds,
                                                    T* __restrict__ Mm, T* __restrict__ Tper, int bid)
@@ -194,13 +198,14 @@ __device__ __forceinline__ void k_spline_warp_body(const double* __restrict__ no
     T* sh_cp = sh_r + 4 * nmax;               // n: modified super-diagonal
     const int f = bid;
     if (f >= nfil) return;
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x, nt = blockDim.x;
     const int64_t o = off[f];
     const int n = (int)(off[f + 1] - o);
     const double s0 = shift[3 * f], s1 = shift[3 * f + 1], s2 = shift[3 * f + 2];
 
+    const bool closed = s0 == 0.0 && s1 == 0.0 && s2 == 0.0;
     double tpart = 0.0;
-    for (int j = lane; j < n; j += 32) {
+    for (int j = lane; j < n; j += nt) {
         const double* a = nodes + 3 * (o + j);
         const double* b = nodes + 3 * (j + 1 < n ? o + j + 1 : o);
         const double w0 = (j + 1 < n) ? 0.0 : s0, w1 = (j + 1 < n) ? 0.0 : s1, w2 = (j + 1 < n) ? 0.0 : s2;
@@ -212,13 +217,25 @@ __device__ __forceinline__ void k_spline_warp_body(const double* __restrict__ no
         ds[3 * (o + j) + 0] = (T)d0;
         ds[3 * (o + j) + 1] = (T)d1;
         ds[3 * (o + j) + 2] = (T)d2;
+        if (closed) {
+            sh_dp[j] = (T)d0;
+            sh_dp[nmax + j] = (T)d1;
+            sh_dp[2 * nmax + j] = (T)d2;
+            dp[3 * (o + j) + 0] = (T)d0;
+            dp[3 * (o + j) + 1] = (T)d1;
+            dp[3 * (o + j) + 2] = (T)d2;
+        }
     }
+    __shared__ double sh_t[8];
 #pragma unroll
     for (int k = 16; k > 0; k >>= 1) tpart += __shfl_xor_sync(0xffffffffu, tpart, k);
-    const double Tsum = tpart;
+    if ((lane & 31) == 0) sh_t[lane >> 5] = tpart;
+    __syncthreads();
+    double Tsum = sh_t[0];
+    for (int k = 1; k < nt >> 5; ++k) Tsum += sh_t[k];
     if (lane == 0) Tper[f] = (T)Tsum;
     const double invT = 1.0 / Tsum;
-    for (int j = lane; j < n; j += 32) {
+    for (int j = closed ? n : lane; j < n; j += nt) {
         const double* a = nodes + 3 * (o + j);
         const double* b = nodes + 3 * (j + 1 < n ? o + j + 1 : o);
         const double w0 = (j + 1 < n) ? 0.0 : s0, w1 = (j + 1 < n) ? 0.0 : s1, w2 = (j + 1 < n) ? 0.0 : s2;
@@ -234,11 +251,11 @@ __device__ __forceinline__ void k_spline_warp_body(const double* __restrict__ no
         dp[3 * (o + j) + 1] = p1;
         dp[3 * (o + j) + 2] = p2;
     }
-    __syncwarp();
+    __syncthreads();
     // right-hand sides 6 (dp_j / h_j - dp_{j-1} / h_{j-1}) and the vector u
     const T hl = sh_h[n - 1];
     const T gamma = -(T)2 * (hl + sh_h[0]);
-    for (int j = lane; j < n; j += 32) {
+    for (int j = lane; j < n; j += nt) {
         const int jm = j == 0 ? n - 1 : j - 1;
         const T hj = sh_h[j], hm = sh_h[jm];
 #pragma unroll
@@ -246,7 +263,7 @@ __device__ __forceinline__ void k_spline_warp_body(const double* __restrict__ no
             sh_r[c * nmax + j] = (T)6 * (sh_dp[c * nmax + j] / hj - sh_dp[c * nmax + jm] / hm);
         sh_r[3 * nmax + j] = (j == 0) ? gamma : ((j == n - 1) ? hl : (T)0);
     }
-    __syncwarp();
+    __syncthreads();
     if (lane < 4) {
         T* r = sh_r + lane * nmax;
         const T a0 = hl, cn = hl;
@@ -284,25 +301,33 @@ __device__ __forceinline__ void k_spline_warp_body(const double* __restrict__ no
             r[j] = x;
         }
     }
-    __syncwarp();
+    __syncthreads();
     const T vfac = hl / gamma;
     const T* z = sh_r + 3 * nmax;
     const T den = (T)1 + z[0] + vfac * z[n - 1];
     T fc[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) fc[c] = (sh_r[c * nmax] + vfac * sh_r[c * nmax + n - 1]) / den;
-    for (int j = lane; j < n; j += 32) {
+    for (int j = lane; j < n; j += nt) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) Mm[3 * (o + j) + c] = sh_r[c * nmax + j] - fc[c] * z[j];
     }
 }
 
+// Threads of a filament's CTA: a thread a node while the CTAs leave room on the
+// SMs, a warp beyond (more resident filaments hide their sweeps).
+static int spline_threads(long long ctas, int nmax)
+{
+    if (ctas > 152 * 16) return 32;
+    return nmax >= 256 ? 256 : (nmax < 1 ? 32 : (nmax + 31) / 32 * 32);
+}
+
 template <typename T>
-__global__ void k_spline_warp(const double* __restrict__ nodes, const int64_t* __restrict__ off,
+__global__ void __launch_bounds__(256, 4) k_spline_thomas(const double* __restrict__ nodes, const int64_t* __restrict__ off,
                               const double* __restrict__ shift, int nfil, int nmax, T* __restrict__ hseg,
                               T* __restrict__ dp, T* __restrict__ ds, T* __restrict__ Mm, T* __restrict__ Tper)
 {
-    k_spline_warp_body<T>(nodes, off, shift, nfil, nmax, hseg, dp, ds, Mm, Tper, blockIdx.x);
+    k_spline_thomas_body<T>(nodes, off, shift, nfil, nmax, hseg, dp, ds, Mm, Tper, blockIdx.x);
 }
 
 template <typename T>
@@ -759,11 +784,11 @@ __global__ void k_nodes(GeomP P, const double* __restrict__ nodes, const int* __
 
 // Batched forms: every member of a batch in one launch.
 template <typename T>
-__global__ void k_spline_warp_b(const SplineD<T>* __restrict__ d, const int* __restrict__ bs, int n)
+__global__ void __launch_bounds__(256, 4) k_spline_thomas_b(const SplineD<T>* __restrict__ d, const int* __restrict__ bs, int n)
 {
     int bid, nb;
     const SplineD<T>& a = d[batch_member(bs, n, bid, nb)];
-    k_spline_warp_body<T>(a.nodes, a.off, a.shift, a.nfil, a.nmax, a.hseg, a.dp, a.ds, a.Mm, a.Tper, bid);
+    k_spline_thomas_body<T>(a.nodes, a.off, a.shift, a.nfil, a.nmax, a.hseg, a.dp, a.ds, a.Mm, a.Tper, bid);
 }
 
 template <typename T>
@@ -787,11 +812,11 @@ cudaError_t launch_spline_b(const BatchL& L, cudaStream_t s)
 {
     if (L.total <= 0) return cudaSuccess;
     if (L.smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_spline_warp_b<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_spline_thomas_b<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)L.smem);
         if (e != cudaSuccess) return e;
     }
-    k_spline_warp_b<T><<<L.total, 32, L.smem, s>>>((const SplineD<T>*)L.desc, L.bstart, L.n);
+    k_spline_thomas_b<T><<<L.total, spline_threads(L.total, (int)(L.smem / (9 * sizeof(T)))), L.smem, s>>>((const SplineD<T>*)L.desc, L.bstart, L.n);
     return cudaGetLastError();
 }
 
@@ -1687,10 +1712,10 @@ cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStre
     const size_t sm = 9 * (size_t)w.nmax_fil * sizeof(T);
     if (sm <= kSplineSmemMax) {
         if (sm > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(k_spline_warp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            cudaError_t e = cudaFuncSetAttribute(k_spline_thomas<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
             if (e != cudaSuccess) return e;
         }
-        k_spline_warp<T><<<nfil, 32, sm, s>>>(nodes, w.off, w.shift, nfil, w.nmax_fil, (T*)w.hseg, (T*)w.dp,
+        k_spline_thomas<T><<<nfil, spline_threads(nfil, w.nmax_fil), sm, s>>>(nodes, w.off, w.shift, nfil, w.nmax_fil, (T*)w.hseg, (T*)w.dp,
                                                (T*)w.ds, (T*)w.Mm, (T*)w.Tper);
         return cudaGetLastError();
     }

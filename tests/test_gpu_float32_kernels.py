@@ -4,6 +4,7 @@ import math
 import numpy as np
 import pytest
 
+import oracle
 from paper_2406_07366_gb300 import workloads as W
 
 torch = pytest.importorskip("torch")
@@ -94,3 +95,34 @@ def test_gather_interpolation_by_a_warp_per_node(w, n):
         out.append(bs.parts(torch.from_numpy(f.nodes).cuda(), want_psi=True)[1][2].cpu().numpy())
         bs.close()
     assert np.abs(out[1] - out[0]).max() < 3e-5 * np.abs(out[0]).max()
+
+
+@pytest.mark.parametrize("closing", [0, 1])
+@pytest.mark.parametrize("n,copies", [(4, 1), (31, 1), (33, 1), (256, 1), (257, 1), (600, 1), (40, 2433)])
+def test_cubic_fit_by_a_block_per_filament(n, copies, closing):
+    """A thread a node up to 2432 filaments, a warp beyond; closed curves and
+    infinite ones.  Points and charges against the float64 fit of the oracle
+    (its first filament): float32 chords and moments of a system with chord
+    ratios below 3 are good to 20 roundings, 2.4e-6 of the longest chord for
+    the points and of the largest charge."""
+    B = _B()
+    rng = np.random.default_rng(n)
+    L = np.full(3, 2 * math.pi)
+    th = np.cumsum(rng.uniform(0.5, 1.5, n))
+    th *= 2 * math.pi / th[-1]
+    X = np.stack([np.cos(th), np.sin(th), (th - th[0]) if closing else 0.3 * np.sin(2 * th)], 1) + L / 2
+    # the closing offsets of a box sum to zero: each infinite curve with its reverse
+    pair, close = ([X, X[::-1]], [[0, 0, 1], [0, 0, -1]]) if closing else ([X], [[0, 0, 0]])
+    f = W._pack(pair * copies, L, closing=close * copies)
+    p = B.make_params(f.L, M=32, Q=3, w=8, precision=B.BS_MIXED)
+    bs = B.BiotSavart(p, f.offsets, f.closing)
+    qX, qq = bs.quadrature(torch.from_numpy(f.nodes).cuda())
+    torch.cuda.synchronize()
+    bs.close()
+    g = oracle.geometry(X, f.offsets[:2], f.closing[:1], f.L, 4, 3)
+    shift = np.array([0, 0, closing * L[2]])
+    chord = np.linalg.norm(np.diff(np.vstack([X, X[:1] + shift]), axis=0), axis=1).max()
+    d = qX[:3 * n].cpu().numpy() - g.qX
+    d -= f.L * np.round(d / f.L)
+    assert np.abs(d).max() < 2.4e-6 * chord
+    assert np.abs(qq[:3 * n].cpu().numpy() - g.qq).max() < 2.4e-6 * np.abs(g.qq).max()
