@@ -41,9 +41,10 @@ import numpy as np  # noqa: E402
 METRIC = "filament nodes/s per Biot–Savart eval at 1e-6 rel. err; FP32/batched vs FP64"
 UNIT = "nodes/s"
 L2_FLUSH_BYTES = 512 << 20
-# spline, nodes, 3 x (count, 3 scan, scatter: short-range cells, spread blocks, node blocks), short range,
-# spread + z FFT, y FFT, x FFT + k-space, inverse y, inverse z + interpolation, final sum
-KERNELS_PER_STEP = 24
+# spline, nodes, clear, 3 x (count, 2 scan, scatter: short-range cells, spread blocks, node blocks), short range,
+# spread + z FFT, y FFT, x FFT + k-space, inverse y, inverse z + interpolation, final sum (grids of the
+# benchmark's sizes; small ones scan in one launch)
+KERNELS_PER_STEP = 22
 
 
 def parse():

@@ -54,7 +54,7 @@ enum {
 
 /* ---- precision forms ------------------------------------------------- */
 enum {
-    BS_FP64 = 0,   /* every stage in float64 (cuFFT D2Z/Z2D)                */
+    BS_FP64 = 0,   /* every stage in float64                                */
     BS_MIXED = 1   /* float32 spread/FFT/k-space/interp/short range; float64
                       node positions, cell-relative offsets and the final sum */
 };
@@ -317,7 +317,7 @@ int bs_rk4_launch(bs_ctx* ctx, int nsteps);
  * kernel width and z-column CTA size of the first of them.  Each stage of
  * the group's evaluation is ONE launch for all its members: member m runs
  * its own blocks of the launch with its own parameters, taken from a device
- * table (about 30 launches whatever the member count).  Every other member's
+ * table (22 launches whatever the member count).  Every other member's
  * evaluation is issued by itself on an internal pool of up to 8 streams,
  * concurrently with the group.  Passing both batch flags on one member is
  * BS_ERR_ARG.  With a non-default

@@ -13,7 +13,7 @@ namespace bsw {
 constexpr int kMaxQ = 8;
 constexpr int kMaxW = 16;
 constexpr int kThreads = 256;
-constexpr size_t kSplineSmemMax = 96 * 1024;  // warp-per-filament spline fit up to this smem
+constexpr size_t kSplineSmemMax = 96 * 1024;  // Thomas spline fit up to this smem
 constexpr double kPi = 3.14159265358979323846264338327950288;
 
 // Device status bits (bs_status).

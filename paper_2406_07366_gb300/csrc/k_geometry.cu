@@ -1560,7 +1560,7 @@ __device__ const double* q_solve_cta(int n, const double* __restrict__ sm)
 // dependent float64 operations, a few thousand cycles per step of the
 // reduction: the one-thread elimination walks n dependent 2 x 2 blocks
 // through global memory.  One step of two leapfrogging 32-node rings (four
-// evaluations): 3.65 -> 1.80 ms, the fit 513 -> about 50 us an evaluation.
+// evaluations): 3.65 -> 1.80 ms, the fit 513 -> 37 us an evaluation.
 template <typename T>
 __global__ void __launch_bounds__(256) k_spline_quintic_cta(const double* __restrict__ nodes,
                                                             const int64_t* __restrict__ off,
@@ -1709,15 +1709,17 @@ cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStre
             return cudaGetLastError();
         }
     }
-    const size_t sm = 9 * (size_t)w.nmax_fil * sizeof(T);
-    if (sm <= kSplineSmemMax) {
-        if (sm > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(k_spline_thomas<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 4) {
+        const size_t sm = 9 * (size_t)w.nmax_fil * sizeof(T);
+        if (sm <= kSplineSmemMax) {
+            if (sm > 48 * 1024) {
+                cudaError_t e = cudaFuncSetAttribute(k_spline_thomas<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                if (e != cudaSuccess) return e;
+            }
+            k_spline_thomas<T><<<nfil, spline_threads(nfil, w.nmax_fil), sm, s>>>(nodes, w.off, w.shift, nfil, w.nmax_fil, (T*)w.hseg, (T*)w.dp,
+                                                   (T*)w.ds, (T*)w.Mm, (T*)w.Tper);
+            return cudaGetLastError();
         }
-        k_spline_thomas<T><<<nfil, spline_threads(nfil, w.nmax_fil), sm, s>>>(nodes, w.off, w.shift, nfil, w.nmax_fil, (T*)w.hseg, (T*)w.dp,
-                                               (T*)w.ds, (T*)w.Mm, (T*)w.Tper);
-        return cudaGetLastError();
     }
     // filaments too long for shared memory: one thread per filament, in global memory
     const int tb = 64;

@@ -1037,9 +1037,9 @@ cudaError_t launch_short(const ShortP& P, const Work& w, cudaStream_t s)
     // ms on the 1e5-node one), the tiled kernel only on request
     const bool tiled = P.m <= kShortTileMaxM && P.kernel == 1;
     if (!tiled) {
-        // one warp per target; in float64 few nodes are spread over the SMs (the
-        // warps of a CTA share one slow float64 pipe: 64 nodes
-        // 38.5 -> 27 us)
+        // one warp per target (or pair of targets); in float64 few nodes are spread
+        // over the SMs (the warps of a CTA share one slow float64 pipe: 64 nodes
+        // 38.5 -> 27 us); from 152 x 8 nodes on every SM has a CTA of 8 warps
         int nw = kShortWarps;
         if (sizeof(T) == 8)
             while (nw > 1 && P.N < 152 * nw) nw /= 2;

@@ -1,6 +1,6 @@
 // Counting sorts that bin the quadrature sources: by short-range cell (the
 // cell lists of Sec. 5.3) and by spreading tile (the long-range spread).
-// count (atomics) -> exclusive scan (three launches, no inter-block waits)
+// count (atomics) -> exclusive scan (one to three launches, no inter-block waits)
 // -> scatter of the records into their bins.
 #include "bs_internal.cuh"
 
