@@ -6,6 +6,8 @@
 #include <cufft.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "bsewald.h"
 
 namespace bsw {
@@ -79,6 +81,25 @@ template <> struct __align__(16) LrRec<double> {
     int base;
     int pad[3];
 };
+
+// Allows a kernel all the dynamic shared memory a CTA can have: the 227 KB of
+// sm_103a less the kernel's static part.  A launch needs it once the two
+// together pass 48 KB, and the static part is easily forgotten in a comparison
+// against that; the launches that may come near therefore always ask.
+template <auto Kernel>
+cudaError_t allow_smem()
+{
+    static std::atomic<int> most{ 0 };  // a property of the compiled kernel
+    int m = most.load(std::memory_order_relaxed);
+    if (m == 0) {
+        cudaFuncAttributes a;
+        const cudaError_t e = cudaFuncGetAttributes(&a, Kernel);
+        if (e != cudaSuccess) return e;
+        m = 227 * 1024 - (int)a.sharedSizeBytes;
+        most.store(m, std::memory_order_relaxed);
+    }
+    return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
+}
 
 // ---- float64 helpers (float64 runs at 1/64 of the float32 rate: library
 // square roots, divisions and conversions are avoided where they are many) ----

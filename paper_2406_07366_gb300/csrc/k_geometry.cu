@@ -811,11 +811,8 @@ template <typename T>
 cudaError_t launch_spline_b(const BatchL& L, cudaStream_t s)
 {
     if (L.total <= 0) return cudaSuccess;
-    if (L.smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_spline_thomas_b<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)L.smem);
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = allow_smem<k_spline_thomas_b<T>>();
+    if (e != cudaSuccess) return e;
     k_spline_thomas_b<T><<<L.total, spline_threads(L.total, (int)(L.smem / (9 * sizeof(T)))), L.smem, s>>>((const SplineD<T>*)L.desc, L.bstart, L.n);
     return cudaGetLastError();
 }
@@ -1164,13 +1161,6 @@ __global__ void __launch_bounds__(256) k_energy_line_quintic_cta(const int64_t* 
 // Threads and shared memory of the CTA-per-filament quintic kernels.
 inline int quintic_threads(int nmax) { return nmax >= 256 ? 256 : (nmax + 31) & ~31; }
 
-template <typename K>
-cudaError_t quintic_smem(K kernel, size_t sm)
-{
-    return sm > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-                          : cudaSuccess;
-}
-
 template <typename T>
 cudaError_t launch_energy_line(const double* nodes, const Work& w, int nfil, int nmax, cudaStream_t s, bool det)
 {
@@ -1178,7 +1168,7 @@ cudaError_t launch_energy_line(const double* nodes, const Work& w, int nfil, int
     if (nfil <= 0) return cudaSuccess;
     if (w.Dd && kQuinticRow * (size_t)nmax <= kQuinticSmemMax) {  // quintic curves
         const size_t sm = kQuinticRow * (size_t)nmax;
-        cudaError_t e = quintic_smem(k_energy_line_quintic_cta<T>, sm);
+        cudaError_t e = allow_smem<k_energy_line_quintic_cta<T>>();
         if (e != cudaSuccess) return e;
         k_energy_line_quintic_cta<T><<<nfil, quintic_threads(nmax), sm, s>>>(
             w.off, w.shift, (const T*)w.hseg, (const T*)w.Dd, (const T*)w.Tper, w.pls, w.psr, w.energy_acc + 1,
@@ -1194,7 +1184,7 @@ cudaError_t launch_energy_line(const double* nodes, const Work& w, int nfil, int
     }
     if (kLineRow * (size_t)nmax <= kCubicSmemMax) {
         const size_t sc = kLineRow * (size_t)nmax;
-        cudaError_t e = quintic_smem(k_energy_line_cta<T>, sc);
+        cudaError_t e = allow_smem<k_energy_line_cta<T>>();
         if (e != cudaSuccess) return e;
         k_energy_line_cta<T><<<nfil, quintic_threads(nmax), sc, s>>>(w.off, w.shift, (const T*)w.hseg,
                                                                      (const T*)w.dp, (const T*)w.Mm, (const T*)w.Tper,
@@ -1203,10 +1193,8 @@ cudaError_t launch_energy_line(const double* nodes, const Work& w, int nfil, int
         return cudaGetLastError();
     }
     const size_t sm = 5 * (size_t)nmax * sizeof(double);
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_energy_line<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = allow_smem<k_energy_line<T>>();
+    if (e != cudaSuccess) return e;
     k_energy_line<T><<<nfil, 32, sm, s>>>(w.off, w.shift, nfil, nmax, (const T*)w.hseg, (const T*)w.dp,
                                           (const T*)w.Mm, (const T*)w.Tper, w.pls, w.psr,
                                           w.energy_acc + 1, det ? w.lpart : nullptr);
@@ -1687,7 +1675,7 @@ cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStre
     if (nfil <= 0) return cudaSuccess;
     if (w.Dd && kQuinticRow * (size_t)w.nmax_fil <= kQuinticSmemMax) {  // quintic
         const size_t sm = kQuinticRow * (size_t)w.nmax_fil;
-        cudaError_t e = quintic_smem(k_spline_quintic_cta<T>, sm);
+        cudaError_t e = allow_smem<k_spline_quintic_cta<T>>();
         if (e != cudaSuccess) return e;
         k_spline_quintic_cta<T><<<nfil, quintic_threads(w.nmax_fil), sm, s>>>(
             nodes, w.off, w.shift, (T*)w.hseg, (T*)w.dp, (T*)w.ds, (T*)w.Mm, (T*)w.Dd, (T*)w.Tper);
@@ -1702,7 +1690,7 @@ cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStre
     if constexpr (sizeof(T) == 8) {
         const size_t sc = kCubicRow * (size_t)w.nmax_fil;
         if (sc <= kCubicSmemMax) {
-            cudaError_t e = quintic_smem(k_spline_cta, sc);
+            cudaError_t e = allow_smem<k_spline_cta>();
             if (e != cudaSuccess) return e;
             k_spline_cta<<<nfil, quintic_threads(w.nmax_fil), sc, s>>>(nodes, w.off, w.shift, (T*)w.hseg, (T*)w.dp,
                                                                      (T*)w.ds, (T*)w.Mm, (T*)w.Tper);
@@ -1712,10 +1700,8 @@ cudaError_t launch_spline(const double* nodes, const Work& w, int nfil, cudaStre
     if constexpr (sizeof(T) == 4) {
         const size_t sm = 9 * (size_t)w.nmax_fil * sizeof(T);
         if (sm <= kSplineSmemMax) {
-            if (sm > 48 * 1024) {
-                cudaError_t e = cudaFuncSetAttribute(k_spline_thomas<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                if (e != cudaSuccess) return e;
-            }
+            cudaError_t e = allow_smem<k_spline_thomas<T>>();
+            if (e != cudaSuccess) return e;
             k_spline_thomas<T><<<nfil, spline_threads(nfil, w.nmax_fil), sm, s>>>(nodes, w.off, w.shift, nfil, w.nmax_fil, (T*)w.hseg, (T*)w.dp,
                                                    (T*)w.ds, (T*)w.Mm, (T*)w.Tper);
             return cudaGetLastError();
