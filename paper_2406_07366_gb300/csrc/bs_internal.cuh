@@ -209,6 +209,10 @@ struct ShortP {
     int want_psi;
     int nb[3];          // target blocks of m x m x m cells per axis, ceil(nc / m)
     int kernel;         // 0: by size, 1: tiled, 2: warp per node (BS_SHORT_TILED / BS_SHORT_PER_NODE)
+    // hc, L, rc2 and alpha rounded to float32 for the mixed form: a conversion
+    // in the kernel shares the slow float64 pipe, and where registers are short
+    // the compiler repeats it for every candidate
+    float hcf[3], Lf[3], rc2f, alphaf;
 };
 
 // The tiled short range takes cells per cut-off up to this (larger m: the

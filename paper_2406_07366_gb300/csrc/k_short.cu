@@ -171,6 +171,16 @@ __device__ __forceinline__ void st_pair(T rx, T ry, T rz, T r2, const T* q, T al
     }
 }
 
+// A length, squared radius or splitting parameter of ShortP in the kernels' precision.
+template <typename T>
+__device__ __forceinline__ T in_t(double d, float f)
+{
+    if constexpr (sizeof(T) == 4)
+        return f;
+    else
+        return d;
+}
+
 constexpr int kShortWarps = 8;  // warps per CTA of the warp-per-node kernel
 
 // Row tables of a CTA, per warp: a round's non-empty rows (first source of
@@ -207,10 +217,10 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
     const int cx = t.cell % nc0;
     const int cy = (t.cell / nc0) % nc1;
     const int cz = t.cell / (nc0 * nc1);
-    const T h0 = (T)P.hc[0], h1 = (T)P.hc[1], h2 = (T)P.hc[2];
-    const T L0 = (T)P.L[0], L1 = (T)P.L[1], L2 = (T)P.L[2];
-    const T rc2 = (T)P.rc2;
-    const T alpha = (T)P.alpha;
+    const T h0 = in_t<T>(P.hc[0], P.hcf[0]), h1 = in_t<T>(P.hc[1], P.hcf[1]), h2 = in_t<T>(P.hc[2], P.hcf[2]);
+    const T L0 = in_t<T>(P.L[0], P.Lf[0]), L1 = in_t<T>(P.L[1], P.Lf[1]), L2 = in_t<T>(P.L[2], P.Lf[2]);
+    const T rc2 = in_t<T>(P.rc2, P.rc2f);
+    const T alpha = in_t<T>(P.alpha, P.alphaf);
     const double alpha16 = 16.0 * P.alpha;  // float64: the tables' argument
     const T two_over_sqrtpi = (T)1.12837916709551257390;
     const int m = P.m;
@@ -426,9 +436,9 @@ __device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>
     const int cx = ta.cell % nc0;
     const int cy = (ta.cell / nc0) % nc1;
     const int cz = ta.cell / (nc0 * nc1);
-    const float h0 = (float)P.hc[0], h1 = (float)P.hc[1], h2 = (float)P.hc[2];
-    const float rc2 = (float)P.rc2;
-    const float alpha = (float)P.alpha;
+    const float h0 = P.hcf[0], h1 = P.hcf[1], h2 = P.hcf[2];
+    const float rc2 = P.rc2f;
+    const float alpha = P.alphaf;
     const int m = P.m;
     const int ny = 2 * m + 1 + abs(dy), nz = 2 * m + 1 + abs(dz);
     const int y0 = min(dy, 0) - m, z0 = min(dz, 0) - m;  // first row offsets from the first node's cell
@@ -616,8 +626,8 @@ __host__ __device__ __forceinline__ bool short_pairs(const ShortP& P)
 
 // One warp of the kernels below: a node, or with PAIR a pair of nodes where
 // the grid allows (pairs whose cells are further apart one after the other).
-// The two are separate kernels: the paired walk's registers would cost the
-// small grids that cannot use it half of their warps.
+// The two are separate kernels: in one of 91 registers the small grids, which
+// cannot pair, took 4 % longer over a batch.
 template <typename T, bool PAIR>
 __device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __restrict__ tgt,
                                              const int* __restrict__ prev, const int* __restrict__ start,
@@ -646,8 +656,11 @@ __device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __
     for (; j < je && j < P.N; ++j) k_short_body<T>(P, tgt, prev, start, src, vsr, psr, j, tab, rows);
 }
 
+// Four CTAs per SM in float32 (64 registers).  Five (48) left too few to keep
+// the cell edges and box lengths of the minimum-image walk: 2e4 nodes with the
+// cut-off at half the box 3.65 -> 7.25 ms, nothing gained elsewhere.
 template <typename T, bool PAIR>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (PAIR ? 4 : 5) : 3) k_short(ShortP P, const SrTgt<T>* __restrict__ tgt, const int* __restrict__ prev,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short(ShortP P, const SrTgt<T>* __restrict__ tgt, const int* __restrict__ prev,
                                                const int* __restrict__ start, const SrRec<T>* __restrict__ src,
                                                double* __restrict__ vsr, double* __restrict__ psr)
 {
@@ -663,7 +676,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (PAIR ? 4 : 5) : 3) k_sh
 }
 
 template <typename T, bool PAIR>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (PAIR ? 4 : 5) : 3) k_short_b(const ShortD<T>* __restrict__ d, const int* __restrict__ bs, int n)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short_b(const ShortD<T>* __restrict__ d, const int* __restrict__ bs, int n)
 {
     __shared__ ShortRows<T> rows;
     int bid, nb;

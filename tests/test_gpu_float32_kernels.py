@@ -126,3 +126,22 @@ def test_cubic_fit_by_a_block_per_filament(n, copies, closing):
     d -= f.L * np.round(d / f.L)
     assert np.abs(d).max() < 2.4e-6 * chord
     assert np.abs(qq[:3 * n].cpu().numpy() - g.qq).max() < 2.4e-6 * np.abs(g.qq).max()
+
+
+@pytest.mark.parametrize("rc_over_L", [0.5, 0.4, 0.35])
+def test_short_range_with_whole_axes_and_minimum_images(rc_over_L):
+    """Cut-offs above a third of the box: every cell of an axis is a neighbour
+    and separations wrap.  Velocity and streamfunction against the float64
+    form at float32's 1e-5 (rms), as for the smaller cut-offs."""
+    B, f = _B(), W.ellipses(7, 45, seed=5)
+    rc = rc_over_L * 2 * math.pi
+    out = []
+    for prec in (B.BS_MIXED, B.BS_FP64):
+        p = B.make_params(f.L, M=32, Q=2, w=8, alpha=3.5 / rc, rc=rc, flags=B.BS_WANT_PSI, precision=prec)
+        bs = B.BiotSavart(p, f.offsets, f.closing)
+        v, psi = bs.parts(torch.from_numpy(f.nodes).cuda(), want_psi=True)
+        torch.cuda.synchronize()
+        bs.close()
+        out.append((v[1].cpu().numpy(), psi[1].cpu().numpy()))
+    for a, b in zip(*out):
+        assert np.sqrt(((a - b) ** 2).mean()) <= 1e-5 * np.sqrt((b ** 2).mean())
