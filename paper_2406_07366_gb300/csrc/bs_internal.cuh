@@ -85,7 +85,10 @@ template <> struct __align__(16) LrRec<double> {
 // Allows a kernel all the dynamic shared memory a CTA can have: the 227 KB of
 // sm_103a less the kernel's static part.  A launch needs it once the two
 // together pass 48 KB, and the static part is easily forgotten in a comparison
-// against that; the launches that may come near therefore always ask.
+// against that; the launches that may come near therefore always ask.  Always
+// for the same amount: the limit belongs to the kernel on the device, not to a
+// context, and set to each launch's own size it could be lowered by one thread
+// between another's setting and launch.
 template <auto Kernel>
 cudaError_t allow_smem()
 {

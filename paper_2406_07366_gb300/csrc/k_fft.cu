@@ -2945,8 +2945,7 @@ struct SpzLaunch {
     {
         using C = typename Cx<T>::t;
         const size_t sm = spread_zfft_smem<T>(P);
-        cudaError_t e =
-            cudaFuncSetAttribute(k_spread_zfft<T, W, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = allow_smem<k_spread_zfft<T, W, RM>>();
         if (e != cudaSuccess) return e;
         k_spread_zfft<T, W, RM><<<P.nbx * P.nby, z_threads<T>(P), sm, s>>>(
             P, w.col_cnt, w.col_rec, (const SpPt<T, W>*)w.col_pts, (const C*)w.tw + P.ng[0] + P.ng[1],
@@ -2989,8 +2988,7 @@ struct ZiLaunch {
     {
         using C = typename Cx<T>::t;
         const size_t sm = zlines_bytes<T>(3 * P.tx * P.ty / 2, P.cls);
-        cudaError_t e =
-            cudaFuncSetAttribute(k_zfft_interp<T, W, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = allow_smem<k_zfft_interp<T, W, RM>>();
         if (e != cudaSuccess) return e;
         k_zfft_interp<T, W, RM><<<P.nbx * P.nby, z_threads<T>(P), sm, s>>>(
             P, w.ncol_cnt, (const NdW<T, W>*)w.nd_sorted, (const C*)w.spec, (const C*)w.tw + P.ng[0] + P.ng[1],
@@ -3045,7 +3043,7 @@ struct FftYLaunch {
         }
         size_t sm = (size_t)MC * P.ls * sizeof(C);
         if (Q.tnb > 0) sm = (size_t)MC * std::max(P.ls, Q.tnb * Q.tby) * sizeof(C) + 128;
-        cudaError_t e = cudaFuncSetAttribute(k_fft_y<T, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = allow_smem<k_fft_y<T, RM>>();
         if (e != cudaSuccess) return e;
         const int nk = P.K[2] + 1;
         const int nch = (nk + MC - 1) / MC;
@@ -3147,8 +3145,7 @@ struct FftXLaunch {
         if (Q.tnbx > 0) sm = (size_t)3 * MC * Q.tnbx * Q.tbx * sizeof(C) + 128;
         if (P.spectrum) sm = std::max(sm, (size_t)3 * MC * P.ls * sizeof(C) + sizeof(double) * (size_t)P.nbins);
         if (P.epart) sm += sizeof(double) * (kZThreadsMax / 32);
-        cudaError_t e =
-            cudaFuncSetAttribute(k_fft_x_kspace<T, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = allow_smem<k_fft_x_kspace<T, RM>>();
         if (e != cudaSuccess) return e;
         const int nk = P.K[2] + 1;
         const int nch = (nk + MC - 1) / MC;
@@ -3187,8 +3184,7 @@ struct FftZLaunch {
     {
         using C = typename Cx<T>::t;
         const size_t sm = (size_t)(P.yc / 2) * P.cls * sizeof(C);
-        cudaError_t e =
-            cudaFuncSetAttribute(k_fft_z_c2r<T, RM, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = allow_smem<k_fft_z_c2r<T, RM, TO>>();
         if (e != cudaSuccess) return e;
         k_fft_z_c2r<T, RM, TO><<<3 * P.ng[0] * (P.ng[1] / P.yc), kThreads, sm, s>>>(
             P, (const C*)w.spec, (const C*)w.tw + P.ng[0] + P.ng[1], out);
@@ -3321,8 +3317,7 @@ cudaError_t launch_col_scatter_b(int w, const BatchL& L, cudaStream_t s)
 template <typename T, int W>
 static cudaError_t spz_b(const BatchL& L, cudaStream_t s)
 {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_spread_zfft_b<T, W, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    cudaError_t e = allow_smem<k_spread_zfft_b<T, W, 8>>();
     if (e != cudaSuccess) return e;
     k_spread_zfft_b<T, W, 8><<<L.total, L.threads, L.smem, s>>>((const SpzD<T>*)L.desc, L.bstart, L.n);
     return cudaGetLastError();
@@ -3346,7 +3341,7 @@ template <typename T>
 cudaError_t launch_fft_y_b(const BatchL& L, cudaStream_t s)
 {
     if (L.total <= 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_fft_y_b<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    cudaError_t e = allow_smem<k_fft_y_b<T, 8>>();
     if (e != cudaSuccess) return e;
     k_fft_y_b<T, 8><<<L.total, kThreads, L.smem, s>>>((const FftYD<T>*)L.desc, L.bstart, L.n);
     return cudaGetLastError();
@@ -3362,8 +3357,7 @@ template <typename T>
 cudaError_t launch_fft_x_kspace_b(const BatchL& L, cudaStream_t s)
 {
     if (L.total <= 0) return cudaSuccess;
-    cudaError_t e =
-        cudaFuncSetAttribute(k_fft_x_kspace_b<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    cudaError_t e = allow_smem<k_fft_x_kspace_b<T, 8>>();
     if (e != cudaSuccess) return e;
     const int nt = std::min(L.threads, x_threads_max<T>());
     k_fft_x_kspace_b<T, 8><<<L.total, nt, L.smem, s>>>((const FftXD<T>*)L.desc, L.bstart, L.n);
@@ -3395,8 +3389,7 @@ size_t zfft_interp_smem(const SpZP& P)
 template <typename T, int W>
 static cudaError_t zi_b(const BatchL& L, cudaStream_t s)
 {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_zfft_interp_b<T, W, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    cudaError_t e = allow_smem<k_zfft_interp_b<T, W, 8>>();
     if (e != cudaSuccess) return e;
     k_zfft_interp_b<T, W, 8><<<L.total, L.threads, L.smem, s>>>((const SpzD<T>*)L.desc, L.bstart, L.n);
     return cudaGetLastError();

@@ -407,10 +407,8 @@ template <typename T, int W>
 static cudaError_t spread_w(const SpreadP& P, const Work& w, int ntiles, cudaStream_t s)
 {
     const size_t sm = spread_smem<T>(P);
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_spread<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = allow_smem<k_spread<T, W>>();
+    if (e != cudaSuccess) return e;
     k_spread<T, W><<<ntiles, kThreads, sm, s>>>(P, w.tile_cnt, (const LrRec<T>*)w.lr_sorted, (T*)w.grid);
     return cudaGetLastError();
 }

@@ -85,3 +85,45 @@ def test_staged_batch_whose_fit_nearly_fills_48_kb(n):
     bs.status()
     bs.close()
     assert float((got - ref).abs().max()) < 1e-6 * float(ref.abs().max())
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+def test_contexts_of_different_sizes_in_several_threads(prec):
+    """A kernel's shared memory limit belongs to the function, not to a context:
+    contexts whose launches need different amounts (grids of 48 to 192 points,
+    filaments of 64 to 1500 nodes), each driven by a thread of its own, must not
+    lower it for one another.  Every evaluation equals the context's first one
+    (float32 atomics reorder the mixed sums: 1e-6; float64 1e-12)."""
+    import threading
+    B = _B()
+    out, err = {}, []
+
+    def drive(k, M, n):
+        try:
+            f = _ring(n)
+            s = torch.cuda.Stream()
+            p = B.make_params(f.L, M=M, Q=2, w=8, precision=B.BS_FP64 if prec == "fp64" else B.BS_MIXED)
+            bs = B.BiotSavart(p, f.offsets, f.closing, stream=s)
+            nodes = torch.from_numpy(f.nodes).cuda()
+            v = [torch.empty_like(nodes) for _ in range(2)]
+            torch.cuda.synchronize()
+            bs.velocity(nodes, v[0])
+            ready.wait(60)
+            for _ in range(400):
+                bs.velocity(nodes, v[1])
+            bs.status()
+            out[k] = float((v[1] - v[0]).abs().max() / v[0].abs().max())
+            bs.close()
+        except Exception as e:  # noqa: BLE001 (shown by the main thread)
+            err.append(repr(e))
+            ready.abort()
+
+    sizes = [(32, 64), (64, 400), (96, 1000), (128, 1500)]
+    ready = threading.Barrier(len(sizes))
+    threads = [threading.Thread(target=drive, args=(k, *s)) for k, s in enumerate(sizes)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not err, err
+    assert len(out) == len(sizes) and max(out.values()) < (1e-6 if prec == "mixed" else 1e-12), out
