@@ -656,9 +656,10 @@ __device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __
     for (; j < je && j < P.N; ++j) k_short_body<T>(P, tgt, prev, start, src, vsr, psr, j, tab, rows);
 }
 
-// Four CTAs per SM in float32 (64 registers).  Five (48) left too few to keep
-// the cell edges and box lengths of the minimum-image walk: 2e4 nodes with the
-// cut-off at half the box 3.65 -> 7.25 ms, nothing gained elsewhere.
+// Four CTAs per SM in float32 (64 registers): with five (48) the one-node walk
+// at the minimum image is 2 % slower (2e4 nodes, cut-off at half the box: 3.65
+// and 3.73 ms).  The batched form of that walk hides more latency with five
+// (256 members of 250 to 650 nodes: 1729 against 1750 us).
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short(ShortP P, const SrTgt<T>* __restrict__ tgt, const int* __restrict__ prev,
                                                const int* __restrict__ start, const SrRec<T>* __restrict__ src,
@@ -676,7 +677,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short(ShortP P,
 }
 
 template <typename T, bool PAIR>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short_b(const ShortD<T>* __restrict__ d, const int* __restrict__ bs, int n)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (PAIR ? 4 : 5) : 3) k_short_b(const ShortD<T>* __restrict__ d, const int* __restrict__ bs, int n)
 {
     __shared__ ShortRows<T> rows;
     int bid, nb;
