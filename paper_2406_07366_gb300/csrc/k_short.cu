@@ -112,13 +112,16 @@ __device__ __forceinline__ double erfc_e<double>(double x, double) { return erfc
 //   1/r from the hardware's approximate reciprocal square root and one step
 //   of Householder's third-order iteration (y += y e (1/2 + 3 e / 8), e = 1 -
 //   r2 y^2; the seed's 2^-20 becomes below 2^-58), 5 operations;
-//   g^(n)(x) and erfc(x) from tables of degree-8 polynomials on intervals of
+//   g^(n)(x) and erfc(x) from tables of degree-11 polynomials on intervals of
 //   width 1/16 centred at i / 16, i = 0..128, written once per device from
 //   Chebyshev interpolation of the functions in extended precision
-//   (set_short_tables): 8 operations each, interpolation error below 2^-60
-//   of the largest value on the interval.
+//   (set_short_tables): 11 operations each.  Relative to the function itself
+//   the value is within 2.1e-16 up to x = 7 and 3.8e-16 up to 8, roundings
+//   included (degree 8: 3e-15 at x = 3.5, 2.7e-11 at 8; the functions fall by
+//   e^-(x/8) and more over an interval, and their high derivatives grow like
+//   powers of 2 x).
 // Beyond x = 8 the library functions are called.
-constexpr int kSgN = 129, kSgDeg = 8, kSgStride = 132;
+constexpr int kSgN = 129, kSgDeg = 11, kSgStride = 132;
 constexpr int kSgTable = (kSgDeg + 1) * kSgStride;  // doubles per function, degree-major
 __device__ double g_sg_tab[2 * kSgTable];           // g^(n), then erfc
 

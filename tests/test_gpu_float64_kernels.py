@@ -142,3 +142,75 @@ def test_float64_node_terms_by_lanes_equal_a_thread_per_node(order, total, local
         out.append([x[k, :65].cpu().numpy() for x in (v, psi) for k in (0, 3)])
     for x, y in zip(*out):
         assert np.abs(x - y).max() < 1e-12 * np.abs(x).max()
+
+
+def _erfc_g(x):
+    """erfc(x) and g(x) = erfc(x) + 2/sqrt(pi) x exp(-x^2) of a Decimal, at the context's precision."""
+    from decimal import Decimal
+    c = 2 / Decimal("3.14159265358979323846264338327950288419716939937510582097494459230781640628620899862803").sqrt()
+    term, s, n = x, x, 0
+    while abs(term) > Decimal(10) ** -70:
+        n += 1
+        term *= -x * x / n
+        s += term / (2 * n + 1)
+    e = 1 - c * s
+    return e, e + c * x * (-x * x).exp()
+
+
+@pytest.mark.parametrize("alpha", [0.25, 1.0, 1.5, 2.0])
+def test_float64_pair_functions_relative_to_themselves(alpha):
+    """Two lines at right angles, two lengths apart, with their reverses out of
+    reach: at a node of one line psi points along the other line and the
+    velocity's part across both comes from it alone, from separations r of the
+    node's distance and a little more.  So each node shows erfc(alpha r) and
+    g(alpha r) relative to themselves, up to alpha r = 8.  Coordinates are
+    exact in binary but for the quadrature points along the lines; three
+    roundings of r are amplified by the functions' (x^2 2 relative), the rest
+    is a dozen roundings: (16 x^2 + 32) 2^-53."""
+    from decimal import Decimal, localcontext
+    B, n, rc = _B(), 32, 4.0
+    L = np.full(3, 16.0)
+    t = 0.5 * np.arange(n)
+
+    def line(axis, *at):
+        X = np.empty((n, 3))
+        X[:, axis] = t
+        X[:, [k for k in range(3) if k != axis]] = at
+        return X
+
+    a, b = line(2, 0.5, 8.5), line(1, 2.5, 8.25)              # along z; along y, 2 away in x
+    back_a, back_b = line(2, 8.5, 8.5)[::-1], line(1, 10.5, 8.25)[::-1]
+    f = W._pack([a, b, back_a, back_b], L, closing=[[0, 0, 1], [0, 1, 0], [0, 0, -1], [0, -1, 0]])
+    p = B.make_params(L, M=32, Q=3, w=8, alpha=alpha, rc=rc, flags=B.BS_WANT_PSI, precision=B.BS_FP64)
+    bs = B.BiotSavart(p, f.offsets, f.closing)
+    nodes = torch.from_numpy(f.nodes).cuda()
+    v, psi = bs.parts(nodes, want_psi=True)
+    qX, qq = bs.quadrature(nodes)
+    bs.status()
+    bs.close()
+    vz, py = v[1][:n, 2].cpu().numpy(), psi[1][:n, 1].cpu().numpy()
+    Y, q = qX.cpu().numpy()[3 * n:6 * n], qq.cpu().numpy()[3 * n:6 * n, 1]
+    seen = 0
+    with localcontext() as ctx:
+        ctx.prec = 110
+        for j in range(n):
+            ev = ep = Decimal(0)
+            dz = Decimal(8.25) - Decimal(float(a[j, 2]))
+            for y, c in zip(Y[:, 1], q):
+                dy = Decimal(float(y)) - Decimal(8.5)
+                r2 = 4 + dy * dy + dz * dz
+                if r2 >= 16:
+                    continue
+                r = r2.sqrt()
+                e, g = _erfc_g(Decimal(alpha) * r)
+                ev += 2 * Decimal(float(c)) * g / (r2 * r)    # (r x q)_z = r_x q_y
+                ep += Decimal(float(c)) * e / r
+            if ep == 0:
+                continue
+            seen += 1
+            pre = Decimal(p.kappa / (4 * math.pi))
+            x2 = alpha ** 2 * (4 + float(dz) ** 2)
+            tol = (16 * x2 + 32) * 2.0 ** -53
+            assert abs(Decimal(float(vz[j])) / (pre * ev) - 1) < tol, (j, math.sqrt(x2))
+            assert abs(Decimal(float(py[j])) / (pre * ep) - 1) < tol, (j, math.sqrt(x2))
+    assert seen >= 12
