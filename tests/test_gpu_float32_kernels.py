@@ -145,3 +145,28 @@ def test_short_range_with_whole_axes_and_minimum_images(rc_over_L):
         out.append((v[1].cpu().numpy(), psi[1].cpu().numpy()))
     for a, b in zip(*out):
         assert np.sqrt(((a - b) ** 2).mean()) <= 1e-5 * np.sqrt((b ** 2).mean())
+
+
+@pytest.mark.parametrize("M", [150, 299, 300])
+def test_compiled_transforms_where_the_modes_pass_a_third(M):
+    """sigma = 1.25 keeps K >= n / 3 of the modes on grids of 192 and 384 points,
+    whose passes are compiled for their lengths: the whole transforms then end
+    in a general last pass.  Long-range velocity and psi against full cuFFT
+    transforms: 2e-6 as in the boundary-pass test, one more pass per axis at
+    384 points: 3e-6."""
+    B = _B()
+    f = W.ellipses(3, 40, seed=M)
+    nodes = torch.from_numpy(f.nodes).cuda()
+    got = []
+    for flags in (0, B.BS_WANT_PSI, B.BS_WANT_PSI | B.BS_FFT_CUFFT):
+        p = B.make_params(f.L, M=M, Q=2, w=8, sigma=1.25, flags=flags, alpha=1.2, rc=3.0, precision=B.BS_MIXED)
+        n, _ = B.bs_nufft_setup(p, want_table=False)
+        assert tuple(n) == ((192,) * 3 if M == 150 else (384,) * 3) and 3 * ((M - 1) // 2) >= n[0]
+        bs = B.BiotSavart(p, f.offsets, f.closing)
+        v = bs.parts(nodes, want_psi=bool(flags))
+        got.append([x[2].clone() for x in (v if flags else (v,))])
+        torch.cuda.synchronize()
+        bs.close()
+    ref = got[2]
+    for x, r in ((got[0][0], ref[0]), (got[1][0], ref[0]), (got[1][1], ref[1])):
+        assert float((x - r).abs().max()) < 3e-6 * float(r.abs().max())
