@@ -5,8 +5,10 @@
 #include <cuda_runtime.h>
 #include <cufft.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <atomic>
+#include <mutex>
 
 #include "bsewald.h"
 
@@ -102,6 +104,20 @@ cudaError_t allow_smem()
         most.store(m, std::memory_order_relaxed);
     }
     return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
+}
+
+// Writes a table into a symbol of the current device unless it is there.  The
+// device is asked (for the first 8 bytes, never zero in a table), as a host-side
+// note would outlive a device reset, which clears the symbol.
+template <typename S>
+cudaError_t put_table(const S& symbol, const void* tab, size_t bytes)
+{
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    unsigned long long there = 0;
+    const cudaError_t e = cudaMemcpyFromSymbol(&there, symbol, sizeof there);
+    if (e != cudaSuccess || memcmp(&there, tab, sizeof there) == 0) return e;
+    return cudaMemcpyToSymbol(symbol, tab, bytes);
 }
 
 // ---- float64 helpers (float64 runs at 1/64 of the float32 rate: library

@@ -30,7 +30,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include <cudaTypedefs.h>
 #include <string.h>
@@ -183,7 +182,7 @@ __device__ __forceinline__ unsigned char* smem_align128(unsigned char* p)
 }
 
 // e^{-2 pi i m / R} for the composite in-register sizes R in {6, 9, 12, 16,
-// 24, 32}, m = 0..R-1, written once per device from float64 values
+// 24, 32}, m = 0..R-1, written from float64 values
 // (set_fft_constants).  Indices are compile-time constants after unrolling,
 // so the factors come straight from the constant bank.
 constexpr int kTwOff6 = 0, kTwOff9 = 6, kTwOff12 = 15, kTwOff16 = 27, kTwOff24 = 43, kTwOff32 = 67, kTwCount = 99;
@@ -3431,18 +3430,10 @@ BSW_INST_B(float)
 #endif
 #undef BSW_INST_B
 
-// Writes the composite-radix twiddles into the current device's constant
-// bank (once per device).
+// Writes the composite-radix twiddles into the current device's constant bank.
 template <typename T>
 cudaError_t set_fft_constants()
 {
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
     float2 hf[kTwCount];
     double2 hd[kTwCount];
     const int sizes[6] = { 6, 9, 12, 16, 24, 32 };
@@ -3454,11 +3445,9 @@ cudaError_t set_fft_constants()
             hf[offs[k] + m] = make_float2((float)cos(ph), (float)sin(ph));
         }
     if constexpr (sizeof(T) == 4)
-        e = cudaMemcpyToSymbol(c_twf, hf, sizeof hf);
+        return put_table(c_twf, hf, sizeof hf);
     else
-        e = cudaMemcpyToSymbol(c_twd, hd, sizeof hd);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-    return e;
+        return put_table(c_twd, hd, sizeof hd);
 }
 
 // One object per precision (the two compile in parallel): BSW_FFT_DOUBLE.

@@ -28,8 +28,6 @@
 // T-precision offset from the cell origin.
 #include <math.h>
 
-#include <mutex>
-
 #include "bs_internal.cuh"
 
 namespace bsw {
@@ -391,8 +389,7 @@ __device__ __forceinline__ void make_poly(SegPoly<T>& P, const T* __restrict__ h
 // root and two divisions cost it about 150 float64 operations a point): E(u) =
 // g^(f)(x) / x^3 and P(u) = erf(x) / x are entire functions of u = x^2, taken
 // from degree-8 polynomials on intervals of 1/4 centred at i / 4, i = 0..64
-// (interpolation error below 2^-55), written once per device
-// (set_node_tables).  Beyond u = 16 the library forms below.
+// (interpolation error below 2^-55), written by set_node_tables.  Beyond u = 16 the library forms below.
 constexpr int kSelfN = 65, kSelfDeg = 8;
 __device__ double g_self_tab[2][(kSelfDeg + 1) * kSelfN];  // E, P; degree-major
 
@@ -1795,24 +1792,21 @@ static long double self_p(long double u)
     return erfl(x) / x;
 }
 
-// The float64 self term's tables, once per device.
+// The float64 self term's tables, on the current device.
 cudaError_t set_node_tables()
 {
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-    static double tab[2][(kSelfDeg + 1) * kSelfN];
-    for (int i = 0; i < kSelfN; ++i) {
-        cheb_fit(self_e, i / 4.0L, 1 / 4.0L, kSelfDeg, tab[0] + i, kSelfN);
-        cheb_fit(self_p, i / 4.0L, 1 / 4.0L, kSelfDeg, tab[1] + i, kSelfN);
-    }
-    e = cudaMemcpyToSymbol(g_self_tab, tab, sizeof tab);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-    return e;
+    struct Tables {
+        double v[2][(kSelfDeg + 1) * kSelfN];
+        Tables()
+        {
+            for (int i = 0; i < kSelfN; ++i) {
+                cheb_fit(self_e, i / 4.0L, 1 / 4.0L, kSelfDeg, v[0] + i, kSelfN);
+                cheb_fit(self_p, i / 4.0L, 1 / 4.0L, kSelfDeg, v[1] + i, kSelfN);
+            }
+        }
+    };
+    static const Tables tab;
+    return put_table(g_self_tab, tab.v, sizeof tab.v);
 }
 
 }  // namespace bsw

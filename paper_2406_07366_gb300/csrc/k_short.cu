@@ -20,8 +20,6 @@
 // k_short (larger m): one warp per node walks the (2m+1)^2 neighbour rows.
 #include <math.h>
 
-#include <mutex>
-
 #include "bs_internal.cuh"
 
 namespace bsw {
@@ -113,7 +111,7 @@ __device__ __forceinline__ double erfc_e<double>(double x, double) { return erfc
 //   of Householder's third-order iteration (y += y e (1/2 + 3 e / 8), e = 1 -
 //   r2 y^2; the seed's 2^-20 becomes below 2^-58), 5 operations;
 //   g^(n)(x) and erfc(x) from tables of degree-11 polynomials on intervals of
-//   width 1/16 centred at i / 16, i = 0..128, written once per device from
+//   width 1/16 centred at i / 16, i = 0..128, written from
 //   Chebyshev interpolation of the functions in extended precision
 //   (set_short_tables): 11 operations each.  Relative to the function itself
 //   the value is within 2.1e-16 up to x = 7 and 3.8e-16 up to 8, roundings
@@ -1117,24 +1115,21 @@ static long double sg_near(long double x)
     return erfcl(x) + 1.12837916709551257389615890312154517L * x * expl(-x * x);
 }
 
-// The float64 pair term's tables, once per device.
+// The float64 pair term's tables, on the current device.
 cudaError_t set_short_tables()
 {
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-    static double tab[2 * kSgTable];
-    for (int i = 0; i < kSgN; ++i) {
-        cheb_fit(sg_near, i / 16.0L, 1 / 16.0L, kSgDeg, tab + i, kSgStride);
-        cheb_fit(sg_erfc, i / 16.0L, 1 / 16.0L, kSgDeg, tab + kSgTable + i, kSgStride);
-    }
-    e = cudaMemcpyToSymbol(g_sg_tab, tab, sizeof tab);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-    return e;
+    struct Tables {
+        double v[2 * kSgTable] = {};
+        Tables()
+        {
+            for (int i = 0; i < kSgN; ++i) {
+                cheb_fit(sg_near, i / 16.0L, 1 / 16.0L, kSgDeg, v + i, kSgStride);
+                cheb_fit(sg_erfc, i / 16.0L, 1 / 16.0L, kSgDeg, v + kSgTable + i, kSgStride);
+            }
+        }
+    };
+    static const Tables tab;
+    return put_table(g_sg_tab, tab.v, sizeof tab.v);
 }
 
 // The float32 complementary error function as the short-range kernels take
