@@ -1263,8 +1263,10 @@ int bs_create(bs_ctx** out, const bs_params* p, void* stream)
     }
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = p->precision == BS_FP64 ? set_fft_constants<double>() : set_fft_constants<float>();
-    if (e == cudaSuccess) e = set_short_tables();
-    if (e == cudaSuccess) e = set_node_tables();
+    if (p->precision == BS_FP64) {
+        if (e == cudaSuccess) e = set_short_tables();
+        if (e == cudaSuccess) e = set_node_tables();
+    }
     // the short-range branch runs at the highest stream priority: its few
     // CTAs are dispatched ahead of the long-range kernels' waiting ones, so
     // the branch ends while the spread is still running
