@@ -317,7 +317,13 @@ int bs_rk4_launch(bs_ctx* ctx, int nsteps);
  * kernel width and z-column CTA size of the first of them.  Each stage of
  * the group's evaluation is ONE launch for all its members: member m runs
  * its own blocks of the launch with its own parameters, taken from a device
- * table (22 launches whatever the member count).  Every other member's
+ * table (19 launches whatever the member count; two more for each of the
+ * three scans when a member has more bins than one CTA scans, one more when
+ * only some members' grids let the short range take nodes in pairs).  In
+ * mixed precision a member's result is its single context's up to rounding:
+ * the order of float32 sums, and, at nodes with a neighbour nearer than about
+ * 1e-3 of the box, roundings of their separation (below 1e-5 of the largest
+ * velocity, where either is that far from the float64 form).  Every other member's
  * evaluation is issued by itself on an internal pool of up to 8 streams,
  * concurrently with the group.  Passing both batch flags on one member is
  * BS_ERR_ARG.  With a non-default

@@ -1727,7 +1727,7 @@ struct Arena {
     {
         const size_t o = (bytes.size() + 255) & ~(size_t)255;
         bytes.resize(o + n);
-        memcpy(bytes.data() + o, p, n);
+        if (n) memcpy(bytes.data() + o, p, n);
         return o;
     }
 };
@@ -1860,7 +1860,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, 128, 0);
     }
-    // counting sorts: zero the counts, count, scan, copy to the cursors, scatter
+    // counting sorts: zero the counts, count, scan (the starts go to the cursors too), scatter
     // exclusive scan of a counter array per member, the starts copied to cur_of
     // (null: no copy); the second list has one CTA per member: members of up to
     // 8 tiles are scanned by one CTA each in one launch
@@ -1916,21 +1916,16 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, kThreads, 0);
     }
-    {   // 7 short range (warp per node, or per pair when most nodes can pair)
+    // short range: the members that take their nodes in pairs, then (at the end
+    // of the list) those that take them one by one.  Each member's own grid
+    // decides, as in its single context, not the company that it is in.
+    auto short_stage = [&](bool pairs) {
         std::vector<ShortD<T>> D;
-        const int prec = sizeof(T) == 8 ? BS_FP64 : BS_MIXED;
-        long long can = 0, all = 0;
-        for (size_t m = 0; m < nm; ++m) {
-            ShortP P;
-            fill_short(mem[m], false, P);
-            all += P.N;
-            can += short_can_pair(P, prec) ? P.N : 0;
-        }
-        const bool kind = 2 * can > all;
         for (size_t m = 0; m < nm; ++m) {
             const Work& w = mem[m]->w;
             ShortD<T> e;
             fill_short(mem[m], false, e.P);
+            if (short_can_pair(e.P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED) != pairs) continue;
             e.tgt = (const SrTgt<T>*)w.tgt;
             e.prev = w.prev;
             e.start = w.cell_cnt;
@@ -1938,11 +1933,12 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
             e.vsr = w.vsr;
             e.psr = w.psr;
             D.push_back(e);
-            blk.push_back(short_blocks(e.P, kind && short_can_pair(e.P, prec)));
+            blk.push_back(short_blocks(e.P, pairs));
         }
         add(D, 256, 0);
-        st.back().kind = kind;
-    }
+        st.back().kind = pairs;
+    };
+    short_stage(true);                                                                     // 7 short range
     auto col_cnt = [](bs_ctx* c) { return c->w.col_cnt; };
     auto colb_n = [](bs_ctx* c) { return c->d.ncolb; };  // spread bins: blocks x z-buckets
     auto col_n = [](bs_ctx* c) { return c->d.ncols; };   // node bins: blocks
@@ -2096,6 +2092,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, 256, 0);
     }
+    short_stage(false);                                                                    // 22 short range
     // upload, then turn the offsets into device pointers.  The group's
     // streams finish with the old tables first; the copy is ordered on the
     // group's stream and waited for (a plain copy from pageable memory may
@@ -2147,6 +2144,7 @@ int batch_issue_staged(bs_batch* b, cudaStream_t s)
     CE(launch_scan_b(L[4], L[5], ss));
     CE(launch_scatter_b<SrRec<T>>(L[6], ss));
     CE(launch_short_b<T>(L[7], ss));
+    CE(launch_short_b<T>(L[22], ss));
     CE(launch_node_w_b<T>(w, L[16], ss));
     CE(launch_scan_b(L[17], L[18], ss));
     CE(launch_node_scatter_b<T>(w, L[19], ss));

@@ -209,3 +209,50 @@ def test_staged_group_follows_the_size_rule_and_flags():
     with pytest.raises(B.BSError) as e:
         B.bs_batch_create([bad], torch.cuda.current_stream().cuda_stream)
     assert e.value.code == B.BS_ERR_ARG
+
+
+@pytest.mark.parametrize("small_cutoffs", [1, 3])
+def test_group_of_members_with_and_without_node_pairs(small_cutoffs):
+    """The short range takes nodes in pairs where a member's grid has 2 (m + 2)
+    cells per axis, whatever the rest of the group: one or three of four members
+    can, and each gives its single context's result (float32 sums in another
+    order: 1e-6)."""
+    B = _B()
+    fs = [W.fourier_tangle(nfil=4, N_l=50 + k, seed=80 + k, amp=2 * math.pi / 48) for k in range(4)]
+    params = []
+    for k, f in enumerate(fs):
+        rc = (0.12 if k < small_cutoffs else 0.35) * 2 * math.pi
+        p = B.make_params(f.L, M=32, Q=2, w=8, alpha=3.5 / rc, rc=rc, precision=B.BS_MIXED)
+        p.flags |= B.BS_BATCH_STAGED
+        params.append(p)
+    s = torch.cuda.Stream()
+    bt, nodes, vel = _run_batch(B, params, fs, s)
+    off = bt.offsets
+    for i, (p, f) in enumerate(zip(params, fs)):
+        ref = _single(B, p, f)
+        assert (vel[off[i]:off[i + 1]] - ref).abs().max().item() < 1e-6 * ref.abs().max().item(), i
+    bt.close()
+
+
+@pytest.mark.parametrize("d", [1e-2, 1e-3])
+def test_staged_member_with_very_near_neighbours(d):
+    """Two opposite curves a distance d apart.  The staged node kernel and the
+    single one round the float32 offsets from the cell centre (edge h) from
+    float64 values that differ in their last places, so now and then by one
+    place of float32, at most 2^-24 h / 2 each for node and source: twice
+    2^-24 h / d of the near pair's velocity, at most the largest one (2.9e-7 / d
+    at h = 0.8 with the pair's two roundings), plus the 1e-6 of the sums'
+    order."""
+    B = _B()
+    th = 2 * math.pi * np.arange(64) / 64
+    X = np.stack([np.cos(th), np.sin(th), 0.3 * np.sin(2 * th)], 1) + 3.0
+    f = W._pack([X, (X + [0, 0, d])[::-1]], 2 * math.pi)
+    p = B.make_params(f.L, M=33, Q=2, w=8, precision=B.BS_MIXED)
+    p.flags |= B.BS_BATCH_STAGED
+    h = 2 * math.pi / math.floor(2 * 2 * math.pi / p.rc)
+    s = torch.cuda.Stream()
+    bt, nodes, vel = _run_batch(B, [p], [f], s)
+    got = vel.clone()
+    bt.close()
+    ref = _single(B, p, f)
+    assert (got - ref).abs().max().item() < (2 * 2.0 ** -23 * h / d + 1e-6) * ref.abs().max().item()
