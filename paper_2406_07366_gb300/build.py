@@ -23,8 +23,10 @@ LIB = os.path.join(LIBDIR, "libbsewald.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["bs_api.cu", "k_geometry.cu", "k_sort.cu", "k_short.cu", "k_long.cu", "k_fft.cu", "k_static_short.cu", "k_rk4.cu",
            "k_peak.cu"]
-# sources compiled a second time with a macro: the transform kernels, an object per precision
-VARIANTS = [("k_fft.cu", "k_fft_f64.o", ["-DBSW_FFT_DOUBLE"])]
+# sources compiled again with macros: the transform kernels, an object per precision for the single
+# contexts and one for the batches
+VARIANTS = [("k_fft.cu", "k_fft_f64.o", ["-DBSW_FFT_DOUBLE"]), ("k_fft.cu", "k_fft_b.o", ["-DBSW_FFT_BATCH"]),
+            ("k_fft.cu", "k_fft_f64_b.o", ["-DBSW_FFT_DOUBLE", "-DBSW_FFT_BATCH"])]
 
 
 def _nvcc() -> str:

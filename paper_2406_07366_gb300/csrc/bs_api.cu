@@ -2257,6 +2257,10 @@ int bs_batch_create(bs_batch** out, int nconf, const bs_params* params, void* st
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->gmain, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_side, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_group, cudaEventDisableTiming);
+    bool f64 = false, f32 = false;
+    for (int i = 0; i < nconf; ++i) (params[i].precision == BS_FP64 ? f64 : f32) = true;
+    if (e == cudaSuccess && f64) e = set_fft_constants_b<double>();
+    if (e == cudaSuccess && f32) e = set_fft_constants_b<float>();
     if (e != cudaSuccess) {
         const int rc = fail(BS_ERR_CUDA, "CUDA set-up failed: %s", cudaGetErrorString(e));
         bs_batch_destroy(b);

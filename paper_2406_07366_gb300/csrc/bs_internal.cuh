@@ -557,7 +557,9 @@ cudaError_t launch_spread_zfft(const SpZP& P, const Work& w, cudaStream_t s);
 template <typename T>
 size_t col_pt_bytes(int w);
 template <typename T>
-cudaError_t set_fft_constants();
+cudaError_t set_fft_constants();  // of the single contexts' kernels
+template <typename T>
+cudaError_t set_fft_constants_b();  // of the batches'
 cudaError_t set_short_tables();
 cudaError_t set_node_tables();
 // CTAs of the warp-per-node (or pair) short range.

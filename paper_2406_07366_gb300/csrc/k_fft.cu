@@ -3423,16 +3423,22 @@ cudaError_t launch_zfft_interp_b(int w, const BatchL& L, cudaStream_t s)
     template size_t fft_y_smem<T>(const FftYP&);                                       \
     template size_t fft_x_smem<T>(const FftXP&);                                       \
     template size_t zfft_interp_smem<T>(const SpZP&);
+// An object per precision (BSW_FFT_DOUBLE), for the single contexts and for
+// the batches (BSW_FFT_BATCH), which compile in parallel.  Each holds twiddles of
+// its own.
 #ifdef BSW_FFT_DOUBLE
-BSW_INST_B(double)
+using FftT = double;
 #else
-BSW_INST_B(float)
+using FftT = float;
+#endif
+#ifdef BSW_FFT_BATCH
+BSW_INST_B(FftT)
 #endif
 #undef BSW_INST_B
 
 // Writes the composite-radix twiddles into the current device's constant bank.
 template <typename T>
-cudaError_t set_fft_constants()
+static cudaError_t set_twiddles()
 {
     float2 hf[kTwCount];
     double2 hd[kTwCount];
@@ -3450,39 +3456,34 @@ cudaError_t set_fft_constants()
         return put_table(c_twd, hd, sizeof hd);
 }
 
-// One object per precision (the two compile in parallel): BSW_FFT_DOUBLE.
-#ifdef BSW_FFT_DOUBLE
-template bool make_tmap_y<double>(void*, const FftYP&, CUtensorMap*);
-template bool make_tmap_x<double>(void*, const FftXP&, CUtensorMap*);
-template cudaError_t launch_col_sort<double>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
-template cudaError_t launch_spread_zfft<double>(const SpZP&, const Work&, cudaStream_t);
-template cudaError_t launch_zfft_interp<double>(const SpZP&, const Work&, cudaStream_t);
-template cudaError_t launch_node_bin<double>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
-template cudaError_t launch_node_clear<double>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
-template size_t nd_rec_bytes<double>(int);
-template cudaError_t launch_fft_x_kspace<double>(const FftXP&, const Work&, bool, cudaStream_t, const CUtensorMap*);
-template cudaError_t launch_fft_y<double>(const FftYP&, const Work&, void*, int, cudaStream_t, const CUtensorMap*);
-template cudaError_t launch_fft_x_kspace<double>(const FftXP&, const Work&, bool, cudaStream_t);
-template cudaError_t launch_fft_z_c2r<double>(const FftZP&, const Work&, cudaStream_t, double*);
-template size_t col_pt_bytes<double>(int);
-template size_t spread_zfft_smem<double>(const SpZP&);
-template cudaError_t set_fft_constants<double>();
+#ifdef BSW_FFT_BATCH
+template <typename T>
+cudaError_t set_fft_constants_b()
+{
+    return set_twiddles<T>();
+}
+template cudaError_t set_fft_constants_b<FftT>();
 #else
-template bool make_tmap_y<float>(void*, const FftYP&, CUtensorMap*);
-template bool make_tmap_x<float>(void*, const FftXP&, CUtensorMap*);
-template cudaError_t launch_col_sort<float>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
-template cudaError_t launch_spread_zfft<float>(const SpZP&, const Work&, cudaStream_t);
-template cudaError_t launch_zfft_interp<float>(const SpZP&, const Work&, cudaStream_t);
-template cudaError_t launch_node_bin<float>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
-template cudaError_t launch_node_clear<float>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
-template size_t nd_rec_bytes<float>(int);
-template cudaError_t launch_fft_x_kspace<float>(const FftXP&, const Work&, bool, cudaStream_t, const CUtensorMap*);
-template cudaError_t launch_fft_y<float>(const FftYP&, const Work&, void*, int, cudaStream_t, const CUtensorMap*);
-template cudaError_t launch_fft_x_kspace<float>(const FftXP&, const Work&, bool, cudaStream_t);
-template cudaError_t launch_fft_z_c2r<float>(const FftZP&, const Work&, cudaStream_t, double*);
-template size_t col_pt_bytes<float>(int);
-template size_t spread_zfft_smem<float>(const SpZP&);
-template cudaError_t set_fft_constants<float>();
+template <typename T>
+cudaError_t set_fft_constants()
+{
+    return set_twiddles<T>();
+}
+template cudaError_t set_fft_constants<FftT>();
+template bool make_tmap_y<FftT>(void*, const FftYP&, CUtensorMap*);
+template bool make_tmap_x<FftT>(void*, const FftXP&, CUtensorMap*);
+template cudaError_t launch_col_sort<FftT>(const ColP&, const Work&, int, cudaStream_t, bool, bool);
+template cudaError_t launch_spread_zfft<FftT>(const SpZP&, const Work&, cudaStream_t);
+template cudaError_t launch_zfft_interp<FftT>(const SpZP&, const Work&, cudaStream_t);
+template cudaError_t launch_node_bin<FftT>(const ColP&, const InterpP&, const double*, const Work&, cudaStream_t);
+template cudaError_t launch_node_clear<FftT>(const ColP&, const InterpP&, const Work&, int, cudaStream_t);
+template size_t nd_rec_bytes<FftT>(int);
+template cudaError_t launch_fft_x_kspace<FftT>(const FftXP&, const Work&, bool, cudaStream_t, const CUtensorMap*);
+template cudaError_t launch_fft_y<FftT>(const FftYP&, const Work&, void*, int, cudaStream_t, const CUtensorMap*);
+template cudaError_t launch_fft_x_kspace<FftT>(const FftXP&, const Work&, bool, cudaStream_t);
+template cudaError_t launch_fft_z_c2r<FftT>(const FftZP&, const Work&, cudaStream_t, double*);
+template size_t col_pt_bytes<FftT>(int);
+template size_t spread_zfft_smem<FftT>(const SpZP&);
 #endif
 
 }  // namespace bsw
