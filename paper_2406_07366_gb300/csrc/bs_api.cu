@@ -1916,16 +1916,16 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
         }
         add(D, kThreads, 0);
     }
-    // short range: the members that take their nodes in pairs, then (at the end
-    // of the list) those that take them one by one.  Each member's own grid
-    // decides, as in its single context, not the company that it is in.
-    auto short_stage = [&](bool pairs) {
+    // short range: the members of one variant (mixed: nodes in pairs), then (at
+    // the end of the list) those of the other.  Each member's own grid decides,
+    // as in its single context, not the company that it is in.
+    auto short_stage = [&](bool v) {
         std::vector<ShortD<T>> D;
         for (size_t m = 0; m < nm; ++m) {
             const Work& w = mem[m]->w;
             ShortD<T> e;
             fill_short(mem[m], false, e.P);
-            if (short_can_pair(e.P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED) != pairs) continue;
+            if (short_variant(e.P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED) != v) continue;
             e.tgt = (const SrTgt<T>*)w.tgt;
             e.prev = w.prev;
             e.start = w.cell_cnt;
@@ -1933,10 +1933,10 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
             e.vsr = w.vsr;
             e.psr = w.psr;
             D.push_back(e);
-            blk.push_back(short_blocks(e.P, pairs));
+            blk.push_back(short_blocks(e.P, v && sizeof(T) == 4));
         }
         add(D, 256, 0);
-        st.back().kind = pairs;
+        st.back().kind = v;
     };
     short_stage(true);                                                                     // 7 short range
     auto col_cnt = [](bs_ctx* c) { return c->w.col_cnt; };

@@ -562,8 +562,9 @@ template <typename T>
 cudaError_t set_fft_constants_b();  // of the batches'
 cudaError_t set_short_tables();
 cudaError_t set_node_tables();
-// CTAs of the warp-per-node (or pair) short range.
-bool short_can_pair(const ShortP& P, int precision);
+// Variant of the warp-per-node short range: float32 whether the grid lets a
+// warp take two nodes, float64 whether alpha r_c <= 4; and its CTAs.
+bool short_variant(const ShortP& P, int precision);
 int short_blocks(const ShortP& P, bool pairs);
 
 // Threads per CTA of a kernel with a thread per item: whole warps spread over

@@ -72,38 +72,52 @@ __device__ __forceinline__ double erfc_e<double>(double x, double) { return erfc
 //   1/r from the hardware's approximate reciprocal square root and one step
 //   of Householder's third-order iteration (y += y e (1/2 + 3 e / 8), e = 1 -
 //   r2 y^2; the seed's 2^-20 becomes below 2^-58), 5 operations;
-//   g^(n)(x) and erfc(x) from tables of degree-11 polynomials on intervals of
-//   width 1/16 centred at i / 16, i = 0..128, written from
-//   Chebyshev interpolation of the functions in extended precision
-//   (set_short_tables): 11 operations each.  Relative to the function itself
-//   the value is within 2.1e-16 up to x = 7 and 3.8e-16 up to 8, roundings
-//   included (degree 8: 3e-15 at x = 3.5, 2.7e-11 at 8; the functions fall by
-//   e^-(x/8) and more over an interval, and their high derivatives grow like
-//   powers of 2 x).
-// Beyond x = 8 the library functions are called.
-constexpr int kSgN = 129, kSgDeg = 11, kSgStride = 132;
-constexpr int kSgTable = (kSgDeg + 1) * kSgStride;  // doubles per function, degree-major
-__device__ double g_sg_tab[2 * kSgTable];           // g^(n), then erfc
+//   g^(n)(x) and erfc(x) from tables of polynomials in x, written from Chebyshev
+//   interpolation of the functions in extended precision (set_short_tables).
+//   Up to alpha r_c = 4 degree 8 on intervals of width 1/32 centred at i / 32, i
+//   = 0..128; beyond, degree 11 on intervals of 1/16, up to x = 8: 8 or 11
+//   operations each.  Relative to the function itself, roundings included, both
+//   are within 2.4e-16 (4e-16 at x = 8).  The high derivatives grow like powers of
+//   2 x: degree 8 on intervals of 1/16 is 3e-15 off at x = 3.5 and 2.7e-11 at 8.
+//   (2560 nodes, a fifth of the box as the cut-off: 511 us with degree 8, 534
+//   with 11.)
+// Beyond the tables the library functions are called.
+constexpr int kSgN = 129, kSgStride = 132;
+template <bool LO> struct Sg {
+    static constexpr int deg = LO ? 8 : 11, scale = LO ? 32 : 16;
+    static constexpr int table = (deg + 1) * kSgStride;  // doubles per function, degree-major
+};
+__device__ double g_sg_lo[2 * Sg<true>::table], g_sg_hi[2 * Sg<false>::table];  // g^(n), then erfc
 
 // Value at the table argument: t in [-1/2, 1/2], interval i.
+template <bool LO>
 __device__ __forceinline__ double sg_poly(const double* __restrict__ tab, int i, double t)
 {
-    double v = tab[kSgDeg * kSgStride + i];
+    double v = tab[Sg<LO>::deg * kSgStride + i];
 #pragma unroll
-    for (int k = kSgDeg - 1; k >= 0; --k) v = fma(v, t, tab[k * kSgStride + i]);
+    for (int k = Sg<LO>::deg - 1; k >= 0; --k) v = fma(v, t, tab[k * kSgStride + i]);
     return v;
 }
 
+// Shared memory of the staged tables: erfc's only with the streamfunction (the
+// spread's large CTAs share the SMs with this kernel).
+template <typename T, bool LO>
+__host__ __device__ constexpr size_t sg_bytes(bool want_psi)
+{
+    return sizeof(T) == 8 ? (want_psi ? 2 : 1) * Sg<LO>::table * sizeof(double) : 0;
+}
+
 // Copies the tables into shared memory (float64; the whole block).
-template <typename T>
+template <typename T, bool LO>
 __device__ __forceinline__ const double* sg_stage(int want_psi)
 {
     if constexpr (sizeof(T) == 8) {
-        __shared__ double s_tab[2 * kSgTable];
-        const int n = want_psi ? 2 * kSgTable : kSgTable;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) s_tab[i] = g_sg_tab[i];
+        extern __shared__ __align__(16) double s_sg[];
+        const double* src = LO ? g_sg_lo : g_sg_hi;
+        const int n = want_psi ? 2 * Sg<LO>::table : Sg<LO>::table;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) s_sg[i] = src[i];
         __syncthreads();
-        return s_tab;
+        return s_sg;
     } else {
         return nullptr;
     }
@@ -165,7 +179,7 @@ template <typename T> struct ShortRows {
 // one OR-reduction per 32 candidates (which rows start in the window) and a
 // population count, and reads the row from the table.  The per-lane partial
 // sums are reduced at the end.
-template <typename T>
+template <typename T, bool LO>
 __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __restrict__ tgt,
                                              const int* __restrict__ prev, const int* __restrict__ start,
                                              const SrRec<T>* __restrict__ src, double* __restrict__ vsr,
@@ -184,7 +198,7 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
     const T L0 = in_t<T>(P.L[0], P.Lf[0]), L1 = in_t<T>(P.L[1], P.Lf[1]), L2 = in_t<T>(P.L[2], P.Lf[2]);
     const T rc2 = in_t<T>(P.rc2, P.rc2f);
     const T alpha = in_t<T>(P.alpha, P.alphaf);
-    const double alpha16 = 16.0 * P.alpha;  // float64: the tables' argument
+    const double alphas = Sg<LO>::scale * P.alpha;  // float64: the tables' argument
     const T two_over_sqrtpi = (T)1.12837916709551257390;
     const int m = P.m;
     // neighbour ranges per axis: all cells when 2m+1 >= n
@@ -318,15 +332,15 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
             T ir, g, ec = (T)0;
             if constexpr (sizeof(T) == 8) {
                 ir = rsqrt_h(r2);
-                const double xs = alpha16 * (r2 * ir);  // 16 x
+                const double xs = alphas * (r2 * ir);  // scale x
                 if (xs < 128.0) {
                     const double mi = xs + 4503599627370496.0;  // 2^52: the low word is rint(xs)
                     const double tt = xs - (mi - 4503599627370496.0);
                     const int it = __double2loint(mi);
-                    g = sg_poly(tab, it, tt);
-                    if (P.want_psi) ec = sg_poly(tab + kSgTable, it, tt);
+                    g = sg_poly<LO>(tab, it, tt);
+                    if (P.want_psi) ec = sg_poly<LO>(tab + Sg<LO>::table, it, tt);
                 } else {
-                    const double x = 0.0625 * xs;
+                    const double x = xs * (1.0 / Sg<LO>::scale);
                     ec = erfc(x);
                     g = ec + two_over_sqrtpi * x * exp(-x * x);
                 }
@@ -587,11 +601,12 @@ __host__ __device__ __forceinline__ bool short_pairs(const ShortP& P)
     return sizeof(T) == 4 && P.nc[0] >= need && P.nc[1] >= need && P.nc[2] >= need;
 }
 
-// One warp of the kernels below: a node, or with PAIR a pair of nodes where
+// One warp of the kernels below, in the variant V that short_variant gives:
+// float64 with the tables up to alpha r = 4 or 8; float32 a node, or a pair of nodes where
 // the grid allows (pairs whose cells are further apart one after the other).
 // The two are separate kernels: in one of 91 registers the small grids, which
 // cannot pair, took 4 % longer over a batch.
-template <typename T, bool PAIR>
+template <typename T, bool V>
 __device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __restrict__ tgt,
                                              const int* __restrict__ prev, const int* __restrict__ start,
                                              const SrRec<T>* __restrict__ src, double* __restrict__ vsr,
@@ -599,7 +614,7 @@ __device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __
                                              ShortRows<T>& rows)
 {
     int j = w, je = w + 1;
-    if constexpr (PAIR) {
+    if constexpr (sizeof(T) == 4 && V) {
         if (short_pairs<T>(P)) {
             j = 2 * w;
             je = j + 2;
@@ -616,41 +631,44 @@ __device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __
             }
         }
     }
-    for (; j < je && j < P.N; ++j) k_short_body<T>(P, tgt, prev, start, src, vsr, psr, j, tab, rows);
+    for (; j < je && j < P.N; ++j) k_short_body<T, sizeof(T) == 8 && V>(P, tgt, prev, start, src, vsr, psr, j, tab, rows);
 }
 
 // Four CTAs per SM in float32 (64 registers): with five (48) the one-node walk
 // at the minimum image is 2 % slower (2e4 nodes, cut-off at half the box: 3.65
 // and 3.73 ms).  The batched form of that walk hides more latency with five
 // (256 members of 250 to 650 nodes: 1729 against 1750 us).
-template <typename T, bool PAIR>
+template <typename T, bool V>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short(ShortP P, const SrTgt<T>* __restrict__ tgt, const int* __restrict__ prev,
                                                const int* __restrict__ start, const SrRec<T>* __restrict__ src,
                                                double* __restrict__ vsr, double* __restrict__ psr)
 {
     __shared__ ShortRows<T> rows;
-    const double* tab = sg_stage<T>(P.want_psi);
+    const double* tab = sg_stage<T, V>(P.want_psi);
     const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if constexpr (sizeof(T) == 8) {  // several groups of nodes per CTA: the tables are staged once
         for (int b = blockIdx.x; b * nw < P.N; b += gridDim.x)
-            k_short_warp<T, PAIR>(P, tgt, prev, start, src, vsr, psr, b * nw + wid, tab, rows);
+            k_short_warp<T, V>(P, tgt, prev, start, src, vsr, psr, b * nw + wid, tab, rows);
     } else {
-        k_short_warp<T, PAIR>(P, tgt, prev, start, src, vsr, psr, blockIdx.x * kShortWarps + wid, tab, rows);
+        k_short_warp<T, V>(P, tgt, prev, start, src, vsr, psr, blockIdx.x * kShortWarps + wid, tab, rows);
     }
 }
 
-template <typename T, bool PAIR>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (PAIR ? 4 : 5) : 3) k_short_b(const ShortD<T>* __restrict__ d, const int* __restrict__ bs, int n)
+template <typename T, bool V>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (V ? 4 : 5) : 3) k_short_b(const ShortD<T>* __restrict__ d, const int* __restrict__ bs, int n)
 {
     __shared__ ShortRows<T> rows;
     int bid, nb;
     const ShortD<T>& a = d[batch_member(bs, n, bid, nb)];
-    const double* tab = sg_stage<T>(a.P.want_psi);
-    k_short_warp<T, PAIR>(a.P, a.tgt, a.prev, a.start, a.src, a.vsr, a.psr,
+    const double* tab = sg_stage<T, V>(a.P.want_psi);
+    k_short_warp<T, V>(a.P, a.tgt, a.prev, a.start, a.src, a.vsr, a.psr,
                           bid * kShortWarps + (int)(threadIdx.x >> 5), tab, rows);
 }
 
-bool short_can_pair(const ShortP& P, int precision) { return precision == BS_MIXED && short_pairs<float>(P); }
+bool short_variant(const ShortP& P, int precision)
+{
+    return precision == BS_MIXED ? short_pairs<float>(P) : P.alpha * P.alpha * P.rc2 <= 16.0;
+}
 
 int short_blocks(const ShortP& P, bool pairs)
 {
@@ -1021,19 +1039,16 @@ cudaError_t launch_short(const ShortP& P, const Work& w, cudaStream_t s)
         if (sizeof(T) == 8)
             while (nw > 1 && P.N < 152 * nw) nw /= 2;
         const int tb = 32 * nw;
-        const bool pairs = short_can_pair(P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED);
-        const long long blocks = sizeof(T) == 8 ? (P.N + nw - 1LL) / nw : short_blocks(P, pairs);
+        const bool v = short_variant(P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED);
+        const long long blocks = sizeof(T) == 8 ? (P.N + nw - 1LL) / nw : short_blocks(P, v);
         // float64: at most 16 CTAs per SM, each on several groups of nodes
         const unsigned g = (unsigned)(sizeof(T) == 8 && blocks > 16 * 152 ? 16 * 152 : blocks);
-        if constexpr (sizeof(T) == 4) {
-            if (pairs) {
-                k_short<T, true><<<g, tb, 0, s>>>(P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt,
-                                                  (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
-                return cudaGetLastError();
-            }
-        }
-        k_short<T, false><<<g, tb, 0, s>>>(P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt,
-                                           (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
+        if (v)
+            k_short<T, true><<<g, tb, sg_bytes<T, true>(P.want_psi), s>>>(
+                P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt, (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
+        else
+            k_short<T, false><<<g, tb, sg_bytes<T, false>(P.want_psi), s>>>(
+                P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt, (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
         return cudaGetLastError();
     }
     // nodes by target block: count, scan, scatter
@@ -1056,13 +1071,13 @@ template <typename T>
 cudaError_t launch_short_b(const BatchL& L, cudaStream_t s)
 {
     if (L.total <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4) {
-        if (L.kind) {
-            k_short_b<T, true><<<L.total, 32 * kShortWarps, 0, s>>>((const ShortD<T>*)L.desc, L.bstart, L.n);
-            return cudaGetLastError();
-        }
-    }
-    k_short_b<T, false><<<L.total, 32 * kShortWarps, 0, s>>>((const ShortD<T>*)L.desc, L.bstart, L.n);
+    // (batches give no streamfunction)
+    if (L.kind)
+        k_short_b<T, true><<<L.total, 32 * kShortWarps, sg_bytes<T, true>(false), s>>>((const ShortD<T>*)L.desc,
+                                                                                      L.bstart, L.n);
+    else
+        k_short_b<T, false><<<L.total, 32 * kShortWarps, sg_bytes<T, false>(false), s>>>((const ShortD<T>*)L.desc,
+                                                                                        L.bstart, L.n);
     return cudaGetLastError();
 }
 
@@ -1081,17 +1096,20 @@ static long double sg_near(long double x)
 cudaError_t set_short_tables()
 {
     struct Tables {
-        double v[2 * kSgTable] = {};
+        double lo[2 * Sg<true>::table] = {}, hi[2 * Sg<false>::table] = {};
         Tables()
         {
             for (int i = 0; i < kSgN; ++i) {
-                cheb_fit(sg_near, i / 16.0L, 1 / 16.0L, kSgDeg, v + i, kSgStride);
-                cheb_fit(sg_erfc, i / 16.0L, 1 / 16.0L, kSgDeg, v + kSgTable + i, kSgStride);
+                cheb_fit(sg_near, i / 32.0L, 1 / 32.0L, Sg<true>::deg, lo + i, kSgStride);
+                cheb_fit(sg_erfc, i / 32.0L, 1 / 32.0L, Sg<true>::deg, lo + Sg<true>::table + i, kSgStride);
+                cheb_fit(sg_near, i / 16.0L, 1 / 16.0L, Sg<false>::deg, hi + i, kSgStride);
+                cheb_fit(sg_erfc, i / 16.0L, 1 / 16.0L, Sg<false>::deg, hi + Sg<false>::table + i, kSgStride);
             }
         }
     };
     static const Tables tab;
-    return put_table(g_sg_tab, tab.v, sizeof tab.v);
+    const cudaError_t e = put_table(g_sg_lo, tab.lo, sizeof tab.lo);
+    return e == cudaSuccess ? put_table(g_sg_hi, tab.hi, sizeof tab.hi) : e;
 }
 
 // The float32 complementary error function as the short-range kernels take
