@@ -170,3 +170,26 @@ def test_compiled_transforms_where_the_modes_pass_a_third(M):
     ref = got[2]
     for x, r in ((got[0][0], ref[0]), (got[1][0], ref[0]), (got[1][1], ref[1])):
         assert float((x - r).abs().max()) < 3e-6 * float(r.abs().max())
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("M", [35, 36, 39, 40])
+def test_y_chunks_of_32_modes_with_tensor_copies(M, prec):
+    """18 or 20 modes along z: the y pass takes them in one chunk of 32 and, the
+    count being even, moves its rows with tensor copies.  Long-range velocity
+    and psi against full cuFFT transforms, bounds of the boundary-pass test."""
+    B, tol = _B(), 2e-6 if prec == "mixed" else 1e-12
+    f = W.ellipses(3, 40, seed=M)
+    nodes = torch.from_numpy(f.nodes).cuda()
+    got = []
+    for flags in (0, B.BS_WANT_PSI, B.BS_WANT_PSI | B.BS_FFT_CUFFT):
+        p = B.make_params(f.L, M=M, Q=2, w=8, flags=flags, alpha=1.2, rc=3.0,
+                          precision=B.BS_MIXED if prec == "mixed" else B.BS_FP64)
+        bs = B.BiotSavart(p, f.offsets, f.closing)
+        v = bs.parts(nodes, want_psi=bool(flags))
+        got.append([x[2].clone() for x in (v if flags else (v,))])
+        torch.cuda.synchronize()
+        bs.close()
+    ref = got[2]
+    for x, r in ((got[0][0], ref[0]), (got[1][0], ref[0]), (got[1][1], ref[1])):
+        assert float((x - r).abs().max()) < tol * float(r.abs().max())
