@@ -186,30 +186,23 @@ double kb_host(double z, double zeta)
 }
 
 // The kernel on the grid spacing of support point t < w / 2 (Appendix A, Eq.
-// kaiser_bessel_bw), as a polynomial in x = f - 1/2: the interpolation
-// polynomial at the Chebyshev points of [-1/2, 1/2], in extended precision
-// (divided differences).  The kernel is sinh(zeta s) / s with s^2 = 1 - z^2,
-// an entire function of z, and zeta 2 / w < 0.995 pi whatever sigma, so the
-// interpolation error at degree 22 is below 2^-53 of the largest value on the
-// spacing.  Point w - 1 - t takes the same polynomial at -x.  The
-// coefficients go out even powers first, then odd ones.
+// kaiser_bessel_bw), as a polynomial in x = f - 1/2 (cheb_fit).  The kernel is
+// sinh(zeta s) / s with s^2 = 1 - z^2, an entire function of z, in grid spacings of
+// type zeta 2 / w = 1.99 pi (1 - 1 / (2 sigma)) < 1.99 pi, so the interpolation
+// error at degree 22 is below 2^-53 of the largest value on the spacing whatever
+// sigma.  Point w - 1 - t takes the same polynomial at -x.  The coefficients go out
+// even powers first, then odd ones.
 void kb_poly(double zeta, int w, int t, double* out)
 {
-    constexpr int n = kKbDeg + 1;
-    long double x[n], c[n], p[n] = {};
     const long double zl = zeta, scale = 2.0L * expl(-zl) / (1.0L - expl(-2.0L * zl));
-    for (int k = 0; k < n; ++k) {
-        x[k] = 0.5L * cosl(3.14159265358979323846264338327950288L * (k + 0.5L) / n);
-        const long double z = (x[k] + 0.5L + (w / 2 - 1 - t)) * 2.0L / w, sq = sqrtl(1.0L - z * z);
-        c[k] = scale * sinhl(zl * sq) / sq;
-    }
-    for (int j = 1; j < n; ++j)
-        for (int k = n - 1; k >= j; --k) c[k] = (c[k] - c[k - 1]) / (x[k] - x[k - j]);
-    for (int k = n - 1; k >= 0; --k) {  // p <- p (x - x_k) + c_k
-        for (int j = n - 1; j > 0; --j) p[j] = p[j - 1] - x[k] * p[j];
-        p[0] = c[k] - x[k] * p[0];
-    }
-    for (int j = 0; j < n; ++j) out[(j & 1) ? (kKbDeg / 2 + 1) + j / 2 : j / 2] = (double)p[j];
+    double p[kKbDeg + 1];
+    bsw::cheb_fit(
+        [&](long double x) {
+            const long double z = (x + 0.5L + (w / 2 - 1 - t)) * 2.0L / w, sq = sqrtl(1.0L - z * z);
+            return scale * sinhl(zl * sq) / sq;
+        },
+        0.0L, 1.0L, kKbDeg, p, 1);
+    for (int j = 0; j <= kKbDeg; ++j) out[(j & 1) ? (kKbDeg / 2 + 1) + j / 2 : j / 2] = p[j];
 }
 
 // F(m) = (w/2) int_{-1}^{1} psi(z) cos(kappa z) dz, kappa = pi m w / n_g: the
@@ -409,7 +402,7 @@ int derive(const bs_params* p, Derived* d)
 
 }  // namespace
 
-void bsw::cheb_fit(long double (*f)(long double), long double c, long double w, int deg, double* out, int stride)
+void bsw::cheb_fit(const std::function<long double(long double)>& f, long double c, long double w, int deg, double* out, int stride)
 {
     long double t[32], v[32], p[32] = {};
     const int n = deg + 1;

@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <atomic>
+#include <functional>
 #include <mutex>
 
 #include "bsewald.h"
@@ -172,45 +173,6 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
 }
 __device__ __forceinline__ unsigned long long dup2(float a) { return pk2(a, a); }
 
-// erfc(x) exp(x^2), x >= 0, in float32: a least-squares fit (weighted for
-// relative error, degree 10 in t = 1 / (1 + x / 2), on [0, 8]) written by
-// gen_erfcx_fit.py; 3.4e-7 relative error evaluated in float32.  Beyond
-// x = 8 the factor exp(-x^2) it multiplies is below 2e-28.
-__device__ __forceinline__ float erfcx_f(float x)
-{
-    constexpr float c[11] = { 1.441113045e-05f, 2.817091850e-01f, 2.866406861e-01f, 2.157398867e-01f,
-                              3.128657818e-01f, -3.176314365e-01f, 7.893466267e-01f, -1.078447950e+00f,
-                              7.163310796e-01f, -2.393311398e-01f, 3.276285984e-02f };
-    const float t = __frcp_rn(1.0f + 0.5f * x);  // the correctly rounded 1 / (1 + x/2)
-    float v = c[10];
-#pragma unroll
-    for (int k = 9; k >= 0; --k) v = fmaf(v, t, c[k]);
-    return v;
-}
-
-// erfcx_f of two arguments; 1 / (1 + x/2) from the hardware's approximation and
-// one Newton step, which gives the correctly rounded value for every float32
-// 1 + x/2 in [1, 5]: the same results as erfcx_f.
-__device__ __forceinline__ unsigned long long erfcx_2(unsigned long long x)
-{
-    using U = unsigned long long;
-    constexpr float c[11] = { 1.441113045e-05f, 2.817091850e-01f, 2.866406861e-01f, 2.157398867e-01f,
-                              3.128657818e-01f, -3.176314365e-01f, 7.893466267e-01f, -1.078447950e+00f,
-                              7.163310796e-01f, -2.393311398e-01f, 3.276285984e-02f };
-    const U d = fma2(dup2(0.5f), x, dup2(1.0f));
-    const float2 df = upk2(d);
-    float t0, t1;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(df.x));
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(df.y));
-    const U y = pk2(t0, t1);
-    const U e = fma2(pk2(-df.x, -df.y), y, dup2(1.0f));
-    const U t = fma2(y, e, y);
-    U v = dup2(c[10]);
-#pragma unroll
-    for (int k = 9; k >= 0; --k) v = fma2(v, t, dup2(c[k]));
-    return v;
-}
-
 // x wrapped into [0, L) (iL = 1/L); non-finite input maps to 0 and raises the
 // flag.  The comparisons are made on the bits (float64 comparisons share the
 // slow pipe).
@@ -229,7 +191,7 @@ __device__ __forceinline__ double wrap_box(double x, double L, double iL, bool& 
 // Monomial coefficients in t (stride apart) of the degree-deg polynomial
 // through f(c + w t) at the Chebyshev points t of [-1/2, 1/2] (divided
 // differences, extended precision; host, deg < 32).
-void cheb_fit(long double (*f)(long double), long double c, long double w, int deg, double* out, int stride);
+void cheb_fit(const std::function<long double(long double)>& f, long double c, long double w, int deg, double* out, int stride);
 
 // Parameters of the geometry / node kernel.
 struct GeomP {

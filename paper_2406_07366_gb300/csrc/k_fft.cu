@@ -2416,14 +2416,8 @@ __device__ __forceinline__ void k_fft_x_tma(const FftXP& P, typename Cx<T>::t* _
     }
 }
 
-// Threads of an x-pass CTA.
-template <typename T>
-constexpr int x_threads_max()
-{
-    return z_threads_max<T>();
-}
 template <typename T, int RM>
-__global__ void __launch_bounds__(x_threads_max<T>(), 2) k_fft_x_kspace(FftXP P, typename Cx<T>::t* __restrict__ F2,
+__global__ void __launch_bounds__(z_threads_max<T>(), 2) k_fft_x_kspace(FftXP P, typename Cx<T>::t* __restrict__ F2,
                                                            typename Cx<T>::t* __restrict__ F2psi,
                                                            const typename Cx<T>::t* __restrict__ tw0,
                                                            const T* __restrict__ tab0, const T* __restrict__ tab1,
@@ -3160,7 +3154,7 @@ struct FftXLaunch {
         const T* tab0 = (const T*)w.ktab + (P.single_decon ? ntab : 0);
         const T* tab1 = tab0 + (P.K[0] + 1);
         const T* tab2 = tab1 + (P.K[1] + 1);
-        const int nt = P.nthreads > 0 ? std::min(P.nthreads, x_threads_max<T>()) : kThreads;
+        const int nt = P.nthreads > 0 ? std::min(P.nthreads, z_threads_max<T>()) : kThreads;
         k_fft_x_kspace<T, RM><<<(2 * P.K[1] + 1) * nch, nt, sm, s>>>(
             Q, (C*)w.f2, want_psi ? (C*)w.f2psi : nullptr, (const C*)w.tw, tab0, tab1, tab2, map, w.status);
         return cudaGetLastError();
@@ -3253,7 +3247,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_fft_y_b(co
 }
 
 template <typename T, int RM>
-__global__ void __launch_bounds__(x_threads_max<T>(), 2) k_fft_x_kspace_b(const FftXD<T>* __restrict__ d,
+__global__ void __launch_bounds__(z_threads_max<T>(), 2) k_fft_x_kspace_b(const FftXD<T>* __restrict__ d,
                                                                         const int* __restrict__ bs, int n)
 {
     using C = typename Cx<T>::t;
@@ -3366,7 +3360,7 @@ cudaError_t launch_fft_x_kspace_b(const BatchL& L, cudaStream_t s)
     if (L.total <= 0) return cudaSuccess;
     cudaError_t e = allow_smem<k_fft_x_kspace_b<T, 8>>();
     if (e != cudaSuccess) return e;
-    const int nt = std::min(L.threads, x_threads_max<T>());
+    const int nt = std::min(L.threads, z_threads_max<T>());
     k_fft_x_kspace_b<T, 8><<<L.total, nt, L.smem, s>>>((const FftXD<T>*)L.desc, L.bstart, L.n);
     return cudaGetLastError();
 }

@@ -1042,7 +1042,6 @@ __device__ __forceinline__ void q_node(const double* __restrict__ t, int m, cons
 constexpr size_t kQuinticRow = 32 * sizeof(double);  // shared memory per node: h, 3 increments, 2 x 14 of the solver
 constexpr size_t kQuinticSmemMax = 200 * 1024;       // filaments up to 800 nodes
 __device__ const double* q_solve_cta(int n, const double* __restrict__ sm);
-__device__ __forceinline__ double block_sum(double v);
 
 // The same line integral on a quintic curve (order 6): f_j = psi_j .
 // sdot(tau_j), with sdot = D_j + n_l L / T the first derivative of the

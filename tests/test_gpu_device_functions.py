@@ -1,5 +1,5 @@
 """The kernels' own elementary functions on the device (``-m gpu``), compiled
-from the library's header into a probe: the packed float32 erfcx of the paired
+from the library's source into a probe: the packed float32 erfcx of the paired
 short range (``test_gpu_erfc.py`` takes the scalar one) and the float64
 reciprocal square root."""
 import ctypes
@@ -13,7 +13,14 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 PROBE = r"""
-#include "bs_internal.cuh"
+#include "k_short.cu"
+
+// what else k_short.cu calls, never reached here
+namespace bsw {
+cudaError_t scan_exclusive(int*, int, int*, cudaStream_t, int*) { return cudaErrorNotSupported; }
+void set_last_error(const char*) {}
+void cheb_fit(const std::function<long double(long double)>&, long double, long double, int, double*, int) {}
+}
 using namespace bsw;
 
 // out[0..n): erfcx_f; out[n..2n): erfcx_2 of neighbouring arguments, the last of an odd count with itself
