@@ -173,10 +173,10 @@ def test_compiled_transforms_where_the_modes_pass_a_third(M):
 
 
 @pytest.mark.parametrize("prec", ["mixed", "fp64"])
-@pytest.mark.parametrize("M", [35, 36, 39, 40])
+@pytest.mark.parametrize("M", [35, 36, 39, 40, 41, 44, 47, 48])
 def test_y_chunks_of_32_modes_with_tensor_copies(M, prec):
-    """18 or 20 modes along z: the y pass takes them in one chunk of 32 and, the
-    count being even, moves its rows with tensor copies.  Long-range velocity
+    """18 to 24 modes along z: the y pass takes them in one chunk of 32 and moves
+    its rows with tensor copies where the count is even.  Long-range velocity
     and psi against full cuFFT transforms, bounds of the boundary-pass test."""
     B, tol = _B(), 2e-6 if prec == "mixed" else 1e-12
     f = W.ellipses(3, 40, seed=M)
