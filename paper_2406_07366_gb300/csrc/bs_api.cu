@@ -804,12 +804,6 @@ void fill_short(const bs_ctx* c, bool want_psi, ShortP& S)
     S.kernel = (p.flags & BS_SHORT_TILED) ? 1 : ((p.flags & BS_SHORT_PER_NODE) ? 2 : 0);
     S.rc2 = p.rc * p.rc;
     S.alpha = p.alpha;
-    for (int k = 0; k < 3; ++k) {
-        S.hcf[k] = (float)S.hc[k];
-        S.Lf[k] = (float)S.L[k];
-    }
-    S.rc2f = (float)S.rc2;
-    S.alphaf = (float)S.alpha;
     S.pref = p.kappa / (4.0 * kPi);
     S.want_psi = want_psi ? 1 : 0;
 }
@@ -1922,6 +1916,7 @@ int batch_build(bs_batch* b, const double* nodes, double* vel)
             ShortD<T> e;
             fill_short(mem[m], false, e.P);
             if (short_variant(e.P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED) != v) continue;
+            e.F = short_f(e.P);
             e.tgt = (const SrTgt<T>*)w.tgt;
             e.prev = w.prev;
             e.start = w.cell_cnt;

@@ -229,11 +229,23 @@ struct ShortP {
     int want_psi;
     int nb[3];          // target blocks of m x m x m cells per axis, ceil(nc / m)
     int kernel;         // 0: by size, 1: tiled, 2: warp per node (BS_SHORT_TILED / BS_SHORT_PER_NODE)
-    // hc, L, rc2 and alpha rounded to float32 for the mixed form: a conversion
-    // in the kernel shares the slow float64 pipe, and where registers are short
-    // the compiler repeats it for every candidate
-    float hcf[3], Lf[3], rc2f, alphaf;
 };
+
+// Its lengths, squared radius and splitting parameter in float32, for the mixed
+// form: a conversion in the kernel shares the slow float64 pipe, and where
+// registers are short the compiler repeats it for every candidate.  (A struct of
+// its own: with ShortP above 128 bytes the compiler reads its members again in
+// the loops, 5 % more instructions in float64.)
+struct ShortF {
+    float hc[3], L[3], rc2, alpha;
+};
+inline ShortF short_f(const ShortP& P)
+{
+    return { { (float)P.hc[0], (float)P.hc[1], (float)P.hc[2] },
+             { (float)P.L[0], (float)P.L[1], (float)P.L[2] },
+             (float)P.rc2,
+             (float)P.alpha };
+}
 
 // The tiled short range takes cells per cut-off up to this (larger m: the
 // warp-per-node kernel).
@@ -679,6 +691,7 @@ template <typename T> struct NodesD {
 };
 template <typename T> struct ShortD {
     ShortP P;
+    ShortF F;
     const SrTgt<T>* tgt;
     const int* prev;
     const int* start;

@@ -118,7 +118,7 @@ __device__ __forceinline__ double erfc_e<double>(double x, double) { return erfc
 //   operations each.  Relative to the function itself, roundings included, both
 //   are within 2.4e-16 (4e-16 at x = 8).  The high derivatives grow like powers of
 //   2 x: degree 8 on intervals of 1/16 is 3e-15 off at x = 3.5 and 2.7e-11 at 8.
-//   (2560 nodes, a fifth of the box as the cut-off: 511 us with degree 8, 534
+//   (2560 nodes, a fifth of the box as the cut-off: 512 us with degree 8, 534
 //   with 11.)
 // Beyond the tables the library functions are called.
 constexpr int kSgN = 129, kSgStride = 132;
@@ -187,7 +187,7 @@ __device__ __forceinline__ void st_pair(T rx, T ry, T rz, T r2, const T* q, T al
     }
 }
 
-// A length, squared radius or splitting parameter of ShortP in the kernels' precision.
+// A length, squared radius or splitting parameter in the kernels' precision.
 template <typename T>
 __device__ __forceinline__ T in_t(double d, float f)
 {
@@ -219,7 +219,7 @@ template <typename T> struct ShortRows {
 // population count, and reads the row from the table.  The per-lane partial
 // sums are reduced at the end.
 template <typename T, bool LO>
-__device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __restrict__ tgt,
+__device__ __forceinline__ void k_short_body(const ShortP& P, const ShortF& F, const SrTgt<T>* __restrict__ tgt,
                                              const int* __restrict__ prev, const int* __restrict__ start,
                                              const SrRec<T>* __restrict__ src, double* __restrict__ vsr,
                                              double* __restrict__ psr, int j, const double* __restrict__ tab,
@@ -233,10 +233,10 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
     const int cx = t.cell % nc0;
     const int cy = (t.cell / nc0) % nc1;
     const int cz = t.cell / (nc0 * nc1);
-    const T h0 = in_t<T>(P.hc[0], P.hcf[0]), h1 = in_t<T>(P.hc[1], P.hcf[1]), h2 = in_t<T>(P.hc[2], P.hcf[2]);
-    const T L0 = in_t<T>(P.L[0], P.Lf[0]), L1 = in_t<T>(P.L[1], P.Lf[1]), L2 = in_t<T>(P.L[2], P.Lf[2]);
-    const T rc2 = in_t<T>(P.rc2, P.rc2f);
-    const T alpha = in_t<T>(P.alpha, P.alphaf);
+    const T h0 = in_t<T>(P.hc[0], F.hc[0]), h1 = in_t<T>(P.hc[1], F.hc[1]), h2 = in_t<T>(P.hc[2], F.hc[2]);
+    const T L0 = in_t<T>(P.L[0], F.L[0]), L1 = in_t<T>(P.L[1], F.L[1]), L2 = in_t<T>(P.L[2], F.L[2]);
+    const T rc2 = in_t<T>(P.rc2, F.rc2);
+    const T alpha = in_t<T>(P.alpha, F.alpha);
     const double alphas = Sg<LO>::scale * P.alpha;  // float64: the tables' argument
     const T two_over_sqrtpi = (T)1.12837916709551257390;
     const int m = P.m;
@@ -439,7 +439,7 @@ __device__ __forceinline__ void k_short_body(const ShortP& P, const SrTgt<T>* __
 // operation by operation (erfcx_2 equals erfcx_f).
 // Needs at least 2 (m + 2) cells per axis (no axis taken whole, the nearest
 // cell image is the minimum image of every candidate for both nodes).
-__device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>& ta, const SrTgt<float>& tb, int dx,
+__device__ __forceinline__ void k_short_pair(const ShortP& P, const ShortF& F, const SrTgt<float>& ta, const SrTgt<float>& tb, int dx,
                                              int dy, int dz, const int* __restrict__ prev,
                                              const int* __restrict__ start, const SrRec<float>* __restrict__ src,
                                              double* __restrict__ vsr, double* __restrict__ psr, int j,
@@ -452,9 +452,9 @@ __device__ __forceinline__ void k_short_pair(const ShortP& P, const SrTgt<float>
     const int cx = ta.cell % nc0;
     const int cy = (ta.cell / nc0) % nc1;
     const int cz = ta.cell / (nc0 * nc1);
-    const float h0 = P.hcf[0], h1 = P.hcf[1], h2 = P.hcf[2];
-    const float rc2 = P.rc2f;
-    const float alpha = P.alphaf;
+    const float h0 = F.hc[0], h1 = F.hc[1], h2 = F.hc[2];
+    const float rc2 = F.rc2;
+    const float alpha = F.alpha;
     const int m = P.m;
     const int ny = 2 * m + 1 + abs(dy), nz = 2 * m + 1 + abs(dz);
     const int y0 = min(dy, 0) - m, z0 = min(dz, 0) - m;  // first row offsets from the first node's cell
@@ -646,7 +646,7 @@ __host__ __device__ __forceinline__ bool short_pairs(const ShortP& P)
 // The two are separate kernels: in one of 91 registers the small grids, which
 // cannot pair, took 4 % longer over a batch.
 template <typename T, bool V>
-__device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __restrict__ tgt,
+__device__ __forceinline__ void k_short_warp(const ShortP& P, const ShortF& F, const SrTgt<T>* __restrict__ tgt,
                                              const int* __restrict__ prev, const int* __restrict__ start,
                                              const SrRec<T>* __restrict__ src, double* __restrict__ vsr,
                                              double* __restrict__ psr, int w, const double* __restrict__ tab,
@@ -664,13 +664,13 @@ __device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __
                 const int dy = cdiff((tb.cell / nc0) % nc1, (ta.cell / nc0) % nc1, nc1);
                 const int dz = cdiff(tb.cell / (nc0 * nc1), ta.cell / (nc0 * nc1), nc2);
                 if (abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1) {
-                    k_short_pair(P, ta, tb, dx, dy, dz, prev, start, src, vsr, psr, j, rows);
+                    k_short_pair(P, F, ta, tb, dx, dy, dz, prev, start, src, vsr, psr, j, rows);
                     return;
                 }
             }
         }
     }
-    for (; j < je && j < P.N; ++j) k_short_body<T, sizeof(T) == 8 && V>(P, tgt, prev, start, src, vsr, psr, j, tab, rows);
+    for (; j < je && j < P.N; ++j) k_short_body<T, sizeof(T) == 8 && V>(P, F, tgt, prev, start, src, vsr, psr, j, tab, rows);
 }
 
 // Four CTAs per SM in float32 (64 registers): with five (48) the one-node walk
@@ -678,7 +678,7 @@ __device__ __forceinline__ void k_short_warp(const ShortP& P, const SrTgt<T>* __
 // and 3.73 ms).  The batched form of that walk hides more latency with five
 // (256 members of 250 to 650 nodes: 1729 against 1750 us).
 template <typename T, bool V>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short(ShortP P, const SrTgt<T>* __restrict__ tgt, const int* __restrict__ prev,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short(ShortP P, ShortF F, const SrTgt<T>* __restrict__ tgt, const int* __restrict__ prev,
                                                const int* __restrict__ start, const SrRec<T>* __restrict__ src,
                                                double* __restrict__ vsr, double* __restrict__ psr)
 {
@@ -687,9 +687,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_short(ShortP P,
     const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if constexpr (sizeof(T) == 8) {  // several groups of nodes per CTA: the tables are staged once
         for (int b = blockIdx.x; b * nw < P.N; b += gridDim.x)
-            k_short_warp<T, V>(P, tgt, prev, start, src, vsr, psr, b * nw + wid, tab, rows);
+            k_short_warp<T, V>(P, F, tgt, prev, start, src, vsr, psr, b * nw + wid, tab, rows);
     } else {
-        k_short_warp<T, V>(P, tgt, prev, start, src, vsr, psr, blockIdx.x * kShortWarps + wid, tab, rows);
+        k_short_warp<T, V>(P, F, tgt, prev, start, src, vsr, psr, blockIdx.x * kShortWarps + wid, tab, rows);
     }
 }
 
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (V ? 4 : 5) : 3) k_short
     int bid, nb;
     const ShortD<T>& a = d[batch_member(bs, n, bid, nb)];
     const double* tab = sg_stage<T, V>(a.P.want_psi);
-    k_short_warp<T, V>(a.P, a.tgt, a.prev, a.start, a.src, a.vsr, a.psr,
+    k_short_warp<T, V>(a.P, a.F, a.tgt, a.prev, a.start, a.src, a.vsr, a.psr,
                           bid * kShortWarps + (int)(threadIdx.x >> 5), tab, rows);
 }
 
@@ -1079,15 +1079,16 @@ cudaError_t launch_short(const ShortP& P, const Work& w, cudaStream_t s)
             while (nw > 1 && P.N < 152 * nw) nw /= 2;
         const int tb = 32 * nw;
         const bool v = short_variant(P, sizeof(T) == 8 ? BS_FP64 : BS_MIXED);
+        const ShortF F = short_f(P);
         const long long blocks = sizeof(T) == 8 ? (P.N + nw - 1LL) / nw : short_blocks(P, v);
         // float64: at most 16 CTAs per SM, each on several groups of nodes
         const unsigned g = (unsigned)(sizeof(T) == 8 && blocks > 16 * 152 ? 16 * 152 : blocks);
         if (v)
             k_short<T, true><<<g, tb, sg_bytes<T, true>(P.want_psi), s>>>(
-                P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt, (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
+                P, F, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt, (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
         else
             k_short<T, false><<<g, tb, sg_bytes<T, false>(P.want_psi), s>>>(
-                P, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt, (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
+                P, F, (const SrTgt<T>*)w.tgt, w.prev, w.cell_cnt, (const SrRec<T>*)w.sr_sorted, w.vsr, w.psr);
         return cudaGetLastError();
     }
     // nodes by target block: count, scan, scatter
