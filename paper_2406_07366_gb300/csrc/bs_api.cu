@@ -378,12 +378,13 @@ int derive(const bs_params* p, Derived* d)
     const size_t mcy = 50000 / ((size_t)(d->ng[1] + 1) * cb);
     d->lmcy = 0;
     while (d->lmcy < 4 && ((size_t)2 << d->lmcy) <= mcy) ++d->lmcy;
-    // 17 to 24 modes: one chunk of 32 in place of a full one and one with 1 to 8
-    // modes.  Measured against two chunks of 16: batches of 128 members 1.29 ->
-    // 1.09 ms at 17 modes, 1.36 -> 1.15 at 21, 1.79 -> 1.54 at 24; single contexts
-    // 1 to 2 % faster.  From 25 to 32 modes batches would gain as much (2.63 -> 2.31
-    // ms at 32), but single contexts lose 1 %: the line is at 24.
-    if (d->lmcy == 4 && d->K[2] + 1 > 16 && d->K[2] + 1 <= 24 && 32 <= mcy) d->lmcy = 5;
+    // 17 to 24 modes (20 in float64): one chunk of 32 in place of a full one and one
+    // with 1 to 8 modes.  Measured against two chunks of 16: float32 batches of 128
+    // members 1.29 -> 1.09 ms at 17 modes, 1.36 -> 1.15 at 21, 1.79 -> 1.54 at 24;
+    // single contexts 1 to 2 % faster.  From 25 to 32 modes batches would gain as much
+    // (2.63 -> 2.31 ms at 32), but single contexts lose 1 %; in float64 they lose 3 %
+    // at 22 already (390 -> 400 us on 2560 nodes).
+    if (d->lmcy == 4 && d->K[2] + 1 > 16 && d->K[2] + 1 <= (rb == 4 ? 24 : 20) && 32 <= mcy) d->lmcy = 5;
     const int lines_x = (p->flags & BS_WANT_PSI) ? 6 : 3;
     // the x pass gets the same larger CTAs as the z-column blocks (two
     // 512-thread CTAs per SM; measured on the 384^3 grid: 0.29 ms against
